@@ -114,7 +114,7 @@ avq_status avq_assign(const avq_problem* prob, const void* K, const void* Cp, co
     return AVQ_ERR_ALIGN;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (use_tensor_path(*prob)) return tc_assign(*prob, K, Cp, Cc, parent_idx, child_idx, nullptr, nullptr, 0, nullptr, st);
-  return simt_assign(*prob, K, Cp, Cc, parent_idx, child_idx, st);
+  return simt_assign(*prob, K, Cp, Cc, parent_idx, child_idx, nullptr, 0, st);
 }
 
 avq_status avq_aggregate(const avq_problem* prob, const void* V, const int32_t* parent_idx,
@@ -129,7 +129,7 @@ avq_status avq_aggregate(const avq_problem* prob, const void* V, const int32_t* 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (use_tensor_path(*prob))
     return tc_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, nullptr, nullptr, nullptr, nullptr, false, nullptr, st);
-  return simt_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, st);
+  return simt_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, false, nullptr, st);
 }
 
 namespace {
@@ -163,7 +163,7 @@ avq_status attend_stage(const avq_problem& p, const Regions& r, const void* Q, c
   if (use_tensor_path(p))
     return tc_attend(p, Q, Cp, Cc, r.np_, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, P, Y, topp_out, importance_out, r.status_word,
                      chained, st);
-  return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, 0, st);
+  return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, 0, chained, st);
 }
 avq_status check_workspace(const avq_problem* prob, int32_t P, int32_t block_q, void* workspace,
                            size_t workspace_bytes, Layout* L) {
@@ -200,10 +200,9 @@ avq_status avq_forward(const avq_problem* prob, const void* Q, const void* K, co
     if (s != AVQ_OK) return s;
     s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, r.status_word, st);
   } else {
-    if (cudaMemsetAsync(r.status_word, 0, 256, st) != cudaSuccess) return AVQ_ERR_CUDA;
-    s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, st);
+    s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, workspace, L.zero_end, st);   // clears the accumulators on the side
     if (s != AVQ_OK) return s;
-    s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, st);
+    s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
   }
   if (s != AVQ_OK) return s;
   return attend_stage(p, r, Q, Cp, Cc, P, block_q, Y, topp_out, importance_out, true, st);
@@ -229,12 +228,11 @@ avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void*
   if (s != AVQ_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const Regions r = carve(workspace, L);
-  if (cudaMemsetAsync(r.status_word, 0, 256, st) != cudaSuccess) return AVQ_ERR_CUDA;
-  s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, st);
+  s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, workspace, L.zero_end, st);
   if (s != AVQ_OK) return s;
-  s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, st);
+  s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
   if (s != AVQ_OK) return s;
-  return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, st);
+  return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, true, st);
 }
 
 avq_status avq_attend(const avq_problem* prob, const void* Q, const void* Cp, const void* Cc, int32_t P,

@@ -43,16 +43,19 @@ Layout make_layout(const avq_problem& p, int32_t P, int32_t block_q);
 
 // ---- plain CUDA-core kernels (avq_simt.cu) ----
 avq_status simt_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
-                       int32_t* parent_idx, int32_t* child_idx, cudaStream_t st);
+                       int32_t* parent_idx, int32_t* child_idx, void* zero_base, size_t zero_bytes,
+                       cudaStream_t st);                 // zero_base / zero_bytes: as in tc_assign
 avq_status simt_aggregate(const avq_problem& p, const void* V, const int32_t* parent_idx,
                           const int32_t* child_idx, float* Vp, float* np_, float* Vc, float* nc,
-                          cudaStream_t st);
+                          bool pre_zeroed, int32_t* status_word,
+                          cudaStream_t st);              // pre_zeroed: launched right behind simt_assign
 avq_status simt_attend(const avq_problem& p, const void* Q, const void* Cp, const void* Cc,
                        const float* Vp, const float* np_, const float* Vc, const float* nc, int32_t P,
                        int32_t block_q, void* Y, int32_t* topp_out, float* importance_out,
-                       int32_t tile_m, cudaStream_t st);   // tile_m: 0 = exact importance
+                       int32_t tile_m, bool chained,
+                       cudaStream_t st);   // tile_m: 0 = exact importance; chained: right behind simt_aggregate
 
-// Shared memory the CUDA-core attention kernel needs for a problem, and the most it may ask for.
+// Size of the CUDA-core attention problem in the header's envelope formula, and its limit.
 size_t simt_attend_smem_bytes(int d, int M, int C, int P, int block_q, int tile_m);
 constexpr size_t kSimtAttendSmemLimit = 200 * 1024;
 

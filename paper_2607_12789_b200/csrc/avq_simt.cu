@@ -1,164 +1,309 @@
-// Plain CUDA-core (FFMA) kernels for the three stages of the AVQ-attention forward.
+// CUDA-core (FFMA) kernels for the three stages of the AVQ-attention forward.
 // They carry the float32 path (tensor-core inputs are 16-bit, too coarse for a 1e-4
 // output tolerance) and any shape outside the tensor-core envelope, for either dtype.
 //
-//   assign_simt_kernel     Algorithm 1, parent and child argmin, one thread per key
-//   aggregate_simt_kernel  Eq. "aggregates": value sums and counts, one warp per key
+//   assign_simt_kernel     Algorithm 1, parent and child argmin, a tile of 64 keys per CTA
+//   aggregate_simt_kernel  Eq. "aggregates": value sums and counts, one warp per 4 keys
 //   attend_simt_kernel     Algorithm 2 in its masked form: parent pass, Eq. "importance",
 //                          top-P, then one softmax over {unrefined parents} U {children of the
 //                          refined parents} with the maximum taken over non-empty codewords
+//
+// The products (distances, logits, weighted value sums) are register-tiled: both operands of a product are
+// staged in shared memory as [contraction index][row or column], a thread keeps an RT x 4 block of results and
+// reads RT + 4 operands per step with 16-byte loads.
 #include <cuda_bf16.h>
 #include <math.h>
 
 #include "avq_internal.h"
+#include "avq_tc_common.cuh"
 
 namespace avq {
 namespace {
+
+using tc::ld_after_wait;
 
 template <typename T> __device__ __forceinline__ float ldf(const T* p);
 template <> __device__ __forceinline__ float ldf<float>(const float* p) { return __ldg(p); }
 template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) {
   return __bfloat162float(*p);
 }
-template <typename T> __device__ __forceinline__ void stf(T* p, float v);
-template <> __device__ __forceinline__ void stf<float>(float* p, float v) { *p = v; }
-template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p, float v) {
-  *p = __float2bfloat16_rn(v);
+// four consecutive elements (d % 4 == 0 and 16-byte aligned bases: 16 bytes of float, 8 of bfloat16)
+__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xFFFF0000u));
+}
+__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16* p, const float4& v) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  uint2 u;
+  u.x = *reinterpret_cast<uint32_t*>(&lo);
+  u.y = *reinterpret_cast<uint32_t*>(&hi);
+  *reinterpret_cast<uint2*>(p) = u;
 }
 
-constexpr int kAssignKeys = 128;   // keys (= threads) per CTA
-constexpr int kAssignCodes = 16;   // parent codewords staged in shared memory at a time
+constexpr int kThreads = 256;      // 16 x 16: thread (ty, tx) owns rows ty*4 (+64), columns tx*4
+constexpr int kCols = 64;          // columns (codewords) of a tile
+constexpr int kLdC = kCols + 4;    // row pitch of a [k][column] operand, floats
+
+// Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r], k < d: the transposed
+// operand of the register-tiled products.  A warp takes 8 rows x 4 chunks of 4 elements: 64-byte pieces of a
+// row in global memory, at most two-way bank conflicts in shared memory.
+template <typename Src>
+__device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Src src) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int kc = lane & 3, rr = lane >> 2;
+  const int chunks = d >> 2, cblocks = (chunks + 3) >> 2;
+  for (int u = warp; u < (rows >> 3) * cblocks; u += kThreads / 32) {
+    const int rb = u / cblocks, cb = u - rb * cblocks;
+    const int r = rb * 8 + rr, c = cb * 4 + kc;
+    if (c < chunks) {
+      const auto* p = src(r);
+      const float4 v = p ? ld4(p + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float* o = dst + (size_t)(4 * c) * ld + r;
+      o[0] = v.x; o[ld] = v.y; o[2 * ld] = v.z; o[3 * ld] = v.w;
+    }
+  }
+}
+
+// acc[i][j] += sum_k A[k][row(i)] * B[k][tx*4 + j], k ascending (one accumulator per result: the sums do not
+// depend on the tiling)
+template <int RT>
+__device__ __forceinline__ void mul_tile(float (&acc)[RT][4], const float* A, int lda, const float* B, int ldb, int K,
+                                         int ty, int tx) {
+  const float* a_ = A + ty * 4;
+  const float* b_ = B + tx * 4;
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    float a[RT];
+    *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(a_ + k * lda);
+    if constexpr (RT == 8) *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(a_ + k * lda + 64);
+    const float4 b = *reinterpret_cast<const float4*>(b_ + k * ldb);
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      acc[i][0] = fmaf(a[i], b.x, acc[i][0]);
+      acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
+      acc[i][2] = fmaf(a[i], b.z, acc[i][2]);
+      acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
+    }
+  }
+}
+
 // Two distances closer than this (relative) are re-evaluated in float64.  The float32 direct
 // form carries about d * 2^-24 relative error, far below it.
 constexpr float kNearTie = 1e-4f;
 
 template <typename T>
-__device__ double exact_dist(const float* krow, const T* c, int d) {
+__device__ double exact_dist(const T* krow, const T* c, int d) {
   double s = 0.0;
   for (int k = 0; k < d; ++k) {
-    double t = (double)krow[k] - (double)ldf(c + k);
+    double t = (double)ldf(krow + k) - (double)ldf(c + k);
     s += t * t;
   }
   return s;
 }
 
 // ------------------------------------------------------------------------------- assign
+constexpr int kAssignKeys = 64;    // keys per CTA
+
+// Parents: 64 keys x 64 codewords at a time, squared differences in the direct form.  Children: four lanes per
+// key.  zero_base / zero_units: 16-byte words this grid clears on the side (the accumulators of the
+// aggregation behind it), each CTA an equal slice.
 template <typename T>
-__global__ void __launch_bounds__(kAssignKeys)
+__global__ void __launch_bounds__(kThreads)
 assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* __restrict__ Cc,
                    int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int d, int M,
-                   int C, int parent_stays) {
-  extern __shared__ float smem[];
-  const int ldk = d + 1;
-  float* ks = smem;                        // [kAssignKeys][d+1]
-  float* cs = smem + kAssignKeys * ldk;    // [kAssignCodes][d]
+                   int C, int parent_stays, uint4* __restrict__ zero_base, uint32_t zero_units) {
+  extern __shared__ __align__(16) float smem[];
+  float* ks = smem;                            // [d][kLdC] keys
+  float* cs = ks + (size_t)d * kLdC;           // [d][kLdC] codewords of the current tile
+  __shared__ int s_par[kAssignKeys];
+  __shared__ float s_d1[kAssignKeys];
+  __shared__ int s_redo[kAssignKeys];          // 1: parent decided in float64 (its exact distance in s_dp)
+  __shared__ double s_dp[kAssignKeys];
+  tc::pdl_launch_dependents();
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int bh = blockIdx.y, h = bh % H;
-  const int j0 = blockIdx.x * kAssignKeys, t = threadIdx.x, j = j0 + t;
-  const int rows = min(kAssignKeys, Nk - j0);
+  const int j0 = blockIdx.x * kAssignKeys;
+  if (zero_units) {
+    const uint32_t ncta = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
+    const uint32_t per = (zero_units + ncta - 1) / ncta;
+    const uint32_t u0 = cta * per, u1 = min(zero_units, u0 + per);
+    for (uint32_t u = u0 + tid; u < u1; u += kThreads) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
+  }
   const T* Kb = K + ((size_t)bh * Nk + j0) * d;
-  for (int e = t; e < rows * d; e += kAssignKeys) ks[(e / d) * ldk + (e % d)] = ldf(Kb + e);
-  const float* kr = ks + t * ldk;
+  const int rows = min(kAssignKeys, Nk - j0);
   const T* Cph = Cp + (size_t)h * M * d;
+  load_transposed(ks, kLdC, kAssignKeys, d, [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; });
 
-  float d1 = INFINITY, d2 = INFINITY;
-  int i1 = 0;
-  for (int m0 = 0; m0 < M; m0 += kAssignCodes) {
-    const int mc = min(kAssignCodes, M - m0);
+  float d1[4], d2[4];
+  int i1[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { d1[i] = INFINITY; d2[i] = INFINITY; i1[i] = 0; }
+  for (int m0 = 0; m0 < M; m0 += kCols) {
+    const int w = min(kCols, M - m0);
     __syncthreads();
-    for (int e = t; e < mc * d; e += kAssignKeys) cs[e] = ldf(Cph + (size_t)m0 * d + e);
+    load_transposed(cs, kLdC, kCols, d, [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; });
     __syncthreads();
-    if (j < Nk) {
-      for (int mm = 0; mm < mc; ++mm) {
-        const float* c = cs + mm * d;
-        float s = 0.f;
-        for (int k = 0; k < d; ++k) {
-          float df = kr[k] - c[k];
-          s = fmaf(df, df, s);
+    float acc[4][4] = {};
+#pragma unroll 4
+    for (int k = 0; k < d; ++k) {
+      const float4 a4 = *reinterpret_cast<const float4*>(ks + k * kLdC + ty * 4);
+      const float4 b4 = *reinterpret_cast<const float4*>(cs + k * kLdC + tx * 4);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float df = a[i] - b[j];
+          acc[i][j] = fmaf(df, df, acc[i][j]);
         }
-        if (s < d1) { d2 = d1; d1 = s; i1 = m0 + mm; }
-        else if (s < d2) { d2 = s; }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (tx * 4 + j < w) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float s = acc[i][j];
+          if (s < d1[i]) { d2[i] = d1[i]; d1[i] = s; i1[i] = m0 + tx * 4 + j; }
+          else if (s < d2[i]) { d2[i] = s; }
+        }
       }
-    }
   }
-  if (j >= Nk) return;
-
-  double dp64 = -1.0;   // exact parent distance, if it had to be computed
-  if (M > 1 && !(d2 - d1 > kNearTie * d2)) {
+  // ---- merge the 16 threads of a key (the lower index wins a tie); near-ties are redone in float64 by them
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const float b1 = __shfl_xor_sync(0xffffffffu, d1[i], o), b2 = __shfl_xor_sync(0xffffffffu, d2[i], o);
+      const int bi = __shfl_xor_sync(0xffffffffu, i1[i], o);
+      d2[i] = fminf(fmaxf(d1[i], b1), fminf(d2[i], b2));
+      if (b1 < d1[i] || (b1 == d1[i] && bi < i1[i])) { d1[i] = b1; i1[i] = bi; }
+    }
+    const int key = ty * 4 + i;
+    const bool redo = M > 1 && key < rows && !(d2[i] - d1[i] > kNearTie * d2[i]);
     double best = INFINITY;
-    int bi = 0;
-    for (int m = 0; m < M; ++m) {
-      double s = exact_dist(kr, Cph + (size_t)m * d, d);
-      if (s < best) { best = s; bi = m; }
+    if (__any_sync(0xffffffffu, redo)) {
+      int bi = 0x7fffffff;
+      if (redo)
+        for (int m = tx; m < M; m += 16) {
+          const double s = exact_dist(Kb + (size_t)key * d, Cph + (size_t)m * d, d);
+          if (s < best) { best = s; bi = m; }
+        }
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      }
+      if (redo) { i1[i] = bi < M ? bi : 0; d1[i] = (float)best; }
     }
-    i1 = bi;
-    dp64 = best;
-    d1 = (float)best;
+    if (tx == 0) {
+      s_par[key] = i1[i];
+      s_d1[key] = d1[i];
+      s_redo[key] = redo ? 1 : 0;
+      s_dp[key] = best;
+    }
   }
+  __syncthreads();
 
-  const T* Cch = Cc + ((size_t)h * M + i1) * C * d;
+  // ---- children of the key's parent: four lanes per key, each over every fourth 4-element chunk
+  const int key = tid >> 2, s4 = tid & 3;
+  const int par = s_par[key];
+  const T* Cch = Cc + ((size_t)h * M + par) * C * d;
   float e1 = INFINITY, e2 = INFINITY;
   int c1 = 0;
   for (int c = 0; c < C; ++c) {
-    const T* cc = Cch + (size_t)c * d;
     float s = 0.f;
-    for (int k = 0; k < d; ++k) {
-      float df = kr[k] - ldf(cc + k);
-      s = fmaf(df, df, s);
+    for (int ch = s4; ch < (d >> 2); ch += 4) {
+      const float4 v = ld4(Cch + (size_t)c * d + 4 * ch);
+      const float* kp = ks + (size_t)(4 * ch) * kLdC + key;
+      const float x0 = kp[0] - v.x, x1 = kp[kLdC] - v.y, x2 = kp[2 * kLdC] - v.z, x3 = kp[3 * kLdC] - v.w;
+      s = fmaf(x0, x0, s); s = fmaf(x1, x1, s); s = fmaf(x2, x2, s); s = fmaf(x3, x3, s);
     }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
     if (s < e1) { e2 = e1; e1 = s; c1 = c; }
     else if (s < e2) { e2 = s; }
   }
   double dc64 = -1.0;
-  if (C > 1 && !(e2 - e1 > kNearTie * e2)) {
+  const bool redo = C > 1 && key < rows && !(e2 - e1 > kNearTie * e2);
+  if (__any_sync(0xffffffffu, redo)) {
     double best = INFINITY;
-    int bi = 0;
-    for (int c = 0; c < C; ++c) {
-      double s = exact_dist(kr, Cch + (size_t)c * d, d);
-      if (s < best) { best = s; bi = c; }
+    int bi = 0x7fffffff;
+    if (redo)
+      for (int c = s4; c < C; c += 4) {
+        const double s = exact_dist(Kb + (size_t)key * d, Cch + (size_t)c * d, d);
+        if (s < best) { best = s; bi = c; }
+      }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
     }
-    c1 = bi;
-    dc64 = best;
-    e1 = (float)best;
+    if (redo) { c1 = bi < C ? bi : 0; dc64 = best; e1 = (float)best; }
   }
-  if (parent_stays) {
-    bool moved = e1 < d1;
-    float hi = fmaxf(e1, d1);
-    if (!(fabsf(e1 - d1) > kNearTie * hi)) {
-      if (dp64 < 0.0) dp64 = exact_dist(kr, Cph + (size_t)i1 * d, d);
-      if (dc64 < 0.0) dc64 = exact_dist(kr, Cch + (size_t)c1 * d, d);
-      moved = dc64 < dp64;
+  if (s4 == 0 && key < rows) {
+    if (parent_stays) {
+      const float d1k = s_d1[key];
+      bool moved = e1 < d1k;
+      if (!(fabsf(e1 - d1k) > kNearTie * fmaxf(e1, d1k))) {
+        const double dp64 = s_redo[key] ? s_dp[key] : exact_dist(Kb + (size_t)key * d, Cph + (size_t)par * d, d);
+        if (dc64 < 0.0) dc64 = exact_dist(Kb + (size_t)key * d, Cch + (size_t)c1 * d, d);
+        moved = dc64 < dp64;
+      }
+      if (!moved) c1 = -1;
     }
-    if (!moved) c1 = -1;
+    pidx[(size_t)bh * Nk + j0 + key] = par;
+    cidx[(size_t)bh * Nk + j0 + key] = c1;
   }
-  pidx[(size_t)bh * Nk + j] = i1;
-  cidx[(size_t)bh * Nk + j] = c1;
 }
 
 // ------------------------------------------------------------------------------- aggregate
+constexpr int kAggKeysPerWarp = 4;
+
+// One warp = 4 keys: lane l adds elements 4l.. of each value row to the parent's and the child's sums with
+// 16-byte reductions.  The value rows are the caller's, so they are loaded before the dependency wait.
 template <typename T>
-__global__ void __launch_bounds__(256)
-aggregate_simt_kernel(const T* __restrict__ V, const int32_t* __restrict__ pidx,
-                      const int32_t* __restrict__ cidx, float* __restrict__ Vp, float* __restrict__ np_,
-                      float* __restrict__ Vc, float* __restrict__ nc, int Nk, int d, int M, int C,
-                      int keys_per_cta) {
+__global__ void __launch_bounds__(kThreads)
+aggregate_simt_kernel(const T* __restrict__ V, const int32_t* pidx, const int32_t* cidx, float* Vp, float* np_,
+                      float* Vc, float* nc, int Nk, int d, int M, int C, int32_t* status_word) {
+  tc::pdl_launch_dependents();
   const int bh = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int j0 = blockIdx.x * keys_per_cta;
-  const int j1 = min(Nk, j0 + keys_per_cta);
-  for (int j = j0 + warp; j < j1; j += nwarps) {
-    const int a = pidx[(size_t)bh * Nk + j];
-    const int c = cidx[(size_t)bh * Nk + j];
-    const T* v = V + ((size_t)bh * Nk + j) * d;
-    float* vp = Vp + ((size_t)bh * M + a) * d;
-    float* vc = (c >= 0) ? Vc + (((size_t)bh * M + a) * C + c) * d : nullptr;
-    for (int k = lane; k < d; k += 32) {
-      float x = ldf(v + k);
-      atomicAdd(vp + k, x);
-      if (vc) atomicAdd(vc + k, x);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j0 = (blockIdx.x * (kThreads / 32) + warp) * kAggKeysPerWarp;
+  const int chunks = d >> 2;                              // <= 64: two per lane
+  float4 v[kAggKeysPerWarp][2];
+#pragma unroll
+  for (int t = 0; t < kAggKeysPerWarp; ++t)
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (j0 + t < Nk && lane + 32 * u < chunks) v[t][u] = ld4(V + ((size_t)bh * Nk + j0 + t) * d + 4 * (lane + 32 * u));
+  tc::pdl_wait();
+#pragma unroll
+  for (int t = 0; t < kAggKeysPerWarp; ++t) {
+    const int j = j0 + t;
+    if (j >= Nk) break;
+    const int a = ld_after_wait(pidx + (size_t)bh * Nk + j);
+    const int c = ld_after_wait(cidx + (size_t)bh * Nk + j);
+    if (a < 0 || a >= M || c < -1 || c >= C) {            // caller-supplied index out of range: skip the key, flag it
+      if (lane == 0 && status_word) atomicCAS(status_word, 0, DEV_BAD_INDEX);
+      continue;
+    }
+    const size_t prow = (size_t)bh * M + a, crow = prow * C + c;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int ch = lane + 32 * u;
+      if (ch < chunks) {
+        atomicAdd(reinterpret_cast<float4*>(Vp + prow * d) + ch, v[t][u]);
+        if (c >= 0) atomicAdd(reinterpret_cast<float4*>(Vc + crow * d) + ch, v[t][u]);
+      }
     }
     if (lane == 0) {
-      atomicAdd(np_ + (size_t)bh * M + a, 1.0f);
-      if (c >= 0) atomicAdd(nc + ((size_t)bh * M + a) * C + c, 1.0f);
+      atomicAdd(np_ + prow, 1.0f);
+      if (c >= 0) atomicAdd(nc + crow, 1.0f);
     }
   }
 }
@@ -174,52 +319,86 @@ struct AttendArgs {
   int correcting; // Algorithm 2's literal child pass: mean-recovered parent logit and Delta A = A_c - A_p
   int tile_m;     // 0: exact importance; else parents visited in tiles of tile_m (Eq. "aproxdenom")
   int Nk;
+  int keep;       // the block's parent logits stay in shared memory between the passes
   float scale;
 };
 
-template <typename T>
-__device__ __forceinline__ float logit(const float* q, const T* c, int d, float scale) {
-  float s = 0.f;
-  for (int k = 0; k < d; ++k) s = fmaf(q[k], ldf(c + k), s);
-  return s * scale;
+// Shared memory of attend_simt_kernel, in floats from the base (doubles first).
+struct AttendSmem {
+  int ldr;                                   // pitch of a [k][row] operand
+  size_t w, wpart, q, c, v, s, rm, rz, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
+};
+// RT = 8: 128 query rows at a time (d <= 128), RT = 4: 64 rows.  v == c where the two tiles share one buffer.
+__host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int block_q, int tile_m,
+                                                         int keep) {
+  AttendSmem L;
+  L.ldr = 16 * RT + 4;
+  const int ntiles = tile_m > 0 ? (M + tile_m - 1) / tile_m : 0;
+  size_t o = 0;
+  auto take = [&](size_t n) { size_t at = o; o += (n + 3) / 4 * 4; return at; };
+  L.w = take(2 * (size_t)M);
+  L.wpart = take(2 * (size_t)(kThreads / 32) * kCols);
+  L.q = take((size_t)d * L.ldr);
+  if (DT <= 2) {
+    L.c = take((size_t)d * kLdC);
+    L.v = take((size_t)kCols * DT * 64);
+  } else {
+    const size_t a = (size_t)d * kLdC, b = (size_t)kCols * DT * 64;
+    L.c = L.v = take(a > b ? a : b);
+  }
+  L.s = take((size_t)(keep ? (M + kCols - 1) / kCols * kCols : kCols) * L.ldr);
+  L.rm = take(block_q);
+  L.rz = take(block_q);
+  L.np = take(M);
+  L.nstay = take(M);
+  L.zt = take((size_t)block_q * ntiles);
+  L.nseen = take(ntiles);
+  L.sel = take(M);
+  L.list = take(P > 0 ? P : 1);
+  L.total = o;
+  return L;
 }
 
-__device__ __forceinline__ float warp_max(float v) {
-  for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+__device__ __forceinline__ float max16(float v) {         // over the 16 threads of a row
+#pragma unroll
+  for (int o = 8; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+__device__ __forceinline__ float sum16(float v) {
+#pragma unroll
+  for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-constexpr int kAttendThreads = 256;
-constexpr int kMaxDPerLane = 8;   // d <= 256
-
-template <typename T>
-__global__ void __launch_bounds__(kAttendThreads) attend_simt_kernel(AttendArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+// One CTA = one query block.  Passes over the parents in tiles of 64 codewords:
+//   A  logits, row maximum over non-empty parents and denominator (running maximum)
+//   B  importance: column sums of A_ij / z_i in float64
+//   C  softmax over unrefined parents and the children of the refined ones, weights through shared memory
+//      into the value product (running maximum, register accumulators rescaled)
+// Where the block's logits fit (a.keep) they are computed once and reused by B and C.  Bound: FFMA issue and
+// the shared-memory pipe (RT + 4 operands per 4 RT products).  Against one warp per query row with a lane per
+// logit, operands read from global memory for every product: whole forward fp32 B2 H12 N1024 d64 M64 C4 P8
+// 2660 -> 84 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.40 ms.
+template <typename T, int RT, int DT>
+__global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kernel(const AttendArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int R = 16 * RT;
   const int d = a.d, M = a.M, C = a.C, P = a.P;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = kAttendThreads / 32;
+  const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.block_q, a.tile_m, a.keep);
+  const int ldr = L.ldr;
+  double* w = reinterpret_cast<double*>(sm + L.w);
+  double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [8][64]
+  float *qs = sm + L.q, *cs = sm + L.c, *vs = sm + L.v, *ss = sm + L.s, *rm = sm + L.rm, *rz = sm + L.rz;
+  float *npS = sm + L.np, *nstay = sm + L.nstay, *zt = sm + L.zt, *nseen = sm + L.nseen;
+  int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
+  constexpr int ldv = DT * 64;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = tid & 15, ty = tid >> 4;
   const int blk = blockIdx.x, bh = blockIdx.y, h = bh % a.H;
   const int i0 = blk * a.block_q;
   const int rows = min(a.block_q, a.Nq - i0);
-  const int ncols = M + P * C;
-
-  // shared memory carve-up (doubles first for alignment)
-  double* w = reinterpret_cast<double*>(smem_raw);                 // [M]
-  float* qs = reinterpret_cast<float*>(w + M);                     // [block_q][d]
-  float* rm = qs + (size_t)a.block_q * d;                          // [block_q]
-  float* rz = rm + a.block_q;                                      // [block_q]
-  float* npS = rz + a.block_q;                                     // [M]
-  float* nstay = npS + M;                                          // [M]
-  float* sbuf = nstay + M;                                         // [nwarps][ncols]
-  int* sel = reinterpret_cast<int*>(sbuf + (size_t)nwarps * ncols);   // [M]
-  int* sel_list = sel + M;                                         // [max(P,1)]
+  const int nrt = (rows + R - 1) / R;
   const int ntiles = a.tile_m > 0 ? (M + a.tile_m - 1) / a.tile_m : 0;
-  float* zt = reinterpret_cast<float*>(sel_list + (P > 0 ? P : 1));   // [block_q][ntiles] denominators seen up to a tile
-  float* nseen = zt + (size_t)a.block_q * ntiles;                  // [ntiles] keys of the tiles seen up to a tile
-
   const T* Qb = static_cast<const T*>(a.Q) + ((size_t)bh * a.Nq + i0) * d;
   const T* Cph = static_cast<const T*>(a.Cp) + (size_t)h * M * d;
   const T* Cch = static_cast<const T*>(a.Cc) + (size_t)h * M * C * d;
@@ -228,174 +407,355 @@ __global__ void __launch_bounds__(kAttendThreads) attend_simt_kernel(AttendArgs 
   const float* np_ = a.np_ + (size_t)bh * M;
   const float* nc = a.nc + (size_t)bh * M * C;
 
-  for (int e = tid; e < rows * d; e += kAttendThreads) qs[e] = ldf(Qb + e);
-  for (int j = tid; j < M; j += kAttendThreads) {
-    float n = np_[j], s = 0.f;
-    for (int c = 0; c < C; ++c) s += nc[j * C + c];
+  auto row_of = [&](int i) { return (i < 4 ? 0 : 64) + ty * 4 + (i & 3); };
+  auto load_q = [&](int rt) {
+    load_transposed(qs, ldr, R, d, [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; });
+  };
+  // Logits of this thread's RT x 4 block of a tile of n columns (row c of the tile at code(c)).  Ends with the
+  // operands still being read by other threads: the caller synchronises before they are overwritten.
+  auto logits = [&](float (&acc)[RT][4], int n, auto code) {
+    load_transposed(cs, kLdC, kCols, d, [&](int c) { return c < n ? code(c) : (const T*)nullptr; });
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    mul_tile<RT>(acc, qs, ldr, cs, kLdC, d, ty, tx);
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] *= a.scale;
+  };
+  auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * 4;
+      *reinterpret_cast<float4*>(o) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+      if constexpr (RT == 8) *reinterpret_cast<float4*>(o + 64) = make_float4(acc[4][j], acc[5][j], acc[6][j], acc[7][j]);
+    }
+  };
+  auto load_s = [&](const float* s0, float (&acc)[RT][4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * 4;
+      const float4 x = *reinterpret_cast<const float4*>(o);
+      acc[0][j] = x.x; acc[1][j] = x.y; acc[2][j] = x.z; acc[3][j] = x.w;
+      if constexpr (RT == 8) {
+        const float4 y = *reinterpret_cast<const float4*>(o + 64);
+        acc[4][j] = y.x; acc[5][j] = y.y; acc[6][j] = y.z; acc[7][j] = y.w;
+      }
+    }
+  };
+
+  load_q(0);                                              // the caller's Q: before the dependency wait
+  tc::pdl_wait();
+  for (int j = tid; j < M; j += kThreads) {
+    const float n = ld_after_wait(np_ + j);
+    float s = 0.f;
+    for (int c = 0; c < C; ++c) s += ld_after_wait(nc + (size_t)j * C + c);
     npS[j] = n;
     nstay[j] = n - s;
+    w[j] = 0.0;
+    sel[j] = 0;
   }
   __syncthreads();
-
-  // ---- parent pass: row maximum over non-empty parents and z_i = sum_j A_ij n_j
-  float* sb = sbuf + (size_t)warp * ncols;
-  for (int i = warp; i < rows; i += nwarps) {
-    float mx = -INFINITY;
-    for (int j = lane; j < M; j += 32) {
-      float s = logit(qs + (size_t)i * d, Cph + (size_t)j * d, d, a.scale);
-      sb[j] = s;
-      if (npS[j] > 0.f) mx = fmaxf(mx, s);
-    }
-    mx = warp_max(mx);
-    float z = 0.f;
-    for (int j = lane; j < M; j += 32)
-      if (npS[j] > 0.f) z += expf(sb[j] - mx) * npS[j];
-    z = warp_sum(z);
-    if (lane == 0) { rm[i] = mx; rz[i] = z; }
-    // tiled importance: the part of the denominator contributed by the tiles visited so far
-    float prefix = 0.f;
-    for (int t = 0; t < ntiles; ++t) {
-      float zp = 0.f;
-      const int j1 = min(M, (t + 1) * a.tile_m);
-      for (int j = t * a.tile_m + lane; j < j1; j += 32)
-        if (npS[j] > 0.f) zp += expf(sb[j] - mx) * npS[j];
-      prefix += warp_sum(zp);
-      if (lane == 0) zt[(size_t)i * ntiles + t] = prefix;
-    }
-  }
-  if (tid == 0) {
+  if (tid < ntiles) {                                     // keys of each tile; turned into prefix sums after pass A
     float seen = 0.f;
-    for (int t = 0; t < ntiles; ++t) {
-      const int j1 = min(M, (t + 1) * a.tile_m);
-      for (int j = t * a.tile_m; j < j1; ++j) seen += npS[j];
-      nseen[t] = seen;
-    }
+    const int j1 = min(M, (tid + 1) * a.tile_m);
+    for (int j = tid * a.tile_m; j < j1; ++j) seen += npS[j];
+    nseen[tid] = seen;
   }
-  __syncthreads();
-
-  // ---- importance w_j = n_j * sum_i exp(s_ij - m_i) / z_i, fixed summation order, float64 sum
-  for (int j = tid; j < M; j += kAttendThreads) {
-    double acc = 0.0;
-    if (npS[j] > 0.f) {
-      // exact: the row's full denominator.  Tiled (appendix "Computing Importance with Tiled Codewords"):
-      // the denominator seen up to this codeword's tile, extrapolated by N / N_seen (Eq. "aproxdenom").
-      const int t = ntiles ? j / a.tile_m : 0;
-      for (int i = 0; i < rows; ++i) {
-        float s = logit(qs + (size_t)i * d, Cph + (size_t)j * d, d, a.scale);
-        acc += (double)expf(s - rm[i]) / (double)(ntiles ? zt[(size_t)i * ntiles + t] : rz[i]);
+  // the choice of parents needs the importances only if there is one to make
+  const bool need_w = (P > 0 && P < M) || a.importance_out != nullptr;
+  // width of the parent tile that starts at c0: it ends where a tile of the tiled importance ends
+  auto width_at = [&](int c0) {
+    int n = min(kCols, M - c0);
+    if (ntiles) n = min(n, (c0 / a.tile_m + 1) * a.tile_m - c0);
+    return n;
+  };
+  // with a.keep the tiles start at multiples of 64 (validated by the launcher), so S is [M][rows]
+  for (int rt = 0; rt < nrt && need_w; ++rt) {
+    if (rt > 0) { __syncthreads(); load_q(rt); }
+    // ---- pass A
+    float m[RT], z[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) { m[i] = -INFINITY; z[i] = 0.f; }
+    for (int c0 = 0; c0 < M;) {
+      const int n = width_at(c0);
+      float acc[RT][4];
+      logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+      if (a.keep) store_s(ss + (size_t)c0 * ldr, acc);
+      float cnt[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cnt[j] = tx * 4 + j < n ? npS[c0 + tx * 4 + j] : 0.f;
+      const int t = ntiles ? c0 / a.tile_m : 0;
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
+        mx = max16(mx);
+        if (mx > m[i]) {                                  // uniform over the 16 threads of the row
+          const float alpha = expf(m[i] - mx);
+          z[i] *= alpha;
+          if (tx == 0)                                    // denominators already recorded follow the reference
+            for (int u = 0; u < t; ++u) if (rt * R + row_of(i) < rows) zt[(size_t)(rt * R + row_of(i)) * ntiles + u] *= alpha;
+          m[i] = mx;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) z[i] = fmaf(expf(acc[i][j] - m[i]), cnt[j], z[i]);
+        if (ntiles && (c0 + n == M || (c0 + n) % a.tile_m == 0)) {
+          const float zp = sum16(z[i]);
+          if (tx == 0 && rt * R + row_of(i) < rows) zt[(size_t)(rt * R + row_of(i)) * ntiles + t] = zp;
+        }
       }
-      acc *= (double)npS[j];
-      if (ntiles) acc *= (double)nseen[t] / (double)a.Nk;
+      c0 += n;
+      __syncthreads();
     }
-    w[j] = acc;
+    double inv[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      const float zi = sum16(z[i]);
+      inv[i] = (!ntiles && rt * R + row_of(i) < rows) ? 1.0 / (double)zi : 0.0;
+    }
+    // ---- pass B
+    int t_inv = -1;
+    for (int c0 = 0; c0 < M;) {
+      const int n = width_at(c0);
+      float acc[RT][4];
+      if (a.keep) load_s(ss + (size_t)c0 * ldr, acc);
+      else logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+      if (ntiles && c0 / a.tile_m != t_inv) {
+        // exact: the row's full denominator.  Tiled (appendix "Computing Importance with Tiled Codewords"):
+        // the denominator seen up to this codeword's tile (Eq. "aproxdenom").
+        t_inv = c0 / a.tile_m;
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+          inv[i] = rt * R + row_of(i) < rows ? 1.0 / (double)zt[(size_t)(rt * R + row_of(i)) * ntiles + t_inv] : 0.0;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        double s = 0.0;
+        if (tx * 4 + j < n && npS[c0 + tx * 4 + j] > 0.f) {
+#pragma unroll
+          for (int i = 0; i < RT; ++i)
+            if (rt * R + row_of(i) < rows) s = fma((double)expf(acc[i][j] - m[i]), inv[i], s);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (lane < 16) wpart[warp * kCols + tx * 4 + j] = s;
+      }
+      __syncthreads();
+      if (tid < n) {
+        double s = 0.0;
+#pragma unroll
+        for (int u = 0; u < kThreads / 32; ++u) s += wpart[u * kCols + tid];
+        w[c0 + tid] += s;
+      }
+      c0 += n;
+      __syncthreads();
+    }
+  }
+  if (need_w) {
+    for (int j = tid; j < M; j += kThreads) {
+      double x = w[j] * (double)npS[j];
+      if (ntiles) {                                       // extrapolated by the keys seen up to the tile
+        float seen = 0.f;
+        for (int t = 0; t <= j / a.tile_m; ++t) seen += nseen[t];
+        x *= (double)seen / (double)a.Nk;
+      }
+      w[j] = x;
+      if (a.importance_out) a.importance_out[((size_t)bh * a.nblk + blk) * M + j] = (float)x;
+    }
   }
   __syncthreads();
-  if (a.importance_out) {
-    float* io = a.importance_out + ((size_t)bh * a.nblk + blk) * M;
-    for (int j = tid; j < M; j += kAttendThreads) io[j] = (float)w[j];
+
+  // ---- top-P by rank (ties -> lower index), then an ascending list.  Non-negative doubles order like their
+  // bit patterns.
+  if (P > 0) {
+    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(w);
+    for (int j = tid; j < M; j += kThreads) {
+      int rank = 0;
+      if (P < M) {
+        const unsigned long long kj = key[j];
+        for (int k = 0; k < j; ++k) rank += key[k] >= kj;
+        for (int k = j + 1; k < M; ++k) rank += key[k] > kj;
+      }
+      sel[j] = rank < P;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int base = 0;
+      for (int j = lane; j < ((M + 31) & ~31); j += 32) {
+        const bool on = j < M && sel[j] != 0;
+        const uint32_t bal = __ballot_sync(0xffffffffu, on);
+        if (on) sel_list[base + __popc(bal & ((1u << lane) - 1u))] = j;
+        base += __popc(bal);
+      }
+    }
+    __syncthreads();
+    if (a.topp_out) {
+      int32_t* to = a.topp_out + ((size_t)bh * a.nblk + blk) * P;
+      for (int r = tid; r < P; r += kThreads) to[r] = sel_list[r];
+    }
   }
 
-  // ---- top-P by rank (ties -> lower index), then an ascending list
-  for (int j = tid; j < M; j += kAttendThreads) {
-    int rank = 0;
-    const double wj = w[j];
-    for (int k = 0; k < M; ++k) {
-      const double wk = w[k];
-      rank += (wk > wj) || (wk == wj && k < j);
-    }
-    sel[j] = rank < P;
-  }
-  __syncthreads();
-  for (int j = tid; j < M; j += kAttendThreads) {
-    if (sel[j]) {
-      int pos = 0;
-      for (int k = 0; k < j; ++k) pos += sel[k];
-      sel_list[pos] = j;
-    }
-  }
-  __syncthreads();
-  if (a.topp_out) {
-    int32_t* to = a.topp_out + ((size_t)bh * a.nblk + blk) * P;
-    for (int r = tid; r < P; r += kAttendThreads) to[r] = sel_list[r];
-  }
-
-  // ---- merged softmax over unrefined parents, stay residuals and children of refined parents
+  // ---- pass C: merged softmax over unrefined parents, stay residuals and children of refined parents
   T* Yb = static_cast<T*>(a.Y) + ((size_t)bh * a.Nq + i0) * d;
-  for (int i = warp; i < rows; i += nwarps) {
-    const float* q = qs + (size_t)i * d;
-    float mx = -INFINITY;
-    for (int j = lane; j < M; j += 32) {
-      float s = logit(q, Cph + (size_t)j * d, d, a.scale);
-      sb[j] = s;
-      const float cnt = (sel[j] && !a.correcting) ? (a.stays ? nstay[j] : 0.f) : npS[j];
-      if (cnt > 0.f) mx = fmaxf(mx, s);
-    }
-    for (int e = lane; e < P * C; e += 32) {
-      const int p = sel_list[e / C], c = e % C;
-      float s = logit(q, Cch + ((size_t)p * C + c) * d, d, a.scale);
-      sb[M + e] = s;
-      if (nc[p * C + c] > 0.f) mx = fmaxf(mx, s);
-    }
-    mx = warp_max(mx);
-    __syncwarp();
-    float x[kMaxDPerLane];
+  const int child_w = (kCols / C) * C;                    // whole families per tile
+  const int vch = d >> 2;
+  for (int rt = 0; rt < nrt; ++rt) {
+    if (rt > 0 || (nrt > 1 && need_w)) { __syncthreads(); load_q(rt); }
+    float m[RT], z[RT], o[DT][RT][4];
 #pragma unroll
-    for (int u = 0; u < kMaxDPerLane; ++u) x[u] = 0.f;
-    float z = 0.f;
-    for (int j = 0; j < M; ++j) {
-      // correcting form: every parent keeps its full term here, the children add differences below
-      const bool s_ = sel[j] != 0 && !a.correcting;
-      const float cnt = s_ ? (a.stays ? nstay[j] : 0.f) : npS[j];
-      if (!(cnt > 0.f)) continue;
-      const float av = expf(sb[j] - mx);
-      z += av * cnt;
+    for (int i = 0; i < RT; ++i) {
+      m[i] = -INFINITY; z[i] = 0.f;
 #pragma unroll
-      for (int u = 0; u < kMaxDPerLane; ++u) {
-        const int k = lane + 32 * u;
-        if (k < d) {
-          float v = Vp[(size_t)j * d + k];
-          if (s_)
-            for (int c = 0; c < C; ++c) v -= Vc[((size_t)j * C + c) * d + k];
-          x[u] = fmaf(av, v, x[u]);
+      for (int t = 0; t < DT; ++t)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o[t][i][j] = 0.f;
+    }
+    // value rows of a tile (padding rows and columns zero): vs[c][k]
+    auto load_v = [&](auto val) {
+      for (int u = tid; u < kCols * (ldv / 4); u += kThreads) {
+        const int c = u / (ldv / 4), ch = u - c * (ldv / 4);
+        *reinterpret_cast<float4*>(vs + c * ldv + 4 * ch) = ch < vch ? val(c, ch) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    const int ptiles = (M + kCols - 1) / kCols;
+    const int ctiles = P > 0 ? (P * C + child_w - 1) / child_w : 0;
+    for (int tt = 0; tt < ptiles + ctiles; ++tt) {
+      const bool child = tt >= ptiles;
+      const int c0 = child ? (tt - ptiles) * child_w : tt * kCols;
+      const int n = child ? min(child_w, P * C - c0) : min(kCols, M - c0);
+      float acc[RT][4], cnt[4];
+      float* sw = ss;                                     // weights of this tile, [column][row]
+      auto val_parent = [&](int c, int ch) {
+        const int j = c0 + c;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < n) {
+          const bool refined = sel[j] != 0 && !a.correcting;
+          const float nn = refined ? (a.stays ? nstay[j] : 0.f) : npS[j];
+          if (nn > 0.f) {
+            v = ld_after_wait(reinterpret_cast<const float4*>(Vp + (size_t)j * d) + ch);
+            if (refined)
+              for (int cc = 0; cc < C; ++cc) {
+                const float4 x = ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)j * C + cc) * d) + ch);
+                v.x -= x.x; v.y -= x.y; v.z -= x.z; v.w -= x.w;
+              }
+          }
+        }
+        return v;
+      };
+      auto val_child = [&](int c, int ch) {
+        if (c >= n) return make_float4(0.f, 0.f, 0.f, 0.f);
+        const int e = c0 + c, p = sel_list[e / C];
+        return ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)p * C + e % C) * d) + ch);
+      };
+      if (DT <= 2) {                                      // its own buffer: loads fly together with the codewords'
+        if (child) load_v(val_child);
+        else load_v(val_parent);
+      }
+      if (child) {
+        logits(acc, n, [&](int c) { const int e = c0 + c; return Cch + ((size_t)sel_list[e / C] * C + e % C) * d; });
+      } else if (a.keep && need_w) {
+        sw = ss + (size_t)c0 * ldr;                       // the tile's logits, overwritten by its weights
+        load_s(sw, acc);
+      } else {
+        logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = tx * 4 + j;
+        cnt[j] = 0.f;
+        if (c < n) {
+          if (child) {
+            const int e = c0 + c;
+            cnt[j] = ld_after_wait(nc + (size_t)sel_list[e / C] * C + e % C);
+          } else {
+            // correcting form: every parent keeps its full term here, the children add differences below
+            cnt[j] = (sel[c0 + c] && !a.correcting) ? (a.stays ? nstay[c0 + c] : 0.f) : npS[c0 + c];
+          }
+        }
+      }
+      float mean[RT][4];                                  // correcting form only
+      const bool corr = child && a.correcting;
+      if (corr) {
+        // Eq. "parent_recovery": under parent = mean(children) the parent's logit is the mean of its
+        // children's; Eq. "correcting_attention": the child's keys trade the parent's weight for their own
+        store_s(sw, acc);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = tx * 4 + j, f = c / C * C;
+#pragma unroll
+          for (int i = 0; i < RT; ++i) {
+            float sp = 0.f;
+            if (c < n) for (int c2 = 0; c2 < C; ++c2) sp += sw[(size_t)(f + c2) * ldr + row_of(i)];
+            mean[i][j] = sp / (float)C;
+          }
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
+        mx = max16(mx);
+        if (mx > m[i]) {
+          const float alpha = expf(m[i] - mx);
+          z[i] *= alpha;
+#pragma unroll
+          for (int t = 0; t < DT; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[t][i][j] *= alpha;
+          m[i] = mx;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float av = 0.f;
+          if (cnt[j] > 0.f) {
+            av = expf(acc[i][j] - m[i]);
+            if (corr) av -= expf(mean[i][j] - m[i]);
+            z[i] = fmaf(av, cnt[j], z[i]);
+          }
+          acc[i][j] = av;
+        }
+      }
+      store_s(sw, acc);
+      __syncthreads();
+      if (DT > 2) {                                       // shared buffer: the codewords are done with
+        if (child) load_v(val_child);
+        else load_v(val_parent);
+        __syncthreads();
+      }
+#pragma unroll
+      for (int t = 0; t < DT; ++t) mul_tile<RT>(o[t], sw, ldr, vs + t * 64, ldv, (n + 3) & ~3, ty, tx);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      const float inv = 1.f / sum16(z[i]);
+      const int r = rt * R + row_of(i);
+      if (r < rows) {
+#pragma unroll
+        for (int t = 0; t < DT; ++t) {
+          const int k = t * 64 + tx * 4;
+          if (k < d) st4(Yb + (size_t)r * d + k, make_float4(o[t][i][0] * inv, o[t][i][1] * inv, o[t][i][2] * inv, o[t][i][3] * inv));
         }
       }
     }
-    for (int e = 0; e < P * C; ++e) {
-      const int p = sel_list[e / C], c = e % C;
-      const float cnt = nc[p * C + c];
-      if (!(cnt > 0.f)) continue;
-      float av = expf(sb[M + e] - mx);
-      if (a.correcting) {
-        // Eq. "parent_recovery": under parent = mean(children) the parent's logit is the mean of its
-        // children's; Eq. "correcting_attention": the child's keys trade the parent's weight for their own
-        float sp = 0.f;
-        for (int c2 = 0; c2 < C; ++c2) sp += sb[M + (e / C) * C + c2];
-        av -= expf(sp / (float)C - mx);
-      }
-      z += av * cnt;
-#pragma unroll
-      for (int u = 0; u < kMaxDPerLane; ++u) {
-        const int k = lane + 32 * u;
-        if (k < d) x[u] = fmaf(av, Vc[((size_t)p * C + c) * d + k], x[u]);
-      }
-    }
-    const float inv = 1.f / z;
-#pragma unroll
-    for (int u = 0; u < kMaxDPerLane; ++u) {
-      const int k = lane + 32 * u;
-      if (k < d) stf(Yb + (size_t)i * d + k, x[u] * inv);
-    }
-    __syncwarp();
   }
 }
 
-}  // namespace (the size below is also used by the host-side validation)
+}  // namespace
 
+// The envelope of the entry points (header): what the problem may ask for.  The kernel's own shared memory is
+// attend_smem_layout(), at most 227 KiB for every problem inside it.
 size_t simt_attend_smem_bytes(int d, int M, int C, int P, int block_q, int tile_m) {
   const size_t ncols = (size_t)M + (size_t)P * C;
   size_t b = sizeof(double) * M;
-  b += sizeof(float) * ((size_t)block_q * d + 2 * (size_t)block_q + 2 * (size_t)M +
-                        (kAttendThreads / 32) * ncols);
+  b += sizeof(float) * ((size_t)block_q * d + 2 * (size_t)block_q + 2 * (size_t)M + 8 * ncols);
   b += sizeof(int) * ((size_t)M + (size_t)(P > 0 ? P : 1));
   if (tile_m > 0) b += sizeof(float) * ((size_t)block_q + 1) * ((M + tile_m - 1) / tile_m);
   return b;
@@ -403,68 +763,98 @@ size_t simt_attend_smem_bytes(int d, int M, int C, int P, int block_q, int tile_
 
 namespace {
 
+constexpr size_t kSmemMax = 227 * 1024;                   // per CTA on sm_100
+constexpr size_t kSmemHalf = 113 * 1024;                  // two CTAs on an SM
+
 template <typename T>
 avq_status launch_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
-                         int32_t* pidx, int32_t* cidx, cudaStream_t st) {
-  const size_t smem = sizeof(float) * ((size_t)kAssignKeys * (p.d + 1) + (size_t)kAssignCodes * p.d);
+                         int32_t* pidx, int32_t* cidx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
+  const size_t smem = sizeof(float) * 2 * (size_t)p.d * kLdC;
   auto kern = assign_simt_kernel<T>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return AVQ_ERR_CUDA;
   dim3 grid((p.Nk + kAssignKeys - 1) / kAssignKeys, p.B * p.H);
-  kern<<<grid, kAssignKeys, smem, st>>>(static_cast<const T*>(K), static_cast<const T*>(Cp),
-                                        static_cast<const T*>(Cc), pidx, cidx, p.H, p.Nk, p.d, p.M, p.C,
-                                        (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0);
+  kern<<<grid, kThreads, smem, st>>>(static_cast<const T*>(K), static_cast<const T*>(Cp),
+                                     static_cast<const T*>(Cc), pidx, cidx, p.H, p.Nk, p.d, p.M, p.C,
+                                     (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0, static_cast<uint4*>(zero_base),
+                                     (uint32_t)(zero_bytes / 16));
   return cuda_ok(cudaGetLastError());
 }
 
 template <typename T>
 avq_status launch_aggregate(const avq_problem& p, const void* V, const int32_t* pidx, const int32_t* cidx,
-                            float* Vp, float* np_, float* Vc, float* nc, cudaStream_t st) {
-  const int keys_per_cta = 256;
-  dim3 grid((p.Nk + keys_per_cta - 1) / keys_per_cta, p.B * p.H);
-  aggregate_simt_kernel<T><<<grid, 256, 0, st>>>(static_cast<const T*>(V), pidx, cidx, Vp, np_, Vc, nc,
-                                                p.Nk, p.d, p.M, p.C, keys_per_cta);
-  return cuda_ok(cudaGetLastError());
+                            float* Vp, float* np_, float* Vc, float* nc, bool chained, int32_t* status_word,
+                            cudaStream_t st) {
+  const int per_cta = kAggKeysPerWarp * (kThreads / 32);
+  dim3 grid((p.Nk + per_cta - 1) / per_cta, p.B * p.H);
+  return cuda_ok(tc::launch_pdl(aggregate_simt_kernel<T>, grid, dim3(kThreads), 0, st, chained,
+                                static_cast<const T*>(V), pidx, cidx, Vp, np_, Vc, nc, p.Nk, p.d, p.M, p.C,
+                                status_word));
+}
+
+template <typename T, int RT, int DT>
+avq_status launch_attend_rd(AttendArgs a, int B, bool chained, cudaStream_t st) {
+  auto bytes = [&](int keep) {
+    return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.block_q, a.tile_m, keep).total;
+  };
+  // The block's logits stay in shared memory when one row tile holds the block and that leaves room for two
+  // CTAs per SM (or all of an SM's memory is there for the taking because the grid has a CTA per SM at most).
+  int sms = 148, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  const bool one_wave = (int64_t)a.nblk * B * a.H <= sms;
+  const size_t most = one_wave ? kSmemMax : kSmemHalf;
+  a.keep = (a.block_q <= 16 * RT && (a.tile_m == 0 || a.tile_m % kCols == 0) && bytes(1) <= most) ? 1 : 0;
+  const size_t smem = bytes(a.keep);
+  if (smem > kSmemMax) return AVQ_ERR_UNSUPPORTED;
+  auto kern = attend_simt_kernel<T, RT, DT>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return AVQ_ERR_CUDA;
+  return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kThreads), smem, st, chained, a));
 }
 
 template <typename T>
-avq_status launch_attend(const AttendArgs& a, int B, cudaStream_t st) {
-  const size_t smem = simt_attend_smem_bytes(a.d, a.M, a.C, a.P, a.block_q, a.tile_m);
-  if (smem > kSimtAttendSmemLimit) return AVQ_ERR_UNSUPPORTED;   // validate_forward rejects these up front
-  auto kern = attend_simt_kernel<T>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return AVQ_ERR_CUDA;
-  dim3 grid(a.nblk, B * a.H);
-  kern<<<grid, kAttendThreads, smem, st>>>(a);
-  return cuda_ok(cudaGetLastError());
+avq_status launch_attend(const AttendArgs& a, int B, bool chained, cudaStream_t st) {
+  if (simt_attend_smem_bytes(a.d, a.M, a.C, a.P, a.block_q, a.tile_m) > kSimtAttendSmemLimit)
+    return AVQ_ERR_UNSUPPORTED;                           // validate_forward rejects these up front
+  // 128 rows at a time where the block has them and the accumulators fit the registers (d <= 128), else 64
+  if (a.block_q > 64 && a.d <= 64) return launch_attend_rd<T, 8, 1>(a, B, chained, st);
+  if (a.block_q > 64 && a.d <= 128) return launch_attend_rd<T, 8, 2>(a, B, chained, st);
+  if (a.d <= 64) return launch_attend_rd<T, 4, 1>(a, B, chained, st);
+  if (a.d <= 128) return launch_attend_rd<T, 4, 2>(a, B, chained, st);
+  return launch_attend_rd<T, 4, 4>(a, B, chained, st);
 }
 
 }  // namespace
 
 avq_status simt_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
-                       int32_t* parent_idx, int32_t* child_idx, cudaStream_t st) {
-  return p.dtype == AVQ_F32 ? launch_assign<float>(p, K, Cp, Cc, parent_idx, child_idx, st)
-                            : launch_assign<__nv_bfloat16>(p, K, Cp, Cc, parent_idx, child_idx, st);
+                       int32_t* parent_idx, int32_t* child_idx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
+  if (zero_bytes % 16 != 0 || (zero_bytes / 16) >> 31) return AVQ_ERR_WORKSPACE;
+  return p.dtype == AVQ_F32
+             ? launch_assign<float>(p, K, Cp, Cc, parent_idx, child_idx, zero_base, zero_bytes, st)
+             : launch_assign<__nv_bfloat16>(p, K, Cp, Cc, parent_idx, child_idx, zero_base, zero_bytes, st);
 }
 
 avq_status simt_aggregate(const avq_problem& p, const void* V, const int32_t* parent_idx,
-                          const int32_t* child_idx, float* Vp, float* np_, float* Vc, float* nc,
-                          cudaStream_t st) {
-  const size_t BH = (size_t)p.B * p.H;
-  cudaError_t e = cudaMemsetAsync(Vp, 0, sizeof(float) * BH * p.M * p.d, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(np_, 0, sizeof(float) * BH * p.M, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(Vc, 0, sizeof(float) * BH * p.M * p.C * p.d, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(nc, 0, sizeof(float) * BH * p.M * p.C, st);
-  if (e != cudaSuccess) return AVQ_ERR_CUDA;
+                          const int32_t* child_idx, float* Vp, float* np_, float* Vc, float* nc, bool pre_zeroed,
+                          int32_t* status_word, cudaStream_t st) {
+  if (!pre_zeroed) {
+    const size_t BH = (size_t)p.B * p.H;
+    cudaError_t e = cudaMemsetAsync(Vp, 0, sizeof(float) * BH * p.M * p.d, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(np_, 0, sizeof(float) * BH * p.M, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(Vc, 0, sizeof(float) * BH * p.M * p.C * p.d, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(nc, 0, sizeof(float) * BH * p.M * p.C, st);
+    if (e != cudaSuccess) return AVQ_ERR_CUDA;
+  }
   return p.dtype == AVQ_F32
-             ? launch_aggregate<float>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, st)
-             : launch_aggregate<__nv_bfloat16>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, st);
+             ? launch_aggregate<float>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, pre_zeroed, status_word, st)
+             : launch_aggregate<__nv_bfloat16>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, pre_zeroed, status_word, st);
 }
 
 avq_status simt_attend(const avq_problem& p, const void* Q, const void* Cp, const void* Cc,
                        const float* Vp, const float* np_, const float* Vc, const float* nc, int32_t P,
                        int32_t block_q, void* Y, int32_t* topp_out, float* importance_out,
-                       int32_t tile_m, cudaStream_t st) {
+                       int32_t tile_m, bool chained, cudaStream_t st) {
   AttendArgs a;
   a.tile_m = tile_m;
   a.Nk = p.Nk;
@@ -474,8 +864,10 @@ avq_status simt_attend(const avq_problem& p, const void* Q, const void* Cp, cons
   a.nblk = (p.Nq + block_q - 1) / block_q;
   a.stays = (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0;
   a.correcting = (p.flags & AVQ_FLAG_CORRECTING) ? 1 : 0;
+  a.keep = 0;
   a.scale = p.scale;
-  return p.dtype == AVQ_F32 ? launch_attend<float>(a, p.B, st) : launch_attend<__nv_bfloat16>(a, p.B, st);
+  return p.dtype == AVQ_F32 ? launch_attend<float>(a, p.B, chained, st)
+                            : launch_attend<__nv_bfloat16>(a, p.B, chained, st);
 }
 
 }  // namespace avq

@@ -121,3 +121,21 @@ def test_correcting_form_matches_the_oracle_and_the_masked_form_on_recentred_cod
     dev = (Yc.float() - Ym.float()).abs().max().item()
     print(f"correcting vs masked form, bf16-rounded re-centred codebooks: max-abs {dev:.3e}")
     assert dev <= 0.25
+
+
+@pytest.mark.parametrize("d,M,C,P,bq,N", [(4, 1, 1, 1, 1, 70), (64, 64, 4, 8, 65, 131), (68, 65, 5, 7, 129, 300),
+                                          (128, 130, 16, 3, 200, 450), (132, 70, 2, 70, 64, 200),
+                                          (256, 33, 3, 0, 100, 210), (64, 300, 4, 20, 128, 256)])
+def test_tile_edges_of_the_register_tiled_kernels(d, M, C, P, bq, N):
+    """64-key, 64-codeword and 64- / 128-row tiles: one element past and short of a tile, several row tiles per
+    query block, every head-dimension variant, logits kept in shared memory and recomputed."""
+    wl = synth.Workload("edges", B=1, H=2, N=N, d=d, M=M, C=C, P=P, block_q=bq, dtype="f32", seed=70 + d, alpha=0.6)
+    parity.full_parity(wl)
+    x = synth.generate(wl)
+    dv = parity.to_device(x, "f32")
+    if P in (0, M) or M < 64:
+        return
+    # importance over tiles of 32 parents (narrower than a codeword tile)
+    _, topp, imp = binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, bq, 32, scale=wl.scale)
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, bq, wl.scale, form="factorised", tile_m=32)
+    parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
