@@ -326,7 +326,7 @@ struct AttendArgs {
 // Shared memory of attend_simt_kernel, in floats from the base (doubles first).
 struct AttendSmem {
   int ldr;                                   // pitch of a [k][row] operand
-  size_t w, wpart, q, c, v, s, rm, rz, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
+  size_t w, wpart, q, c, v, s, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
 };
 // RT = 8: 128 query rows at a time (d <= 128), RT = 4: 64 rows.  v == c where the two tiles share one buffer.
 __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int block_q, int tile_m,
@@ -347,8 +347,6 @@ __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, 
     L.c = L.v = take(a > b ? a : b);
   }
   L.s = take((size_t)(keep ? (M + kCols - 1) / kCols * kCols : kCols) * L.ldr);
-  L.rm = take(block_q);
-  L.rz = take(block_q);
   L.np = take(M);
   L.nstay = take(M);
   L.zt = take((size_t)block_q * ntiles);
@@ -388,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
   const int ldr = L.ldr;
   double* w = reinterpret_cast<double*>(sm + L.w);
   double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [8][64]
-  float *qs = sm + L.q, *cs = sm + L.c, *vs = sm + L.v, *ss = sm + L.s, *rm = sm + L.rm, *rz = sm + L.rz;
+  float *qs = sm + L.q, *cs = sm + L.c, *vs = sm + L.v, *ss = sm + L.s;
   float *npS = sm + L.np, *nstay = sm + L.nstay, *zt = sm + L.zt, *nseen = sm + L.nseen;
   int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
   constexpr int ldv = DT * 64;

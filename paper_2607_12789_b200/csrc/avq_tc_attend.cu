@@ -1,24 +1,32 @@
 // Tensor-core attention pass of AVQ-attention (Algorithm 2 in its masked form) for bf16 inputs.
 //
-// One CTA = one query tile of 128 rows of one (batch, head) at a time; each row is handled by NQ threads
-// (column slices).  Values enter as per-codeword MEANS with the key counts multiplied into the weights.
+// One CTA = one query tile of 128 rows of one (batch, head) at a time; 4 NQ warps, warp w holds rows
+// 32 (w % 4) .. +31 of the column slice w / 4.  Inside a warp the accumulator is read in the layout of an MMA
+// result (tcgen05.ld.16x256b): lane 4 g + t holds rows g, g + 8, g + 16, g + 24 and column pairs 2 t, 2 t + 1 of every
+// 8-column block.  Against one row per lane this (a) needs a quarter of the per-column operands (bias, counts) per
+// thread, (b) sums a column over its rows mostly in registers (14 shuffles per 64 columns instead of 62), (c) puts
+// neighbouring columns into neighbouring registers for the packed fp32 instructions and for the weights' stores.
+// Parent codewords (and their value rows) stand in an order of their own in shared memory: inside every group of 8
+// rows, codeword 4 v + t at row 2 t + v (the tensor map does it), so that lane t of a quad holds the codewords t,
+// t + 4, t + 8, ... of its slice and the denominator's four partial sums stay what they are with one row per lane:
+// which parents are selected does not depend on the layout.
+// Values enter as per-codeword MEANS with the key counts multiplied into the weights.
 // Flow of a tile:
-//   parents   S = Q . Cp^T                 tcgen05.mma, fp32 accumulator in TMEM columns [0, M)
-//             read once into registers: row maximum over non-empty parents, exp2, exact
-//             denominator z                                         (Eq. "vqflashattention");
-//             in the same loop the bf16 weights A_ij n_j -> shared memory (over the dead codebook)
+//   parents   S = Q . Cp^T                 tcgen05.mma, fp32 accumulator in TMEM, issued at the end of the tile before
+//             read once into registers: row maximum over non-empty parents, exp2, exact denominator z
+//                                                                   (Eq. "vqflashattention")
 //             importance w_j = n_j sum_i A_ij / z_i from the fp32 weights  (Eq. "importance")
-//             top-P by rank, ties to the lower index                ("Child spawning")
-//             a refined parent's row of the value tile becomes its stay row (zeros by default) and its
-//             rounded weights leave the denominator
-//             O = (A n) . mean_p           tcgen05.mma into TMEM columns [CT, CT + d)
+//             top-P, ties to the lower index                        ("Child spawning")
+//             bf16 weights A_ij n_j (zero for a refined parent) -> A operand
+//             O = (A n) . mean_p           tcgen05.mma
 //   children  of the selected parents, in chunks of <= CHW columns: gathered codeword rows,
-//             S_c = Q . Cc_sel^T, running maximum (non-empty children only), O rescaled in TMEM if a
-//             row's maximum moved, bf16 weights, O += A_c . Vbar_c   (Algorithm 2, child loop)
+//             S_c = Q . Cc_sel^T, bf16 weights, O += A_c . Vbar_c   (Algorithm 2, child loop); O is rescaled in
+//             TMEM only if the children's weights against the row's reference pass 2^64
 //   Y = O / z, z accumulated from the same bf16-rounded weights as the numerator.
-// Empty codewords are excluded from every maximum and contribute nothing (their count and value sum
-// are zero; their weight is clamped so that it stays finite) - appendix on numerical stability.
-// The gathers of the first child chunk are issued as soon as the selection is known.
+// Empty codewords are excluded from every maximum and contribute nothing (their logit is -inf, their count and
+// value sum are zero) - appendix on numerical stability.
+// A CTA takes a run of consecutive tiles: codebook, parent values and counts stay in shared memory while the
+// (batch, head) does not change.
 #include "avq_tc_common.cuh"
 
 namespace avq {
@@ -27,6 +35,8 @@ namespace {
 using namespace tc;
 
 constexpr int kRows = 128;
+// shared-memory row / TMEM column of parent codeword c
+__device__ __forceinline__ int parent_pos(int c) { return (c & ~7) | ((c & 3) << 1) | ((c >> 2) & 1); }
 
 struct AttendParams {
   const __nv_bfloat16* Cc;    // [H, M, C, d]
@@ -42,7 +52,6 @@ struct AttendParams {
   int H, Nq, M, C, P, nblk;
   int total_tiles;            // nblk * B * H
   int logC;                   // log2(C)
-  uint32_t tmem_cols;
   float scale_log2e;
 };
 
@@ -56,26 +65,171 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Column sums over the 32 lanes of a warp of V values per lane.  Returns, in every lane, the
-// sum of column (lane >> (5 - log2 V)).  V = 32: 31 shuffles instead of 160.
-template <int V>
-__device__ __forceinline__ float transpose_reduce(float (&v)[V], int lane) {
-  int n = V;
+// ---- packed pairs of fp32 (two neighbouring columns of one row)
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 pack2u(uint32_t lo, uint32_t hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// z += both halves of a bf16 pair (mixed-precision adds: no widening instructions)
+__device__ __forceinline__ void add_bf16x2(float& z, uint32_t pk) {
+  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %0, h, %0;\n\t}"
+      : "+f"(z) : "r"(pk));
+}
+
+// ---- accumulator fragments: NB blocks of 8 columns x 32 rows per warp.  r[half][4 b + 2 u + v] = row
+// 16 half + 8 u + g, column 8 b + 2 t + v.
+template <int NB>
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[2][4 * NB]) {
+  static_assert(NB == 2 || NB == 4, "16 or 32 columns");
 #pragma unroll
-  for (int b = 16; b >= 1; b >>= 1) {
+  for (int h = 0; h < 2; ++h) {
+    uint32_t* q = r[h];
+    const uint32_t a = taddr + ((uint32_t)(16 * h) << 16);
+    if constexpr (NB == 4)
+      asm volatile(
+          "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+          : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
+            "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+          : "r"(a) : "memory");
+    else
+      asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7])
+                   : "r"(a) : "memory");
+  }
+}
+// M codeword rows of 64 columns in the order of parent_pos: dimensions (column, v, t, group of 8)
+__device__ __forceinline__ void tma_load_codes(void* dst, const CUtensorMap* map, int x, int group, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %4, %5}], [%2];"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(0), "r"(group)
+      : "memory");
+}
+// Waits for this warp's TMEM loads; the registers pass through so that no use of them moves ahead of the wait.
+template <int NB>
+__device__ __forceinline__ void tmem_ld_wait_frag(uint32_t (&r)[2][4 * NB]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int c = 0; c < NB / 2; ++c) {
+      uint32_t* q = r[h] + 8 * c;
+      if (h == 0 && c == 0)
+        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                     : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7])::"memory");
+      else
+        asm volatile("" : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7])::"memory");
+    }
+}
+template <int NB>
+__device__ __forceinline__ void tmem_st_frag(uint32_t taddr, const uint32_t (&r)[2][4 * NB]) {
+  static_assert(NB == 2, "16 columns");
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t* q = r[h];
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
+                     taddr + ((uint32_t)(16 * h) << 16)),
+                 "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
+                 : "memory");
+  }
+}
+// bf16 weights of 32 columns x 32 rows (16 TMEM columns, the K-major A operand of the value MMA):
+// r[half][2 b + u] = columns 8 b + 2 t, + 1 of row 16 half + 8 u + g.
+__device__ __forceinline__ void tmem_st_weights(uint32_t taddr, const uint32_t (&r)[2][8]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t* q = r[h];
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
+                     taddr + ((uint32_t)(16 * h) << 16)),
+                 "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
+                 : "memory");
+  }
+}
+// D += A . B with A (bf16, K-major) in TMEM
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                             bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
+// Four 8 x 8 bf16 blocks (rows 0-7, 8-15, 16-23, 24-31 of the warp, one 8-column block): lane l supplies the
+// address of row l's 16 bytes.
+__device__ __forceinline__ void stmatrix4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2),
+               "r"(r3)
+               : "memory");
+}
+// One lane of a converged warp.  With a warp-uniform condition around it (the warp index comes from a shuffle) the
+// compiler keeps descriptors and coordinates in uniform registers; behind `if (lane == 0)` every tcgen05.mma or TMA
+// instruction moved them there again, which took 130 instead of 50 cycles each beside busy warps.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ float quad_max(float v) {
+  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
+  return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+__device__ __forceinline__ float quad_sum(float v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+__device__ __forceinline__ float pick4(const float (&v)[4], int t) {
+  const float a = (t & 1) ? v[1] : v[0], b = (t & 1) ? v[3] : v[2];
+  return (t & 2) ? b : a;
+}
+
+// Column sums over the 8 lanes (stride 4) that share a column: v[NB] pairs per lane; lane 4 g + t returns the pair
+// of block g (NB = 8) or g / 2 (NB = 4).
+template <int NB>
+__device__ __forceinline__ f32x2 reduce_rows(f32x2 (&v)[NB], int lane) {
+  int n = NB;
+#pragma unroll
+  for (int b = 16; b >= 4; b >>= 1) {
     if (n > 1) {
       n >>= 1;
       const bool hi = (lane & b) != 0;
 #pragma unroll
-      for (int i = 0; i < V / 2; ++i) {
+      for (int i = 0; i < NB / 2; ++i)
         if (i < n) {
-          const float send = hi ? v[i] : v[i + n];
-          const float keep = hi ? v[i + n] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, b);
+          const f32x2 send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+          v[i] = add2(keep, __shfl_xor_sync(0xffffffffu, send, b));
         }
-      }
     } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], b);
+      v[0] = add2(v[0], __shfl_xor_sync(0xffffffffu, v[0], b));
     }
   }
   return v[0];
@@ -88,50 +242,54 @@ __device__ __forceinline__ void row_sync(int q) {
   asm volatile("bar.sync %0, %1;" ::"r"(q + 1), "r"(32 * NQ) : "memory");
 }
 
-// Multiplies 16 fp32 weights by their codewords' key counts, rounds the products to bf16, stores them at
-// (row r, columns col0..col0+15) of the K-major swizzled A tile, and returns the sum of the rounded
-// products (the denominator is built from exactly what the value MMA multiplies).  KEEP: each product
-// enters that sum times keep16[] (the share of its own term a parent keeps once it is refined).
-template <bool KEEP>
-__device__ __forceinline__ float store_weights16(unsigned char* A, int r, int col0, const float* cnt16,
-                                                 const float* keep16, const float (&a)[16]) {
-  const float4* n4 = reinterpret_cast<const float4*>(cnt16);
-  const float4* k4 = reinterpret_cast<const float4*>(keep16);
-  uint32_t pk[8];
-  float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;         // independent partial sums: no 16-deep add chain
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const float4 n = n4[u];
-    const uint32_t p0 = pack_bf16(a[4 * u] * n.x, a[4 * u + 1] * n.y);
-    const uint32_t p1 = pack_bf16(a[4 * u + 2] * n.z, a[4 * u + 3] * n.w);
-    if constexpr (KEEP) {
-      const float4 k = k4[u];
-      z0 = fmaf(__uint_as_float(p0 << 16), k.x, z0);
-      z1 = fmaf(__uint_as_float(p0 & 0xFFFF0000u), k.y, z1);
-      z2 = fmaf(__uint_as_float(p1 << 16), k.z, z2);
-      z3 = fmaf(__uint_as_float(p1 & 0xFFFF0000u), k.w, z3);
-    } else {
-      z0 += __uint_as_float(p0 << 16);
-      z1 += __uint_as_float(p0 & 0xFFFF0000u);
-      z2 += __uint_as_float(p1 << 16);
-      z3 += __uint_as_float(p1 & 0xFFFF0000u);
-    }
-    pk[2 * u] = p0;
-    pk[2 * u + 1] = p1;
-  }
-  const float z = (z0 + z1) + (z2 + z3);
-  unsigned char* sub = A + (col0 >> 6) * (kRows * 128);
-  *reinterpret_cast<uint4*>(sub + sw128_offset(r, col0 & 63)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  *reinterpret_cast<uint4*>(sub + sw128_offset(r, (col0 & 63) + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-  return z;
-}
-
-// NQ = threads per query row: 1, 2 or 4.  Small tiles take NQ = 1 so that four CTAs share an SM and
+// Shared-memory and TMEM plan of one instantiation.
+// NQ = warps (column slices) per 32 query rows: 1, 2 or 4.  Small tiles take NQ = 1 so that four CTAs share an SM and
 // overlap each other's load / MMA / softmax phases; the largest take NQ = 4.
 // CT = parent tile width (64, 128 or 256, >= M), a compile-time constant so that every shared-memory
 // offset folds into the instruction stream instead of occupying a register.
-// FUSE = the weight conversion runs inside the exponential loop (chosen by the launcher from CT, P and M).
-template <int D, int NQ, int CT, bool FUSE>
+template <int D, int NQ, int CT>
+struct Plan {
+  static constexpr int kThreads = 128 * NQ;
+  static constexpr int kSubD = D / 64;
+  static constexpr int CHW = CT < 128 ? CT : 128;        // child chunk width
+  static constexpr int QT = kSubD * kRows * 128;         // bytes of a query / output tile
+  // Weights as the A operand in TMEM: nothing to swizzle or fence, the MMA reads half the shared memory, and the
+  // codebook survives the tile.  The smallest tile has no TMEM columns left (four CTAs of 128 columns share an
+  // SM): its weights overwrite the codebook in shared memory, which is then loaded again (8 KB).
+  static constexpr bool kTW = !(CT == 64 && D == 64);
+  // The children's codes and value rows have a buffer each, so that both gathers run ahead of the logits.  The largest
+  // tile has room for the values only: the codes go over the parent codebook, whose logits are done by then, and the
+  // overwritten half of the codebook is loaded again behind the child logits.  The smallest gathers the values into
+  // the codes' place once the child logits are done (four CTAs fill each other's gaps).
+  static constexpr bool kCodesInCA = CT == 256 && D == 128;
+  static constexpr bool kSepCV = kTW;
+  // The output tile is staged in the child buffers where they are as large as a query tile, else across the
+  // parent values and the child buffer (the parent values are then loaded again).
+  static constexpr bool kStageInCC = CT >= 128 || kSepCV;
+  static constexpr int cp_bytes = CT * D * 2;
+  static constexpr int ca_bytes = kTW ? cp_bytes : (cp_bytes > kRows * CT * 2 ? cp_bytes : kRows * CT * 2);
+  static constexpr int oQ = 0, oCA = QT, oV = oCA + ca_bytes, oCC = oV + CT * D * 2,
+                       oCV = oCC + (kSepCV && !kCodesInCA ? CHW * D * 2 : 0);
+  static constexpr int oStage = kStageInCC ? oCC : oV;
+  static constexpr int oF = oCV + CHW * D * 2;           // fp32 / word arrays from here
+  // TMEM columns: logits, weights (kTW), output.  With 256 logit columns the child logits use half of them and the
+  // children's weights go into the other half, so they need not wait for the parents' value MMA.
+  static constexpr bool kSepW = CT == 256;
+  static constexpr int tW = kTW ? CT : 0, tWc = kSepW ? 128 : tW, tO = kTW ? CT + CT / 2 : CT;
+  static constexpr int tmem_used = tO + D;
+  static constexpr uint32_t tmem_cols = tmem_used <= 128 ? 128 : (tmem_used <= 256 ? 256 : 512);
+  static_assert(CHW * D * 2 * (kSepCV && !kCodesInCA ? 2 : 1) >= QT || !kStageInCC, "the output tile fits its staging area");
+  static_assert(kStageInCC || CT * D * 2 + CHW * D * 2 >= QT, "the output tile fits its staging area");
+};
+
+template <int D, int NQ, int CT>
+size_t attend_smem(int MC) {
+  using L = Plan<D, NQ, CT>;
+  return L::oF + 4 * ((size_t)2 * CT + CT + L::CHW + CT + 4 * CT + 2 * NQ * kRows + 2 * CT + MC + CT + 32 + 18) + 8 * 6 + 16;
+}
+
+// STAYS = the PARENT_STAYS rule: a refined parent keeps the keys that stayed with it.
+template <int D, int NQ, int CT, bool STAYS>
 __global__ void __launch_bounds__(128 * NQ, 4 / NQ)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmCp,
                  const __grid_constant__ CUtensorMap tmVpb, const __grid_constant__ CUtensorMap tmY,
@@ -139,723 +297,805 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
-  constexpr int kThreads = 128 * NQ;
-  constexpr int kScLane = kThreads / 2;                  // lane 0 of a warp in the other half of the CTA
-  constexpr int kSubD = D / 64;
+  using L = Plan<D, NQ, CT>;
+  constexpr int kThreads = L::kThreads, kSubD = L::kSubD, CHW = L::CHW;
+  constexpr bool kTW = L::kTW, kSepCV = L::kSepCV;
+  constexpr int kVWarp = kThreads / 64;                  // issues S and the value MMAs (warp 0: child logits, TMA)
   constexpr int kLogD = (D == 128) ? 7 : 6;
   constexpr int kLogChunks = kLogD - 3;                  // 16-byte chunks per codeword row
-  constexpr int CHW = CT < 128 ? CT : 128;               // child chunk width
   constexpr int QW = CT / NQ, QWC = CHW / NQ;
-  constexpr int subA = CT >> 6;                          // 64-column sub-tiles of an A / value tile
-  constexpr int ca_bytes = (CT * D * 2 > subA * kRows * 128) ? CT * D * 2 : subA * kRows * 128;
+  constexpr int NB = QW / 8, NC = QW / 32;               // 8-column blocks and 32-column chunks of a warp's parents
+  constexpr int NCC = QWC / 32;                          // and of its children
   const int M = p.M, C = p.C, P = p.P, logC = p.logC;
-  unsigned char* Qs = smem;                              // kSubD x [128 x 128 B]
-  unsigned char* CA = Qs + kSubD * kRows * 128;          // parent codes, later the bf16 weights
-  unsigned char* Vs = CA + ca_bytes;                     // value rows: kSubD x [rows x 128 B], rows = M or a chunk's children
-  unsigned char* CC = Vs + subA * D * 128;               // kSubD x [CHW x 128 B] gathered child codes
-  float* cnt = reinterpret_cast<float*>(CC + CHW * D * 2);   // [CT] key counts of the parents
+  unsigned char* Qs = smem + L::oQ;                      // kSubD x [128 x 128 B]
+  unsigned char* CA = smem + L::oCA;                     // parent codes: kSubD x [M x 128 B] (kTW false: later the bf16 weights)
+  unsigned char* Vs = smem + L::oV;                      // parent value rows: kSubD x [M x 128 B]
+  unsigned char* CC = L::kCodesInCA ? CA : smem + L::oCC;   // gathered child codes: kSubD x [rows x 128 B]
+  unsigned char* CV = smem + L::oCV;                     // gathered child values
+  unsigned char* stage = smem + L::oStage;
+  // per-parent operands, by column (parent_pos)
+  float* cnt = reinterpret_cast<float*>(smem + L::oF);   // [CT] key counts
   float* bias = cnt + CT;                                // [CT] 0 for non-empty parents, -inf for empty
-  float* cntk = bias + CT;                               // [CT] share of its own term a parent keeps: 1, or once refined 0 / its stay share
-  float* cntc = cntk + CT;                               // [CHW] key counts of the child chunk
-  float* biasc = cntc + CHW;                             // [CHW]
-  float* w = biasc + CHW;                                // [CT] importance
-  float* wpart = w + CT;                                 // [4][CT]
-  float* xm = wpart + 4 * CT;                            // [NQ][128] exchange between the threads of a row
+  // what a parent's term is multiplied by: default rule, the bf16 mask of its weight (0xFFFF, once refined 0);
+  // PARENT_STAYS, the share of its own denominator term it keeps (1, once refined its stay share)
+  float* keep_f = bias + CT;                             // [CT] STAYS
+  uint16_t* keep_m = reinterpret_cast<uint16_t*>(keep_f);   // [CT] default rule
+  float* l2n = keep_f + CT;                              // [CHW] log2 of the key counts of the child chunk
+  float* w = l2n + CHW;                                  // [CT] importance, by parent
+  float* wpart = w + CT;                                 // [4][CT] by column
+  float* xm = wpart + 4 * CT;                            // [NQ][128] exchange between the warps of a row
   float* xz = xm + NQ * kRows;                           // [NQ][128]
-  float* xz2 = xz + NQ * kRows;                          // [NQ][128]
-  float* ncs = xz2 + NQ * kRows;                         // [M * C] key counts of every child of this (b, h)
-  int* sel_list = reinterpret_cast<int*>(ncs + p.M * p.C);    // [CT]
-  uint32_t* wmask = reinterpret_cast<uint32_t*>(sel_list + CT);    // [16]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(wmask + 18);        // [5]  (wmask[16] is a scratch word)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
+  uint64_t* cand = reinterpret_cast<uint64_t*>(xz + NQ * kRows);   // [CT] top-P candidates
+  float* ncs = reinterpret_cast<float*>(cand + CT);      // [M * C] log2 of the key counts of every child of this (b, h)
+  int* sel_list = reinterpret_cast<int*>(ncs + M * C);   // [CT] refined parents
+  int* wcount = sel_list + CT;                           // [32] keys at or above a sample key
+  uint32_t* nzmask = reinterpret_cast<uint32_t*>(wcount + 32);   // [8] parents with an importance above zero
+  uint32_t* selmask = nzmask + 8;                        // [8] refined parents
+  int* ncand_s = reinterpret_cast<int*>(selmask + 8);    // candidates listed (+ 1 word of padding)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ncand_s + 2);     // [6]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int q = warp & 3, cq = warp >> 2, r = q * 32 + lane;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
+  const int q = warp & 3, cq = warp >> 2, r = q * 32 + lane;   // r: the row this lane stands for in exchanges
+  const int g = lane >> 2, t4 = lane & 3;                // fragment rows q*32 + g + 8 h, column pairs 2 t4
   const int colbase = cq * QW;
   uint64_t* bar_q = &bars[0];                            // query tile landed
-  uint64_t* bar_ld1 = &bars[1];                          // parent value rows landed
-  uint64_t* bar_s = &bars[2];
-  uint64_t* bar_pv = &bars[3];
+  uint64_t* bar_v = &bars[1];                            // parent value rows landed
+  uint64_t* bar_s = &bars[2];                            // parent or child logits done
+  uint64_t* bar_pv = &bars[3];                           // children's value MMA done
   uint64_t* bar_cp = &bars[4];                           // parent codebook landed
-  // A CTA works through the tiles blockIdx.x, blockIdx.x + gridDim.x, ... (the grid is one wave of CTAs).
-  // The next tile's Q is loaded as soon as this tile's last logits are done, its codebook as soon as this
-  // tile's last value MMA is done, so the set-up, the loads and the first MMA of a tile hide behind the tail
-  // of the tile before.  The output is staged where the next tile's first loads do not go: in the child-code
-  // buffer when that is as large as a Q tile (CT >= 128), else across the value tile and the child-code
-  // buffer, which are adjacent and together as large (the next tile's value rows then load a little later).
-  constexpr bool kChain = true;
-  constexpr bool kStageInCC = CT >= 128;
-  // weight conversion inside the exponential loop (see there): pays where few CTAs share the SM and P is small
-  // against M; measured slower for the 64-column tiles (four CTAs per SM already fill each other's gaps) and
-  // for P near M (the P look-ups per row cost more than the overlap gains)
-  constexpr bool fuse = FUSE;
-  auto issue_q = [&](int t) {                            // thread 0 only
-    const int tb = t / p.nblk, ti0 = (t - tb * p.nblk) * kRows;
-    mbar_expect_tx(bar_q, (uint32_t)(kSubD * kRows * 128));
+  uint64_t* bar_o = &bars[5];                            // parents' value MMA done
+  auto issue_q = [&](int bh, int blk) {                  // one thread (as the next two)
+    mbar_expect_tx(bar_q, (uint32_t)L::QT);
 #pragma unroll
-    for (int s = 0; s < kSubD; ++s) tma_load_3d(Qs + s * kRows * 128, &tmQ, s * 64, ti0, tb, bar_q);
+    for (int s = 0; s < kSubD; ++s) tma_load_3d(Qs + s * kRows * 128, &tmQ, s * 64, blk * kRows, bh, bar_q);
   };
-  auto issue_cp = [&](int t) {
-    const int th = (t / p.nblk) % p.H;
-    mbar_expect_tx(bar_cp, (uint32_t)(kSubD * M * 128));
-#pragma unroll
-    for (int s = 0; s < kSubD; ++s) tma_load_2d(CA + s * M * 128, &tmCp, s * 64, th * M, bar_cp);
+  auto issue_cp = [&](int bh, int subs) {                // the first `subs` halves of the codebook
+    mbar_expect_tx(bar_cp, (uint32_t)(subs * M * 128));
+    for (int s = 0; s < subs; ++s) tma_load_codes(CA + s * M * 128, &tmCp, s * 64, ((bh % p.H) * M) >> 3, bar_cp);
   };
-  auto issue_vp = [&](int t) {
-    const int tb = t / p.nblk;
-    mbar_expect_tx(bar_ld1, (uint32_t)(kSubD * M * 128));
+  auto issue_v = [&](int bh) {
+    mbar_expect_tx(bar_v, (uint32_t)(kSubD * M * 128));
 #pragma unroll
-    for (int s = 0; s < kSubD; ++s) tma_load_2d(Vs + s * M * 128, &tmVpb, s * 64, tb * M, bar_ld1);
-  };
-
-  auto issue_s = [&](uint32_t tmem_d, uint32_t parity) {  // one thread: S = Q . Cp^T once both tiles have landed
-    const bool q_ok = mbar_wait(bar_q, parity, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-    const bool c_ok = mbar_wait(bar_cp, parity, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-    if (q_ok && c_ok) {
-      tc_fence_after();
-      const uint32_t idesc = umma_idesc_bf16(kRows, M);
-      const uint32_t qa = smem_u32(Qs), ca = smem_u32(CA);
-#pragma unroll
-      for (int k = 0; k < D / 16; ++k)
-        umma_bf16(tmem_d, umma_desc_sw128(qa + (k / 4) * kRows * 128 + (k % 4) * 32),
-                  umma_desc_sw128(ca + (k / 4) * M * 128 + (k % 4) * 32), idesc, k > 0);
-    }
-    umma_commit(bar_s);
+    for (int s = 0; s < kSubD; ++s) tma_load_codes(Vs + s * M * 128, &tmVpb, s * 64, (bh * M) >> 3, bar_v);
   };
 
   __shared__ int early_exit;
+  // This CTA's run of consecutive tiles.  The CTAs with one tile more are the first ones of the grid: CTAs that
+  // share an SM are a multiple of the SM count apart, so every SM gets its share of them.
+  const int per = p.total_tiles / gridDim.x, more = p.total_tiles - per * gridDim.x;
+  const int tile0 = (int)blockIdx.x * per + min((int)blockIdx.x, more);
+  const int tile1 = tile0 + per + ((int)blockIdx.x < more ? 1 : 0);
+  int bh = tile0 / p.nblk, blk = tile0 - bh * p.nblk;
 
   // ---- Part 1 touches only the caller's Q and Cp, so it may run while the kernel that produces the
   // aggregates is still finishing (programmatic dependent launch): barriers, TMEM, the Q / Cp loads and
   // S = Q . Cp^T.
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     prefetch_tmap(&tmQ);
     prefetch_tmap(&tmCp);
     prefetch_tmap(&tmVpb);
-    mbar_init(bar_q, 1);
-    mbar_init(bar_cp, 1);
-    mbar_init(bar_ld1, 1);
-    mbar_init(bar_s, 1);
-    mbar_init(bar_pv, 1);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) mbar_init(&bars[i], 1);
     mbar_fence_init();
     *abort_flag = 0;
-    issue_q(blockIdx.x);
-    issue_cp(blockIdx.x);
+    issue_q(bh, blk);
+    issue_cp(bh, kSubD);
   }
   // TMEM is allocated before the dependency wait.  tcgen05.alloc blocks until the columns are free and the
   // wait returns only when the kernels before this one have finished; neither can hold the other up: the
   // columns an earlier kernel's CTAs own are released when those CTAs end, which needs nothing from this
   // kernel, and CTAs of this kernel release theirs on every path (including the early exit below).
-  if (warp == 1) {                                   // not the warp whose lane 0 is busy issuing the loads
-    tmem_alloc(tmem_slot, p.tmem_cols);
+  if (warp == 1) {                                   // not the warp whose lane is busy issuing the loads
+    tmem_alloc(tmem_slot, L::tmem_cols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
   const uint32_t t_s = t_row + (uint32_t)colbase;
   const uint32_t t_sc = t_row + (uint32_t)(cq * QWC);
-  const uint32_t t_o = t_row + (uint32_t)(CT + cq * (D / NQ));
+  const uint32_t t_o = t_row + (uint32_t)(L::tO + cq * (D / NQ));
   const uint32_t idesc_o = umma_idesc_bf16(kRows, D) | (1u << 16);   // B (the value rows) is MN-major
   const float sc = p.scale_log2e;
-  uint32_t ph_s = 0, ph_pv = 0, ph_in = 0;               // ph_in: parity of the three load barriers (once per tile)
+  uint32_t ph_s = 0, ph_pv = 0, ph_v = 0, ph_o = 0;
+  uint32_t ph_q = 0, ph_cp = 0;                          // used by the issuing warp
   const int PC = P * C;
-  const int my_cols = min(max(M - colbase, 0), QW);      // multiple of 16 (M % 32 == 0, QW % 16 == 0)
-  bool first = true;
-  bool store_pending = false;                            // thread 0: a TMA store may still be reading CC
-  for (int tile = blockIdx.x; tile < p.total_tiles; tile += gridDim.x) {
-  const int bh = tile / p.nblk, blk = tile - bh * p.nblk, h = bh % p.H;
-  const int i0 = blk * kRows;
-  const int rows_valid = min(kRows, p.Nq - i0);
-  const int next_tile = tile + gridDim.x;
-  const bool has_next = kChain && next_tile < p.total_tiles;
-  // Key counts of this (b, h): one parent count and one 16-byte group of child counts per thread.  Their loads
-  // are started before thread 0 turns to the MMA issue so that its warp is not a load latency behind the
-  // others at the next barrier (first tile: only after the dependency wait below - the kernel before this
-  // one writes them, so they are loaded with statements the compiler cannot move ahead of that wait).
-  static_assert(CT <= kThreads && 2 * CT <= 4 * kThreads, "one count load per thread");
-  float n_reg = 0.f;
-  float4 nc_reg = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto load_counts = [&]() {
-    if (tid < M) n_reg = ld_after_wait(p.np_ + (size_t)bh * M + tid);
-    if (PC > 0 && tid < ((M * C) >> 2))
-      nc_reg = ld_after_wait(reinterpret_cast<const float4*>(p.nc + (size_t)bh * M * C) + tid);
-  };
-  if (!first) load_counts();
-  if (tid == 0) {
-    issue_s(tmem_base, ph_in);
-    if (!kStageInCC && !first) {
-      // the value tile was the staging area of the tile before: reload it once that store has read it
-      tma_store_wait_read();
-      store_pending = false;
-      issue_vp(tile);
-    }
-  }
+  const int my_cols = min(max(M - colbase, 0), QW);      // multiple of 32
 
-  // ---- Part 2 reads what the earlier kernels of this call wrote: status word, counts, value sums.
-  if (first) {
-    pdl_wait();
-    load_counts();                                     // in flight before thread 0 blocks on the status word
-    if (tid == 0) {
-      issue_vp(tile);
-      // a wait that expired in an earlier CTA or kernel of this call: do not start more work
-      early_exit = (p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0);
-    }
-  }
-  if (tid < CT) {
-    cnt[tid] = n_reg;
-    bias[tid] = n_reg > 0.f ? 0.f : -INFINITY;
-    cntk[tid] = 1.f;
-  }
-  // every child's key count: the gathers below pick theirs from shared memory instead of waiting for a
-  // dependent global load once the selection is known
-  if (PC > 0 && tid < ((M * C) >> 2)) reinterpret_cast<float4*>(ncs)[tid] = nc_reg;
-  __syncthreads();
-  if (first && early_exit) {
-    // let the MMA and the load already in flight finish, then leave cleanly
-    mbar_wait(bar_s, 0, abort_flag, nullptr, 0);
-    mbar_wait(bar_ld1, 0, abort_flag, nullptr, 0);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, p.tmem_cols);
-    return;
-  }
-  first = false;
-
-  // ---- parents: row maximum over non-empty codewords (empty ones carry a -inf bias)
-  mbar_wait(bar_s, ph_s, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-  ph_s ^= 1;
-  tc_fence_after();
-  if (tid == 0 && has_next && PC == 0) issue_q(next_tile);   // no child logits will read this Q tile
-  // This thread's QW (<= 64) parent logits are read from TMEM once and stay in registers through the
-  // maximum, the exponentials, the importance sums and the conversion to bf16.
-  float a[QW];
-  float mx = -INFINITY, mx2 = -INFINITY;
-#pragma unroll
-  for (int c0 = 0; c0 < QW; c0 += 16) {
-    if (c0 < my_cols) {                                  // warp-uniform
-      float s[16];
-      tmem_ld16(t_s + c0, s);
-      const float4* b4 = reinterpret_cast<const float4*>(bias + colbase + c0);
-      // the biased logit stays in the register: an empty parent's -inf becomes a weight of exactly 0
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float4 b = b4[u];
-        a[c0 + 4 * u] = s[4 * u] + b.x;
-        a[c0 + 4 * u + 1] = s[4 * u + 1] + b.y;
-        a[c0 + 4 * u + 2] = s[4 * u + 2] + b.z;
-        a[c0 + 4 * u + 3] = s[4 * u + 3] + b.w;
-        mx = fmaxf(mx, fmaxf(a[c0 + 4 * u], a[c0 + 4 * u + 1]));
-        mx2 = fmaxf(mx2, fmaxf(a[c0 + 4 * u + 2], a[c0 + 4 * u + 3]));
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) a[c0 + e] = 0.f;
-    }
-  }
-  float m_run = fmaxf(mx, mx2) * sc;                    // scale > 0: the maximum commutes with it
-  if (NQ > 1) {
-    xm[cq * kRows + r] = m_run;
-    row_sync<NQ>(q);
-#pragma unroll
-    for (int u = 0; u < NQ; ++u) m_run = fmaxf(m_run, xm[u * kRows + r]);
-  }
-  // m_run is finite: at least one parent holds a key.
-
-  // ---- fp32 weights; exact denominator of the parent pass.  Empty parents carry a logit of -inf, hence
-  // a weight of exactly zero; every other logit is at most the maximum (up to one rounding).
-  float zfull = 0.f, zall = 0.f;                          // zall: sum of this thread's bf16-rounded weights x counts
-  {
-    float zf0 = 0.f, zf1 = 0.f, zf2 = 0.f, zf3 = 0.f;
-    const float negm = -m_run;
-#pragma unroll
-    for (int c0 = 0; c0 < QW; c0 += 16) {
-      if (c0 < my_cols) {
-        const float4* n4 = reinterpret_cast<const float4*>(cnt + colbase + c0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float4 n = n4[u];
-          a[c0 + 4 * u] = ex2(fmaf(a[c0 + 4 * u], sc, negm));
-          a[c0 + 4 * u + 1] = ex2(fmaf(a[c0 + 4 * u + 1], sc, negm));
-          a[c0 + 4 * u + 2] = ex2(fmaf(a[c0 + 4 * u + 2], sc, negm));
-          a[c0 + 4 * u + 3] = ex2(fmaf(a[c0 + 4 * u + 3], sc, negm));
-          zf0 = fmaf(a[c0 + 4 * u], n.x, zf0);
-          zf1 = fmaf(a[c0 + 4 * u + 1], n.y, zf1);
-          zf2 = fmaf(a[c0 + 4 * u + 2], n.z, zf2);
-          zf3 = fmaf(a[c0 + 4 * u + 3], n.w, zf3);
-        }
-        // Large tiles with few parents to refine: the bf16 weights go to shared memory (over the dead
-        // codebook) right here - the exponentials keep the XU pipe busy and the conversion (ALU pipe, stores)
-        // fills the issue slots they leave empty.  The selection is not known yet; what it removes is taken
-        // out of the denominator afterwards (P look-ups per row).
-        if constexpr (fuse) {
-          float am[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) am[e] = a[c0 + e];
-          zall += store_weights16<false>(CA, r, colbase + c0, cnt + colbase + c0, nullptr, am);
-        }
-      }
-    }
-    zfull = (zf0 + zf1) + (zf2 + zf3);
-    if (NQ > 1) {
-      xz[cq * kRows + r] = zfull;
-      row_sync<NQ>(q);
-      zfull = 0.f;
-#pragma unroll
-      for (int u = 0; u < NQ; ++u) zfull += xz[u * kRows + r];
-    }
-  }
-  // The importances are needed only to choose which parents to refine: with P = 0 (nothing refined) or
-  // P >= M (everything refined) the choice is fixed and the pass is skipped unless the caller wants them.
-  const bool need_w = (P > 0 && P < M) || p.importance_out != nullptr;
-  if (need_w) {
-    const float inv = (r < rows_valid) ? 1.f / zfull : 0.f;
-    // ---- importance: column sums of A_ij / z_i over the 128 rows (32 per warp, then 4 warps)
-    if constexpr ((QW & 31) == 0) {
-#pragma unroll
-      for (int c0 = 0; c0 < QW; c0 += 32) {
-        if (c0 < my_cols) {
-          float v[32];
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] = a[c0 + e] * inv;
-          const float colsum = transpose_reduce<32>(v, lane);
-          wpart[q * CT + colbase + c0 + lane] = colsum;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int c0 = 0; c0 < QW; c0 += 16) {
-        if (c0 < my_cols) {
-          float v[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] = a[c0 + e] * inv;
-          const float colsum = transpose_reduce<16>(v, lane);
-          if ((lane & 1) == 0) wpart[q * CT + colbase + c0 + (lane >> 1)] = colsum;
-        }
-      }
-    }
-  }
-  if (need_w) {
-    __syncthreads();
-    if (tid < M) {
-      const float wj = cnt[tid] * ((wpart[tid] + wpart[CT + tid]) + (wpart[2 * CT + tid] + wpart[3 * CT + tid]));
-      w[tid] = wj;
-      if (p.importance_out) p.importance_out[((size_t)bh * p.nblk + blk) * M + tid] = wj;
-    }
-    __syncthreads();
-  }
-
-  // ---- top-P by rank.  Non-negative floats order like their bit patterns, so the comparisons run on
-  // integers.  gt_j = number of strictly larger importances; parent j is selected if gt_j < P, except
-  // that when a group of EQUAL importances straddles the boundary only its lowest indices are kept.
-  // kT threads share one parent's scan.
-  {
-    const int kT = (kThreads >= 2 * M) ? 2 : 1;          // threads that share one parent's scan
-    const int j = (kT == 2) ? (tid >> 1) : tid, part = (kT == 2) ? (tid & 1) : 0;
-    const uint32_t* keys = reinterpret_cast<const uint32_t*>(w);
-    int* gstar = reinterpret_cast<int*>(&wmask[16]);
-    bool mine = false;
-    if (P >= M) {
-      mine = (j < M) && (part == 0);
-    } else if (P > 0) {
-      int gt = 0;
-      if (j < M) {
-        const uint32_t kj = keys[j];
-        const int span = M / kT, kb = part * span;
-        int g0 = 0, g1 = 0, g2 = 0, g3 = 0;              // four independent counters: no serial add chain
-        // 16 keys per trip (span is a multiple of 16): the four 16-byte loads are in flight together
-        // instead of one load -> compare -> add chain per trip
-        for (int k = kb; k < kb + span; k += 16) {
-          uint4 kq[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) kq[u] = *reinterpret_cast<const uint4*>(keys + k + 4 * u);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            asm("{\n\t.reg .pred p0, p1, p2, p3;\n\t"
-                "setp.gt.u32 p0, %4, %8;\n\tsetp.gt.u32 p1, %5, %8;\n\t"
-                "setp.gt.u32 p2, %6, %8;\n\tsetp.gt.u32 p3, %7, %8;\n\t"
-                "@p0 add.s32 %0, %0, 1;\n\t@p1 add.s32 %1, %1, 1;\n\t"
-                "@p2 add.s32 %2, %2, 1;\n\t@p3 add.s32 %3, %3, 1;\n\t}"
-                : "+r"(g0), "+r"(g1), "+r"(g2), "+r"(g3)
-                : "r"(kq[u].x), "r"(kq[u].y), "r"(kq[u].z), "r"(kq[u].w), "r"(kj));
-          }
-        }
-        gt = (g0 + g1) + (g2 + g3);
-      }
-      if (kT == 2) gt += __shfl_xor_sync(0xffffffffu, gt, 1);
-      const bool cand = (j < M) && (part == 0) && (gt < P);
-      if (tid == 0) *gstar = 0;
-      const int ncand = __syncthreads_count(cand);
-      mine = cand;
-      if (ncand > P) {                                   // uniform: equal importances straddle the boundary
-        if (cand) atomicMax(gstar, gt);                  // the tied group has the largest gt among candidates
-        __syncthreads();
-        const int g = *gstar;
-        const bool tied = cand && gt == g;
-        const uint32_t beq = __ballot_sync(0xffffffffu, tied);
-        if (lane == 0) wmask[warp] = beq;
-        __syncthreads();
-        int epos = __popc(beq & ((1u << lane) - 1u));
-        for (int u = 0; u < warp; ++u) epos += __popc(wmask[u]);
-        mine = cand && (gt < g || epos < P - g);
-        __syncthreads();
-      }
-    }
-    const uint32_t bal = __ballot_sync(0xffffffffu, mine);
-    if (lane == 0) wmask[warp] = bal;
-    __syncthreads();
-    if (mine) {
-      int pos = __popc(bal & ((1u << lane) - 1u));
-      for (int u = 0; u < warp; ++u) pos += __popc(wmask[u]);
-      sel_list[pos] = j;
-      cntk[j] = p.rho ? __ldg(p.rho + (size_t)bh * M + j) : 0.f;   // the share of its keys that stays with it
-      if (p.topp_out) p.topp_out[((size_t)bh * p.nblk + blk) * P + pos] = j;
-    }
-  }
-  // the output tile of the tile before must have left the child-code buffer before it is refilled (its
-  // store was issued a whole parent pass ago, so this does not wait in practice)
-  if (tid == 0 && store_pending) {
-    tma_store_wait_read();
-    store_pending = false;
-  }
-  __syncthreads();
-
-  // ---- first child chunk: start the asynchronous gather of its codeword rows now; it lands while the
-  // weight conversion below runs
-  const __nv_bfloat16* Cch = p.Cc + (size_t)h * M * C * D;
-  int ncols = min(PC, CHW);
-  int np16 = (ncols + 15) & ~15;
-  // Rows of a chunk, gathered into a K-major / row-per-codeword tile of np16 rows (kSubD sub-tiles of 64
-  // columns): local row e = src[sel_list[(e_first+e)/C] * C + (e_first+e)%C, :]; padding rows are zero.
-  // A thread keeps its 16-byte chunk column and walks down the rows (kThreads is a multiple of the chunks
-  // per row).
-  auto gather_rows = [&](unsigned char* tile, const __nv_bfloat16* src, int e_first) {
-    constexpr int kRowsPerPass = kThreads >> kLogChunks;   // a multiple of 8: a thread's swizzle phase is fixed
-    constexpr int kPasses = (CHW + kRowsPerPass - 1) / kRowsPerPass;
-    const int ch = tid & ((1 << kLogChunks) - 1), row0 = tid >> kLogChunks;
-    const uint32_t dst0 = smem_u32(tile) + (uint32_t)((ch >> 3) * (np16 * 128)) + sw128_offset(row0, (ch & 7) * 8);
-    const __nv_bfloat16* src_col = src + ch * 8;
-    int sel[kPasses];
-#pragma unroll
-    for (int it = 0; it < kPasses; ++it) {                 // the list look-ups first, all in flight together
-      const int e = e_first + row0 + it * kRowsPerPass;
-      sel[it] = (row0 + it * kRowsPerPass < ncols) ? sel_list[e >> logC] : 0;
-    }
-#pragma unroll
-    for (int it = 0; it < kPasses; ++it) {
-      const int row = row0 + it * kRowsPerPass;
-      const uint32_t dst = dst0 + (uint32_t)(it * kRowsPerPass * 128);
-      if (row < ncols) {
-        const int e = e_first + row;
-        const uint32_t off = (uint32_t)(((sel[it] << logC) + (e & (C - 1))) << kLogD);   // elements: < 2^31
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src_col + off) : "memory");
-      } else if (row < np16) {
-        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
-      }
-    }
-  };
-  auto gather_codes = [&](int e_first) {
-    float n_child = 0.f;
-    if (tid < ncols) {                                   // CHW <= 128 <= kThreads
-      const int e = e_first + tid;
-      n_child = ncs[(sel_list[e >> logC] << logC) + (e & (C - 1))];
-    }
-    gather_rows(CC, Cch, e_first);
-    if (tid < CHW) {
-      cntc[tid] = n_child;
-      biasc[tid] = n_child > 0.f ? 0.f : -INFINITY;
-    }
-  };
-  gather_codes(0);
-
-  // ---- bf16 weights into shared memory (over the dead codebook) + their denominator.  A refined parent
-  // is removed from the numerator by clearing its row of the value tile (d / 8 16-byte stores) and from the
-  // denominator by its zeroed count, so the weights themselves need no mask.
-  mbar_wait(bar_ld1, ph_in, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);   // value sums have landed
-  for (int u = tid; u < (min(P, M) << kLogChunks); u += kThreads) {
-    const int row = sel_list[u >> kLogChunks], ch = u & ((1 << kLogChunks) - 1);
-    // a refined parent keeps only the keys that stayed with it (Algorithm 1's masked scatter): its value row
-    // becomes the stay residual, Vbar_stay = Vbar_p - sum_c Vbar_c, in the same per-n_p units (all zero under
-    // the default rule, where every key moves to a child)
-    uint4 stay = make_uint4(0, 0, 0, 0);
-    if (p.Vsb) stay = __ldg(reinterpret_cast<const uint4*>(p.Vsb + ((size_t)bh * M + row) * D) + ch);
-    *reinterpret_cast<uint4*>(Vs + (ch >> 3) * (M * 128) + sw128_offset(row, (ch & 7) * 8)) = stay;
-  }
-  if constexpr (!fuse) {
-    // bf16 weights into shared memory (over the dead codebook) + their denominator; a refined parent's
-    // rounded weight enters the denominator with the share of its own term that it keeps (cntk)
-    float zloc = 0.f;
-#pragma unroll
-    for (int c0 = 0; c0 < QW; c0 += 16) {
-      if (c0 < my_cols) {
-        float am[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) am[e] = a[c0 + e];
-        zloc += store_weights16<true>(CA, r, colbase + c0, cnt + colbase + c0, cntk + colbase + c0, am);
-      }
-    }
-    xz2[cq * kRows + r] = zloc;
-  } else {
-    // denominator of the parent pass from the rounded weights, less what the refined parents no longer carry
-    // (all of it under the default rule, the share of the keys that moved to children under PARENT_STAYS);
-    // the row's NQ threads split the P look-ups
-    float fix = 0.f;
-    const int nsel = min(P, M);
-    for (int u0 = cq; u0 < nsel; u0 += 4 * NQ) {         // four look-ups in flight per trip
-      int jj[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) jj[t] = sel_list[min(u0 + t * NQ, nsel - 1)];
-      float wv[4], kv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const uint16_t hv =
-            *reinterpret_cast<const uint16_t*>(CA + (jj[t] >> 6) * (kRows * 128) + sw128_offset(r, jj[t] & 63));
-        wv[t] = __uint_as_float((uint32_t)hv << 16);
-        kv[t] = (u0 + t * NQ < nsel) ? 1.f - cntk[jj[t]] : 0.f;
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t) fix = fmaf(wv[t], kv[t], fix);
-    }
-    xz2[cq * kRows + r] = zall - fix;
-  }
-  cp_async_wait_all();
-  fence_proxy_async();
-  tc_fence_before();
-  __syncthreads();
-  float z_run = 0.f;
-#pragma unroll
-  for (int u = 0; u < NQ; ++u) z_run += xz2[u * kRows + r];
-
-  // ---- O = A . Vbar_p, and right behind it the first child chunk's logits
-  if (tid == 0) {
-    tc_fence_after();
-    if (mbar_wait(bar_ld1, ph_in, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND)) {
-      const uint32_t aa = smem_u32(CA), va = smem_u32(Vs);
-      for (int k = 0; k < M / 16; ++k)
-        umma_bf16(tmem_base + CT, umma_desc_sw128(aa + (k / 4) * kRows * 128 + (k % 4) * 32),
-                  umma_desc_sw128_mn(va + k * 2048, (uint32_t)(M * 128)), idesc_o, k > 0);
-    }
-    umma_commit(bar_pv);
-  }
-  // The child-score MMAs are issued by a lane of another warp: an issuing lane stalls at the tensor pipe's
-  // pace, and two short stalls side by side delay the next CTA-wide barrier less than one long one.
-  if (tid == kScLane && PC > 0) {
-    tc_fence_after();
-    const uint32_t idesc = umma_idesc_bf16(kRows, np16);
-    const uint32_t qa = smem_u32(Qs), ca = smem_u32(CC);
+  // Q . rows^T into the logit columns.  (Descriptors count 16-byte units: 2 per 32 bytes, 8 per 128-byte row.)
+  auto logits_mma = [&](uint64_t bdesc, int rows) {
+    const uint32_t idesc = umma_idesc_bf16(kRows, rows);
+    const uint64_t qd = umma_desc_sw128(smem_u32(Qs));
 #pragma unroll
     for (int k = 0; k < D / 16; ++k)
-      umma_bf16(tmem_base, umma_desc_sw128(qa + (k / 4) * kRows * 128 + (k % 4) * 32),
-                umma_desc_sw128(ca + (k / 4) * np16 * 128 + (k % 4) * 32), idesc, k > 0);
-    umma_commit(bar_s);
-  }
-
-  // ---- child chunks
-  const __nv_bfloat16* Vch = p.Vcb + (size_t)bh * M * C * D;
-  for (int e0 = 0; e0 < PC; e0 += CHW) {
-    // The previous second MMA must have released A and Vs before they are rewritten.
-    mbar_wait(bar_pv, ph_pv, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-    ph_pv ^= 1;
-    tc_fence_after();
-    // value rows of this chunk (the same gather as for its codeword rows).  Asynchronous copies: they land
-    // while the chunk's logits are turned into weights.  Padding rows are zero: they meet finite weights.
-    gather_rows(Vs, Vch, e0);
-
-    // ---- child logits: running maximum over non-empty children
-    mbar_wait(bar_s, ph_s, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-    ph_s ^= 1;
-    tc_fence_after();
-    if (tid == 0 && has_next && e0 + CHW >= PC) issue_q(next_tile);   // the last logits are done: Q is dead
-    const int my_c = min(max(np16 - cq * QWC, 0), QWC);
-    // With 32 child columns per thread the chunk's logits are read from TMEM once and stay in registers with
-    // their bias (an empty child's -inf becomes a weight of exactly 0); with 64 per thread they are read twice
-    // (the register copy measured slower there: N=16384 M=64 P=16 attend 43.4 -> 46.5 us; c3 179.7 -> 176.2).
-    constexpr bool kChildRegs = QWC <= 32;
-    float cl[kChildRegs ? QWC : 1];
-    float mxc = -INFINITY;
-    if constexpr (kChildRegs) {
-#pragma unroll
-      for (int c0 = 0; c0 < QWC; c0 += 16) {
-        if (c0 < my_c) {                                 // warp-uniform
-          float s[16];
-          tmem_ld16(t_sc + c0, s);
-          const float4* b4 = reinterpret_cast<const float4*>(biasc + cq * QWC + c0);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float4 b = b4[u];
-            cl[c0 + 4 * u] = s[4 * u] + b.x;
-            cl[c0 + 4 * u + 1] = s[4 * u + 1] + b.y;
-            cl[c0 + 4 * u + 2] = s[4 * u + 2] + b.z;
-            cl[c0 + 4 * u + 3] = s[4 * u + 3] + b.w;
-            mxc = fmaxf(mxc, fmaxf(cl[c0 + 4 * u], cl[c0 + 4 * u + 1]));
-            mxc = fmaxf(mxc, fmaxf(cl[c0 + 4 * u + 2], cl[c0 + 4 * u + 3]));
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) cl[c0 + e] = -INFINITY;
-        }
+      umma_bf16(tmem_base, qd + (uint64_t)((k / 4) * (kRows * 8) + (k % 4) * 2),
+                bdesc + (uint64_t)((k / 4) * rows * 8 + (k % 4) * 2), idesc, k > 0);
+  };
+  // One warp: S = Q . Cp^T of a tile once its operands have landed.
+  auto issue_s = [&](bool new_cp) {
+    if (elect_one()) {
+      bool ok = mbar_wait(bar_q, ph_q, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+      if (new_cp) ok = mbar_wait(bar_cp, ph_cp, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND) && ok;
+      if (ok) {
+        tc_fence_after();
+        logits_mma(umma_desc_sw128(smem_u32(CA)), M);
       }
+      umma_commit(bar_s);
+    }
+    __syncwarp();
+    ph_q ^= 1;
+    if (new_cp) ph_cp ^= 1;
+  };
+  auto issue_sc = [&](int rows) {                        // one warp: child logits
+    if (elect_one()) {
+      tc_fence_after();
+      logits_mma(umma_desc_sw128(smem_u32(CC)), rows);
+      umma_commit(bar_s);
+    }
+    __syncwarp();
+  };
+  // One warp: O (+)= weights (TMEM columns from w_col) . value rows
+  auto issue_o = [&](const unsigned char* values, int rows, int w_col, bool accumulate, uint64_t* bar) {
+    if (elect_one()) {
+      tc_fence_after();
+      const uint64_t vd = umma_desc_sw128_mn(smem_u32(values), (uint32_t)(rows * 128));
+      const uint64_t ad = umma_desc_sw128(smem_u32(CA));
+#pragma unroll
+      for (int k = 0; k < CT / 16; ++k)
+        if (16 * k < rows) {
+          if constexpr (kTW)
+            umma_bf16_ts(tmem_base + L::tO, tmem_base + w_col + 8 * k, vd + (uint64_t)(128 * k), idesc_o, accumulate || k > 0);
+          else
+            umma_bf16(tmem_base + L::tO, ad + (uint64_t)((k / 4) * (kRows * 8) + (k % 4) * 2), vd + (uint64_t)(128 * k),
+                      idesc_o, accumulate || k > 0);
+        }
+      umma_commit(bar);
+    }
+    __syncwarp();
+  };
+  // Weights of 32 columns (col0 a multiple of 32) of this warp's rows -> A operand: pk[b][h] = block b, row h.
+  const uint32_t a_row = smem_u32(CA) + (uint32_t)(r * 128 + ((lane & 7) << 4));
+  auto put_weights = [&](int w_col, int col0, const uint32_t (&pk)[4][4]) {
+    if constexpr (kTW) {
+      const uint32_t v[2][8] = {{pk[0][0], pk[0][1], pk[1][0], pk[1][1], pk[2][0], pk[2][1], pk[3][0], pk[3][1]},
+                                {pk[0][2], pk[0][3], pk[1][2], pk[1][3], pk[2][2], pk[2][3], pk[3][2], pk[3][3]}};
+      tmem_st_weights(t_row + (uint32_t)(w_col + (col0 >> 1)), v);
     } else {
-      for (int c0 = 0; c0 < my_c; c0 += 16) {
-        float s[16];
-        tmem_ld16(t_sc + c0, s);
-        const float4* b4 = reinterpret_cast<const float4*>(biasc + cq * QWC + c0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float4 b = b4[u];
-          mxc = fmaxf(mxc, fmaxf(s[4 * u] + b.x, s[4 * u + 1] + b.y));
-          mxc = fmaxf(mxc, fmaxf(s[4 * u + 2] + b.z, s[4 * u + 3] + b.w));
-        }
+      for (int b = 0; b < 4; ++b) {
+        const int col = col0 + 8 * b;
+        stmatrix4((a_row + (uint32_t)((col >> 6) * (kRows * 128))) ^ (uint32_t)(((col >> 3) & 7) << 4), pk[b][0], pk[b][1],
+                  pk[b][2], pk[b][3]);
       }
     }
-    float m_c = mxc * sc;
-    if (NQ > 1) {
-      xm[cq * kRows + r] = m_c;
-      row_sync<NQ>(q);
-#pragma unroll
-      for (int u = 0; u < NQ; ++u) m_c = fmaxf(m_c, xm[u * kRows + r]);
-    }
-    // Any reference value works as long as numerator and denominator share it.  The running one is
-    // kept unless the children exceed it by more than 2^kLazyLog2 (weights up to that factor above 1 are
-    // harmless in fp32 and bf16), which spares most rows the rescaling of O and z.
-    constexpr float kLazyLog2 = 8.f;
-    const float m_new = (m_c > m_run + kLazyLog2) ? m_c : m_run;
-    const float negm = -m_new;
-    // ---- rescale what has been accumulated if this row's maximum moved
-    const float alpha = ex2(m_run + negm);
-    if (__any_sync(0xffffffffu, alpha < 1.f)) {
-      for (int c0 = 0; c0 < D / NQ; c0 += 16) {
-        float o[16];
-        tmem_ld16(t_o + c0, o);
-#pragma unroll
-        for (int e = 0; e < 16; ++e) o[e] *= alpha;
-        tmem_st16(t_o + c0, o);
-      }
-      tmem_st_wait();
-    }
-    z_run *= alpha;
-    m_run = m_new;
-    // ---- bf16 weights of the children over the parents' (consumed) weights
-    {
-      float zloc = 0.f;
-      if constexpr (kChildRegs) {
-#pragma unroll
-        for (int c0 = 0; c0 < QWC; c0 += 16) {
-          if (c0 < my_c) {
-            float a[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) a[e] = ex2(fmaf(cl[c0 + e], sc, negm));
-            zloc += store_weights16<false>(CA, r, cq * QWC + c0, cntc + cq * QWC + c0, nullptr, a);
-          }
-        }
-      } else {
-        for (int c0 = 0; c0 < my_c; c0 += 16) {
-          float a[16];
-          tmem_ld16(t_sc + c0, a);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) a[e] = ex2(fminf(fmaf(a[e], sc, negm), kLazyLog2));   // clamp: empty children
-          zloc += store_weights16<false>(CA, r, cq * QWC + c0, cntc + cq * QWC + c0, nullptr, a);
-        }
-      }
-      xz2[cq * kRows + r] = zloc;
-    }
+  };
+  auto weights_done = [&]() {                            // before the barrier ahead of the MMA that reads them
+    if constexpr (kTW) tmem_st_wait();
     cp_async_wait_all();
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
+  };
+  // The values a fragment thread needs of rows g + 8 h, from the lane that stands for the row.
+  auto to_frag = [&](float v, float (&out)[4]) {
 #pragma unroll
-    for (int u = 0; u < NQ; ++u) z_run += xz2[u * kRows + r];
+    for (int h = 0; h < 4; ++h) out[h] = __shfl_sync(0xffffffffu, v, g + 8 * h);
+  };
 
-    // ---- O += A_c . Vbar_c; then stage the next chunk's codes (the logits MMA of this chunk is done)
-    const int e_next = e0 + CHW;
-    if (tid == 0) {
-      tc_fence_after();
-      const uint32_t aa = smem_u32(CA), va = smem_u32(Vs);
-      for (int k = 0; k < np16 / 16; ++k)
-        umma_bf16(tmem_base + CT, umma_desc_sw128(aa + (k / 4) * kRows * 128 + (k % 4) * 32),
-                  umma_desc_sw128_mn(va + k * 2048, (uint32_t)(np16 * 128)), idesc_o, true);
-      umma_commit(bar_pv);
-    }
-    if (e_next < PC) {
-      ncols = min(PC - e_next, CHW);
-      np16 = (ncols + 15) & ~15;
-      gather_codes(e_next);
-      cp_async_wait_all();
-      fence_proxy_async();
-      tc_fence_before();
+  if (warp == kVWarp) issue_s(true);
+  bool first = true, new_bh = true;                      // new_bh: counts (and V) of another (b, h) than the tile before
+  bool store_pending = false;                            // warp 0: a TMA store may still be reading the staging area
+  for (int tile = tile0; tile < tile1; ++tile) {
+    const int i0 = blk * kRows;
+    const int rows_valid = min(kRows, p.Nq - i0);
+    const bool has_next = tile + 1 < tile1;
+    const int nbh = blk + 1 == p.nblk ? bh + 1 : bh, nblk_ = blk + 1 == p.nblk ? 0 : blk + 1;
+    const bool next_new_bh = has_next && nbh != bh;
+    const bool next_new_head = next_new_bh && p.H > 1;
+    const bool next_new_cp = has_next && (!kTW || next_new_head || (L::kCodesInCA && PC > 0));
+    const bool next_new_v = has_next && (STAYS || !L::kStageInCC || next_new_bh);
+    // V of this tile: loaded behind the last use of the one before (below), except for the first tile
+    const bool new_v = STAYS || !L::kStageInCC || new_bh;
+
+    if (new_bh) {
+      // ---- Part 2 reads what the earlier kernels of this call wrote: status word, counts, value means.  (Loaded
+      // with statements the compiler cannot move ahead of the dependency wait.)
+      static_assert(CT <= kThreads && 2 * CT <= 4 * kThreads, "one count load per thread");
+      if (first) pdl_wait();
+      float n_reg = 0.f;
+      float4 nc_reg = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tid < M) n_reg = ld_after_wait(p.np_ + (size_t)bh * M + tid);
+      if (PC > 0 && tid < ((M * C) >> 2))
+        nc_reg = ld_after_wait(reinterpret_cast<const float4*>(p.nc + (size_t)bh * M * C) + tid);
+      if (first && warp == 0 && elect_one()) {
+        issue_v(bh);
+        // a wait that expired in an earlier CTA or kernel of this call: do not start more work
+        early_exit = (p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0);
+      }
+      if (tid < CT) {
+        cnt[parent_pos(tid)] = n_reg;
+        bias[parent_pos(tid)] = n_reg > 0.f ? 0.f : -INFINITY;
+      }
+      // every child's key count: the gathers below pick theirs from shared memory instead of waiting for a
+      // dependent global load once the selection is known (log2 0 = -inf: an empty child's weight is exactly 0)
+      if (PC > 0 && tid < ((M * C) >> 2))
+        reinterpret_cast<float4*>(ncs)[tid] = make_float4(log2f(nc_reg.x), log2f(nc_reg.y), log2f(nc_reg.z), log2f(nc_reg.w));
       __syncthreads();
-      if (tid == kScLane) {
-        tc_fence_after();
-        const uint32_t idesc = umma_idesc_bf16(kRows, np16);
-        const uint32_t qa = smem_u32(Qs), ca = smem_u32(CC);
+      if (first && early_exit) {
+        // let the MMA and the load already in flight finish, then leave cleanly
+        mbar_wait(bar_s, 0, abort_flag, nullptr, 0);
+        mbar_wait(bar_v, 0, abort_flag, nullptr, 0);
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 1) tmem_dealloc(tmem_base, L::tmem_cols);
+        return;
+      }
+      first = false;
+    }
+
+    // ---- parents: this thread's logits (4 rows x QW / 8 column pairs) are read from TMEM once and stay in
+    // registers through the exponentials, the importance sums and the conversion to bf16.  An empty parent's
+    // -inf bias becomes a weight of exactly 0.
+    mbar_wait(bar_s, ph_s, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+    ph_s ^= 1;
+    tc_fence_after();
+    if (warp == 0 && PC == 0 && has_next && elect_one()) issue_q(nbh, nblk_);   // no child logits will read this Q tile
+    if (warp == 0 && kTW && next_new_cp && !(L::kCodesInCA && PC > 0) && elect_one())
+      issue_cp(nbh, kSubD);                              // the codebook of the head that follows
+    f32x2 a[4][NB];                                      // [row h][block]
+    float m_run[4];                                      // maximum of the rows, log2 units
 #pragma unroll
-        for (int k = 0; k < D / 16; ++k)
-          umma_bf16(tmem_base, umma_desc_sw128(qa + (k / 4) * kRows * 128 + (k % 4) * 32),
-                    umma_desc_sw128(ca + (k / 4) * np16 * 128 + (k % 4) * 32), idesc, k > 0);
-        umma_commit(bar_s);
+    for (int h = 0; h < 4; ++h) m_run[h] = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (32 * c < my_cols) {                            // warp-uniform
+        uint32_t s[2][16];
+        tmem_ld_frag<4>(t_s + 32 * c, s);
+        f32x2 bi[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) bi[b] = *reinterpret_cast<const f32x2*>(bias + colbase + 32 * c + 8 * b + 2 * t4);
+        tmem_ld_wait_frag<4>(s);
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const f32x2 v = add2(pack2u(s[h >> 1][4 * b + 2 * (h & 1)], s[h >> 1][4 * b + 2 * (h & 1) + 1]), bi[b]);
+            a[h][4 * c + b] = v;
+            float lo, hi;
+            unpack2(v, lo, hi);
+            m_run[h] = max3(m_run[h], lo, hi);
+          }
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int h = 0; h < 4; ++h) a[h][4 * c + b] = 0;
       }
     }
-  }
-
-  // ---- epilogue: Y = O / z
-  const bool o_ok = mbar_wait(bar_pv, ph_pv, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
-  ph_pv ^= 1;
-  tc_fence_after();
-  // the last value MMA has released the weight tile and the value tile: the next tile's codebook and
-  // parent value rows load while this tile's output is written
-  if (tid == 0 && has_next) {
-    issue_cp(next_tile);
-    if (kStageInCC) issue_vp(next_tile);
-  }
-  // The output tile is staged in shared memory in the layout of the Q load and written with TMA tile
-  // stores; rows past Nq are clipped by the tensor map.  Staging area: see the top of the tile loop.
-  unsigned char* stage = kStageInCC ? CC : Vs;
-  if (o_ok) {
-    const float inv = 1.f / z_run;
-    for (int c0 = 0; c0 < D / NQ; c0 += 16) {
-      float o[16];
-      tmem_ld16(t_o + c0, o);
-      uint32_t pk[8];
 #pragma unroll
-      for (int e = 0; e < 16; e += 2) pk[e >> 1] = pack_bf16(o[e] * inv, o[e + 1] * inv);
-      const int col0 = cq * (D / NQ) + c0;
-      unsigned char* sub = stage + (col0 >> 6) * (kRows * 128);
-      *reinterpret_cast<uint4*>(sub + sw128_offset(r, col0 & 63)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-      *reinterpret_cast<uint4*>(sub + sw128_offset(r, (col0 & 63) + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    for (int h = 0; h < 4; ++h) m_run[h] = quad_max(m_run[h]) * sc;   // scale > 0: the maximum commutes with it
+    if (NQ > 1) {
+      xm[cq * kRows + q * 32 + g + 8 * t4] = pick4(m_run, t4);
+      row_sync<NQ>(q);
+      float m = xm[r];                                   // of row `lane`
+#pragma unroll
+      for (int u = 1; u < NQ; ++u) m = fmaxf(m, xm[u * kRows + r]);
+      to_frag(m, m_run);
     }
-    fence_proxy_async();
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (tid == 0 && o_ok) {
+    // m_run is finite: at least one parent holds a key.
+
+    // ---- fp32 weights and the exact denominator.  This lane's columns are the codewords t, t + 4, ... of the slice
+    // in ascending order: one chain per row, the quad adds (0 + 1) + (2 + 3).
+    float iz[4];                                         // 1 / z, 0 for rows past the end
+    {
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+      const f32x2 sc2 = pack2(sc, sc);
+      f32x2 nm[4];
 #pragma unroll
-    for (int s2 = 0; s2 < kSubD; ++s2) tma_store_3d(&tmY, stage + s2 * kRows * 128, s2 * 64, i0, bh);
-    tma_store_commit();
-    if (has_next) store_pending = true;                // waited for before the next tile refills CC
-    else tma_store_wait_read();                        // before the CTA may leave
-  }
-  ph_in ^= 1;
+      for (int h = 0; h < 4; ++h) nm[h] = pack2(-m_run[h], -m_run[h]);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (32 * c < my_cols) {                          // 64 independent exponentials per step
+          float2 n2[4];
+#pragma unroll
+          for (int b = 0; b < 4; ++b) n2[b] = *reinterpret_cast<const float2*>(cnt + colbase + 32 * c + 8 * b + 2 * t4);
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+              f32x2& x = a[h][4 * c + b];
+              float lo, hi;
+              unpack2(fma2(x, sc2, nm[h]), lo, hi);
+              lo = ex2(lo);
+              hi = ex2(hi);
+              z[h] = fmaf(hi, n2[b].y, fmaf(lo, n2[b].x, z[h]));
+              x = pack2(lo, hi);
+            }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) z[h] = quad_sum(z[h]);
+      float zr;                                          // of row `lane`
+      if (NQ > 1) {
+        xz[cq * kRows + q * 32 + g + 8 * t4] = pick4(z, t4);
+        row_sync<NQ>(q);
+        zr = xz[r];
+#pragma unroll
+        for (int u = 1; u < NQ; ++u) zr += xz[u * kRows + r];
+      } else {
+        zr = __shfl_sync(0xffffffffu, pick4(z, t4), 4 * (lane & 7) + (lane >> 3));
+      }
+      to_frag(r < rows_valid ? 1.f / zr : 0.f, iz);
+    }
+
+    // The importances are needed only to choose which parents to refine: with P = 0 (nothing refined) or
+    // P >= M (everything refined) the choice is fixed and the pass is skipped unless the caller wants them.
+    const bool need_w = (P > 0 && P < M) || p.importance_out != nullptr;
+    uint32_t key = 0;                                    // importance of parent `tid` (non-negative float bits)
+    int nz = 0;                                          // parents with an importance above zero
+    if (tid < CT) {                                      // nothing is refined yet
+      if constexpr (STAYS) keep_f[tid] = 1.f;
+      else keep_m[tid] = 0xFFFFu;
+    }
+    if (need_w) {
+      // ---- importance: column sums of A_ij / z_i over the 128 rows (4 in registers, 8 lanes, 4 warps)
+      f32x2 inv[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) inv[h] = pack2(iz[h], iz[h]);
+      f32x2 v[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+        v[b] = add2(add2(mul2(a[0][b], inv[0]), mul2(a[2][b], inv[2])), add2(mul2(a[1][b], inv[1]), mul2(a[3][b], inv[3])));
+      const f32x2 colsum = reduce_rows<NB>(v, lane);
+      const int b = NB == 8 ? g : g >> 1;
+      if (NB == 8 || (g & 1) == 0) *reinterpret_cast<f32x2*>(wpart + q * CT + colbase + 8 * b + 2 * t4) = colsum;
+      __syncthreads();
+      float wj = 0.f;
+      if (tid < M) {
+        const int c = parent_pos(tid);
+        wj = cnt[c] * ((wpart[c] + wpart[CT + c]) + (wpart[2 * CT + c] + wpart[3 * CT + c]));
+        w[tid] = wj;
+        const uint32_t m_ = __ballot_sync(0xffffffffu, wj > 0.f);   // M is a multiple of 32
+        if (lane == 0) { nzmask[warp] = m_; selmask[warp] = 0u; }
+        if (p.importance_out) p.importance_out[((size_t)bh * p.nblk + blk) * M + tid] = wj;
+      }
+      if (tid == 0) *ncand_s = 0;
+      key = __float_as_uint(wj);
+      nz = __syncthreads_count(wj > 0.f);
+    }
+
+    // ---- top-P, ties to the lower index.  Non-negative floats order like their bit patterns, so the comparisons
+    // run on integers.
+    auto choose = [&](int j, int pos) {
+      sel_list[pos] = j;
+      if constexpr (STAYS) keep_f[parent_pos(j)] = __ldg(p.rho + (size_t)bh * M + j);   // the share of its keys that stays with it
+      else keep_m[parent_pos(j)] = 0;
+    };
+    int32_t* topp_out = p.topp_out ? p.topp_out + ((size_t)bh * p.nblk + blk) * P : nullptr;
+    if (P >= M) {
+      if (!need_w) __syncthreads();                      // keep[] reset above by other threads
+      if (tid < M) {
+        choose(tid, tid);
+        if (topp_out) topp_out[tid] = tid;
+      }
+    } else if (P > 0) {
+      const int K = M >> 5;                              // keys per lane (32 k + lane), <= 8
+      const uint32_t below = (1u << lane) - 1u;
+      if (nz <= P) {
+        // Peaked attention leaves most importances at exactly zero: all others are refined, and as many of the
+        // zeros as are missing, lowest index first.  No ranking.
+        if (warp < K) {
+          int nz_before = 0;
+          for (int k = 0; k < warp; ++k) nz_before += __popc(nzmask[k]);
+          const uint32_t mk = nzmask[warp];
+          const int zr = 32 * warp - nz_before + __popc(~mk & below);   // zeros before this parent
+          if (((mk >> lane) & 1u) || zr < P - nz) {
+            const int pos = nz_before + __popc(mk & below) + min(zr, P - nz);
+            choose(warp * 32 + lane, pos);
+            if (topp_out) topp_out[pos] = warp * 32 + lane;
+          }
+        }
+      } else {
+        // Only candidates are ranked, those at or above a bound that at least P keys reach.  The bound is the
+        // largest of 32 sample keys (the first 32 parents') that has at least P keys at or above it, else the
+        // smallest key above zero; each warp counts for its share of the samples.
+        constexpr int kPer = 32 / (kThreads / 32);       // samples per warp
+        uint32_t kk[CT / 32];
+#pragma unroll
+        for (int k = 0; k < CT / 32; ++k) kk[k] = k < K ? reinterpret_cast<const uint32_t*>(w)[32 * k + lane] : 0u;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+          const uint32_t smp = __shfl_sync(0xffffffffu, kk[0], warp * kPer + j);
+          int c = 0;
+#pragma unroll
+          for (int k = 0; k < CT / 32; ++k) c += kk[k] >= smp;
+          c = __reduce_add_sync(0xffffffffu, c);
+          if (lane == 0) wcount[warp * kPer + j] = smp > 0u ? c : 0;
+        }
+        __syncthreads();
+        const uint32_t bound = max(__reduce_max_sync(0xffffffffu, wcount[lane] >= P ? kk[0] : 0u), 1u);
+        if (warp < K) {                                  // candidates of this warp's 32 parents -> list, in any order
+          const uint32_t mk = __ballot_sync(0xffffffffu, key >= bound);
+          int base = 0;
+          if (lane == 0) base = atomicAdd(ncand_s, __popc(mk));
+          base = __shfl_sync(0xffffffffu, base, 0);
+          // importance above, complement of the index below: larger means refined earlier, no two are equal
+          if ((mk >> lane) & 1u) cand[base + __popc(mk & below)] = ((uint64_t)key << 32) | (uint32_t)(0xFFFF - tid);
+        }
+        __syncthreads();
+        // rank of every candidate among them; 2^lt threads share a candidate.  The list of refined parents is
+        // ordered by rank.
+        const int ncand = *ncand_s;
+        constexpr int kLogT = NQ == 4 ? 9 : (NQ == 2 ? 8 : 7);
+        const int lt = max(0, min(4, kLogT - (32 - __clz(ncand - 1))));
+        const int i = tid >> lt, part = tid & ((1 << lt) - 1);
+        const uint64_t mine = i < ncand ? cand[i] : 0;
+        int rank = 0;
+        for (int k = part; k < ncand; k += 4 << lt) {    // four in flight; past the end only the comparison is masked
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int ku = k + (u << lt);
+            rank += (cand[min(ku, CT - 1)] > mine) & (ku < ncand);
+          }
+        }
+#pragma unroll
+        for (int o = 1; o <= 8; o <<= 1) {
+          const int other = __shfl_xor_sync(0xffffffffu, rank, o);
+          if (o < (1 << lt)) rank += other;
+        }
+        if (i < ncand && part == 0 && rank < P) {
+          const int j = 0xFFFF - (int)((uint32_t)mine & 0xFFFFu);
+          choose(j, rank);
+          if (topp_out) atomicOr(&selmask[j >> 5], 1u << (j & 31));
+        }
+        if (topp_out) {                                  // the caller's list is ascending
+          __syncthreads();
+          if (warp < K) {
+            const uint32_t mk = selmask[warp];
+            int pos = __popc(mk & below);
+            for (int k = 0; k < warp; ++k) pos += __popc(selmask[k]);
+            if ((mk >> lane) & 1u) topp_out[pos] = tid;
+          }
+        }
+      }
+    }
+    // the output tile of the tile before must have left its staging area before that is refilled (its store was
+    // issued a whole parent pass ago, so this does not wait in practice)
+    if (warp == 0 && store_pending) {
+      if (elect_one()) {
+        tma_store_wait_read();
+        if (!L::kStageInCC) issue_v(bh);                 // this tile's values: their buffer was the staging area
+      }
+      store_pending = false;
+    }
+    __syncthreads();
+
+    // ---- first child chunk: start the asynchronous gather of its codeword rows now; it lands while the
+    // weight conversion below runs
+    const __nv_bfloat16* Cch = p.Cc + (size_t)(bh % p.H) * M * C * D;
+    const __nv_bfloat16* Vch = p.Vcb + (size_t)bh * M * C * D;
+    int ncols = min(PC, CHW);
+    int np32 = (ncols + 31) & ~31;
+    // Rows of a chunk, gathered into a row-per-codeword tile of np32 rows (kSubD sub-tiles of 64 columns): local
+    // row e = src[sel_list[(e_first+e)/C] * C + (e_first+e)%C, :]; padding rows are zero.  A thread keeps its
+    // 16-byte chunk column and walks down the rows (kThreads is a multiple of the chunks per row).
+    auto gather_rows = [&](unsigned char* dst_tile, const __nv_bfloat16* src, int e_first) {
+      constexpr int kRowsPerPass = kThreads >> kLogChunks;   // a multiple of 8: a thread's swizzle phase is fixed
+      constexpr int kPasses = (CHW + kRowsPerPass - 1) / kRowsPerPass;
+      const int ch = tid & ((1 << kLogChunks) - 1), row0 = tid >> kLogChunks;
+      const uint32_t dst0 = smem_u32(dst_tile) + (uint32_t)((ch >> 3) * (np32 * 128)) + sw128_offset(row0, (ch & 7) * 8);
+      const __nv_bfloat16* src_col = src + ch * 8;
+      int sel[kPasses];
+#pragma unroll
+      for (int it = 0; it < kPasses; ++it) {                 // the list look-ups first, all in flight together
+        const int e = e_first + row0 + it * kRowsPerPass;
+        sel[it] = (row0 + it * kRowsPerPass < ncols) ? sel_list[e >> logC] : 0;
+      }
+#pragma unroll
+      for (int it = 0; it < kPasses; ++it) {
+        const int row = row0 + it * kRowsPerPass;
+        const uint32_t dst = dst0 + (uint32_t)(it * kRowsPerPass * 128);
+        if (row < ncols) {
+          const int e = e_first + row;
+          const uint32_t off = (uint32_t)(((sel[it] << logC) + (e & (C - 1))) << kLogD);   // elements: < 2^31
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src_col + off) : "memory");
+        } else if (row < np32) {
+          asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
+        }
+      }
+    };
+    auto gather_codes = [&](int e_first) {
+      float l2 = -INFINITY;
+      if (tid < ncols) {                                   // CHW <= 128 <= kThreads
+        const int e = e_first + tid;
+        l2 = ncs[(sel_list[e >> logC] << logC) + (e & (C - 1))];
+      }
+      gather_rows(CC, Cch, e_first);
+      if (tid < CHW) l2n[tid] = l2;
+    };
+    if (PC > 0) gather_codes(0);
+
+    // ---- bf16 weights -> A operand, and their denominator (this thread's share of its rows; put together at the
+    // end of the tile).  Default rule: a refined parent's weight is masked to zero.
+    if (new_v) {                                           // parent values have landed (needed by the MMA and the stay rows)
+      mbar_wait(bar_v, ph_v, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+      ph_v ^= 1;
+    }
+    if constexpr (STAYS) {
+      // a refined parent keeps only the keys that stayed with it (Algorithm 1's masked scatter): its value row
+      // becomes the stay residual, Vbar_stay = Vbar_p - sum_c Vbar_c, in the same per-n_p units
+      for (int u = tid; u < (min(P, M) << kLogChunks); u += kThreads) {
+        const int row = sel_list[u >> kLogChunks], ch = u & ((1 << kLogChunks) - 1);
+        *reinterpret_cast<uint4*>(Vs + (ch >> 3) * (M * 128) + sw128_offset(parent_pos(row), (ch & 7) * 8)) =
+            __ldg(reinterpret_cast<const uint4*>(p.Vsb + ((size_t)bh * M + row) * D) + ch);
+      }
+    }
+    float z_run[4] = {0.f, 0.f, 0.f, 0.f};
+    {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (32 * c < my_cols) {
+          uint32_t pk[4][4];
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const f32x2 n2 = *reinterpret_cast<const f32x2*>(cnt + colbase + 32 * c + 8 * b + 2 * t4);
+            uint32_t km = 0;
+            float2 kf = make_float2(0.f, 0.f);
+            if constexpr (STAYS) kf = *reinterpret_cast<const float2*>(keep_f + colbase + 32 * c + 8 * b + 2 * t4);
+            else km = *reinterpret_cast<const uint32_t*>(keep_m + colbase + 32 * c + 8 * b + 2 * t4);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+              float lo, hi;
+              unpack2(mul2(a[h][4 * c + b], n2), lo, hi);
+              pk[b][h] = pack_bf16(lo, hi);
+              if constexpr (STAYS) {
+                z_run[h] = fmaf(__uint_as_float(pk[b][h] << 16), kf.x, z_run[h]);
+                z_run[h] = fmaf(__uint_as_float(pk[b][h] & 0xFFFF0000u), kf.y, z_run[h]);
+              } else {
+                pk[b][h] &= km;
+                add_bf16x2(z_run[h], pk[b][h]);
+              }
+            }
+          }
+          put_weights(L::tW, colbase + 32 * c, pk);
+        }
+      }
+    }
+    weights_done();
+    __syncthreads();
+
+    // ---- the first child chunk's logits, and behind them O = A . Vbar_p: the tensor pipe works in order, the
+    // children's logits are waited for, O is not.  An issuing lane is held up at the tensor pipe's pace, so O has
+    // another warp, which does its share of the gather first.
+    auto pair_barrier = [&](bool wait) {                   // warp 0 arrives, kVWarp waits
+      if (wait) asm volatile("bar.sync 5, 64;" ::: "memory");
+      else asm volatile("bar.arrive 5, 64;" ::: "memory");
+    };
+    if (warp == 0 && PC > 0) {
+      issue_sc(np32);
+      pair_barrier(false);
+    }
+    if (kSepCV && PC > 0) gather_rows(CV, Vch, 0);         // while the logits are computed
+    if (warp == kVWarp) {
+      if (PC > 0) pair_barrier(true);
+      issue_o(Vs, M, L::tW, false, bar_o);
+    }
+
+    // ---- child chunks
+    for (int e0 = 0; e0 < PC; e0 += CHW) {
+      mbar_wait(bar_s, ph_s, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+      ph_s ^= 1;
+      tc_fence_after();
+      const bool last = e0 + CHW >= PC;
+      if (warp == 0 && last && has_next && elect_one()) {  // the last logits are done: Q is dead, and so are the codes
+        issue_q(nbh, nblk_);
+        if (L::kCodesInCA) issue_cp(nbh, (next_new_head || M < CT) ? kSubD : 1);
+      }
+      if (e0 > 0) {                                        // the chunk before has left the weights and the value rows
+        mbar_wait(bar_pv, ph_pv, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+        ph_pv ^= 1;
+      }
+      if constexpr (!kSepCV) gather_rows(CC, Vch, e0);     // the codes are dead: the values take their place
+      else if (e0 > 0) gather_rows(CV, Vch, e0);
+      tc_fence_after();
+      bool o_done = L::kSepW || e0 > 0;                    // the weights' columns are free
+      const int my_c = min(max(np32 - cq * QWC, 0), QWC);  // multiple of 32
+      float zc[4];
+      for (;;) {
+        // bf16 weights exp2(s - m + log2 n) of the children, their sum
+        const f32x2 sc2 = pack2(sc, sc);
+        f32x2 nm[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) { nm[h] = pack2(-m_run[h], -m_run[h]); zc[h] = 0.f; }
+#pragma unroll
+        for (int c = 0; c < NCC; ++c)
+          if (32 * c < my_c) {                             // warp-uniform
+            uint32_t s[2][16];
+            tmem_ld_frag<4>(t_sc + 32 * c, s);
+            f32x2 ln[4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) ln[b] = *reinterpret_cast<const f32x2*>(l2n + cq * QWC + 32 * c + 8 * b + 2 * t4);
+            tmem_ld_wait_frag<4>(s);
+            uint32_t pk[4][4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                const f32x2 x = pack2u(s[h >> 1][4 * b + 2 * (h & 1)], s[h >> 1][4 * b + 2 * (h & 1) + 1]);
+                float lo, hi;
+                unpack2(add2(fma2(x, sc2, nm[h]), ln[b]), lo, hi);
+                pk[b][h] = pack_bf16(ex2(lo), ex2(hi));
+                add_bf16x2(zc[h], pk[b][h]);
+              }
+            if (!o_done) {
+              mbar_wait(bar_o, ph_o, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+              tc_fence_after();
+              o_done = true;
+            }
+            put_weights(L::tWc, cq * QWC + 32 * c, pk);
+          }
+        // Any reference value works as long as numerator and denominator share it: the parents' maximum is kept
+        // unless the children's weights grow so large against it that fp32 sums could overflow.  That is found out
+        // at the barrier that publishes the weights; the rare case goes round the loop once more.
+        constexpr float kLargest = 1.8446744e19f;          // 2^64
+        weights_done();
+        if (!__syncthreads_or(fmaxf(fmaxf(zc[0], zc[1]), fmaxf(zc[2], zc[3])) > kLargest)) break;
+        // ---- row maxima of the chunk (non-empty children); where they exceed the reference it moves up and O and z
+        // are rescaled
+        float m_c[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < NCC; ++c)
+          if (32 * c < my_c) {
+            uint32_t s[2][16];
+            tmem_ld_frag<4>(t_sc + 32 * c, s);
+            tmem_ld_wait_frag<4>(s);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const float2 ln = *reinterpret_cast<const float2*>(l2n + cq * QWC + 32 * c + 8 * b + 2 * t4);
+#pragma unroll
+              for (int h = 0; h < 4; ++h)
+                m_c[h] = max3(m_c[h], ln.x + sc * __uint_as_float(s[h >> 1][4 * b + 2 * (h & 1)]),
+                              ln.y + sc * __uint_as_float(s[h >> 1][4 * b + 2 * (h & 1) + 1]));
+            }
+          }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) m_c[h] = quad_max(m_c[h]);
+        if (NQ > 1) {
+          xm[cq * kRows + q * 32 + g + 8 * t4] = pick4(m_c, t4);
+          row_sync<NQ>(q);
+          float m = xm[r];
+#pragma unroll
+          for (int u = 1; u < NQ; ++u) m = fmaxf(m, xm[u * kRows + r]);
+          to_frag(m, m_c);
+        }
+        float alpha[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          alpha[h] = 1.f;
+          if (m_c[h] > m_run[h]) {
+            alpha[h] = ex2(m_run[h] - m_c[h]);
+            m_run[h] = m_c[h];
+          }
+          z_run[h] *= alpha[h];
+        }
+        if (e0 == 0) mbar_wait(bar_o, ph_o, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+        tc_fence_after();
+        for (int c0 = 0; c0 < D / NQ; c0 += 16) {
+          uint32_t o[2][8];
+          tmem_ld_frag<2>(t_o + c0, o);
+          tmem_ld_wait_frag<2>(o);
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {                  // blocks 0, 1 x columns 0, 1
+              uint32_t& x = o[h >> 1][4 * (e >> 1) + 2 * (h & 1) + (e & 1)];
+              x = __float_as_uint(__uint_as_float(x) * alpha[h]);
+            }
+          tmem_st_frag<2>(t_o + c0, o);
+        }
+        tmem_st_wait();
+        // a second turn sees weights of at most about the chunk's width and ends
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) z_run[h] += zc[h];
+
+      // ---- O += A_c . Vbar_c
+      if (warp == kVWarp) issue_o(kSepCV ? CV : CC, np32, L::tWc, true, bar_pv);
+      if (!last) {
+        ncols = min(PC - e0 - CHW, CHW);
+        np32 = (ncols + 31) & ~31;
+        if constexpr (!kSepCV) mbar_wait(bar_pv, ph_pv, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);   // values have left CC
+        gather_codes(e0 + CHW);
+        cp_async_wait_all();
+        fence_proxy_async();
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 0) issue_sc(np32);
+      }
+    }
+
+    // ---- epilogue: Y = O / z.  The rows' denominators are put together while the last MMA runs.
+    float inv[4];
+    {
+      float zt[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) zt[h] = quad_sum(z_run[h]);
+      float z;                                             // of row `lane`
+      if (NQ > 1) {
+        xz[cq * kRows + q * 32 + g + 8 * t4] = pick4(zt, t4);
+        row_sync<NQ>(q);
+        z = xz[r];
+#pragma unroll
+        for (int u = 1; u < NQ; ++u) z += xz[u * kRows + r];
+      } else {
+        z = __shfl_sync(0xffffffffu, pick4(zt, t4), 4 * (lane & 7) + (lane >> 3));
+      }
+      to_frag(1.f / z, inv);
+    }
+    const bool o_ok = mbar_wait(PC > 0 ? bar_pv : bar_o, PC > 0 ? ph_pv : ph_o, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);
+    if (PC > 0) ph_pv ^= 1;
+    ph_o ^= 1;                                             // (the children's MMA is behind the parents')
+    tc_fence_after();
+    // the next tile's logits: every thread has read this tile's, and the last value MMA its weights
+    if (kTW && has_next && warp == kVWarp) issue_s(next_new_cp);
+    if (warp == 0 && has_next && elect_one()) {
+      // the last value MMA has released the weights (here: the codebook's place) and the parent values
+      if (!kTW) issue_cp(nbh, kSubD);
+      if (L::kStageInCC && next_new_v) issue_v(nbh);
+    }
+    // The output tile is staged in shared memory in the layout of the Q load and written with TMA tile
+    // stores; rows past Nq are clipped by the tensor map.
+    if (o_ok) {
+      constexpr int OW = D / NQ, ONB = OW >= 32 ? 4 : 2;   // output columns of this warp, blocks per step
+      const uint32_t st_row = smem_u32(stage) + (uint32_t)(r * 128 + ((lane & 7) << 4));
+#pragma unroll
+      for (int c = 0; c < OW / (8 * ONB); ++c) {
+        uint32_t o[2][4 * ONB];
+        tmem_ld_frag<ONB>(t_o + 8 * ONB * c, o);
+        tmem_ld_wait_frag<ONB>(o);
+#pragma unroll
+        for (int b = 0; b < ONB; ++b) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const uint32_t* x = &o[h >> 1][4 * b + 2 * (h & 1)];
+            pk[h] = pack_bf16(__uint_as_float(x[0]) * inv[h], __uint_as_float(x[1]) * inv[h]);
+          }
+          const int col = cq * OW + 8 * ONB * c + 8 * b;
+          stmatrix4((st_row + (uint32_t)((col >> 6) * (kRows * 128))) ^ (uint32_t)(((col >> 3) & 7) << 4), pk[0], pk[1], pk[2],
+                    pk[3]);
+        }
+      }
+      fence_proxy_async();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0 && o_ok) {
+      if (elect_one()) {
+#pragma unroll
+        for (int s2 = 0; s2 < kSubD; ++s2) tma_store_3d(&tmY, stage + s2 * kRows * 128, s2 * 64, i0, bh);
+        tma_store_commit();
+        if (!has_next) tma_store_wait_read();              // before the CTA may leave
+      }
+      store_pending = has_next;                            // waited for before the staging area is refilled
+    }
+    if (!kTW && has_next && warp == kVWarp) issue_s(true);
+    new_bh = next_new_bh;
+    bh = nbh;
+    blk = nblk_;
   }   // tiles
-  if (warp == 1) tmem_dealloc(tmem_base, p.tmem_cols);
+  if (warp == 1) tmem_dealloc(tmem_base, L::tmem_cols);
 }
 
-size_t attend_smem(int D, int CT, int CHW, int NQ, int MC) {
-  const int subA = CT / 64;
-  const size_t ca = (size_t)max(CT * D * 2, subA * kRows * 128);
-  size_t b = (size_t)(D / 64) * kRows * 128 + ca + (size_t)subA * D * 128 + (size_t)CHW * D * 2;
-  b += sizeof(float) * (3 * (size_t)CT + 2 * (size_t)CHW + (size_t)CT + 4 * (size_t)CT + 3 * (size_t)NQ * kRows);
-  b += sizeof(int) * (size_t)CT + sizeof(uint32_t) * 18 + sizeof(uint64_t) * 5 + 2 * sizeof(uint32_t);
-  return b + 64 + sizeof(float) * (size_t)MC;
-}
-
-template <int D, int NQ, int CT, bool FUSE>
-avq_status launch_nq_f(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CUtensorMap& tmVpb,
-                     const CUtensorMap& tmY, const AttendParams& a, unsigned BH, size_t smem, bool chained,
-                     cudaStream_t st) {
-  auto kern = tc_attend_kernel<D, NQ, CT, FUSE>;
+template <int D, int NQ, int CT, bool STAYS>
+avq_status launch_plan(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CUtensorMap& tmVpb,
+                       const CUtensorMap& tmY, const AttendParams& a, bool chained, cudaStream_t st) {
+  auto kern = tc_attend_kernel<D, NQ, CT, STAYS>;
+  const size_t smem = attend_smem<D, NQ, CT>(a.M * a.C);
   // The limit is set once per device and instantiation (setting it again is harmless if two threads race).
   static size_t configured[64] = {};
   int dev = 0;
@@ -865,7 +1105,7 @@ avq_status launch_nq_f(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CU
       return AVQ_ERR_CUDA;
     if (dev >= 0 && dev < 64) configured[dev] = smem;
   }
-  // Grid: one wave of CTAs (4 / NQ per SM), each taking every gridDim.x-th tile.
+  // Grid: one wave of CTAs (4 / NQ per SM), each taking an equal run of tiles.
   static int sm_count[64] = {};
   int sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
   if (sms <= 0) {
@@ -874,24 +1114,17 @@ avq_status launch_nq_f(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CU
   }
   int ctas = a.total_tiles;
   if (ctas > (4 / NQ) * sms) ctas = (4 / NQ) * sms;
-  const dim3 grid((unsigned)ctas);
   // Inside avq_forward (`chained`) the kernel before it in the stream is the aggregate's finalize kernel
   // and Q was complete before the call, so the attention kernel may start as its programmatic dependent.
   // A stand-alone avq_attend is launched plainly: the work before it in the stream may be producing Q.
-  return cuda_ok(launch_pdl(kern, grid, dim3(128 * NQ), smem, st, chained, tmQ, tmCp, tmVpb, tmY, a));
+  return cuda_ok(launch_pdl(kern, dim3((unsigned)ctas), dim3(128 * NQ), smem, st, chained, tmQ, tmCp, tmVpb, tmY, a));
 }
 
 template <int D, int NQ, int CT>
 avq_status launch_nq(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CUtensorMap& tmVpb,
-                     const CUtensorMap& tmY, const AttendParams& a, unsigned BH, size_t smem, bool chained,
-                     cudaStream_t st) {
-  // conversion inside the exponential loop: measured to pay for the larger tiles when P is small against M
-  // (c2 45.1 -> 43.3 us, c3 188 -> 184 us) and to cost for 64-column tiles (N=16384 M=64 P=16: 43 -> 47 us)
-  // and for P near M (N=65536 M=128 P=128: 615 -> 649 us)
-  if constexpr (CT >= 128) {
-    if (4 * a.P <= a.M) return launch_nq_f<D, NQ, CT, true>(tmQ, tmCp, tmVpb, tmY, a, BH, smem, chained, st);
-  }
-  return launch_nq_f<D, NQ, CT, false>(tmQ, tmCp, tmVpb, tmY, a, BH, smem, chained, st);
+                     const CUtensorMap& tmY, const AttendParams& a, bool chained, cudaStream_t st) {
+  return a.rho ? launch_plan<D, NQ, CT, true>(tmQ, tmCp, tmVpb, tmY, a, chained, st)
+               : launch_plan<D, NQ, CT, false>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
 }
 
 template <int D>
@@ -909,15 +1142,9 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
     if (s != AVQ_OK) return s;
   }
   {
-    const uint64_t dims[2] = {(uint64_t)D, (uint64_t)p.H * p.M};
-    const uint32_t box[2] = {64, (uint32_t)p.M};
-    avq_status s = make_tmap_bf16(&tmCp, Cp, 2, dims, box);
+    avq_status s = make_tmap_codes(&tmCp, Cp, D, (uint64_t)p.H * p.M, (uint32_t)p.M);
     if (s != AVQ_OK) return s;
-  }
-  {
-    const uint64_t dims[2] = {(uint64_t)D, BH * p.M};
-    const uint32_t box[2] = {64, (uint32_t)p.M};
-    avq_status s = make_tmap_bf16(&tmVpb, Vpb, 2, dims, box);
+    s = make_tmap_codes(&tmVpb, Vpb, D, BH * p.M, (uint32_t)p.M);
     if (s != AVQ_OK) return s;
   }
   AttendParams a;
@@ -936,25 +1163,18 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
   if ((uint64_t)a.nblk * BH > 0x7fffffffull) return AVQ_ERR_UNSUPPORTED;
   a.total_tiles = (int)(a.nblk * BH);
   const int CT = p.M <= 64 ? 64 : (p.M <= 128 ? 128 : 256);
-  const int CHW = CT < 128 ? CT : 128;
   a.logC = p.C == 8 ? 3 : 2;
-  uint32_t cols = 32;
-  while ((int)cols < CT + D) cols <<= 1;
-  a.tmem_cols = cols;
   a.scale_log2e = p.scale * 1.4426950408889634f;
-  const int NQ = (D == 64) ? (CT == 64 ? 1 : (CT == 128 ? 2 : 4)) : (CT == 64 ? 2 : 4);
-  const size_t smem = attend_smem(D, CT, CHW, NQ, p.M * p.C);
-  // Threads per query row follow from how many CTAs can share an SM (TMEM columns, shared memory):
+  // Warps per query row follow from how many CTAs can share an SM (TMEM columns, shared memory):
   // four small CTAs of 128 threads, two of 256, or one of 512.
-  const unsigned bh = (unsigned)BH;
-  if (D == 64) {
-    if (CT == 64) return launch_nq<D, 1, 64>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
-    if (CT == 128) return launch_nq<D, 2, 128>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
-    return launch_nq<D, 4, 256>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
+  if constexpr (D == 64) {
+    if (CT == 64) return launch_nq<D, 1, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+    if (CT == 128) return launch_nq<D, 2, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+  } else {
+    if (CT == 64) return launch_nq<D, 2, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+    if (CT == 128) return launch_nq<D, 4, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
   }
-  if (CT == 64) return launch_nq<D, 2, 64>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
-  if (CT == 128) return launch_nq<D, 4, 128>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
-  return launch_nq<D, 4, 256>(tmQ, tmCp, tmVpb, tmY, a, bh, smem, chained, st);
+  return launch_nq<D, 4, 256>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
 }
 
 }  // namespace

@@ -293,6 +293,9 @@ EncodeTiledFn encode_tiled_fn();   // nullptr if the driver entry point cannot b
 // and 128-byte swizzle; out-of-range elements read as zero.
 avq_status make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
                           const uint32_t* box);
+// Codeword rows [rows, d] bf16 in boxes of `box_rows` rows x 64 columns that land in shared memory with row 4 v + t of
+// every group of 8 at position 2 t + v: a 4-dimensional view (column, v, t, group).
+avq_status make_tmap_codes(CUtensorMap* map, const void* base, int d, uint64_t rows, uint32_t box_rows);
 
 }  // namespace tc
 }  // namespace avq

@@ -20,16 +20,20 @@ EncodeTiledFn encode_tiled_fn() {
 
 namespace {
 // Encoding a tensor map costs a few microseconds of host time and a forward needs seven of them, so
-// recent encodings are kept: the result depends only on (base, rank, dims, box).
+// recent encodings are kept: the result depends only on (base, rank, dims, strides, box).
+constexpr int kMaxRank = 4;
 struct TmapKey {
   const void* base;
   int rank;
-  uint64_t dims[3];
-  uint32_t box[3];
+  uint64_t dims[kMaxRank];
+  uint64_t strides[kMaxRank - 1];   // bytes, of dimensions 1..
+  uint32_t box[kMaxRank];
   bool operator==(const TmapKey& o) const {
     if (base != o.base || rank != o.rank) return false;
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < rank; ++i)
       if (dims[i] != o.dims[i] || box[i] != o.box[i]) return false;
+    for (int i = 0; i + 1 < rank; ++i)
+      if (strides[i] != o.strides[i]) return false;
     return true;
   }
 };
@@ -38,15 +42,8 @@ std::mutex g_tmap_mu;
 TmapKey g_tmap_keys[kTmapCache];
 CUtensorMap g_tmap_vals[kTmapCache];
 int g_tmap_used = 0, g_tmap_next = 0;
-}  // namespace
 
-avq_status make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
-                          const uint32_t* box) {
-  if (rank < 1 || rank > 3) return AVQ_ERR_UNSUPPORTED;
-  TmapKey key = {};
-  key.base = base;
-  key.rank = rank;
-  for (int i = 0; i < rank; ++i) { key.dims[i] = dims[i]; key.box[i] = box[i]; }
+avq_status encode(CUtensorMap* map, const TmapKey& key) {
   {
     std::lock_guard<std::mutex> lock(g_tmap_mu);
     for (int i = 0; i < g_tmap_used; ++i)
@@ -54,18 +51,15 @@ avq_status make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const ui
   }
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return AVQ_ERR_CUDA;
-  cuuint64_t gdim[5];
-  cuuint64_t gstride[4];
-  cuuint32_t bdim[5], estr[5];
-  uint64_t pitch = 2;
-  for (int i = 0; i < rank; ++i) {
-    gdim[i] = dims[i];
-    bdim[i] = box[i];
+  cuuint64_t gdim[kMaxRank], gstride[kMaxRank];
+  cuuint32_t bdim[kMaxRank], estr[kMaxRank];
+  for (int i = 0; i < key.rank; ++i) {
+    gdim[i] = key.dims[i];
+    bdim[i] = key.box[i];
     estr[i] = 1;
-    pitch *= dims[i];
-    if (i + 1 < rank) gstride[i] = pitch;   // byte stride of dimension i+1
+    if (i + 1 < key.rank) gstride[i] = key.strides[i];
   }
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gdim,
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)key.rank, const_cast<void*>(key.base), gdim,
                   gstride, bdim, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return AVQ_ERR_CUDA;
@@ -74,6 +68,35 @@ avq_status make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const ui
   g_tmap_keys[slot] = key;
   g_tmap_vals[slot] = *map;
   return AVQ_OK;
+}
+}  // namespace
+
+avq_status make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
+                          const uint32_t* box) {
+  if (rank < 1 || rank > 3) return AVQ_ERR_UNSUPPORTED;
+  TmapKey key = {};
+  key.base = base;
+  key.rank = rank;
+  uint64_t pitch = 2;
+  for (int i = 0; i < rank; ++i) {
+    key.dims[i] = dims[i];
+    key.box[i] = box[i];
+    pitch *= dims[i];
+    if (i + 1 < rank) key.strides[i] = pitch;   // byte stride of dimension i+1
+  }
+  return encode(map, key);
+}
+
+avq_status make_tmap_codes(CUtensorMap* map, const void* base, int d, uint64_t rows, uint32_t box_rows) {
+  if (rows % 8 != 0 || box_rows % 8 != 0) return AVQ_ERR_UNSUPPORTED;
+  const uint64_t row = 2 * (uint64_t)d;
+  TmapKey key = {};
+  key.base = base;
+  key.rank = 4;
+  key.dims[0] = (uint64_t)d; key.dims[1] = 2; key.dims[2] = 4; key.dims[3] = rows / 8;
+  key.strides[0] = 4 * row; key.strides[1] = row; key.strides[2] = 8 * row;
+  key.box[0] = 64; key.box[1] = 2; key.box[2] = 4; key.box[3] = box_rows / 8;
+  return encode(map, key);
 }
 
 }  // namespace tc

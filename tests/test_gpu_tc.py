@@ -242,3 +242,17 @@ def test_chained_tiles_with_several_child_chunks():
     that each tile runs through several child chunks before the next tile's loads are issued."""
     parity.sampled_parity(synth.sweep_point(16384, 64, 64), heads=[(0, 7)], blocks_per_head=4)
     parity.sampled_parity(synth.sweep_point(16384, 256, 64).with_(H=4), heads=[(0, 2)], blocks_per_head=3)
+
+
+@pytest.mark.parametrize("d,M,C,P,N", [(64, 64, 4, 16, 300), (64, 96, 8, 40, 260), (128, 64, 4, 5, 129), (128, 256, 4, 48, 400),
+                                       (64, 160, 4, 33, 257)])
+def test_children_far_above_the_parents_move_the_reference(d, M, C, P, N):
+    """Children so far from their parents that their logits exceed the parents' maximum by more than 64 powers of two:
+    the attention kernel's rescaling turn, in every tile plan, over one and several child chunks."""
+    wl = synth.Workload("far", B=1, H=2, N=N, d=d, M=M, C=C, P=P, block_q=128, seed=900 + M + d, alpha=0.6,
+                        hot_queries=True, sigma_c=12.0)
+    x = synth.generate(wl)
+    s = np.einsum("hnd,hmd->hnm", x["Q"][0].astype(np.float64), x["Cp"].astype(np.float64)).max(-1)
+    c = np.einsum("hnd,hmcd->hnmc", x["Q"][0].astype(np.float64), x["Cc"].astype(np.float64)).max((-1, -2))
+    assert ((c - s) * wl.scale * np.log2(np.e) > 80).mean() > 0.5
+    parity.full_parity(wl, x=x)
