@@ -244,13 +244,14 @@ def test_chained_tiles_with_several_child_chunks():
     parity.sampled_parity(synth.sweep_point(16384, 256, 64).with_(H=4), heads=[(0, 2)], blocks_per_head=3)
 
 
-@pytest.mark.parametrize("d,M,C,P,N", [(64, 64, 4, 16, 300), (64, 96, 8, 40, 260), (128, 64, 4, 5, 129), (128, 256, 4, 48, 400),
+@pytest.mark.parametrize("d,M,C,P,N", [(64, 64, 4, 16, 300), (64, 96, 8, 40, 260), (128, 64, 4, 5, 250), (128, 256, 4, 48, 400),
                                        (64, 160, 4, 33, 257)])
 def test_children_far_above_the_parents_move_the_reference(d, M, C, P, N):
     """Children so far from their parents that their logits exceed the parents' maximum by more than 64 powers of two:
-    the attention kernel's rescaling turn, in every tile plan, over one and several child chunks."""
+    the attention kernel's rescaling turn, in every tile plan, over one and several child chunks.  (P small against a tile of few queries
+    is left out: the P-th importance then lies below 2^-126, the smallest weight fp32 holds, and the choice is open.)"""
     wl = synth.Workload("far", B=1, H=2, N=N, d=d, M=M, C=C, P=P, block_q=128, seed=900 + M + d, alpha=0.6,
-                        hot_queries=True, sigma_c=12.0)
+                        hot_queries=True, sigma_c=20.0)
     x = synth.generate(wl)
     s = np.einsum("hnd,hmd->hnm", x["Q"][0].astype(np.float64), x["Cp"].astype(np.float64)).max(-1)
     c = np.einsum("hnd,hmcd->hnmc", x["Q"][0].astype(np.float64), x["Cc"].astype(np.float64)).max((-1, -2))
