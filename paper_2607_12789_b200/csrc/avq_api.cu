@@ -113,7 +113,7 @@ avq_status avq_assign(const avq_problem* prob, const void* K, const void* Cp, co
   if (!aligned16(K) || !aligned16(Cp) || !aligned16(Cc) || !aligned16(parent_idx) || !aligned16(child_idx))
     return AVQ_ERR_ALIGN;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (use_tensor_path(*prob)) return tc_assign(*prob, K, Cp, Cc, parent_idx, child_idx, nullptr, nullptr, 0, nullptr, st);
+  if (use_tensor_path(*prob)) return tc_assign(*prob, K, Cp, Cc, parent_idx, child_idx, nullptr, nullptr, 0, nullptr, false, st);
   return simt_assign(*prob, K, Cp, Cc, parent_idx, child_idx, nullptr, 0, st);
 }
 
@@ -128,7 +128,7 @@ avq_status avq_aggregate(const avq_problem* prob, const void* V, const int32_t* 
     return AVQ_ERR_ALIGN;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (use_tensor_path(*prob))
-    return tc_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, nullptr, nullptr, nullptr, nullptr, false, nullptr, st);
+    return tc_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, nullptr, nullptr, nullptr, nullptr, false, false, nullptr, st);
   return simt_aggregate(*prob, V, parent_idx, child_idx, Vp, np_, Vc, nc, false, nullptr, st);
 }
 
@@ -159,10 +159,10 @@ Regions carve(void* workspace, const Layout& L) {
 }
 avq_status attend_stage(const avq_problem& p, const Regions& r, const void* Q, const void* Cp, const void* Cc,
                         int32_t P, int32_t block_q, void* Y, int32_t* topp_out, float* importance_out,
-                        bool chained, cudaStream_t st) {
+                        bool chained, const int32_t* perm, cudaStream_t st) {
   if (use_tensor_path(p))
     return tc_attend(p, Q, Cp, Cc, r.np_, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, P, Y, topp_out, importance_out, r.status_word,
-                     chained, st);
+                     chained, perm, st);
   return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, 0, chained, st);
 }
 avq_status check_workspace(const avq_problem* prob, int32_t P, int32_t block_q, void* workspace,
@@ -174,6 +174,33 @@ avq_status check_workspace(const avq_problem* prob, int32_t P, int32_t block_q, 
   return AVQ_OK;
 }
 }  // namespace
+}  // extern "C"
+
+namespace avq {
+avq_status forward_core(const avq_problem& p, const void* Q, const void* K, const void* V, const void* Cp,
+                        const void* Cc, int32_t P, int32_t block_q, void* Y, int32_t* topp_out, float* importance_out,
+                        void* workspace, const Layout& L, const int32_t* perm, cudaStream_t st) {
+  avq_status s;
+  const Regions r = carve(workspace, L);
+  if (use_tensor_path(p)) {
+    // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
+    // The codeword norms as a pass of their own pay once many CTAs share them and a codebook is large: measured
+    // c3 (128 CTAs per head, M d = 32768) -4 us, c2 (M d = 8192) +-0, c1 +1.4 us (the extra launch).
+    const bool norms_pass = (size_t)p.M * p.d >= 16384 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
+    s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);
+    if (s != AVQ_OK) return s;
+    s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, false, r.status_word, st);
+  } else {
+    s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, workspace, L.zero_end, st);   // clears the accumulators on the side
+    if (s != AVQ_OK) return s;
+    s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
+  }
+  if (s != AVQ_OK) return s;
+  return attend_stage(p, r, Q, Cp, Cc, P, block_q, Y, topp_out, importance_out, true, perm, st);
+}
+}  // namespace avq
+
+extern "C" {
 
 avq_status avq_forward(const avq_problem* prob, const void* Q, const void* K, const void* V,
                        const void* Cp, const void* Cc, int32_t P, int32_t block_q, void* Y,
@@ -188,24 +215,8 @@ avq_status avq_forward(const avq_problem* prob, const void* Q, const void* K, co
   Layout L;
   s = check_workspace(prob, P, block_q, workspace, workspace_bytes, &L);
   if (s != AVQ_OK) return s;
-  const avq_problem& p = *prob;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const Regions r = carve(workspace, L);
-  if (use_tensor_path(p)) {
-    // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
-    // The codeword norms as a pass of their own pay once many CTAs share them and a codebook is large: measured
-    // c3 (128 CTAs per head, M d = 32768) -4 us, c2 (M d = 8192) +-0, c1 +1.4 us (the extra launch).
-    const bool norms_pass = (size_t)p.M * p.d >= 16384 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
-    s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, st);
-    if (s != AVQ_OK) return s;
-    s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, r.status_word, st);
-  } else {
-    s = simt_assign(p, K, Cp, Cc, r.pidx, r.cidx, workspace, L.zero_end, st);   // clears the accumulators on the side
-    if (s != AVQ_OK) return s;
-    s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
-  }
-  if (s != AVQ_OK) return s;
-  return attend_stage(p, r, Q, Cp, Cc, P, block_q, Y, topp_out, importance_out, true, st);
+  return forward_core(*prob, Q, K, V, Cp, Cc, P, block_q, Y, topp_out, importance_out, workspace, L, nullptr,
+                      static_cast<cudaStream_t>(stream));
 }
 
 avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void* K, const void* V,
@@ -247,7 +258,7 @@ avq_status avq_attend(const avq_problem* prob, const void* Q, const void* Cp, co
   Layout L;
   s = check_workspace(prob, P, block_q, workspace, workspace_bytes, &L);
   if (s != AVQ_OK) return s;
-  return attend_stage(*prob, carve(workspace, L), Q, Cp, Cc, P, block_q, Y, topp_out, importance_out, false,
+  return attend_stage(*prob, carve(workspace, L), Q, Cp, Cc, P, block_q, Y, topp_out, importance_out, false, nullptr,
                       static_cast<cudaStream_t>(stream));
 }
 

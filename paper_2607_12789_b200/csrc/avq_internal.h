@@ -40,6 +40,11 @@ bool use_tensor_path(const avq_problem& p);
 avq_status validate_problem(const avq_problem* p);
 avq_status validate_forward(const avq_problem* p, int32_t P, int32_t block_q);
 Layout make_layout(const avq_problem& p, int32_t P, int32_t block_q);
+// The three stages on validated arguments.  perm (tensor-core path only, may be null): Q is in tile order, written by
+// the kernel just launched on the stream, and Y rows go to their places perm[i].
+avq_status forward_core(const avq_problem& p, const void* Q, const void* K, const void* V, const void* Cp,
+                        const void* Cc, int32_t P, int32_t block_q, void* Y, int32_t* topp_out, float* importance_out,
+                        void* workspace, const Layout& L, const int32_t* perm, cudaStream_t st);
 
 // ---- plain CUDA-core kernels (avq_simt.cu) ----
 avq_status simt_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
@@ -65,16 +70,19 @@ constexpr size_t kSimtAttendSmemLimit = 200 * 1024;
 // null every assign CTA computes the norms of its head itself
 avq_status tc_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
                      int32_t* parent_idx, int32_t* child_idx, int32_t* status_word, void* zero_base,
-                     size_t zero_bytes, float* cnorm, cudaStream_t st);
+                     size_t zero_bytes, float* cnorm, bool beside, cudaStream_t st);   // beside: may overlap the kernel
+                                                         // before it on the stream (which it does not depend on)
 avq_status tc_aggregate(const avq_problem& p, const void* V, const int32_t* parent_idx,
                         const int32_t* child_idx, float* Vp, float* np_, float* Vc, float* nc,
-                        void* Vpb, void* Vcb, void* Vsb, float* rho, bool pre_zeroed, int32_t* status_word,
-                        cudaStream_t st);   // Vsb, rho: stay rows and stay shares (PARENT_STAYS), may be null
+                        void* Vpb, void* Vcb, void* Vsb, float* rho, bool pre_zeroed, bool leaves_only,
+                        int32_t* status_word, cudaStream_t st);   // Vsb, rho: stay rows and stay shares (PARENT_STAYS),
+                                            // may be null; leaves_only: Vp / np_ keep the stay part alone
 avq_status tc_attend(const avq_problem& p, const void* Q, const void* Cp, const void* Cc,
                      const float* np_, const float* nc, const void* Vpb, const void* Vcb, const void* Vsb,
                      const float* rho, int32_t P,
                      void* Y, int32_t* topp_out, float* importance_out, int32_t* status_word,
-                     bool chained, cudaStream_t st);   // chained: launched right behind tc_aggregate
+                     bool chained, const int32_t* perm, cudaStream_t st);   // chained: launched right behind tc_aggregate;
+                                                         // perm: see forward_core
 
 inline avq_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AVQ_OK : AVQ_ERR_CUDA; }
 

@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(256) clear_accumulators_kernel(float* a, size_
 template <int D, int C>
 avq_status run(const avq_problem& p, const void* V, const int32_t* pidx, const int32_t* cidx, float* Vp,
                float* np_, float* Vc, float* nc, void* Vpb, void* Vcb, void* Vsb, float* rho, bool pre_zeroed,
-               int32_t* status_word, cudaStream_t st) {
+               bool leaves_only, int32_t* status_word, cudaStream_t st) {
   const unsigned BH = (unsigned)(p.B * p.H);
   if (!pre_zeroed) {                                   // the stand-alone call: one launch clears the four accumulators
     const size_t n_c = (size_t)BH * p.M * C, n_p = (size_t)BH * p.M;
@@ -365,6 +365,7 @@ avq_status run(const avq_problem& p, const void* V, const int32_t* pidx, const i
                        status_word) != cudaSuccess)
       return AVQ_ERR_CUDA;
   }
+  if (leaves_only) return AVQ_OK;
   dim3 g2(p.M / (C == 4 ? 8 : 4), BH);
   return cuda_ok(tc::launch_pdl(finalize_kernel<D, C>, g2, dim3(D, C == 4 ? 8 : 4), 0, st, true, static_cast<const float*>(Vc),
                                 static_cast<const float*>(nc), Vp, np_, static_cast<__nv_bfloat16*>(Vpb),
@@ -375,12 +376,13 @@ avq_status run(const avq_problem& p, const void* V, const int32_t* pidx, const i
 
 avq_status tc_aggregate(const avq_problem& p, const void* V, const int32_t* parent_idx,
                         const int32_t* child_idx, float* Vp, float* np_, float* Vc, float* nc, void* Vpb,
-                        void* Vcb, void* Vsb, float* rho, bool pre_zeroed, int32_t* status_word, cudaStream_t st) {
+                        void* Vcb, void* Vsb, float* rho, bool pre_zeroed, bool leaves_only, int32_t* status_word,
+                        cudaStream_t st) {
   if (p.d == 64)
-    return p.C == 4 ? run<64, 4>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, status_word, st)
-                    : run<64, 8>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, status_word, st);
-  return p.C == 4 ? run<128, 4>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, status_word, st)
-                  : run<128, 8>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, status_word, st);
+    return p.C == 4 ? run<64, 4>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, leaves_only, status_word, st)
+                    : run<64, 8>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, leaves_only, status_word, st);
+  return p.C == 4 ? run<128, 4>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, leaves_only, status_word, st)
+                  : run<128, 8>(p, V, parent_idx, child_idx, Vp, np_, Vc, nc, Vpb, Vcb, Vsb, rho, pre_zeroed, leaves_only, status_word, st);
 }
 
 }  // namespace avq

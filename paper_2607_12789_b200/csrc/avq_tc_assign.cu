@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(256) code_norms_kernel(const __nv_bfloat16* __
   s += __shfl_xor_sync(0xffffffffu, s, 2);
   s += __shfl_xor_sync(0xffffffffu, s, 4);
   if (row < rows && part == 0) cnorm[row] = s;
+  pdl_wait();                // this grid's completion implies that of the one it ran beside
 }
 
 // NL = 16-byte loads per lane that cover one parent's C x d block of children: C * d / 256.
@@ -108,7 +109,7 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
                  int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int M, int C,
                  uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, uint32_t zero_units,
-                 const float* cnorm_g) {
+                 const float* cnorm_g, int beside) {
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -393,6 +394,7 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     pidx[(size_t)bh * Nk + j0 + tid] = par[tid];
     cidx[(size_t)bh * Nk + j0 + tid] = chi[tid];
   }
+  if (beside) pdl_wait();    // this grid's completion then implies that of the one it ran beside
 }
 
 uint32_t pow2_cols(int n) {
@@ -403,7 +405,8 @@ uint32_t pow2_cols(int n) {
 
 template <int D, int NL, bool STAYS>
 avq_status launch(const avq_problem& p, const void* K, const void* Cp, const void* Cc, int32_t* pidx,
-                  int32_t* cidx, int32_t* status_word, void* zero_base, size_t zero_bytes, float* cnorm, cudaStream_t st) {
+                  int32_t* cidx, int32_t* status_word, void* zero_base, size_t zero_bytes, float* cnorm, bool beside,
+                  cudaStream_t st) {
   CUtensorMap tmK, tmCp;
   const uint64_t BH = (uint64_t)p.B * p.H;
   {
@@ -434,26 +437,27 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   dim3 grid((p.Nk + kKeys - 1) / kKeys, (unsigned)BH);
   if (cnorm) {
     const int rows = p.H * p.M;
-    code_norms_kernel<D><<<(rows * 8 + 255) / 256, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(Cp), cnorm, rows);
-    if (cudaGetLastError() != cudaSuccess) return AVQ_ERR_CUDA;
+    if (launch_pdl(code_norms_kernel<D>, dim3((rows * 8 + 255) / 256), dim3(256), 0, st, beside,
+                   static_cast<const __nv_bfloat16*>(Cp), cnorm, rows) != cudaSuccess)
+      return AVQ_ERR_CUDA;
   }
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
-  return cuda_ok(launch_pdl(kern, grid, dim3(kThreadsA), smem, st, cnorm != nullptr, tmK, tmCp,
+  return cuda_ok(launch_pdl(kern, grid, dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
                             static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,
                             p.H, p.Nk, p.M, p.C, pow2_cols(p.M), status_word, static_cast<uint4*>(zero_base),
-                            (uint32_t)(zero_bytes / 16), static_cast<const float*>(cnorm)));
+                            (uint32_t)(zero_bytes / 16), static_cast<const float*>(cnorm), beside ? 1 : 0));
 }
 
 }  // namespace
 
 avq_status tc_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
                      int32_t* parent_idx, int32_t* child_idx, int32_t* status_word, void* zero_base,
-                     size_t zero_bytes, float* cnorm, cudaStream_t st) {
+                     size_t zero_bytes, float* cnorm, bool beside, cudaStream_t st) {
   if (zero_bytes % 16 != 0 || (zero_bytes / 16) >> 31) return AVQ_ERR_WORKSPACE;
   const bool stays = (p.flags & AVQ_FLAG_PARENT_STAYS) != 0;
 #define AVQ_ASSIGN(DD, NN)                                                                                     \
-  (stays ? launch<DD, NN, true>(p, K, Cp, Cc, parent_idx, child_idx, status_word, zero_base, zero_bytes, cnorm, st) \
-         : launch<DD, NN, false>(p, K, Cp, Cc, parent_idx, child_idx, status_word, zero_base, zero_bytes, cnorm, st))
+  (stays ? launch<DD, NN, true>(p, K, Cp, Cc, parent_idx, child_idx, status_word, zero_base, zero_bytes, cnorm, beside, st) \
+         : launch<DD, NN, false>(p, K, Cp, Cc, parent_idx, child_idx, status_word, zero_base, zero_bytes, cnorm, beside, st))
   if (p.d == 64) return p.C == 4 ? AVQ_ASSIGN(64, 1) : AVQ_ASSIGN(64, 2);
   return p.C == 4 ? AVQ_ASSIGN(128, 2) : AVQ_ASSIGN(128, 4);
 #undef AVQ_ASSIGN

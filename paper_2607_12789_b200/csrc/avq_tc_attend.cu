@@ -49,6 +49,7 @@ struct AttendParams {
   int32_t* topp_out;          // optional
   float* importance_out;      // optional
   int32_t* status_word;
+  const int32_t* perm;        // Y row of query i of the head is perm[i] (else nullptr; an entry out of range is flagged and skipped)
   int H, Nq, M, C, P, nblk;
   int total_tiles;            // nblk * B * H
   int logC;                   // log2(C)
@@ -289,7 +290,8 @@ size_t attend_smem(int MC) {
 }
 
 // STAYS = the PARENT_STAYS rule: a refined parent keeps the keys that stayed with it.
-template <int D, int NQ, int CT, bool STAYS>
+// PERM = output rows go to p.perm's places (a branch at run time cost the plain call 1 us of 43).
+template <int D, int NQ, int CT, bool STAYS, bool PERM>
 __global__ void __launch_bounds__(128 * NQ, 4 / NQ)
 tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmCp,
                  const __grid_constant__ CUtensorMap tmVpb, const __grid_constant__ CUtensorMap tmY,
@@ -381,6 +383,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     for (int i = 0; i < 6; ++i) mbar_init(&bars[i], 1);
     mbar_fence_init();
     *abort_flag = 0;
+    if (PERM) pdl_wait();                                // Q is then the work of an earlier kernel of the call
     issue_q(bh, blk);
     issue_cp(bh, kSubD);
   }
@@ -513,8 +516,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         nc_reg = ld_after_wait(reinterpret_cast<const float4*>(p.nc + (size_t)bh * M * C) + tid);
       if (first && warp == 0 && elect_one()) {
         issue_v(bh);
-        // a wait that expired in an earlier CTA or kernel of this call: do not start more work
-        early_exit = (p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0);
+        // a wait that expired in an earlier CTA or kernel of this call: do not start more work (a flagged index is
+        // no reason to stop)
+        const int32_t word = p.status_word != nullptr ? *reinterpret_cast<volatile int32_t*>(p.status_word) : 0;
+        early_exit = word != 0 && word != DEV_BAD_INDEX;
       }
       if (tid < CT) {
         cnt[parent_pos(tid)] = n_reg;
@@ -1075,13 +1080,27 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     tc_fence_before();
     __syncthreads();
     if (warp == 0 && o_ok) {
-      if (elect_one()) {
+      if (!PERM && elect_one()) {
 #pragma unroll
         for (int s2 = 0; s2 < kSubD; ++s2) tma_store_3d(&tmY, stage + s2 * kRows * 128, s2 * 64, i0, bh);
         tma_store_commit();
         if (!has_next) tma_store_wait_read();              // before the CTA may leave
       }
-      store_pending = has_next;                            // waited for before the staging area is refilled
+      store_pending = !PERM && has_next;                   // waited for before the staging area is refilled
+    }
+    if constexpr (PERM) {                                  // every row to its place: d / 8 lanes per row, 16 bytes each
+      if (o_ok) {
+        for (int u = tid; u < (rows_valid << kLogChunks); u += kThreads) {
+          const int row = u >> kLogChunks, ch = u & ((1 << kLogChunks) - 1);
+          const int j = __ldg(p.perm + i0 + row);
+          const uint4 v = *reinterpret_cast<const uint4*>(stage + (ch >> 3) * (kRows * 128) + sw128_offset(row, (ch & 7) * 8));
+          if (j >= 0 && j < p.Nq) reinterpret_cast<uint4*>(p.Y + ((size_t)bh * p.Nq + j) * D)[ch] = v;
+          else if (ch == 0 && p.status_word) atomicCAS(p.status_word, 0, DEV_BAD_INDEX);
+        }
+      }
+      fence_proxy_async();
+      __syncthreads();                                     // read before the staging area is refilled
+      if (!L::kStageInCC && has_next && warp == 0 && elect_one()) issue_v(nbh);
     }
     if (!kTW && has_next && warp == kVWarp) issue_s(true);
     new_bh = next_new_bh;
@@ -1091,10 +1110,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   if (warp == 1) tmem_dealloc(tmem_base, L::tmem_cols);
 }
 
-template <int D, int NQ, int CT, bool STAYS>
+template <int D, int NQ, int CT, bool STAYS, bool PERM>
 avq_status launch_plan(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CUtensorMap& tmVpb,
                        const CUtensorMap& tmY, const AttendParams& a, bool chained, cudaStream_t st) {
-  auto kern = tc_attend_kernel<D, NQ, CT, STAYS>;
+  auto kern = tc_attend_kernel<D, NQ, CT, STAYS, PERM>;
   const size_t smem = attend_smem<D, NQ, CT>(a.M * a.C);
   // The limit is set once per device and instantiation (setting it again is harmless if two threads race).
   static size_t configured[64] = {};
@@ -1123,14 +1142,17 @@ avq_status launch_plan(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CU
 template <int D, int NQ, int CT>
 avq_status launch_nq(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CUtensorMap& tmVpb,
                      const CUtensorMap& tmY, const AttendParams& a, bool chained, cudaStream_t st) {
-  return a.rho ? launch_plan<D, NQ, CT, true>(tmQ, tmCp, tmVpb, tmY, a, chained, st)
-               : launch_plan<D, NQ, CT, false>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+  if (a.perm)
+    return a.rho ? launch_plan<D, NQ, CT, true, true>(tmQ, tmCp, tmVpb, tmY, a, chained, st)
+                 : launch_plan<D, NQ, CT, false, true>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+  return a.rho ? launch_plan<D, NQ, CT, true, false>(tmQ, tmCp, tmVpb, tmY, a, chained, st)
+               : launch_plan<D, NQ, CT, false, false>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
 }
 
 template <int D>
 avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const void* Cc, const float* np_,
                   const float* nc, const void* Vpb, const void* Vcb, const void* Vsb, const float* rho, int32_t P, void* Y, int32_t* topp_out,
-                  float* importance_out, int32_t* status_word, bool chained, cudaStream_t st) {
+                  float* importance_out, int32_t* status_word, bool chained, const int32_t* perm, cudaStream_t st) {
   const uint64_t BH = (uint64_t)p.B * p.H;
   CUtensorMap tmQ, tmCp, tmVpb, tmY;
   {
@@ -1158,6 +1180,7 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
   a.topp_out = topp_out;
   a.importance_out = importance_out;
   a.status_word = status_word;
+  a.perm = perm;
   a.H = p.H; a.Nq = p.Nq; a.M = p.M; a.C = p.C; a.P = P;
   a.nblk = (p.Nq + kRows - 1) / kRows;
   if ((uint64_t)a.nblk * BH > 0x7fffffffull) return AVQ_ERR_UNSUPPORTED;
@@ -1181,9 +1204,9 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
 
 avq_status tc_attend(const avq_problem& p, const void* Q, const void* Cp, const void* Cc, const float* np_,
                      const float* nc, const void* Vpb, const void* Vcb, const void* Vsb, const float* rho, int32_t P, void* Y, int32_t* topp_out,
-                     float* importance_out, int32_t* status_word, bool chained, cudaStream_t st) {
-  return p.d == 64 ? launch<64>(p, Q, Cp, Cc, np_, nc, Vpb, Vcb, Vsb, rho, P, Y, topp_out, importance_out, status_word, chained, st)
-                   : launch<128>(p, Q, Cp, Cc, np_, nc, Vpb, Vcb, Vsb, rho, P, Y, topp_out, importance_out, status_word, chained, st);
+                     float* importance_out, int32_t* status_word, bool chained, const int32_t* perm, cudaStream_t st) {
+  return p.d == 64 ? launch<64>(p, Q, Cp, Cc, np_, nc, Vpb, Vcb, Vsb, rho, P, Y, topp_out, importance_out, status_word, chained, perm, st)
+                   : launch<128>(p, Q, Cp, Cc, np_, nc, Vpb, Vcb, Vsb, rho, P, Y, topp_out, importance_out, status_word, chained, perm, st);
 }
 
 }  // namespace avq
