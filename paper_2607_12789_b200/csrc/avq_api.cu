@@ -73,7 +73,7 @@ Layout make_layout(const avq_problem& p, int32_t /*P*/, int32_t /*block_q*/) {
       L.Vsb = take(2 * BH * p.M * p.d);
       L.rho = take(sizeof(float) * BH * p.M);
     }
-    L.cnorm = take(sizeof(float) * (size_t)p.H * p.M);
+    L.cnorm = take(sizeof(float) * (size_t)p.H * p.M * (1 + p.C));
   }
   L.total = off;
   return L;
@@ -184,9 +184,7 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
   const Regions r = carve(workspace, L);
   if (use_tensor_path(p)) {
     // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
-    // The codeword norms as a pass of their own pay once many CTAs share them and a codebook is large: measured
-    // c3 (128 CTAs per head, M d = 32768) -4 us, c2 (M d = 8192) +-0, c1 +1.4 us (the extra launch).
-    const bool norms_pass = (size_t)p.M * p.d >= 16384 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
+    const bool norms_pass = (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
     s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);
     if (s != AVQ_OK) return s;
     s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, false, r.status_word, st);

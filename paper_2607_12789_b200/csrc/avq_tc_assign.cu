@@ -1,16 +1,20 @@
 // Tensor-core key assignment (Algorithm 1, parent and child argmin) for bf16 inputs.
 //
-// One CTA takes 128 consecutive keys of one (batch, head), 8 warps.  TMA stages the key tile and the
-// head's parent codebook in shared memory (K-major, 128-byte swizzle); one elected thread issues the
+// One CTA takes a run of tiles of 128 consecutive keys of one (batch, head), 8 warps.  TMA stages the key tiles (two
+// buffers where they fit) and, once per head, the head's parent codebook in shared memory (K-major, 128-byte swizzle); one elected thread issues the
 // tcgen05 MMA chain  D[128 x M] = K_tile . Cp^T  into TMEM.
-//   parent   two threads per key (column halves) read their TMEM lane, form ||c||^2 - 2 k.c and keep
-//            the best and the runner-up; the halves are merged in shared memory.  Only when best and
-//            runner-up are closer than the MMA's rounding can separate are all M distances redone in
-//            float64 in the direct form (lowest index wins ties).
+//   parent   warp w holds keys 32 (w % 4) .. +31 of the column half w / 4 and reads the products in the fragment layout
+//            (4 keys x column pairs per lane).  Two passes over ||c||^2 - 2 k.c: the minimum of the row; then the
+//            number and the index of the columns within the MMA's rounding of it, added up in one register.  Only
+//            when there is more than one such column are all M distances redone in float64 in the direct form
+//            (lowest index wins ties).  Three instructions per column and row instead of the six of a running best,
+//            runner-up and index, and half of them off the ALU pipe, which bounded the kernel.
 //   child    fp32 direct form sum (k - c)^2 on CUDA cores (2 C d flops per key; a second MMA over all
 //            M C children would cost C times the parent GEMM), float64 recheck for near-ties.
 //            Four lanes per key, each over a quarter of the head dimension for all C children of the
 //            key's parent (one running sum per child); a transposing butterfly merges the four lanes.
+#include <type_traits>
+
 #include "avq_tc_common.cuh"
 
 namespace avq {
@@ -22,36 +26,47 @@ constexpr int kKeys = 128;
 constexpr int kThreadsA = 256;
 // CTAs per SM the register budget is set for: the d = 64 kernels are small enough (24-48 KB of shared
 // memory, at most 128 TMEM columns up to M = 128) for four to share an SM.
-constexpr int assign_min_ctas(int D, int NL) { return D == 64 ? 4 : 2; }
+constexpr int assign_min_ctas(int D) { return D == 64 ? 4 : 2; }
 
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
-// Two packed bf16 widened to a pair of fp32 in one 64-bit register (for the f32x2 instructions).
-__device__ __forceinline__ uint64_t bf2_to_f32x2(uint32_t u) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(u << 16), "r"(u & 0xFFFF0000u));
-  return r;
+// s + the squares of 8 packed bf16 (mixed-precision multiply-add: exact products, fp32 sum)
+__device__ __forceinline__ float norm_bf16x8(float s, const uint4& v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tfma.rn.f32.bf16 %0, l, l, %0;\n\tfma.rn.f32.bf16 %0, h, h, %0;\n\t}"
+        : "+f"(s) : "r"(w[e]));
+  return s;
 }
-struct KeyChunk { uint64_t p[4]; };   // 8 key elements as four fp32 pairs
+// s += k . c over 8 packed bf16 (same instruction)
+__device__ __forceinline__ void dot_bf16x8(float& s, const uint4& k, const uint4& c) {
+  const uint32_t x[4] = {k.x, k.y, k.z, k.w}, y[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    asm("{\n\t.reg .b16 a, b, c, d;\n\tmov.b32 {a, b}, %1;\n\tmov.b32 {c, d}, %2;\n\tfma.rn.f32.bf16 %0, a, c, %0;\n\tfma.rn.f32.bf16 %0, b, d, %0;\n\t}"
+        : "+f"(s) : "r"(x[e]), "r"(y[e]));
+}
+struct KeyChunk { f32x2 p[4]; };      // 8 key elements as four fp32 pairs
 __device__ __forceinline__ KeyChunk widen8(const uint4& a) {
   KeyChunk k;
-  k.p[0] = bf2_to_f32x2(a.x); k.p[1] = bf2_to_f32x2(a.y); k.p[2] = bf2_to_f32x2(a.z); k.p[3] = bf2_to_f32x2(a.w);
+  k.p[0] = pack2(bf_lo(a.x), bf_hi(a.x)); k.p[1] = pack2(bf_lo(a.y), bf_hi(a.y));
+  k.p[2] = pack2(bf_lo(a.z), bf_hi(a.z)); k.p[3] = pack2(bf_lo(a.w), bf_hi(a.w));
   return k;
 }
 // sum over 8 elements of (k - c)^2, two lanes of packed fp32 arithmetic (sub.f32x2 / fma.f32x2)
 __device__ __forceinline__ float sqdiff8(const KeyChunk& k, const uint4& c) {
   const uint32_t y[4] = {c.x, c.y, c.z, c.w};
-  uint64_t acc = 0;   // {0.f, 0.f}
+  f32x2 acc = 0;   // {0.f, 0.f}
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    uint64_t d;
-    const uint64_t cw = bf2_to_f32x2(y[e]);
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(k.p[e]), "l"(cw));
-    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc) : "l"(d));
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(k.p[e]), "l"(pack2(bf_lo(y[e]), bf_hi(y[e]))));
+    acc = fma2(d, d, acc);
   }
   float lo, hi;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc));
+  unpack2(acc, lo, hi);
   return lo + hi;
 }
 
@@ -72,26 +87,20 @@ __device__ double exact_dist_smem(const unsigned char* Ks, int row, const __nv_b
   return s;
 }
 
-// ||c||^2 of every parent codeword of every head, once per call: a per-head constant that otherwise each of
-// the Nk / 128 assign CTAs of every (batch, head) recomputes.  Eight lanes per codeword row.
+// ||c||^2 of every codeword of every head, once per call: parents [H, M], then children [H, M, C].  Eight lanes per
+// codeword row.
 template <int D>
-__global__ void __launch_bounds__(256) code_norms_kernel(const __nv_bfloat16* __restrict__ Cp, float* __restrict__ cnorm,
-                                                         int rows) {
+__global__ void __launch_bounds__(256) code_norms_kernel(const __nv_bfloat16* __restrict__ Cp,
+                                                         const __nv_bfloat16* __restrict__ Cc,
+                                                         float* __restrict__ cnorm, int parents, int rows) {
   pdl_launch_dependents();   // the assign grid may start its set-up and loads
   const int row = (blockIdx.x * 256 + threadIdx.x) >> 3, part = threadIdx.x & 7;
   float s = 0.f;
   if (row < rows) {
-    const uint4* src = reinterpret_cast<const uint4*>(Cp + (size_t)row * D) + part;
+    const __nv_bfloat16* code = row < parents ? Cp + (size_t)row * D : Cc + (size_t)(row - parents) * D;
+    const uint4* src = reinterpret_cast<const uint4*>(code) + part;
 #pragma unroll
-    for (int t = 0; t < D / 64; ++t) {
-      const uint4 v = __ldg(src + 8 * t);
-      const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        s = fmaf(bf_lo(wv[e]), bf_lo(wv[e]), s);
-        s = fmaf(bf_hi(wv[e]), bf_hi(wv[e]), s);
-      }
-    }
+    for (int t = 0; t < D / 64; ++t) s = norm_bf16x8(s, __ldg(src + 8 * t));
   }
   s += __shfl_xor_sync(0xffffffffu, s, 1);
   s += __shfl_xor_sync(0xffffffffu, s, 2);
@@ -103,180 +112,234 @@ __global__ void __launch_bounds__(256) code_norms_kernel(const __nv_bfloat16* __
 // NL = 16-byte loads per lane that cover one parent's C x d block of children: C * d / 256.
 // STAYS: Algorithm 1's masked scatter - a key moves to its nearest child only if that child is strictly
 // closer than the parent (child index -1 otherwise).
-template <int D, int NL, bool STAYS>
-__global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D, NL))
+// RUNS: a CTA takes a run of tiles (else one: no loop state in registers).
+// TABLE: cnorm_g holds the squared norms of all codewords (parents [H, M], then children [H, M, C]); the child distances
+// are then ||c||^2 - 2 k.c at one mixed-precision multiply-add per element, half the instructions of the direct form.
+template <int D, int NL, bool STAYS, bool RUNS, bool TABLE>
+__global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D))
 tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmCp,
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
-                 int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int M, int C,
-                 uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, uint32_t zero_units,
+                 int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int M, int nblk, int total_tiles,
+                 int nbuf, uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, uint32_t zero_units,
                  const float* cnorm_g, int beside) {
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int kSub = D / 64;                       // 64-column sub-tiles along the head dimension
-  unsigned char* Ks = smem;                          // kSub x [128 x 128 B]
-  unsigned char* Cs = Ks + kSub * kKeys * 128;       // kSub x [M x 128 B]
+  constexpr int kKeyBytes = kSub * kKeys * 128;
+  if constexpr (!RUNS) nbuf = 1;
+  unsigned char* Cs = smem + nbuf * kKeyBytes;       // kSub x [M x 128 B]; before it nbuf key tiles, kSub x [128 x 128 B] each
   float* cnorm = reinterpret_cast<float*>(Cs + kSub * M * 128);   // [M]
-  float* xd1 = cnorm + M;                            // [2][128] best distance of each column half
-  float* xd2 = xd1 + 2 * kKeys;                      // [2][128] runner-up
-  float* xkn = xd2 + 2 * kKeys;                      // [2][128] halves of ||k||^2
-  int* xi1 = reinterpret_cast<int*>(xkn + 2 * kKeys);   // [2][128] index of the best
-  int* par = xi1 + 2 * kKeys;                        // [128] final parent of each key
+  float* xd = cnorm + M;                             // [2][128] smallest distance of each column half
+  float* xs = xd + 2 * kKeys;                        // [2][128] columns close to the minimum: sum of 256 + index
+  float* xkn = xs + 2 * kKeys;                       // [2][128] halves of ||k||^2
+  int* par = reinterpret_cast<int*>(xkn + 2 * kKeys);   // [128] final parent of each key
   int* chi = par + kKeys;                            // [128] final child of each key
   uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(chi + kKeys);   // max ||c||^2 (non-negative float bits)
   uint32_t* tmem_slot = cmax_bits + 1;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [2]
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [4]
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 4);
+  uint64_t *bar_k = bars, *bar_mma = bars + 2, *bar_c = bars + 3;   // key tile (per buffer), products, codebook
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
   const int q = warp & 3, hf = warp >> 2, r = q * 32 + lane;
-  const int bh = blockIdx.y, h = bh % H;
-  const int j0 = blockIdx.x * kKeys;
+  const int g = lane >> 2, t4 = lane & 3;            // fragment rows q*32 + g + 8 h, column pairs 2 t4
+  // This CTA's run of consecutive tiles (the CTAs with one more are the first ones: every SM gets its share).
+  int tile0 = (int)blockIdx.x, tile1 = tile0 + 1;
+  if constexpr (RUNS) {
+    const int per_cta = total_tiles / gridDim.x, more = total_tiles - per_cta * gridDim.x;
+    tile0 = (int)blockIdx.x * per_cta + min((int)blockIdx.x, more);
+    tile1 = tile0 + per_cta + ((int)blockIdx.x < more ? 1 : 0);
+  }
+  int bh = tile0 / nblk, blk = tile0 - bh * nblk;
   const int MH = M >> 1;                             // columns per half (multiple of 16: M % 32 == 0)
   pdl_launch_dependents();   // the next kernel of the call may begin its set-up
   // Inside avq_forward the grid also clears the accumulators of the aggregation that follows (status
   // header, leaf sums, leaf counts: zero_units 16-byte words), each CTA an equal slice; the stores drain
   // while the tile loads.  A bounded wait that expires does so long after CTA 0 has cleared the header.
   if (zero_units) {
-    const uint32_t ncta = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
+    const uint32_t ncta = gridDim.x, cta = blockIdx.x;
     const uint32_t per = (zero_units + ncta - 1) / ncta;
     const uint32_t u0 = cta * per, u1 = min(zero_units, u0 + per);
     for (uint32_t u = u0 + tid; u < u1; u += kThreadsA) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
   }
-  if (tid == 0) {
+  auto load_keys = [&](int buf, int b, int t) {      // one thread
+    mbar_expect_tx(&bar_k[buf], (uint32_t)kKeyBytes);
+#pragma unroll
+    for (int s = 0; s < kSub; ++s) tma_load_3d(smem + buf * kKeyBytes + s * kKeys * 128, &tmK, s * 64, t * kKeys, b, &bar_k[buf]);
+  };
+  auto load_codes = [&](int b) {
+    mbar_expect_tx(bar_c, (uint32_t)(kSub * M * 128));
+#pragma unroll
+    for (int s = 0; s < kSub; ++s) tma_load_2d(Cs + s * M * 128, &tmCp, s * 64, (b % H) * M, bar_c);
+  };
+  if (warp == 0 && elect_one()) {
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmCp);
-    mbar_init(&bars[0], 1);
-    mbar_init(&bars[1], 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mbar_init(&bars[i], 1);
     mbar_fence_init();
     *abort_flag = 0;
     *cmax_bits = 0;
-    mbar_expect_tx(&bars[0], (uint32_t)(kSub * (kKeys + M) * 128));
-#pragma unroll
-    for (int s = 0; s < kSub; ++s) {
-      tma_load_3d(Ks + s * kKeys * 128, &tmK, s * 64, j0, bh, &bars[0]);
-      tma_load_2d(Cs + s * M * 128, &tmCp, s * 64, h * M, &bars[0]);
-    }
+    load_keys(0, bh, blk);
+    load_codes(bh);
+    if (RUNS && nbuf == 2 && tile0 + 1 < tile1) load_keys(1, blk + 1 == nblk ? bh + 1 : bh, blk + 1 == nblk ? 0 : blk + 1);
   }
   // tcgen05.alloc blocks while the SM's columns are taken (four CTAs of 256 columns share an SM at d = 64,
   // M > 128: two run, two wait here).  The holders need nothing from the waiters and free their columns
   // before they end, so the wait is finite; it is the one device-side wait without a time limit of its own.
-  if (warp == 1) {                                   // not the warp whose lane 0 is busy issuing the loads
+  if (warp == 1) {                                   // not the warp that is busy issuing the loads
     tmem_alloc(tmem_slot, tmem_cols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
 
-  const bool loaded = mbar_wait(&bars[0], 0, abort_flag, status_word, DEV_TIMEOUT_ASSIGN);
-  if (tid == 0 && loaded) {
-    tc_fence_after();
-    const uint32_t idesc = umma_idesc_bf16(kKeys, M);
-    const uint32_t ka = smem_u32(Ks), ca = smem_u32(Cs);
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  auto issue_mma = [&](const unsigned char* keys) {  // one warp
+    if (elect_one()) {
+      tc_fence_after();
+      const uint32_t idesc = umma_idesc_bf16(kKeys, M);
+      const uint64_t kd = umma_desc_sw128(smem_u32(keys)), cd = umma_desc_sw128(smem_u32(Cs));
 #pragma unroll
-    for (int k = 0; k < D / 16; ++k)
-      umma_bf16(tmem_base, umma_desc_sw128(ka + (k / 4) * kKeys * 128 + (k % 4) * 32),
-                umma_desc_sw128(ca + (k / 4) * M * 128 + (k % 4) * 32), idesc, k > 0);
-    umma_commit(&bars[1]);
-  }
-
-  // ||c_m||^2 (and its maximum): from the array the kernel ahead of this one filled, or from the staged
-  // codebook; half of ||k||^2 per thread
-  if (cnorm_g) {
-    pdl_wait();
+      for (int k = 0; k < D / 16; ++k)
+        umma_bf16(tmem_base, kd + (uint64_t)((k / 4) * (kKeys * 8) + (k % 4) * 2),
+                  cd + (uint64_t)((k / 4) * M * 8 + (k % 4) * 2), idesc, k > 0);
+      umma_commit(bar_mma);
+    }
+    __syncwarp();
+  };
+  uint32_t ph_k = 0, ph_mma = 0, ph_c = 0;           // ph_k: bit per buffer
+  bool new_head = true, mma_issued = false;
+  for (int tile = tile0, buf = 0;; ++tile, buf = RUNS && nbuf == 2 ? buf ^ 1 : 0) {
+  const int h = bh % H, j0 = blk * kKeys;
+  const int nbh = blk + 1 == nblk ? bh + 1 : bh, nblk_ = blk + 1 == nblk ? 0 : blk + 1;
+  const bool has_next = RUNS && tile + 1 < tile1, next_new_head = has_next && nbh != bh && H > 1;
+  const unsigned char* Ks = smem + buf * kKeyBytes;
+  // ||c_m||^2 (and its maximum) of a head: from the array the kernel ahead of this one filled, or from the staged
+  // codebook
+  bool codes = true;
+  if (new_head) {
+    codes = mbar_wait(bar_c, ph_c, abort_flag, status_word, DEV_TIMEOUT_ASSIGN);
+    ph_c ^= 1;
+    if (TABLE) pdl_wait();
     for (int m = tid; m < M; m += kThreadsA) {
-      const float s = ld_after_wait(cnorm_g + (size_t)h * M + m);
+      float s = 0.f;
+      if (TABLE) {
+        s = ld_after_wait(cnorm_g + (size_t)h * M + m);
+      } else {
+#pragma unroll
+        for (int sub = 0; sub < kSub; ++sub)
+#pragma unroll
+          for (int ch = 0; ch < 8; ++ch)
+            s = norm_bf16x8(s, *reinterpret_cast<const uint4*>(Cs + sub * M * 128 + sw128_offset(m, ch * 8)));
+      }
       cnorm[m] = s;
       atomicMax(cmax_bits, __float_as_uint(s));
     }
-  } else
-  for (int m = tid; m < M; m += kThreadsA) {
-    float s = 0.f;
-#pragma unroll
-    for (int sub = 0; sub < kSub; ++sub) {
-#pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {
-        const uint4 v = *reinterpret_cast<const uint4*>(Cs + sub * M * 128 + sw128_offset(m, ch * 8));
-        const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          s = fmaf(bf_lo(wv[e]), bf_lo(wv[e]), s);
-          s = fmaf(bf_hi(wv[e]), bf_hi(wv[e]), s);
-        }
-      }
-    }
-    cnorm[m] = s;
-    atomicMax(cmax_bits, __float_as_uint(s));
   }
-  {
+  const bool loaded = mbar_wait(&bar_k[buf], (ph_k >> buf) & 1u, abort_flag, status_word, DEV_TIMEOUT_ASSIGN) && codes;
+  ph_k ^= 1u << buf;
+  if (warp == 0 && loaded && !mma_issued) issue_mma(Ks);   // (all lanes wait for the same barriers and agree)
+  mma_issued = false;
+
+  {                                                  // half of ||k||^2 per thread
     float s = 0.f;
     constexpr int kChunksHalf = D / 16;              // 16-byte chunks in half a row
 #pragma unroll
     for (int cc = 0; cc < kChunksHalf; ++cc) {
       const int ch = hf * kChunksHalf + cc;          // chunk index in the row, 0 .. D/8-1
-      const uint4 v = *reinterpret_cast<const uint4*>(Ks + (ch >> 3) * kKeys * 128 + sw128_offset(r, (ch & 7) * 8));
-      const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        s = fmaf(bf_lo(wv[e]), bf_lo(wv[e]), s);
-        s = fmaf(bf_hi(wv[e]), bf_hi(wv[e]), s);
-      }
+      s = norm_bf16x8(s, *reinterpret_cast<const uint4*>(Ks + (ch >> 3) * kKeys * 128 + sw128_offset(r, (ch & 7) * 8)));
     }
     xkn[hf * kKeys + r] = s;
   }
   __syncthreads();   // cnorm, cmax visible
 
-  const bool done = mbar_wait(&bars[1], 0, abort_flag, status_word, DEV_TIMEOUT_ASSIGN);
+  const bool done = mbar_wait(bar_mma, ph_mma, abort_flag, status_word, DEV_TIMEOUT_ASSIGN);
+  ph_mma ^= 1;
   tc_fence_after();
 
-  // ---- parent argmin over this thread's half of the columns
-  {
-    float d1 = INFINITY, d2 = INFINITY;
-    int i1 = 0;
-    const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * MH);
-    for (int c0 = 0; c0 < MH; c0 += 16) {
-      float dot[16];
-      tmem_ld16(trow + c0, dot);                     // warp-collective: executed by every lane
-      const float4* cn4 = reinterpret_cast<const float4*>(cnorm + hf * MH + c0);
+  // ---- parents: minimum of ||c||^2 - 2 k.c over this warp's half of the columns
+  const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * MH);
+  const float* cnh = cnorm + hf * MH;
+  const f32x2 minus2 = pack2(-2.f, -2.f);
+  float m[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float4 cn = cn4[u];
-        const float dist[4] = {fmaf(-2.f, dot[4 * u], cn.x), fmaf(-2.f, dot[4 * u + 1], cn.y),
-                               fmaf(-2.f, dot[4 * u + 2], cn.z), fmaf(-2.f, dot[4 * u + 3], cn.w)};
+  for (int h4 = 0; h4 < 4; ++h4) m[h4] = INFINITY;
+  auto blocks = [&](auto nb, int c0, auto&& use) {   // distances of nb 8-column blocks from column c0, pair by pair
+    constexpr int NBk = decltype(nb)::value;
+    uint32_t s[2][4 * NBk];
+    tmem_ld_frag<NBk>(trow + c0, s);                 // warp-collective
+    f32x2 cn[NBk];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          d2 = fminf(d2, fmaxf(dist[e], d1));        // runner-up: second smallest so far
-          if (dist[e] < d1) { d1 = dist[e]; i1 = hf * MH + c0 + 4 * u + e; }
-        }
+    for (int b = 0; b < NBk; ++b) cn[b] = *reinterpret_cast<const f32x2*>(cnh + c0 + 8 * b + 2 * t4);
+    tmem_ld_wait_frag<NBk>(s);
+#pragma unroll
+    for (int b = 0; b < NBk; ++b)
+#pragma unroll
+      for (int h4 = 0; h4 < 4; ++h4) {
+        float lo, hi;
+        unpack2(fma2(pack2u(s[h4 >> 1][4 * b + 2 * (h4 & 1)], s[h4 >> 1][4 * b + 2 * (h4 & 1) + 1]), minus2, cn[b]), lo, hi);
+        use(h4, c0 + 8 * b, lo, hi);
       }
-    }
-    xd1[hf * kKeys + r] = d1;
-    xd2[hf * kKeys + r] = d2;
-    xi1[hf * kKeys + r] = i1;
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
-
-  // ---- merge the halves (the lower half holds the lower indices, so it wins ties); recheck near-ties
-  const __nv_bfloat16* Cph = Cp + (size_t)h * M * D;
-  if (hf == 0) {
-    const float a1 = xd1[r], a2 = xd2[r], b1 = xd1[kKeys + r], b2 = xd2[kKeys + r];
-    int i1 = (b1 < a1) ? xi1[kKeys + r] : xi1[r];
-    const float d1 = fminf(a1, b1);
-    const float d2 = fminf(fmaxf(a1, b1), fminf(a2, b2));
-    const float knorm = xkn[r] + xkn[kKeys + r];
-    const float cmax = __uint_as_float(*cmax_bits);
+  };
+  auto all_blocks = [&](auto&& use) {
+    int c0 = 0;
+    if constexpr (D > 64)                            // (the 64-register budget of d = 64 holds 16 columns at a time)
+      for (; c0 + 32 <= MH; c0 += 32) blocks(std::integral_constant<int, 4>{}, c0, use);
+    for (; c0 < MH; c0 += 16) blocks(std::integral_constant<int, 2>{}, c0, use);
+  };
+  all_blocks([&](int h4, int, float lo, float hi) { m[h4] = min3(m[h4], lo, hi); });
+#pragma unroll
+  for (int h4 = 0; h4 < 4; ++h4) m[h4] = quad_min(m[h4]);
+  xd[hf * kKeys + q * 32 + g + 8 * t4] = pick4(m, t4);
+  asm volatile("bar.sync %0, 64;" ::"r"(q + 1) : "memory");   // the two warps that share these keys
+  float lim[4];
+  {
     // The MMA accumulates k.c in fp32: its error is a small multiple of 2^-24 * ||k|| * ||c||, which
     // 2e-4 * (||k||^2 + max ||c||^2) bounds with a wide margin.
-    if (done && j0 + r < Nk && !(d2 - d1 > 2e-4f * (knorm + cmax))) {
+    const float knorm = xkn[r] + xkn[kKeys + r], cmax = __uint_as_float(*cmax_bits);
+    const float l = fminf(xd[r], xd[kKeys + r]) + 2e-4f * (knorm + cmax);
+#pragma unroll
+    for (int h4 = 0; h4 < 4; ++h4) lim[h4] = __shfl_sync(0xffffffffu, l, g + 8 * h4);
+  }
+  // ---- the columns within that of the minimum: one, as a rule
+  float hits[4] = {0.f, 0.f, 0.f, 0.f};
+  {
+    const float col0 = (float)(256 + hf * MH + 2 * t4);
+    all_blocks([&](int h4, int c, float lo, float hi) {
+      const float w0 = col0 + (float)c;
+      if (lo <= lim[h4]) hits[h4] += w0;
+      if (hi <= lim[h4]) hits[h4] += w0 + 1.f;
+    });
+  }
+#pragma unroll
+  for (int h4 = 0; h4 < 4; ++h4) hits[h4] = quad_sum(hits[h4]);
+  xs[hf * kKeys + q * 32 + g + 8 * t4] = pick4(hits, t4);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1 && !has_next) tmem_dealloc(tmem_base, tmem_cols);
+  // the products have been read: those of the next tile, if its keys have a buffer of their own, run beside the rest
+  if (nbuf == 2 && has_next && !next_new_head) {
+    if (warp == 0 && mbar_wait(&bar_k[buf ^ 1], (ph_k >> (buf ^ 1)) & 1u, abort_flag, status_word, DEV_TIMEOUT_ASSIGN)) {
+      tc_fence_after();
+      issue_mma(smem + (buf ^ 1) * kKeyBytes);
+    }
+    mma_issued = true;
+  }
+
+  const __nv_bfloat16* Cph = Cp + (size_t)h * M * D;
+  if (hf == 0) {
+    const float s = xs[r] + xs[kKeys + r];           // < 512: a single column, 256 + index
+    int i1 = (s >= 256.f && s < 512.f) ? (int)s - 256 : 0;
+    if (done && j0 + r < Nk && !(s >= 256.f && s < 512.f)) {
       double best = INFINITY;
       int bi = 0;
-      for (int m = 0; m < M; ++m) {
-        const double s = exact_dist_smem<D>(Ks, r, Cph + (size_t)m * D);
-        if (s < best) { best = s; bi = m; }
+      for (int mm = 0; mm < M; ++mm) {
+        const double sd = exact_dist_smem<D>(Ks, r, Cph + (size_t)mm * D);
+        if (sd < best) { best = sd; bi = mm; }
       }
       i1 = bi;
     }
@@ -290,39 +353,62 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     // parent's C children (the group reads 64 contiguous bytes of a child row per load), keeps one running
     // sum per child, and a transposing butterfly over the four lanes leaves child s (and s + 4) in lane s.
     // The loads of the next chunk column are in flight while the current one is squared.
-    constexpr int kC = NL * 256 / D;                   // children per parent (4 or 8)
+    constexpr int kC = NL * 256 / D;                   // children per parent (4 or 8), four at a time
     constexpr int kChunks = D / 8;                     // 16-byte chunks per row
     constexpr int kT = kChunks / 4;                    // chunk columns per lane (2 or 4)
-    constexpr int kSteps = 2 * kT;                     // (pass, chunk column) pairs
+    constexpr int kF = kC / 4;                         // groups of four children
+    constexpr int kSteps = 2 * kT * kF;                // (pass, chunk column, group) triples
     const int s4 = lane & 3, grp = lane >> 2;
     const size_t head_base = (size_t)h * M;
-    uint4 buf[2][kC];
-    auto issue = [&](int step, uint4 (&dst)[kC]) {
-      const int key = warp * 16 + (step / kT) * 8 + grp;
-      const uint4* src = reinterpret_cast<const uint4*>(Cc + (head_base + par[key]) * kC * D) + (s4 + 4 * (step % kT));
-  #pragma unroll
-      for (int c = 0; c < kC; ++c) dst[c] = __ldg(src + c * kChunks);
+    uint4 buf4[2][4];
+    auto issue = [&](int step, uint4 (&dst)[4]) {
+      const int key = warp * 16 + (step / (kT * kF)) * 8 + grp;
+      const uint4* src = reinterpret_cast<const uint4*>(Cc + ((head_base + par[key]) * kC + 4 * (step % kF)) * D) +
+                         (s4 + 4 * ((step / kF) % kT));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) dst[c] = __ldg(src + c * kChunks);
     };
     float sum[kC];
-    float sum_p = 0.f;                                   // STAYS: direct-form distance to the parent itself
-    issue(0, buf[0]);
-  #pragma unroll
+    float sum_p = 0.f;                                   // STAYS: the same for the parent itself
+    issue(0, buf4[0]);
+    float ncv[2][kC / 4];                                // TABLE: norms of child s4 (and s4 + 4) of this lane's keys
+    if constexpr (TABLE) {
+#pragma unroll
+      for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+        for (int i = 0; i < kC / 4; ++i)
+          ncv[pass][i] = ld_after_wait(cnorm_g + (size_t)H * M + (head_base + par[warp * 16 + pass * 8 + grp]) * kC + s4 + 4 * i);
+    }
+    typename std::conditional<TABLE, uint4, KeyChunk>::type kv;
+#pragma unroll
     for (int step = 0; step < kSteps; ++step) {
-      const int pass = step / kT, t = step % kT;
+      const int pass = step / (kT * kF), t = (step / kF) % kT, f = step % kF;
       const int key = warp * 16 + pass * 8 + grp;
-      if (step + 1 < kSteps) issue(step + 1, buf[(step + 1) & 1]);
-      if (t == 0) {
-  #pragma unroll
+      if (step + 1 < kSteps) issue(step + 1, buf4[(step + 1) & 1]);
+      if (t == 0 && f == 0) {
+#pragma unroll
         for (int c = 0; c < kC; ++c) sum[c] = 0.f;
         sum_p = 0.f;
       }
       const int ch = s4 + 4 * t;
-      const KeyChunk kv = widen8(*reinterpret_cast<const uint4*>(Ks + (ch >> 3) * (kKeys * 128) + sw128_offset(key, (ch & 7) * 8)));
-  #pragma unroll
-      for (int c = 0; c < kC; ++c) sum[c] += sqdiff8(kv, buf[step & 1][c]);
-      if constexpr (STAYS)
-        sum_p += sqdiff8(kv, __ldg(reinterpret_cast<const uint4*>(Cp + (head_base + par[key]) * D) + ch));
-      if (t == kT - 1) {
+      if (f == 0) {
+        const uint4 kw = *reinterpret_cast<const uint4*>(Ks + (ch >> 3) * (kKeys * 128) + sw128_offset(key, (ch & 7) * 8));
+        if constexpr (TABLE) kv = kw;
+        else kv = widen8(kw);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if constexpr (TABLE) dot_bf16x8(sum[4 * f + c], kv, buf4[step & 1][c]);
+        else sum[4 * f + c] += sqdiff8(kv, buf4[step & 1][c]);
+      }
+      if constexpr (STAYS) {
+        if (f == 0) {
+          const uint4 pw = __ldg(reinterpret_cast<const uint4*>(Cp + (head_base + par[key]) * D) + ch);
+          if constexpr (TABLE) dot_bf16x8(sum_p, kv, pw);
+          else sum_p += sqdiff8(kv, pw);
+        }
+      }
+      if (t == kT - 1 && f == kF - 1) {
         // transpose-reduce over the group: after the two exchanges lane s holds the total of child s
         // (and of child s + 4 when C = 8)
         const bool hi1 = (s4 & 1) != 0, hi2 = (s4 & 2) != 0;
@@ -339,6 +425,21 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           const float send = hi2 ? r[2 * i] : r[2 * i + 1];
           const float keep = hi2 ? r[2 * i + 1] : r[2 * i];
           tot[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+        }
+        // Closer than this two distances are decided in float64.  Direct form: relative.  With the table: the dot
+        // product is a chain of D / 4 exact products in fp32 and two additions, the norms one of D / 8 and three, so a
+        // distance is off by at most 2 (D/4 + 2) 2^-24 |k||c| + (D/8 + 3) 2^-24 |c|^2 < 3.3e-6 (|k|^2 + |c|^2) at D = 128,
+        // two of them by less than 1e-5 (|k|^2 + max |c|^2).
+        float near = 0.f;
+        if constexpr (TABLE) {
+          float cmx = STAYS ? cnorm[par[key]] : 0.f;
+#pragma unroll
+          for (int i = 0; i < kC / 4; ++i) {
+            cmx = fmaxf(cmx, ncv[pass][i]);
+            tot[i] = fmaf(-2.f, tot[i], ncv[pass][i]);
+          }
+          cmx = quad_max(cmx);
+          near = 1e-5f * (xkn[key] + xkn[kKeys + key] + cmx);
         }
         float e1 = tot[0], e2 = INFINITY;
         int c1 = s4;
@@ -358,8 +459,45 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if constexpr (STAYS) {
           dp = sum_p + __shfl_xor_sync(0xffffffffu, sum_p, 1);
           dp += __shfl_xor_sync(0xffffffffu, dp, 2);
+          if constexpr (TABLE) dp = fmaf(-2.f, dp, cnorm[par[key]]);
         }
-        if (s4 == 0) {
+        if constexpr (TABLE) {
+          // float64, direct form, a quarter of the dimensions per lane of the key's group
+          auto exact4 = [&](const __nv_bfloat16* c) {
+            double sd = 0.0;
+            for (int u = 0; u < kT; ++u)
+              for (int e = 0; e < 8; ++e) {
+                const int col = 8 * (s4 + 4 * u) + e;
+                const double x = (double)key_elem<D>(Ks, key, col) - (double)__bfloat162float(c[col]);
+                sd += x * x;
+              }
+            sd += __shfl_xor_sync(0xffffffffu, sd, 1);
+            return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
+          };
+          const bool live = done && j0 + key < Nk;
+          const __nv_bfloat16* Cch = Cc + (head_base + par[key]) * kC * D;
+          bool redo = live && !(e2 - e1 > near);
+          if (__any_sync(0xffffffffu, redo)) {
+            double best = INFINITY;
+            int bi = 0;
+            for (int c = 0; c < kC; ++c) {
+              const double sd = exact4(Cch + (size_t)c * D);
+              if (sd < best) { best = sd; bi = c; }
+            }
+            if (redo) c1 = bi;
+          }
+          if constexpr (STAYS) {
+            // strict '<' against the parent distance; float64 when the two are closer than fp32 separates
+            bool moved = e1 < dp;
+            redo = redo || (live && !(fabsf(e1 - dp) > near));
+            if (__any_sync(0xffffffffu, redo)) {
+              const bool closer = exact4(Cch + (size_t)c1 * D) < exact4(Cp + (head_base + par[key]) * D);
+              if (redo) moved = closer;
+            }
+            if (!moved) c1 = -1;
+          }
+          if (s4 == 0) chi[key] = c1;
+        } else if (s4 == 0) {
           bool rechecked = false;
           double best = INFINITY;
           if (done && j0 + key < Nk && !(e2 - e1 > 1e-4f * e2)) {
@@ -394,6 +532,21 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     pidx[(size_t)bh * Nk + j0 + tid] = par[tid];
     cidx[(size_t)bh * Nk + j0 + tid] = chi[tid];
   }
+  // every thread is past its last read of this key tile (and of the codebook): refill
+  if (warp == 0 && has_next && elect_one()) {
+    if (nbuf == 1) load_keys(0, nbh, nblk_);
+    else if (tile + 2 < tile1) load_keys(buf, nblk_ + 1 == nblk ? nbh + 1 : nbh, nblk_ + 1 == nblk ? 0 : nblk_ + 1);
+    if (next_new_head) {
+      *cmax_bits = 0;
+      load_codes(nbh);
+    }
+  }
+  new_head = next_new_head;
+  bh = nbh;
+  blk = nblk_;
+  if (!has_next) break;
+  if (next_new_head) __syncthreads();                // cmax_bits is clear
+  }   // tiles
   if (beside) pdl_wait();    // this grid's completion then implies that of the one it ran beside
 }
 
@@ -401,6 +554,28 @@ uint32_t pow2_cols(int n) {
   uint32_t c = 32;
   while ((int)c < n) c <<= 1;
   return c;
+}
+
+template <int D, int NL, bool STAYS, bool RUNS, bool TABLE>
+avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const avq_problem& p, const void* Cp,
+                         const void* Cc, int32_t* pidx, int32_t* cidx, int32_t* status_word, void* zero_base,
+                         size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, int nbuf, size_t smem,
+                         unsigned grid, cudaStream_t st) {
+  auto kern = tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>;
+  // The limit is set once per device and instantiation (setting it again is harmless if two threads race).
+  static size_t configured[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return AVQ_ERR_CUDA;
+    if (dev >= 0 && dev < 64) configured[dev] = smem;
+  }
+  // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
+  return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
+                            static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,
+                            p.H, p.Nk, p.M, nblk, total, nbuf, pow2_cols(p.M), status_word,
+                            static_cast<uint4*>(zero_base), (uint32_t)(zero_bytes / 16), cnorm, beside ? 1 : 0));
 }
 
 template <int D, int NL, bool STAYS>
@@ -421,31 +596,47 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
     avq_status s = make_tmap_bf16(&tmCp, Cp, 2, dims, box);
     if (s != AVQ_OK) return s;
   }
-  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 +
-                      sizeof(float) * (p.M + 6 * kKeys) +
-                      sizeof(int) * (4 * kKeys) + 64 + 1024;
-  auto kern = tc_assign_kernel<D, NL, STAYS>;
-  // The limit is set once per device and instantiation (setting it again is harmless if two threads race).
-  static size_t configured[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return AVQ_ERR_CUDA;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
+  // Key tiles: two buffers where that does not cost a resident CTA.
+  auto bytes = [&](int nbuf) {
+    return (size_t)(D / 64) * (nbuf * kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys) + 96;
+  };
+  constexpr size_t kSmSmem = 227 * 1024;
+  auto resident = [&](int nbuf) { return (int)min((size_t)assign_min_ctas(D), kSmSmem / (bytes(nbuf) + 1024)); };
+  const uint32_t cols = pow2_cols(p.M);
+  int sms = 148;
+  {
+    static int sm_count[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+    sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
+    if (sms <= 0) {
+      if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AVQ_ERR_CUDA;
+      if (dev >= 0 && dev < 64) sm_count[dev] = sms;
+    }
   }
-  dim3 grid((p.Nk + kKeys - 1) / kKeys, (unsigned)BH);
+  const int nblk = (p.Nk + kKeys - 1) / kKeys;
+  if ((uint64_t)nblk * BH > 0x7fffffffull) return AVQ_ERR_UNSUPPORTED;
+  const int total = (int)(nblk * BH);
+  // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, pays from four tiles per
+  // CTA on (N16384 H16 d128 M256, 6.9 tiles: 72 -> 63 us); with fewer the uneven last round costs more than the
+  // set-up it saves (B2 H8 N5000 d128, 2.2 tiles: whole call 111 -> 130 us), and where the columns of the resident
+  // CTAs exceed TMEM, so that they take them in turn, it costs too (N65536 d64 M256: whole call 780 -> 960 us).
+  const int nbuf2 = resident(2) >= resident(1) ? 2 : 1;
+  const bool shared_cols = (int)cols * resident(1) > 512;
+  const bool runs = !shared_cols && (int64_t)total >= 4ll * resident(nbuf2) * sms;
+  const int nbuf = runs ? nbuf2 : 1;
+  const size_t smem = bytes(nbuf);
   if (cnorm) {
-    const int rows = p.H * p.M;
+    const int parents = p.H * p.M, rows = parents * (1 + p.C);
     if (launch_pdl(code_norms_kernel<D>, dim3((rows * 8 + 255) / 256), dim3(256), 0, st, beside,
-                   static_cast<const __nv_bfloat16*>(Cp), cnorm, rows) != cudaSuccess)
+                   static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), cnorm, parents,
+                   rows) != cudaSuccess)
       return AVQ_ERR_CUDA;
   }
-  // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
-  return cuda_ok(launch_pdl(kern, grid, dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
-                            static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,
-                            p.H, p.Nk, p.M, p.C, pow2_cols(p.M), status_word, static_cast<uint4*>(zero_base),
-                            (uint32_t)(zero_bytes / 16), static_cast<const float*>(cnorm), beside ? 1 : 0));
+  auto go = cnorm ? (runs ? launch_kernel<D, NL, STAYS, true, true> : launch_kernel<D, NL, STAYS, false, true>)
+                  : (runs ? launch_kernel<D, NL, STAYS, true, false> : launch_kernel<D, NL, STAYS, false, false>);
+  return go(tmK, tmCp, p, Cp, Cc, pidx, cidx, status_word, zero_base, zero_bytes, cnorm, beside, nblk, total, nbuf, smem,
+            (unsigned)(runs ? resident(nbuf) * sms : total), st);
 }
 
 }  // namespace

@@ -66,176 +66,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// ---- packed pairs of fp32 (two neighbouring columns of one row)
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ f32x2 pack2u(uint32_t lo, uint32_t hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-// z += both halves of a bf16 pair (mixed-precision adds: no widening instructions)
-__device__ __forceinline__ void add_bf16x2(float& z, uint32_t pk) {
-  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %0, h, %0;\n\t}"
-      : "+f"(z) : "r"(pk));
-}
-
-// ---- accumulator fragments: NB blocks of 8 columns x 32 rows per warp.  r[half][4 b + 2 u + v] = row
-// 16 half + 8 u + g, column 8 b + 2 t + v.
-template <int NB>
-__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[2][4 * NB]) {
-  static_assert(NB == 2 || NB == 4, "16 or 32 columns");
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t* q = r[h];
-    const uint32_t a = taddr + ((uint32_t)(16 * h) << 16);
-    if constexpr (NB == 4)
-      asm volatile(
-          "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-          : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
-            "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
-          : "r"(a) : "memory");
-    else
-      asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7])
-                   : "r"(a) : "memory");
-  }
-}
-// M codeword rows of 64 columns in the order of parent_pos: dimensions (column, v, t, group of 8)
-__device__ __forceinline__ void tma_load_codes(void* dst, const CUtensorMap* map, int x, int group, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %4, %5}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(0), "r"(group)
-      : "memory");
-}
-// Waits for this warp's TMEM loads; the registers pass through so that no use of them moves ahead of the wait.
-template <int NB>
-__device__ __forceinline__ void tmem_ld_wait_frag(uint32_t (&r)[2][4 * NB]) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int c = 0; c < NB / 2; ++c) {
-      uint32_t* q = r[h] + 8 * c;
-      if (h == 0 && c == 0)
-        asm volatile("tcgen05.wait::ld.sync.aligned;"
-                     : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7])::"memory");
-      else
-        asm volatile("" : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7])::"memory");
-    }
-}
-template <int NB>
-__device__ __forceinline__ void tmem_st_frag(uint32_t taddr, const uint32_t (&r)[2][4 * NB]) {
-  static_assert(NB == 2, "16 columns");
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const uint32_t* q = r[h];
-    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
-                     taddr + ((uint32_t)(16 * h) << 16)),
-                 "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
-                 : "memory");
-  }
-}
-// bf16 weights of 32 columns x 32 rows (16 TMEM columns, the K-major A operand of the value MMA):
-// r[half][2 b + u] = columns 8 b + 2 t, + 1 of row 16 half + 8 u + g.
-__device__ __forceinline__ void tmem_st_weights(uint32_t taddr, const uint32_t (&r)[2][8]) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const uint32_t* q = r[h];
-    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
-                     taddr + ((uint32_t)(16 * h) << 16)),
-                 "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
-                 : "memory");
-  }
-}
-// D += A . B with A (bf16, K-major) in TMEM
-__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                             bool accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
-      : "memory");
-}
-// Four 8 x 8 bf16 blocks (rows 0-7, 8-15, 16-23, 24-31 of the warp, one 8-column block): lane l supplies the
-// address of row l's 16 bytes.
-__device__ __forceinline__ void stmatrix4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2),
-               "r"(r3)
-               : "memory");
-}
-// One lane of a converged warp.  With a warp-uniform condition around it (the warp index comes from a shuffle) the
-// compiler keeps descriptors and coordinates in uniform registers; behind `if (lane == 0)` every tcgen05.mma or TMA
-// instruction moved them there again, which took 130 instead of 50 cycles each beside busy warps.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ float quad_max(float v) {
-  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
-  return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
-}
-__device__ __forceinline__ float quad_sum(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  return v + __shfl_xor_sync(0xffffffffu, v, 2);
-}
-__device__ __forceinline__ float pick4(const float (&v)[4], int t) {
-  const float a = (t & 1) ? v[1] : v[0], b = (t & 1) ? v[3] : v[2];
-  return (t & 2) ? b : a;
-}
-
-// Column sums over the 8 lanes (stride 4) that share a column: v[NB] pairs per lane; lane 4 g + t returns the pair
-// of block g (NB = 8) or g / 2 (NB = 4).
-template <int NB>
-__device__ __forceinline__ f32x2 reduce_rows(f32x2 (&v)[NB], int lane) {
-  int n = NB;
-#pragma unroll
-  for (int b = 16; b >= 4; b >>= 1) {
-    if (n > 1) {
-      n >>= 1;
-      const bool hi = (lane & b) != 0;
-#pragma unroll
-      for (int i = 0; i < NB / 2; ++i)
-        if (i < n) {
-          const f32x2 send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
-          v[i] = add2(keep, __shfl_xor_sync(0xffffffffu, send, b));
-        }
-    } else {
-      v[0] = add2(v[0], __shfl_xor_sync(0xffffffffu, v[0], b));
-    }
-  }
-  return v[0];
-}
-
 // The NQ warps that share a quarter of the rows (warp % 4 == q) exchange per-row values through shared
 // memory; they synchronise among themselves on named barrier q + 1 instead of stalling the whole CTA.
 template <int NQ>
