@@ -43,27 +43,40 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, const float4& v) {
   *reinterpret_cast<uint2*>(p) = u;
 }
 
-constexpr int kThreads = 256;      // 16 x 16: thread (ty, tx) owns rows ty*4 (+64), columns tx*4
+constexpr int kThreads = 256;      // of the assign and aggregate kernels: 16 x 16, thread (ty, tx) owns rows ty*4, columns tx*4
 constexpr int kCols = 64;          // columns (codewords) of a tile
 constexpr int kLdC = kCols + 4;    // row pitch of a [k][column] operand, floats
 
 // Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r], k < d: the transposed
 // operand of the register-tiled products.  A warp takes 8 rows x 4 chunks of 4 elements: 64-byte pieces of a
 // row in global memory, at most two-way bank conflicts in shared memory.
-template <typename Src>
+template <int THREADS, typename Src>
 __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Src src) {
+  constexpr int kWarps = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kc = lane & 3, rr = lane >> 2;
-  const int chunks = d >> 2, cblocks = (chunks + 3) >> 2;
-  for (int u = warp; u < (rows >> 3) * cblocks; u += kThreads / 32) {
-    const int rb = u / cblocks, cb = u - rb * cblocks;
-    const int r = rb * 8 + rr, c = cb * 4 + kc;
-    if (c < chunks) {
-      const auto* p = src(r);
-      const float4 v = p ? ld4(p + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      float* o = dst + (size_t)(4 * c) * ld + r;
-      o[0] = v.x; o[ld] = v.y; o[2 * ld] = v.z; o[3 * ld] = v.w;
+  const int chunks = d >> 2, cblocks = (chunks + 3) >> 2, units = (rows >> 3) * cblocks;
+  for (int u = warp; u < units; u += 2 * kWarps) {        // two loads in flight per trip
+    float4 v[2];
+    int at[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int ue = u + e * kWarps, rb = ue / cblocks, cb = ue - rb * cblocks;
+      const int r = rb * 8 + rr, c = cb * 4 + kc;
+      at[e] = -1;
+      v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ue < units && c < chunks) {
+        at[e] = 4 * c * ld + r;
+        const auto* p = src(r);
+        if (p) v[e] = ld4(p + 4 * c);
+      }
     }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (at[e] >= 0) {
+        float* o = dst + at[e];
+        o[0] = v[e].x; o[ld] = v[e].y; o[2 * ld] = v[e].z; o[3 * ld] = v[e].w;
+      }
   }
 }
 
@@ -72,13 +85,13 @@ __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, in
 template <int RT>
 __device__ __forceinline__ void mul_tile(float (&acc)[RT][4], const float* A, int lda, const float* B, int ldb, int K,
                                          int ty, int tx) {
-  const float* a_ = A + ty * 4;
+  const float* a_ = A + ty * RT;
   const float* b_ = B + tx * 4;
 #pragma unroll 4
   for (int k = 0; k < K; ++k) {
     float a[RT];
-    *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(a_ + k * lda);
-    if constexpr (RT == 8) *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(a_ + k * lda + 64);
+    if constexpr (RT == 4) *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(a_ + k * lda);
+    else *reinterpret_cast<float2*>(a) = *reinterpret_cast<const float2*>(a_ + k * lda);
     const float4 b = *reinterpret_cast<const float4*>(b_ + k * ldb);
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
@@ -135,7 +148,7 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const T* Kb = K + ((size_t)bh * Nk + j0) * d;
   const int rows = min(kAssignKeys, Nk - j0);
   const T* Cph = Cp + (size_t)h * M * d;
-  load_transposed(ks, kLdC, kAssignKeys, d, [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; });
+  load_transposed<kThreads>(ks, kLdC, kAssignKeys, d, [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; });
 
   float d1[4], d2[4];
   int i1[4];
@@ -144,7 +157,7 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   for (int m0 = 0; m0 < M; m0 += kCols) {
     const int w = min(kCols, M - m0);
     __syncthreads();
-    load_transposed(cs, kLdC, kCols, d, [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; });
+    load_transposed<kThreads>(cs, kLdC, kCols, d, [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; });
     __syncthreads();
     float acc[4][4] = {};
 #pragma unroll 4
@@ -323,21 +336,23 @@ struct AttendArgs {
   float scale;
 };
 
+constexpr int kAttThreads = 512;   // 32 x 16: thread (ty, tx) owns rows ty*RT .. , columns tx*4
+
 // Shared memory of attend_simt_kernel, in floats from the base (doubles first).
 struct AttendSmem {
   int ldr;                                   // pitch of a [k][row] operand
   size_t w, wpart, q, c, v, s, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
 };
-// RT = 8: 128 query rows at a time (d <= 128), RT = 4: 64 rows.  v == c where the two tiles share one buffer.
+// RT = 4: 128 query rows at a time (d <= 128), RT = 2: 64 rows.  v == c where the two tiles share one buffer.
 __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int block_q, int tile_m,
                                                          int keep) {
   AttendSmem L;
-  L.ldr = 16 * RT + 4;
+  L.ldr = 32 * RT + 4;
   const int ntiles = tile_m > 0 ? (M + tile_m - 1) / tile_m : 0;
   size_t o = 0;
   auto take = [&](size_t n) { size_t at = o; o += (n + 3) / 4 * 4; return at; };
   L.w = take(2 * (size_t)M);
-  L.wpart = take(2 * (size_t)(kThreads / 32) * kCols);
+  L.wpart = take(2 * (size_t)(kAttThreads / 32) * kCols);
   L.q = take((size_t)d * L.ldr);
   if (DT <= 2) {
     L.c = take((size_t)d * kLdC);
@@ -376,16 +391,18 @@ __device__ __forceinline__ float sum16(float v) {
 // Where the block's logits fit (a.keep) they are computed once and reused by B and C.  Bound: FFMA issue and
 // the shared-memory pipe (RT + 4 operands per 4 RT products).  Against one warp per query row with a lane per
 // logit, operands read from global memory for every product: whole forward fp32 B2 H12 N1024 d64 M64 C4 P8
-// 2660 -> 84 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.40 ms.
-template <typename T, int RT, int DT>
-__global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kernel(const AttendArgs a) {
+// 2660 -> 82 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.36 ms (84 us and 0.40 ms with 256 threads).
+// 512 threads with 4 rows each rather than 256 with 8: the same products per second, twice the warps for everything
+// that is a latency (operand loads, exponentials, exchanges), which was most of the time.
+template <typename T, int RT, int DT, bool CORR>
+__global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) attend_simt_kernel(const AttendArgs a) {
   extern __shared__ __align__(16) float sm[];
-  constexpr int R = 16 * RT;
+  constexpr int R = 32 * RT, kThreads = kAttThreads;
   const int d = a.d, M = a.M, C = a.C, P = a.P;
   const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.block_q, a.tile_m, a.keep);
   const int ldr = L.ldr;
   double* w = reinterpret_cast<double*>(sm + L.w);
-  double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [8][64]
+  double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [16][64]
   float *qs = sm + L.q, *cs = sm + L.c, *vs = sm + L.v, *ss = sm + L.s;
   float *npS = sm + L.np, *nstay = sm + L.nstay, *zt = sm + L.zt, *nseen = sm + L.nseen;
   int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
@@ -405,14 +422,14 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
   const float* np_ = a.np_ + (size_t)bh * M;
   const float* nc = a.nc + (size_t)bh * M * C;
 
-  auto row_of = [&](int i) { return (i < 4 ? 0 : 64) + ty * 4 + (i & 3); };
+  auto row_of = [&](int i) { return ty * RT + i; };
   auto load_q = [&](int rt) {
-    load_transposed(qs, ldr, R, d, [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; });
+    load_transposed<kThreads>(qs, ldr, R, d, [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; });
   };
   // Logits of this thread's RT x 4 block of a tile of n columns (row c of the tile at code(c)).  Ends with the
   // operands still being read by other threads: the caller synchronises before they are overwritten.
   auto logits = [&](float (&acc)[RT][4], int n, auto code) {
-    load_transposed(cs, kLdC, kCols, d, [&](int c) { return c < n ? code(c) : (const T*)nullptr; });
+    load_transposed<kThreads>(cs, kLdC, kCols, d, [&](int c) { return c < n ? code(c) : (const T*)nullptr; });
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < RT; ++i)
@@ -427,20 +444,21 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
   auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * 4;
-      *reinterpret_cast<float4*>(o) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
-      if constexpr (RT == 8) *reinterpret_cast<float4*>(o + 64) = make_float4(acc[4][j], acc[5][j], acc[6][j], acc[7][j]);
+      float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * RT;
+      if constexpr (RT == 4) *reinterpret_cast<float4*>(o) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+      else *reinterpret_cast<float2*>(o) = make_float2(acc[0][j], acc[1][j]);
     }
   };
   auto load_s = [&](const float* s0, float (&acc)[RT][4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * 4;
-      const float4 x = *reinterpret_cast<const float4*>(o);
-      acc[0][j] = x.x; acc[1][j] = x.y; acc[2][j] = x.z; acc[3][j] = x.w;
-      if constexpr (RT == 8) {
-        const float4 y = *reinterpret_cast<const float4*>(o + 64);
-        acc[4][j] = y.x; acc[5][j] = y.y; acc[6][j] = y.z; acc[7][j] = y.w;
+      const float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * RT;
+      if constexpr (RT == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(o);
+        acc[0][j] = x.x; acc[1][j] = x.y; acc[2][j] = x.z; acc[3][j] = x.w;
+      } else {
+        const float2 x = *reinterpret_cast<const float2*>(o);
+        acc[0][j] = x.x; acc[1][j] = x.y;
       }
     }
   };
@@ -571,14 +589,19 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
   // bit patterns.
   if (P > 0) {
     const unsigned long long* key = reinterpret_cast<const unsigned long long*>(w);
-    for (int j = tid; j < M; j += kThreads) {
+    int lt = 0;                                           // 2^lt threads share a key's scan
+    while (lt < 4 && (M << (lt + 1)) <= kThreads) ++lt;
+    const int part = tid & ((1 << lt) - 1);
+    for (int j0 = 0; j0 < M; j0 += kThreads >> lt) {      // uniform
+      const int j = j0 + (tid >> lt);
       int rank = 0;
-      if (P < M) {
+      if (P < M && j < M) {
         const unsigned long long kj = key[j];
-        for (int k = 0; k < j; ++k) rank += key[k] >= kj;
-        for (int k = j + 1; k < M; ++k) rank += key[k] > kj;
+#pragma unroll 8
+        for (int k = part; k < M; k += 1 << lt) rank += (key[k] > kj) | ((key[k] == kj) & (k < j));
       }
-      sel[j] = rank < P;
+      for (int o = 1; o < (1 << lt); o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      if (j < M && part == 0) sel[j] = rank < P;
     }
     __syncthreads();
     if (warp == 0) {
@@ -631,7 +654,7 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
         const int j = c0 + c;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c < n) {
-          const bool refined = sel[j] != 0 && !a.correcting;
+          const bool refined = sel[j] != 0 && !CORR;
           const float nn = refined ? (a.stays ? nstay[j] : 0.f) : npS[j];
           if (nn > 0.f) {
             v = ld_after_wait(reinterpret_cast<const float4*>(Vp + (size_t)j * d) + ch);
@@ -671,13 +694,12 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
             cnt[j] = ld_after_wait(nc + (size_t)sel_list[e / C] * C + e % C);
           } else {
             // correcting form: every parent keeps its full term here, the children add differences below
-            cnt[j] = (sel[c0 + c] && !a.correcting) ? (a.stays ? nstay[c0 + c] : 0.f) : npS[c0 + c];
+            cnt[j] = (sel[c0 + c] && !CORR) ? (a.stays ? nstay[c0 + c] : 0.f) : npS[c0 + c];
           }
         }
       }
-      float mean[RT][4];                                  // correcting form only
-      const bool corr = child && a.correcting;
-      if (corr) {
+      float mean[CORR ? RT : 1][4];                       // correcting form only
+      if (CORR && child) {
         // Eq. "parent_recovery": under parent = mean(children) the parent's logit is the mean of its
         // children's; Eq. "correcting_attention": the child's keys trade the parent's weight for their own
         store_s(sw, acc);
@@ -689,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
           for (int i = 0; i < RT; ++i) {
             float sp = 0.f;
             if (c < n) for (int c2 = 0; c2 < C; ++c2) sp += sw[(size_t)(f + c2) * ldr + row_of(i)];
-            mean[i][j] = sp / (float)C;
+            mean[CORR ? i : 0][j] = sp / (float)C;
           }
         }
         __syncthreads();
@@ -714,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, (DT == 1) ? 2 : 1) attend_simt_kerne
           float av = 0.f;
           if (cnt[j] > 0.f) {
             av = expf(acc[i][j] - m[i]);
-            if (corr) av -= expf(mean[i][j] - m[i]);
+            if (CORR && child) av -= expf(mean[CORR ? i : 0][j] - m[i]);
             z[i] = fmaf(av, cnt[j], z[i]);
           }
           acc[i][j] = av;
@@ -790,8 +812,8 @@ avq_status launch_aggregate(const avq_problem& p, const void* V, const int32_t* 
                                 status_word));
 }
 
-template <typename T, int RT, int DT>
-avq_status launch_attend_rd(AttendArgs a, int B, bool chained, cudaStream_t st) {
+template <typename T, int RT, int DT, bool CORR>
+avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st) {
   auto bytes = [&](int keep) {
     return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.block_q, a.tile_m, keep).total;
   };
@@ -802,25 +824,31 @@ avq_status launch_attend_rd(AttendArgs a, int B, bool chained, cudaStream_t st) 
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AVQ_ERR_CUDA;
   const bool one_wave = (int64_t)a.nblk * B * a.H <= sms;
   const size_t most = one_wave ? kSmemMax : kSmemHalf;
-  a.keep = (a.block_q <= 16 * RT && (a.tile_m == 0 || a.tile_m % kCols == 0) && bytes(1) <= most) ? 1 : 0;
+  a.keep = (a.block_q <= 32 * RT && (a.tile_m == 0 || a.tile_m % kCols == 0) && bytes(1) <= most) ? 1 : 0;
   const size_t smem = bytes(a.keep);
   if (smem > kSmemMax) return AVQ_ERR_UNSUPPORTED;
-  auto kern = attend_simt_kernel<T, RT, DT>;
+  auto kern = attend_simt_kernel<T, RT, DT, CORR>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return AVQ_ERR_CUDA;
-  return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kThreads), smem, st, chained, a));
+  return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kAttThreads), smem, st, chained, a));
+}
+
+template <typename T, int RT, int DT>
+avq_status launch_attend_rd(const AttendArgs& a, int B, bool chained, cudaStream_t st) {
+  return a.correcting ? launch_attend_rdc<T, RT, DT, true>(a, B, chained, st)
+                      : launch_attend_rdc<T, RT, DT, false>(a, B, chained, st);
 }
 
 template <typename T>
 avq_status launch_attend(const AttendArgs& a, int B, bool chained, cudaStream_t st) {
   if (simt_attend_smem_bytes(a.d, a.M, a.C, a.P, a.block_q, a.tile_m) > kSimtAttendSmemLimit)
     return AVQ_ERR_UNSUPPORTED;                           // validate_forward rejects these up front
-  // 128 rows at a time where the block has them and the accumulators fit the registers (d <= 128), else 64
-  if (a.block_q > 64 && a.d <= 64) return launch_attend_rd<T, 8, 1>(a, B, chained, st);
-  if (a.block_q > 64 && a.d <= 128) return launch_attend_rd<T, 8, 2>(a, B, chained, st);
-  if (a.d <= 64) return launch_attend_rd<T, 4, 1>(a, B, chained, st);
-  if (a.d <= 128) return launch_attend_rd<T, 4, 2>(a, B, chained, st);
-  return launch_attend_rd<T, 4, 4>(a, B, chained, st);
+  // 128 rows at a time where the block has them and shared memory holds them (d <= 128), else 64
+  if (a.block_q > 64 && a.d <= 64) return launch_attend_rd<T, 4, 1>(a, B, chained, st);
+  if (a.block_q > 64 && a.d <= 128) return launch_attend_rd<T, 4, 2>(a, B, chained, st);
+  if (a.d <= 64) return launch_attend_rd<T, 2, 1>(a, B, chained, st);
+  if (a.d <= 128) return launch_attend_rd<T, 2, 2>(a, B, chained, st);
+  return launch_attend_rd<T, 2, 4>(a, B, chained, st);
 }
 
 }  // namespace
