@@ -10,9 +10,12 @@
 //
 // The products (distances, logits, weighted value sums) are register-tiled: both operands of a product are
 // staged in shared memory as [contraction index][row or column], a thread keeps an RT x 4 block of results and
-// reads RT + 4 operands per step with 16-byte loads.
+// reads RT + 4 operands per step with 16-byte loads.  The logits of bfloat16 inputs are warp-level tensor-core products
+// (exact products, float32 sums, as on the FFMA path); everything behind them stays float32.
 #include <cuda_bf16.h>
 #include <math.h>
+
+#include <type_traits>
 
 #include "avq_internal.h"
 #include "avq_tc_common.cuh"
@@ -322,6 +325,65 @@ aggregate_simt_kernel(const T* __restrict__ V, const int32_t* pidx, const int32_
 }
 
 // ------------------------------------------------------------------------------- attend
+// `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
+template <int THREADS, typename Src>
+__device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
+  const int per = dpad >> 2, units = rows * per;
+  for (int u = threadIdx.x; u < units; u += 2 * THREADS) {
+    uint2 v[2];
+    int at[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int ue = u + e * THREADS, r = ue / per, c = ue - r * per;
+      at[e] = ue < units ? r * pitch + 4 * c : -1;
+      v[e] = make_uint2(0u, 0u);
+      if (ue < units && 4 * c < d) {
+        const __nv_bfloat16* p = src(r);
+        if (p) v[e] = __ldg(reinterpret_cast<const uint2*>(p + 4 * c));
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (at[e] >= 0) *reinterpret_cast<uint2*>(dst + at[e]) = v[e];
+  }
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+// s[column][row] = scale * Q . codes^T for 32 RT rows x 64 columns, 16 warps: 16 rows x 8 RT columns per warp
+template <int RT>
+__device__ __forceinline__ void mma_logits(float* s, int ldr, const __nv_bfloat16* q, const __nv_bfloat16* c, int pitch,
+                                           int dpad, float scale) {
+  constexpr int NT = RT;                                  // 8-column tiles per warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = (warp % (2 * RT)) * 16, n0 = (warp / (2 * RT)) * 8 * NT;
+  const __nv_bfloat16* ap = q + (r0 + (lane & 15)) * pitch + (lane >> 4) * 8;
+  const __nv_bfloat16* bp = c + (n0 + (lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 8;
+  float acc[NT][4] = {};
+#pragma unroll 4
+  for (int k = 0; k < dpad; k += 16) {
+    uint32_t a[4];
+    ldmatrix4(a, ap + k);
+#pragma unroll
+    for (int j = 0; j < NT; j += 2) {
+      uint32_t b[4];
+      ldmatrix4(b, bp + j * 8 * pitch + k);
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                     : "+f"(acc[j + e][0]), "+f"(acc[j + e][1]), "+f"(acc[j + e][2]), "+f"(acc[j + e][3])
+                     : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[2 * e]), "r"(b[2 * e + 1]));
+    }
+  }
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      s[(size_t)(n0 + 8 * j + 2 * t + (e & 1)) * ldr + r0 + g + 8 * (e >> 1)] = acc[j][e] * scale;
+}
+
 struct AttendArgs {
   const void *Q, *Cp, *Cc;
   const float *Vp, *np_, *Vc, *nc;
@@ -344,8 +406,9 @@ struct AttendSmem {
   size_t w, wpart, q, c, v, s, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
 };
 // RT = 4: 128 query rows at a time (d <= 128), RT = 2: 64 rows.  v == c where the two tiles share one buffer.
+// mma: Q and codewords as bfloat16 rows.
 __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int block_q, int tile_m,
-                                                         int keep) {
+                                                         int keep, bool mma) {
   AttendSmem L;
   L.ldr = 32 * RT + 4;
   const int ntiles = tile_m > 0 ? (M + tile_m - 1) / tile_m : 0;
@@ -353,13 +416,14 @@ __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, 
   auto take = [&](size_t n) { size_t at = o; o += (n + 3) / 4 * 4; return at; };
   L.w = take(2 * (size_t)M);
   L.wpart = take(2 * (size_t)(kAttThreads / 32) * kCols);
-  L.q = take((size_t)d * L.ldr);
+  const size_t pitch = (size_t)(d + 15) / 16 * 8 + 4;       // floats per bfloat16 row: padded to 16 elements, plus 8
+  const size_t cbytes = mma ? kCols * pitch : (size_t)d * kLdC, vbytes = (size_t)kCols * DT * 64;
+  L.q = take(mma ? 32 * RT * pitch : (size_t)d * L.ldr);
   if (DT <= 2) {
-    L.c = take((size_t)d * kLdC);
-    L.v = take((size_t)kCols * DT * 64);
+    L.c = take(cbytes);
+    L.v = take(vbytes);
   } else {
-    const size_t a = (size_t)d * kLdC, b = (size_t)kCols * DT * 64;
-    L.c = L.v = take(a > b ? a : b);
+    L.c = L.v = take(cbytes > vbytes ? cbytes : vbytes);
   }
   L.s = take((size_t)(keep ? (M + kCols - 1) / kCols * kCols : kCols) * L.ldr);
   L.np = take(M);
@@ -391,15 +455,19 @@ __device__ __forceinline__ float sum16(float v) {
 // Where the block's logits fit (a.keep) they are computed once and reused by B and C.  Bound: FFMA issue and
 // the shared-memory pipe (RT + 4 operands per 4 RT products).  Against one warp per query row with a lane per
 // logit, operands read from global memory for every product: whole forward fp32 B2 H12 N1024 d64 M64 C4 P8
-// 2660 -> 82 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.36 ms (84 us and 0.40 ms with 256 threads).
+// 2660 -> 82 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.36 ms (84 us and 0.40 ms with
+// 256 threads); with the bfloat16 logits on the tensor cores 0.27 ms.
 // 512 threads with 4 rows each rather than 256 with 8: the same products per second, twice the warps for everything
 // that is a latency (operand loads, exponentials, exchanges), which was most of the time.
-template <typename T, int RT, int DT, bool CORR>
-__global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) attend_simt_kernel(const AttendArgs a) {
+// WIDE: one CTA per SM with twice the registers, for grids of a wave at most (they measured 3 % faster there, fp32
+// B2 H12 N1024 in 192 CTAs 10 % slower).
+template <typename T, int RT, int DT, bool CORR, bool WIDE>
+__global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 : 1) attend_simt_kernel(const AttendArgs a) {
   extern __shared__ __align__(16) float sm[];
   constexpr int R = 32 * RT, kThreads = kAttThreads;
   const int d = a.d, M = a.M, C = a.C, P = a.P;
-  const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.block_q, a.tile_m, a.keep);
+  constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
+  const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.block_q, a.tile_m, a.keep, kMma);
   const int ldr = L.ldr;
   double* w = reinterpret_cast<double*>(sm + L.w);
   double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [16][64]
@@ -423,23 +491,11 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) atten
   const float* nc = a.nc + (size_t)bh * M * C;
 
   auto row_of = [&](int i) { return ty * RT + i; };
+  const int dpad = (d + 15) & ~15, pitch = dpad + 8;
   auto load_q = [&](int rt) {
-    load_transposed<kThreads>(qs, ldr, R, d, [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; });
-  };
-  // Logits of this thread's RT x 4 block of a tile of n columns (row c of the tile at code(c)).  Ends with the
-  // operands still being read by other threads: the caller synchronises before they are overwritten.
-  auto logits = [&](float (&acc)[RT][4], int n, auto code) {
-    load_transposed<kThreads>(cs, kLdC, kCols, d, [&](int c) { return c < n ? code(c) : (const T*)nullptr; });
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < RT; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    mul_tile<RT>(acc, qs, ldr, cs, kLdC, d, ty, tx);
-#pragma unroll
-    for (int i = 0; i < RT; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] *= a.scale;
+    auto row = [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; };
+    if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(qs), pitch, R, d, dpad, row);
+    else load_transposed<kThreads>(qs, ldr, R, d, row);
   };
   auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
 #pragma unroll
@@ -460,6 +516,32 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) atten
         const float2 x = *reinterpret_cast<const float2*>(o);
         acc[0][j] = x.x; acc[1][j] = x.y;
       }
+    }
+  };
+
+  // Logits of this thread's RT x 4 block of a tile of n columns (row c of the tile at code(c)), by way of s0 where
+  // they come from the tensor cores.  Ends with the operands still being read by other threads: the caller
+  // synchronises before they are overwritten.
+  auto logits = [&](float (&acc)[RT][4], float* s0, int n, auto code) {
+    auto row = [&](int c) { return c < n ? code(c) : (const T*)nullptr; };
+    if constexpr (kMma) {
+      load_rows<kThreads>(reinterpret_cast<T*>(cs), pitch, kCols, d, dpad, row);
+      __syncthreads();
+      mma_logits<RT>(s0, ldr, reinterpret_cast<const T*>(qs), reinterpret_cast<const T*>(cs), pitch, dpad, a.scale);
+      __syncthreads();
+      load_s(s0, acc);
+    } else {
+      load_transposed<kThreads>(cs, kLdC, kCols, d, row);
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+      mul_tile<RT>(acc, qs, ldr, cs, kLdC, d, ty, tx);
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] *= a.scale;
     }
   };
 
@@ -499,8 +581,9 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) atten
     for (int c0 = 0; c0 < M;) {
       const int n = width_at(c0);
       float acc[RT][4];
-      logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
-      if (a.keep) store_s(ss + (size_t)c0 * ldr, acc);
+      float* s0 = a.keep ? ss + (size_t)c0 * ldr : ss;
+      logits(acc, s0, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+      if (!kMma && a.keep) store_s(s0, acc);
       float cnt[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) cnt[j] = tx * 4 + j < n ? npS[c0 + tx * 4 + j] : 0.f;
@@ -540,7 +623,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) atten
       const int n = width_at(c0);
       float acc[RT][4];
       if (a.keep) load_s(ss + (size_t)c0 * ldr, acc);
-      else logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+      else logits(acc, ss, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
       if (ntiles && c0 / a.tile_m != t_inv) {
         // exact: the row's full denominator.  Tiled (appendix "Computing Importance with Tiled Codewords"):
         // the denominator seen up to this codeword's tile (Eq. "aproxdenom").
@@ -677,12 +760,12 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR) ? 2 : 1) atten
         else load_v(val_parent);
       }
       if (child) {
-        logits(acc, n, [&](int c) { const int e = c0 + c; return Cch + ((size_t)sel_list[e / C] * C + e % C) * d; });
+        logits(acc, sw, n, [&](int c) { const int e = c0 + c; return Cch + ((size_t)sel_list[e / C] * C + e % C) * d; });
       } else if (a.keep && need_w) {
         sw = ss + (size_t)c0 * ldr;                       // the tile's logits, overwritten by its weights
         load_s(sw, acc);
       } else {
-        logits(acc, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+        logits(acc, sw, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -814,8 +897,9 @@ avq_status launch_aggregate(const avq_problem& p, const void* V, const int32_t* 
 
 template <typename T, int RT, int DT, bool CORR>
 avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st) {
+  constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
   auto bytes = [&](int keep) {
-    return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.block_q, a.tile_m, keep).total;
+    return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.block_q, a.tile_m, keep, kMma).total;
   };
   // The block's logits stay in shared memory when one row tile holds the block and that leaves room for two
   // CTAs per SM (or all of an SM's memory is there for the taking because the grid has a CTA per SM at most).
@@ -827,7 +911,7 @@ avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st)
   a.keep = (a.block_q <= 32 * RT && (a.tile_m == 0 || a.tile_m % kCols == 0) && bytes(1) <= most) ? 1 : 0;
   const size_t smem = bytes(a.keep);
   if (smem > kSmemMax) return AVQ_ERR_UNSUPPORTED;
-  auto kern = attend_simt_kernel<T, RT, DT, CORR>;
+  auto kern = one_wave ? attend_simt_kernel<T, RT, DT, CORR, true> : attend_simt_kernel<T, RT, DT, CORR, false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return AVQ_ERR_CUDA;
   return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kAttThreads), smem, st, chained, a));
