@@ -53,17 +53,17 @@ constexpr int kLdC = kCols + 4;    // row pitch of a [k][column] operand, floats
 // Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r], k < d: the transposed
 // operand of the register-tiled products.  A warp takes 8 rows x 4 chunks of 4 elements: 64-byte pieces of a
 // row in global memory, at most two-way bank conflicts in shared memory.
-template <int THREADS, typename Src>
+template <int THREADS, int BATCH, typename Src>
 __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Src src) {
   constexpr int kWarps = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kc = lane & 3, rr = lane >> 2;
   const int chunks = d >> 2, cblocks = (chunks + 3) >> 2, units = (rows >> 3) * cblocks;
-  for (int u = warp; u < units; u += 2 * kWarps) {        // two loads in flight per trip
-    float4 v[2];
-    int at[2];
+  for (int u = warp; u < units; u += BATCH * kWarps) {    // BATCH loads in flight per trip
+    float4 v[BATCH];
+    int at[BATCH];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < BATCH; ++e) {
       const int ue = u + e * kWarps, rb = ue / cblocks, cb = ue - rb * cblocks;
       const int r = rb * 8 + rr, c = cb * 4 + kc;
       at[e] = -1;
@@ -75,7 +75,7 @@ __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, in
       }
     }
 #pragma unroll
-    for (int e = 0; e < 2; ++e)
+    for (int e = 0; e < BATCH; ++e)
       if (at[e] >= 0) {
         float* o = dst + at[e];
         o[0] = v[e].x; o[ld] = v[e].y; o[2 * ld] = v[e].z; o[3 * ld] = v[e].w;
@@ -120,11 +120,75 @@ __device__ double exact_dist(const T* krow, const T* c, int d) {
   return s;
 }
 
+// `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
+template <int THREADS, typename Src>
+__device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
+  const int per = dpad >> 2, units = rows * per;
+  for (int u = threadIdx.x; u < units; u += 2 * THREADS) {
+    uint2 v[2];
+    int at[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int ue = u + e * THREADS, r = ue / per, c = ue - r * per;
+      at[e] = ue < units ? r * pitch + 4 * c : -1;
+      v[e] = make_uint2(0u, 0u);
+      if (ue < units && 4 * c < d) {
+        const __nv_bfloat16* p = src(r);
+        if (p) v[e] = __ldg(reinterpret_cast<const uint2*>(p + 4 * c));
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (at[e] >= 0) *reinterpret_cast<uint2*>(dst + at[e]) = v[e];
+  }
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+// One warp: s[column][row] = scale * q . c^T for rows r0 .. +15 and columns n0 .. +8 NT - 1
+template <int NT>
+__device__ __forceinline__ void mma_block(float* s, int ldr, const __nv_bfloat16* q, const __nv_bfloat16* c, int pitch,
+                                          int dpad, float scale, int r0, int n0) {
+  const int lane = threadIdx.x & 31;
+  const __nv_bfloat16* ap = q + (r0 + (lane & 15)) * pitch + (lane >> 4) * 8;
+  const __nv_bfloat16* bp = c + (n0 + (lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 8;
+  float acc[NT][4] = {};
+#pragma unroll 4
+  for (int k = 0; k < dpad; k += 16) {
+    uint32_t a[4];
+    ldmatrix4(a, ap + k);
+#pragma unroll
+    for (int j = 0; j < NT; j += 2) {
+      uint32_t b[4];
+      ldmatrix4(b, bp + j * 8 * pitch + k);
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                     : "+f"(acc[j + e][0]), "+f"(acc[j + e][1]), "+f"(acc[j + e][2]), "+f"(acc[j + e][3])
+                     : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[2 * e]), "r"(b[2 * e + 1]));
+    }
+  }
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      s[(size_t)(n0 + 8 * j + 2 * t + (e & 1)) * ldr + r0 + g + 8 * (e >> 1)] = acc[j][e] * scale;
+}
+
 // ------------------------------------------------------------------------------- assign
 constexpr int kAssignKeys = 64;    // keys per CTA
 
-// Parents: 64 keys x 64 codewords at a time, squared differences in the direct form.  Children: four lanes per
-// key.  zero_base / zero_units: 16-byte words this grid clears on the side (the accumulators of the
+// Shared memory: float32, keys and codewords as [k][row]; bfloat16, both as rows, the products [column][key], norms.
+__host__ __device__ inline size_t assign_smem_floats(int d, bool mma) {
+  if (!mma) return 2 * (size_t)d * kLdC;
+  return 2 * (size_t)kAssignKeys * ((size_t)(d + 15) / 16 * 8 + 4) + (size_t)kCols * kLdC + kAssignKeys + kCols;
+}
+
+// Parents: 64 keys x 64 codewords at a time.  float32: squared differences in the direct form.  bfloat16: norms and
+// tensor-core products (M512 d64, 16384 keys: 74 us with float32 multiply-adds).  Children: four lanes per key,
+// direct form.  zero_base / zero_units: 16-byte words this grid clears on the side (the accumulators of the
 // aggregation behind it), each CTA an equal slice.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
@@ -132,8 +196,13 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
                    int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int d, int M,
                    int C, int parent_stays, uint4* __restrict__ zero_base, uint32_t zero_units) {
   extern __shared__ __align__(16) float smem[];
-  float* ks = smem;                            // [d][kLdC] keys
-  float* cs = ks + (size_t)d * kLdC;           // [d][kLdC] codewords of the current tile
+  constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
+  const int dpad = (d + 15) & ~15, pitch = dpad + 8;
+  float* ks = smem;                                               // [d][kLdC] keys, or rows of pitch bfloat16
+  float* cs = ks + (kMma ? (size_t)kAssignKeys * pitch / 2 : (size_t)d * kLdC);   // codewords of the current tile, alike
+  float* prod = cs + (size_t)kCols * pitch / 2;                   // bfloat16: [kCols][kLdC] products
+  float* kn = prod + (size_t)kCols * kLdC;                        // [kAssignKeys] key norms
+  float* cn = kn + kAssignKeys;                                   // [kCols] codeword norms
   __shared__ int s_par[kAssignKeys];
   __shared__ float s_d1[kAssignKeys];
   __shared__ int s_redo[kAssignKeys];          // 1: parent decided in float64 (its exact distance in s_dp)
@@ -151,7 +220,22 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const T* Kb = K + ((size_t)bh * Nk + j0) * d;
   const int rows = min(kAssignKeys, Nk - j0);
   const T* Cph = Cp + (size_t)h * M * d;
-  load_transposed<kThreads>(ks, kLdC, kAssignKeys, d, [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; });
+  auto key_row = [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; };
+  if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(ks), pitch, kAssignKeys, d, dpad, key_row);
+  else load_transposed<kThreads, 4>(ks, kLdC, kAssignKeys, d, key_row);
+  // squared norm of a staged row, four lanes per row (row tid / 4)
+  auto row_norm = [&](const float* base) {
+    const T* rowp = reinterpret_cast<const T*>(base) + (tid >> 2) * pitch;
+    float s = 0.f;
+    for (int k = 4 * (tid & 3); k < dpad; k += 16) {
+      const uint2 u = *reinterpret_cast<const uint2*>(rowp + k);
+      const float a = __uint_as_float(u.x << 16), b = __uint_as_float(u.x & 0xFFFF0000u);
+      const float c = __uint_as_float(u.y << 16), e = __uint_as_float(u.y & 0xFFFF0000u);
+      s = fmaf(a, a, s); s = fmaf(b, b, s); s = fmaf(c, c, s); s = fmaf(e, e, s);
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    return s + __shfl_xor_sync(0xffffffffu, s, 2);
+  };
 
   float d1[4], d2[4];
   int i1[4];
@@ -159,22 +243,48 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   for (int i = 0; i < 4; ++i) { d1[i] = INFINITY; d2[i] = INFINITY; i1[i] = 0; }
   for (int m0 = 0; m0 < M; m0 += kCols) {
     const int w = min(kCols, M - m0);
-    __syncthreads();
-    load_transposed<kThreads>(cs, kLdC, kCols, d, [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; });
+    if (m0 > 0) __syncthreads();
+    auto code_row = [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; };
+    if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(cs), pitch, kCols, d, dpad, code_row);
+    else load_transposed<kThreads, 4>(cs, kLdC, kCols, d, code_row);
     __syncthreads();
     float acc[4][4] = {};
+    if constexpr (kMma) {
+      if (m0 == 0) {
+        const float s = row_norm(ks);
+        if ((tid & 3) == 0) kn[tid >> 2] = s;
+      }
+      {
+        const float s = row_norm(cs);
+        if ((tid & 3) == 0) cn[tid >> 2] = s;
+      }
+      const int warp = tid >> 5;
+      mma_block<4>(prod, kLdC, reinterpret_cast<const T*>(ks), reinterpret_cast<const T*>(cs), pitch, dpad, -2.f,
+                   (warp & 3) * 16, (warp >> 2) * 32);
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 x = *reinterpret_cast<const float4*>(prod + (tx * 4 + j) * kLdC + ty * 4);
+        const float c = cn[tx * 4 + j];
+        acc[0][j] = kn[ty * 4] + c + x.x;
+        acc[1][j] = kn[ty * 4 + 1] + c + x.y;
+        acc[2][j] = kn[ty * 4 + 2] + c + x.z;
+        acc[3][j] = kn[ty * 4 + 3] + c + x.w;
+      }
+    } else {
 #pragma unroll 4
-    for (int k = 0; k < d; ++k) {
-      const float4 a4 = *reinterpret_cast<const float4*>(ks + k * kLdC + ty * 4);
-      const float4 b4 = *reinterpret_cast<const float4*>(cs + k * kLdC + tx * 4);
-      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+      for (int k = 0; k < d; ++k) {
+        const float4 a4 = *reinterpret_cast<const float4*>(ks + k * kLdC + ty * 4);
+        const float4 b4 = *reinterpret_cast<const float4*>(cs + k * kLdC + tx * 4);
+        const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float df = a[i] - b[j];
-          acc[i][j] = fmaf(df, df, acc[i][j]);
-        }
+          for (int j = 0; j < 4; ++j) {
+            const float df = a[i] - b[j];
+            acc[i][j] = fmaf(df, df, acc[i][j]);
+          }
+      }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -198,7 +308,10 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
       if (b1 < d1[i] || (b1 == d1[i] && bi < i1[i])) { d1[i] = b1; i1[i] = bi; }
     }
     const int key = ty * 4 + i;
-    const bool redo = M > 1 && key < rows && !(d2[i] - d1[i] > kNearTie * d2[i]);
+    // direct form: relative.  Norms and products: each carries a rounding error of a small multiple of 2^-24 of the
+    // norms, which this bounds with a wide margin.
+    const float close = kMma ? 1e-4f * (kn[key] + d2[i]) : kNearTie * d2[i];
+    const bool redo = M > 1 && key < rows && !(d2[i] - d1[i] > close);
     double best = INFINITY;
     if (__any_sync(0xffffffffu, redo)) {
       int bi = 0x7fffffff;
@@ -228,20 +341,54 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const int key = tid >> 2, s4 = tid & 3;
   const int par = s_par[key];
   const T* Cch = Cc + ((size_t)h * M + par) * C * d;
+  // distance to one codeword row, this lane's chunks; four loads in flight
+  auto dist_part = [&](const T* c) {
+    float s = 0.f;
+    for (int c0 = s4; c0 < (d >> 2); c0 += 16) {
+      float4 v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (c0 + 4 * e < (d >> 2)) v[e] = ld4(c + 4 * (c0 + 4 * e));
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (c0 + 4 * e < (d >> 2)) {
+          const int k = 4 * (c0 + 4 * e);
+          float4 x;
+          if constexpr (kMma) {
+            const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const T*>(ks) + key * pitch + k);
+            x = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                            __uint_as_float(u.y & 0xFFFF0000u));
+          } else {
+            const float* kp = ks + (size_t)k * kLdC + key;
+            x = make_float4(kp[0], kp[kLdC], kp[2 * kLdC], kp[3 * kLdC]);
+          }
+          x.x -= v[e].x; x.y -= v[e].y; x.z -= v[e].z; x.w -= v[e].w;
+          s = fmaf(x.x, x.x, s); s = fmaf(x.y, x.y, s); s = fmaf(x.z, x.z, s); s = fmaf(x.w, x.w, s);
+        }
+    }
+    return s;
+  };
   float e1 = INFINITY, e2 = INFINITY;
   int c1 = 0;
-  for (int c = 0; c < C; ++c) {
-    float s = 0.f;
-    for (int ch = s4; ch < (d >> 2); ch += 4) {
-      const float4 v = ld4(Cch + (size_t)c * d + 4 * ch);
-      const float* kp = ks + (size_t)(4 * ch) * kLdC + key;
-      const float x0 = kp[0] - v.x, x1 = kp[kLdC] - v.y, x2 = kp[2 * kLdC] - v.z, x3 = kp[3 * kLdC] - v.w;
-      s = fmaf(x0, x0, s); s = fmaf(x1, x1, s); s = fmaf(x2, x2, s); s = fmaf(x3, x3, s);
+  for (int c = 0; c < C; c += 2) {                        // two children at a time
+    float sa = dist_part(Cch + (size_t)c * d);
+    float sb = c + 1 < C ? dist_part(Cch + (size_t)(c + 1) * d) : INFINITY;
+    sa += __shfl_xor_sync(0xffffffffu, sa, 1);
+    sb += __shfl_xor_sync(0xffffffffu, sb, 1);
+    sa += __shfl_xor_sync(0xffffffffu, sa, 2);
+    sb += __shfl_xor_sync(0xffffffffu, sb, 2);
+    if (sa < e1) { e2 = e1; e1 = sa; c1 = c; }
+    else if (sa < e2) { e2 = sa; }
+    if (c + 1 < C) {
+      if (sb < e1) { e2 = e1; e1 = sb; c1 = c + 1; }
+      else if (sb < e2) { e2 = sb; }
     }
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (s < e1) { e2 = e1; e1 = s; c1 = c; }
-    else if (s < e2) { e2 = s; }
+  }
+  float dpar = 0.f;                                       // the parent's distance in the same form
+  if (kMma && parent_stays) {
+    dpar = dist_part(Cph + (size_t)par * d);
+    dpar += __shfl_xor_sync(0xffffffffu, dpar, 1);
+    dpar += __shfl_xor_sync(0xffffffffu, dpar, 2);
   }
   double dc64 = -1.0;
   const bool redo = C > 1 && key < rows && !(e2 - e1 > kNearTie * e2);
@@ -263,7 +410,7 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   }
   if (s4 == 0 && key < rows) {
     if (parent_stays) {
-      const float d1k = s_d1[key];
+      const float d1k = kMma && !s_redo[key] ? dpar : s_d1[key];
       bool moved = e1 < d1k;
       if (!(fabsf(e1 - d1k) > kNearTie * fmaxf(e1, d1k))) {
         const double dp64 = s_redo[key] ? s_dp[key] : exact_dist(Kb + (size_t)key * d, Cph + (size_t)par * d, d);
@@ -325,65 +472,6 @@ aggregate_simt_kernel(const T* __restrict__ V, const int32_t* pidx, const int32_
 }
 
 // ------------------------------------------------------------------------------- attend
-// `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
-template <int THREADS, typename Src>
-__device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
-  const int per = dpad >> 2, units = rows * per;
-  for (int u = threadIdx.x; u < units; u += 2 * THREADS) {
-    uint2 v[2];
-    int at[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int ue = u + e * THREADS, r = ue / per, c = ue - r * per;
-      at[e] = ue < units ? r * pitch + 4 * c : -1;
-      v[e] = make_uint2(0u, 0u);
-      if (ue < units && 4 * c < d) {
-        const __nv_bfloat16* p = src(r);
-        if (p) v[e] = __ldg(reinterpret_cast<const uint2*>(p + 4 * c));
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-      if (at[e] >= 0) *reinterpret_cast<uint2*>(dst + at[e]) = v[e];
-  }
-}
-__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
-}
-// s[column][row] = scale * Q . codes^T for 32 RT rows x 64 columns, 16 warps: 16 rows x 8 RT columns per warp
-template <int RT>
-__device__ __forceinline__ void mma_logits(float* s, int ldr, const __nv_bfloat16* q, const __nv_bfloat16* c, int pitch,
-                                           int dpad, float scale) {
-  constexpr int NT = RT;                                  // 8-column tiles per warp
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r0 = (warp % (2 * RT)) * 16, n0 = (warp / (2 * RT)) * 8 * NT;
-  const __nv_bfloat16* ap = q + (r0 + (lane & 15)) * pitch + (lane >> 4) * 8;
-  const __nv_bfloat16* bp = c + (n0 + (lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 8;
-  float acc[NT][4] = {};
-#pragma unroll 4
-  for (int k = 0; k < dpad; k += 16) {
-    uint32_t a[4];
-    ldmatrix4(a, ap + k);
-#pragma unroll
-    for (int j = 0; j < NT; j += 2) {
-      uint32_t b[4];
-      ldmatrix4(b, bp + j * 8 * pitch + k);
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                     : "+f"(acc[j + e][0]), "+f"(acc[j + e][1]), "+f"(acc[j + e][2]), "+f"(acc[j + e][3])
-                     : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[2 * e]), "r"(b[2 * e + 1]));
-    }
-  }
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int j = 0; j < NT; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      s[(size_t)(n0 + 8 * j + 2 * t + (e & 1)) * ldr + r0 + g + 8 * (e >> 1)] = acc[j][e] * scale;
-}
-
 struct AttendArgs {
   const void *Q, *Cp, *Cc;
   const float *Vp, *np_, *Vc, *nc;
@@ -495,7 +583,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   auto load_q = [&](int rt) {
     auto row = [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; };
     if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(qs), pitch, R, d, dpad, row);
-    else load_transposed<kThreads>(qs, ldr, R, d, row);
+    else load_transposed<kThreads, WIDE ? 4 : 2>(qs, ldr, R, d, row);
   };
   auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
 #pragma unroll
@@ -527,11 +615,13 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
     if constexpr (kMma) {
       load_rows<kThreads>(reinterpret_cast<T*>(cs), pitch, kCols, d, dpad, row);
       __syncthreads();
-      mma_logits<RT>(s0, ldr, reinterpret_cast<const T*>(qs), reinterpret_cast<const T*>(cs), pitch, dpad, a.scale);
+      // 32 RT rows x 64 columns over 16 warps: 16 rows x 8 RT columns each
+      mma_block<RT>(s0, ldr, reinterpret_cast<const T*>(qs), reinterpret_cast<const T*>(cs), pitch, dpad, a.scale,
+                    (warp % (2 * RT)) * 16, (warp / (2 * RT)) * 8 * RT);
       __syncthreads();
       load_s(s0, acc);
     } else {
-      load_transposed<kThreads>(cs, kLdC, kCols, d, row);
+      load_transposed<kThreads, 2>(cs, kLdC, kCols, d, row);
       __syncthreads();
 #pragma unroll
       for (int i = 0; i < RT; ++i)
@@ -549,10 +639,12 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   tc::pdl_wait();
   for (int j = tid; j < M; j += kThreads) {
     const float n = ld_after_wait(np_ + j);
-    float s = 0.f;
-    for (int c = 0; c < C; ++c) s += ld_after_wait(nc + (size_t)j * C + c);
     npS[j] = n;
-    nstay[j] = n - s;
+    if (a.stays) {                                        // keys that stay with their parent
+      float s = 0.f;
+      for (int c = 0; c < C; ++c) s += ld_after_wait(nc + (size_t)j * C + c);
+      nstay[j] = n - s;
+    }
     w[j] = 0.0;
     sel[j] = 0;
   }
@@ -872,7 +964,7 @@ constexpr size_t kSmemHalf = 113 * 1024;                  // two CTAs on an SM
 template <typename T>
 avq_status launch_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
                          int32_t* pidx, int32_t* cidx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
-  const size_t smem = sizeof(float) * 2 * (size_t)p.d * kLdC;
+  const size_t smem = sizeof(float) * assign_smem_floats(p.d, std::is_same<T, __nv_bfloat16>::value);
   auto kern = assign_simt_kernel<T>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return AVQ_ERR_CUDA;
