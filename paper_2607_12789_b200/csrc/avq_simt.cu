@@ -50,10 +50,14 @@ constexpr int kThreads = 256;      // of the assign and aggregate kernels: 16 x 
 constexpr int kCols = 64;          // columns (codewords) of a tile
 constexpr int kLdC = kCols + 4;    // row pitch of a [k][column] operand, floats
 
-// Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r], k < d: the transposed
+// The columns of a tile of n <= 64 codewords: thread tx owns tx, tx + 16, tx + 32, tx + 48, which stand side by side in
+// the shared-memory operand, so that a narrow tile costs only the columns it has.
+__device__ __forceinline__ int code_pos(int c) { return ((c & 15) << 2) | (c >> 4); }
+
+// Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r] (CODES: dst[k][code_pos(r)]), k < d: the transposed
 // operand of the register-tiled products.  A warp takes 8 rows x 4 chunks of 4 elements: 64-byte pieces of a
 // row in global memory, at most two-way bank conflicts in shared memory.
-template <int THREADS, int BATCH, typename Src>
+template <int THREADS, int BATCH, bool CODES, typename Src>
 __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Src src) {
   constexpr int kWarps = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -69,7 +73,7 @@ __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, in
       at[e] = -1;
       v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (ue < units && c < chunks) {
-        at[e] = 4 * c * ld + r;
+        at[e] = 4 * c * ld + (CODES ? code_pos(r) : r);
         const auto* p = src(r);
         if (p) v[e] = ld4(p + 4 * c);
       }
@@ -83,28 +87,35 @@ __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, in
   }
 }
 
-// acc[i][j] += sum_k A[k][row(i)] * B[k][tx*4 + j], k ascending (one accumulator per result: the sums do not
-// depend on the tiling)
-template <int RT>
+// acc[i][j] += sum_k A[k][ty*RT + i] * B[k][tx*4 + j], j < NJ, k ascending (one accumulator per result: the sums do
+// not depend on the tiling)
+template <int RT, int NJ>
 __device__ __forceinline__ void mul_tile(float (&acc)[RT][4], const float* A, int lda, const float* B, int ldb, int K,
                                          int ty, int tx) {
   const float* a_ = A + ty * RT;
   const float* b_ = B + tx * 4;
 #pragma unroll 4
   for (int k = 0; k < K; ++k) {
-    float a[RT];
+    float a[RT], b[4];
     if constexpr (RT == 4) *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(a_ + k * lda);
     else *reinterpret_cast<float2*>(a) = *reinterpret_cast<const float2*>(a_ + k * lda);
-    const float4 b = *reinterpret_cast<const float4*>(b_ + k * ldb);
+    if constexpr (NJ == 4) *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(b_ + k * ldb);
+    else if constexpr (NJ == 2) *reinterpret_cast<float2*>(b) = *reinterpret_cast<const float2*>(b_ + k * ldb);
+    else b[0] = b_[k * ldb];
 #pragma unroll
-    for (int i = 0; i < RT; ++i) {
-      acc[i][0] = fmaf(a[i], b.x, acc[i][0]);
-      acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
-      acc[i][2] = fmaf(a[i], b.z, acc[i][2]);
-      acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
-    }
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
   }
 }
+template <int RT>
+__device__ __forceinline__ void mul_codes(float (&acc)[RT][4], const float* A, int lda, const float* B, int ldb, int K,
+                                          int ty, int tx, int n) {
+  if (n <= 16) mul_tile<RT, 1>(acc, A, lda, B, ldb, K, ty, tx);
+  else if (n <= 32) mul_tile<RT, 2>(acc, A, lda, B, ldb, K, ty, tx);
+  else mul_tile<RT, 4>(acc, A, lda, B, ldb, K, ty, tx);
+}
+__device__ __forceinline__ int code_rows(int n) { return n <= 16 ? 16 : (n <= 32 ? 32 : 64); }
 
 // Two distances closer than this (relative) are re-evaluated in float64.  The float32 direct
 // form carries about d * 2^-24 relative error, far below it.
@@ -180,18 +191,18 @@ __device__ __forceinline__ void mma_block(float* s, int ldr, const __nv_bfloat16
 // ------------------------------------------------------------------------------- assign
 constexpr int kAssignKeys = 64;    // keys per CTA
 
-// Shared memory: float32, keys and codewords as [k][row]; bfloat16, both as rows, the products [column][key], norms.
+// Shared memory: float32, keys and codewords as [k][row]; bfloat16, both as rows, and the products [column][key]; norms.
 __host__ __device__ inline size_t assign_smem_floats(int d, bool mma) {
-  if (!mma) return 2 * (size_t)d * kLdC;
+  if (!mma) return 2 * (size_t)d * kLdC + kAssignKeys + kCols;
   return 2 * (size_t)kAssignKeys * ((size_t)(d + 15) / 16 * 8 + 4) + (size_t)kCols * kLdC + kAssignKeys + kCols;
 }
 
-// Parents: 64 keys x 64 codewords at a time.  float32: squared differences in the direct form.  bfloat16: norms and
-// tensor-core products (M512 d64, 16384 keys: 74 us with float32 multiply-adds).  Children: four lanes per key,
+// Parents: 64 keys x 64 codewords at a time, ||k||^2 + ||c||^2 - 2 k.c with float64 rechecks; bfloat16 products on the
+// tensor cores (M512 d64, 16384 keys: 74 us with float32 multiply-adds).  Children: four lanes per key,
 // direct form.  zero_base / zero_units: 16-byte words this grid clears on the side (the accumulators of the
 // aggregation behind it), each CTA an equal slice.
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* __restrict__ Cc,
                    int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int d, int M,
                    int C, int parent_stays, uint4* __restrict__ zero_base, uint32_t zero_units) {
@@ -201,10 +212,9 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   float* ks = smem;                                               // [d][kLdC] keys, or rows of pitch bfloat16
   float* cs = ks + (kMma ? (size_t)kAssignKeys * pitch / 2 : (size_t)d * kLdC);   // codewords of the current tile, alike
   float* prod = cs + (size_t)kCols * pitch / 2;                   // bfloat16: [kCols][kLdC] products
-  float* kn = prod + (size_t)kCols * kLdC;                        // [kAssignKeys] key norms
-  float* cn = kn + kAssignKeys;                                   // [kCols] codeword norms
+  float* kn = kMma ? prod + (size_t)kCols * kLdC : cs + (size_t)d * kLdC;   // [kAssignKeys] key norms
+  float* cn = kn + kAssignKeys;                                   // [kCols] codeword norms (float32: by code_pos)
   __shared__ int s_par[kAssignKeys];
-  __shared__ float s_d1[kAssignKeys];
   __shared__ int s_redo[kAssignKeys];          // 1: parent decided in float64 (its exact distance in s_dp)
   __shared__ double s_dp[kAssignKeys];
   tc::pdl_launch_dependents();
@@ -222,16 +232,24 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const T* Cph = Cp + (size_t)h * M * d;
   auto key_row = [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; };
   if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(ks), pitch, kAssignKeys, d, dpad, key_row);
-  else load_transposed<kThreads, 4>(ks, kLdC, kAssignKeys, d, key_row);
-  // squared norm of a staged row, four lanes per row (row tid / 4)
+  else load_transposed<kThreads, 4, false>(ks, kLdC, kAssignKeys, d, key_row);
+  // squared norm of a staged row (float32: column), four lanes per row (row tid / 4)
   auto row_norm = [&](const float* base) {
-    const T* rowp = reinterpret_cast<const T*>(base) + (tid >> 2) * pitch;
     float s = 0.f;
-    for (int k = 4 * (tid & 3); k < dpad; k += 16) {
-      const uint2 u = *reinterpret_cast<const uint2*>(rowp + k);
-      const float a = __uint_as_float(u.x << 16), b = __uint_as_float(u.x & 0xFFFF0000u);
-      const float c = __uint_as_float(u.y << 16), e = __uint_as_float(u.y & 0xFFFF0000u);
-      s = fmaf(a, a, s); s = fmaf(b, b, s); s = fmaf(c, c, s); s = fmaf(e, e, s);
+    if constexpr (kMma) {
+      const T* rowp = reinterpret_cast<const T*>(base) + (tid >> 2) * pitch;
+      for (int k = 4 * (tid & 3); k < dpad; k += 16) {
+        const uint2 u = *reinterpret_cast<const uint2*>(rowp + k);
+        const float a = __uint_as_float(u.x << 16), b = __uint_as_float(u.x & 0xFFFF0000u);
+        const float c = __uint_as_float(u.y << 16), e = __uint_as_float(u.y & 0xFFFF0000u);
+        s = fmaf(a, a, s); s = fmaf(b, b, s); s = fmaf(c, c, s); s = fmaf(e, e, s);
+      }
+    } else {
+#pragma unroll 4
+      for (int k = tid & 3; k < d; k += 4) {
+        const float x = base[(size_t)k * kLdC + (tid >> 2)];
+        s = fmaf(x, x, s);
+      }
     }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     return s + __shfl_xor_sync(0xffffffffu, s, 2);
@@ -246,53 +264,48 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
     if (m0 > 0) __syncthreads();
     auto code_row = [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; };
     if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(cs), pitch, kCols, d, dpad, code_row);
-    else load_transposed<kThreads, 4>(cs, kLdC, kCols, d, code_row);
+    else load_transposed<kThreads, 4, true>(cs, kLdC, code_rows(w), d, code_row);
     __syncthreads();
     float acc[4][4] = {};
+    if (m0 == 0) {
+      const float s = row_norm(ks);
+      if ((tid & 3) == 0) kn[tid >> 2] = s;
+    }
+    {
+      const float s = row_norm(cs);
+      if ((tid & 3) == 0) cn[tid >> 2] = s;
+    }
     if constexpr (kMma) {
-      if (m0 == 0) {
-        const float s = row_norm(ks);
-        if ((tid & 3) == 0) kn[tid >> 2] = s;
-      }
-      {
-        const float s = row_norm(cs);
-        if ((tid & 3) == 0) cn[tid >> 2] = s;
-      }
       const int warp = tid >> 5;
-      mma_block<4>(prod, kLdC, reinterpret_cast<const T*>(ks), reinterpret_cast<const T*>(cs), pitch, dpad, -2.f,
+      mma_block<4>(prod, kLdC, reinterpret_cast<const T*>(ks), reinterpret_cast<const T*>(cs), pitch, dpad, 1.f,
                    (warp & 3) * 16, (warp >> 2) * 32);
       __syncthreads();
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float4 x = *reinterpret_cast<const float4*>(prod + (tx * 4 + j) * kLdC + ty * 4);
-        const float c = cn[tx * 4 + j];
-        acc[0][j] = kn[ty * 4] + c + x.x;
-        acc[1][j] = kn[ty * 4 + 1] + c + x.y;
-        acc[2][j] = kn[ty * 4 + 2] + c + x.z;
-        acc[3][j] = kn[ty * 4 + 3] + c + x.w;
+        const float4 x = *reinterpret_cast<const float4*>(prod + (tx + 16 * j) * kLdC + ty * 4);
+        acc[0][j] = x.x; acc[1][j] = x.y; acc[2][j] = x.z; acc[3][j] = x.w;
       }
     } else {
-#pragma unroll 4
-      for (int k = 0; k < d; ++k) {
-        const float4 a4 = *reinterpret_cast<const float4*>(ks + k * kLdC + ty * 4);
-        const float4 b4 = *reinterpret_cast<const float4*>(cs + k * kLdC + tx * 4);
-        const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+      mul_codes<4>(acc, ks, kLdC, cs, kLdC, d, ty, tx, w);
+      __syncthreads();
+    }
+    {
+      const float4 k4 = *reinterpret_cast<const float4*>(kn + ty * 4);
+      const float kv[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+      for (int j = 0; j < 4; ++j) {
+        const float c = cn[kMma ? tx + 16 * j : tx * 4 + j];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float df = a[i] - b[j];
-            acc[i][j] = fmaf(df, df, acc[i][j]);
-          }
+        for (int i = 0; i < 4; ++i) acc[i][j] = fmaf(-2.f, acc[i][j], kv[i] + c);
       }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (tx * 4 + j < w) {
+      if (tx + 16 * j < w) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float s = acc[i][j];
-          if (s < d1[i]) { d2[i] = d1[i]; d1[i] = s; i1[i] = m0 + tx * 4 + j; }
+          if (s < d1[i]) { d2[i] = d1[i]; d1[i] = s; i1[i] = m0 + tx + 16 * j; }
           else if (s < d2[i]) { d2[i] = s; }
         }
       }
@@ -308,9 +321,9 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
       if (b1 < d1[i] || (b1 == d1[i] && bi < i1[i])) { d1[i] = b1; i1[i] = bi; }
     }
     const int key = ty * 4 + i;
-    // direct form: relative.  Norms and products: each carries a rounding error of a small multiple of 2^-24 of the
-    // norms, which this bounds with a wide margin.
-    const float close = kMma ? 1e-4f * (kn[key] + d2[i]) : kNearTie * d2[i];
+    // norms and products: each carries a rounding error of a small multiple of 2^-24 of the norms, which this bounds
+    // with a wide margin
+    const float close = 1e-4f * (kn[key] + d2[i]);
     const bool redo = M > 1 && key < rows && !(d2[i] - d1[i] > close);
     double best = INFINITY;
     if (__any_sync(0xffffffffu, redo)) {
@@ -330,7 +343,6 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
     }
     if (tx == 0) {
       s_par[key] = i1[i];
-      s_d1[key] = d1[i];
       s_redo[key] = redo ? 1 : 0;
       s_dp[key] = best;
     }
@@ -385,7 +397,7 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
     }
   }
   float dpar = 0.f;                                       // the parent's distance in the same form
-  if (kMma && parent_stays) {
+  if (parent_stays) {
     dpar = dist_part(Cph + (size_t)par * d);
     dpar += __shfl_xor_sync(0xffffffffu, dpar, 1);
     dpar += __shfl_xor_sync(0xffffffffu, dpar, 2);
@@ -410,7 +422,7 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   }
   if (s4 == 0 && key < rows) {
     if (parent_stays) {
-      const float d1k = kMma && !s_redo[key] ? dpar : s_d1[key];
+      const float d1k = dpar;
       bool moved = e1 < d1k;
       if (!(fabsf(e1 - d1k) > kNearTie * fmaxf(e1, d1k))) {
         const double dp64 = s_redo[key] ? s_dp[key] : exact_dist(Kb + (size_t)key * d, Cph + (size_t)par * d, d);
@@ -563,6 +575,8 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   float *npS = sm + L.np, *nstay = sm + L.nstay, *zt = sm + L.zt, *nseen = sm + L.nseen;
   int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
   constexpr int ldv = DT * 64;
+  int* cand = reinterpret_cast<int*>(wpart);              // [M] candidates of the selection (the sums are done by then)
+  __shared__ int s_count[32], s_ncand;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = tid & 15, ty = tid >> 4;
   const int blk = blockIdx.x, bh = blockIdx.y, h = bh % a.H;
@@ -583,12 +597,12 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   auto load_q = [&](int rt) {
     auto row = [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; };
     if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(qs), pitch, R, d, dpad, row);
-    else load_transposed<kThreads, WIDE ? 4 : 2>(qs, ldr, R, d, row);
+    else load_transposed<kThreads, WIDE ? 4 : 2, false>(qs, ldr, R, d, row);
   };
   auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * RT;
+      float* o = s0 + (size_t)(tx + 16 * j) * ldr + ty * RT;
       if constexpr (RT == 4) *reinterpret_cast<float4*>(o) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
       else *reinterpret_cast<float2*>(o) = make_float2(acc[0][j], acc[1][j]);
     }
@@ -596,7 +610,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   auto load_s = [&](const float* s0, float (&acc)[RT][4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float* o = s0 + (size_t)(tx * 4 + j) * ldr + ty * RT;
+      const float* o = s0 + (size_t)(tx + 16 * j) * ldr + ty * RT;
       if constexpr (RT == 4) {
         const float4 x = *reinterpret_cast<const float4*>(o);
         acc[0][j] = x.x; acc[1][j] = x.y; acc[2][j] = x.z; acc[3][j] = x.w;
@@ -621,13 +635,13 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       __syncthreads();
       load_s(s0, acc);
     } else {
-      load_transposed<kThreads, 2>(cs, kLdC, kCols, d, row);
+      load_transposed<kThreads, 2, true>(cs, kLdC, code_rows(n), d, row);
       __syncthreads();
 #pragma unroll
       for (int i = 0; i < RT; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-      mul_tile<RT>(acc, qs, ldr, cs, kLdC, d, ty, tx);
+      mul_codes<RT>(acc, qs, ldr, cs, kLdC, d, ty, tx, n);
 #pragma unroll
       for (int i = 0; i < RT; ++i)
 #pragma unroll
@@ -678,7 +692,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       if (!kMma && a.keep) store_s(s0, acc);
       float cnt[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cnt[j] = tx * 4 + j < n ? npS[c0 + tx * 4 + j] : 0.f;
+      for (int j = 0; j < 4; ++j) cnt[j] = tx + 16 * j < n ? npS[c0 + tx + 16 * j] : 0.f;
       const int t = ntiles ? c0 / a.tile_m : 0;
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
@@ -727,13 +741,13 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         double s = 0.0;
-        if (tx * 4 + j < n && npS[c0 + tx * 4 + j] > 0.f) {
+        if (tx + 16 * j < n && npS[c0 + tx + 16 * j] > 0.f) {
 #pragma unroll
           for (int i = 0; i < RT; ++i)
             if (rt * R + row_of(i) < rows) s = fma((double)expf(acc[i][j] - m[i]), inv[i], s);
         }
         s += __shfl_xor_sync(0xffffffffu, s, 16);
-        if (lane < 16) wpart[warp * kCols + tx * 4 + j] = s;
+        if (lane < 16) wpart[warp * kCols + tx + 16 * j] = s;
       }
       __syncthreads();
       if (tid < n) {
@@ -760,23 +774,56 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   }
   __syncthreads();
 
-  // ---- top-P by rank (ties -> lower index), then an ascending list.  Non-negative doubles order like their
-  // bit patterns.
+  // ---- top-P (ties -> lower index), then an ascending list.  Non-negative doubles order like their bit patterns.
   if (P > 0) {
+    // Only candidates are ranked, those at or above a bound that at least P keys reach: the largest of 32 sample keys
+    // that has P keys at or above it.  (Ranking all of them took 16 of 230 us at M = 512.)
     const unsigned long long* key = reinterpret_cast<const unsigned long long*>(w);
-    int lt = 0;                                           // 2^lt threads share a key's scan
-    while (lt < 4 && (M << (lt + 1)) <= kThreads) ++lt;
-    const int part = tid & ((1 << lt) - 1);
-    for (int j0 = 0; j0 < M; j0 += kThreads >> lt) {      // uniform
-      const int j = j0 + (tid >> lt);
-      int rank = 0;
-      if (P < M && j < M) {
-        const unsigned long long kj = key[j];
-#pragma unroll 8
-        for (int k = part; k < M; k += 1 << lt) rank += (key[k] > kj) | ((key[k] == kj) & (k < j));
+    if (P >= M) {
+      for (int j = tid; j < M; j += kThreads) sel[j] = 1;
+    } else {
+      unsigned long long bound = 0;
+      {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const unsigned long long smp = key[(2 * warp + e) * M / 32];
+          int c = 0;
+          for (int j = lane; j < M; j += 32) c += key[j] >= smp;
+          c = __reduce_add_sync(0xffffffffu, c);
+          if (lane == 0) s_count[2 * warp + e] = c;
+        }
+        if (tid == 0) s_ncand = 0;
+        __syncthreads();
+        if (s_count[lane] >= P) bound = key[lane * M / 32];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+          const unsigned long long other = __shfl_xor_sync(0xffffffffu, bound, o);
+          bound = other > bound ? other : bound;
+        }
       }
-      for (int o = 1; o < (1 << lt); o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-      if (j < M && part == 0) sel[j] = rank < P;
+      for (int j = tid; j < M; j += kThreads)
+        if (key[j] >= bound) cand[atomicAdd(&s_ncand, 1)] = j;   // in any order
+      __syncthreads();
+      const int nc_ = s_ncand;
+      int lt = 0;                                         // 2^lt threads share a candidate's scan
+      while (lt < 4 && (nc_ << (lt + 1)) <= kThreads) ++lt;
+      const int part = tid & ((1 << lt) - 1);
+      for (int i0_ = 0; i0_ < nc_; i0_ += kThreads >> lt) {   // uniform
+        const int i = i0_ + (tid >> lt);
+        const int j = i < nc_ ? cand[i] : 0;
+        const unsigned long long kj = key[j];
+        int rank = 0;
+        if (i < nc_) {
+#pragma unroll 4
+          for (int q = part; q < nc_; q += 1 << lt) {
+            const int k = cand[q];
+            const unsigned long long kk = key[k];
+            rank += (kk > kj) | ((kk == kj) & (k < j));
+          }
+        }
+        for (int o = 1; o < (1 << lt); o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (i < nc_ && part == 0 && rank < P) sel[j] = 1;
+      }
     }
     __syncthreads();
     if (warp == 0) {
@@ -861,7 +908,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int c = tx * 4 + j;
+        const int c = tx + 16 * j;
         cnt[j] = 0.f;
         if (c < n) {
           if (child) {
@@ -881,7 +928,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int c = tx * 4 + j, f = c / C * C;
+          const int c = tx + 16 * j, f = c / C * C;
 #pragma unroll
           for (int i = 0; i < RT; ++i) {
             float sp = 0.f;
@@ -925,7 +972,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         __syncthreads();
       }
 #pragma unroll
-      for (int t = 0; t < DT; ++t) mul_tile<RT>(o[t], sw, ldr, vs + t * 64, ldv, (n + 3) & ~3, ty, tx);
+      for (int t = 0; t < DT; ++t) mul_tile<RT, 4>(o[t], sw, ldr, vs + t * 64, ldv, (n + 3) & ~3, ty, tx);
       __syncthreads();
     }
 #pragma unroll
