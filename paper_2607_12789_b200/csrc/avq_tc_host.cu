@@ -37,17 +37,25 @@ struct TmapKey {
     return true;
   }
 };
-constexpr int kTmapCache = 128;
+// A set-associative table: a call looks at the entries of one set instead of at all of them.
+constexpr int kTmapSets = 64, kTmapWays = 4;
 std::mutex g_tmap_mu;
-TmapKey g_tmap_keys[kTmapCache];
-CUtensorMap g_tmap_vals[kTmapCache];
-int g_tmap_used = 0, g_tmap_next = 0;
+TmapKey g_tmap_keys[kTmapSets][kTmapWays];                // rank 0: empty
+CUtensorMap g_tmap_vals[kTmapSets][kTmapWays];
+uint8_t g_tmap_next[kTmapSets];
+
+unsigned tmap_set(const TmapKey& k) {
+  uint64_t h = reinterpret_cast<uintptr_t>(k.base) >> 8;
+  h = (h ^ (k.dims[1] * 31) ^ ((uint64_t)k.box[1] << 20) ^ (uint64_t)k.rank << 12) * 0x9E3779B97F4A7C15ull;
+  return (unsigned)(h >> 58);
+}
 
 avq_status encode(CUtensorMap* map, const TmapKey& key) {
+  const unsigned set = tmap_set(key);
   {
     std::lock_guard<std::mutex> lock(g_tmap_mu);
-    for (int i = 0; i < g_tmap_used; ++i)
-      if (g_tmap_keys[i] == key) { *map = g_tmap_vals[i]; return AVQ_OK; }
+    for (int i = 0; i < kTmapWays; ++i)
+      if (g_tmap_keys[set][i] == key) { *map = g_tmap_vals[set][i]; return AVQ_OK; }
   }
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return AVQ_ERR_CUDA;
@@ -64,9 +72,9 @@ avq_status encode(CUtensorMap* map, const TmapKey& key) {
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return AVQ_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_tmap_mu);
-  const int slot = g_tmap_used < kTmapCache ? g_tmap_used++ : (g_tmap_next++ % kTmapCache);
-  g_tmap_keys[slot] = key;
-  g_tmap_vals[slot] = *map;
+  const int way = g_tmap_next[set]++ % kTmapWays;
+  g_tmap_keys[set][way] = key;
+  g_tmap_vals[set][way] = *map;
   return AVQ_OK;
 }
 }  // namespace
