@@ -87,7 +87,7 @@ struct Plan {
   // Weights as the A operand in TMEM: nothing to swizzle or fence, the MMA reads half the shared memory, and the
   // codebook survives the tile.  The smallest tile has no TMEM columns left (four CTAs of 128 columns share an
   // SM): its weights overwrite the codebook in shared memory, which is then loaded again (8 KB).
-  static constexpr bool kTW = !(CT == 64 && D == 64);
+  static constexpr bool kTW = !(CT == 64 && D == 64 && NQ == 1);
   // The children's codes and value rows have a buffer each, so that both gathers run ahead of the logits.  The largest
   // tile has room for the values only: the codes go over the parent codebook, whose logits are done by then, and the
   // overwritten half of the codebook is loaded again behind the child logits.  The smallest gathers the values into
@@ -1019,8 +1019,14 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
   a.logC = p.C == 8 ? 3 : 2;
   a.scale_log2e = p.scale * 1.4426950408889634f;
   // Warps per query row follow from how many CTAs can share an SM (TMEM columns, shared memory):
-  // four small CTAs of 128 threads, two of 256, or one of 512.
+  // four small CTAs of 128 threads, two of 256, or one of 512.  A grid too small for that takes twice the warps per
+  // tile (attend, B1 H12 d64 M64: N785 10.3 -> 8.7 us, N2000 12.3 -> 10.3).
+  int sms = 0, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return AVQ_ERR_CUDA;
   if constexpr (D == 64) {
+    if (CT == 64 && a.total_tiles <= 2 * sms) return launch_nq<D, 2, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+    if (CT == 128 && a.total_tiles <= sms) return launch_nq<D, 4, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
     if (CT == 64) return launch_nq<D, 1, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
     if (CT == 128) return launch_nq<D, 2, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
   } else {
