@@ -620,10 +620,12 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, pays from four tiles per
   // CTA on (N16384 H16 d128 M256, 6.9 tiles: 72 -> 63 us); with fewer the uneven last round costs more than the
   // set-up it saves (B2 H8 N5000 d128, 2.2 tiles: whole call 111 -> 130 us), and where the columns of the resident
-  // CTAs exceed TMEM, so that they take them in turn, it costs too (N65536 d64 M256: whole call 780 -> 960 us).
+  // CTAs exceed TMEM, so that they take them in turn, it costs too (N65536 d64 M256: whole call 780 -> 960 us).  A
+  // codebook below 64 KB is set up faster than the loop state costs (B8 H12 N10167 d64 M32: this kernel 122 us with
+  // one tile per CTA, 130 with runs and the norm table).
   const int nbuf2 = resident(2) >= resident(1) ? 2 : 1;
   const bool shared_cols = (int)cols * resident(1) > 512;
-  const bool runs = !shared_cols && (int64_t)total >= 4ll * resident(nbuf2) * sms;
+  const bool runs = !shared_cols && p.M * D >= 32768 && (int64_t)total >= 4ll * resident(nbuf2) * sms;
   const int nbuf = runs ? nbuf2 : 1;
   const size_t smem = bytes(nbuf);
   if (cnorm) {
