@@ -185,9 +185,9 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
   if (use_tensor_path(p)) {
     // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
     // The norm table pays for its launch where a head has four waves of tiles to share it and the codebook is not so
-    // small that a CTA's own norms are nearly free (16 KB: N32768 H16 d64 M128 C4, this kernel 65 -> 61 us with it;
-    // 4 KB: B8 H12 N10167 d64 M32 C8, whole call 270 us without, 276 with).
-    const bool norms_pass = (size_t)p.M * p.d >= 8192 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
+    // small that a CTA's own norms are nearly free (8 KB: B8 H12 N1024 d64 M64, whole call 43.6 -> 43.1 us with it;
+    // 4 KB: B8 H12 N10167 d64 M32 C8, 270 us without, 276 with).
+    const bool norms_pass = (size_t)p.M * p.d >= 4096 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
     s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);
     if (s != AVQ_OK) return s;
     s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, false, r.status_word, st);
