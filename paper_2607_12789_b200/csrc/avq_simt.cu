@@ -524,12 +524,12 @@ constexpr int kAttThreads = 512;   // 32 x 16: thread (ty, tx) owns rows ty*RT .
 // Shared memory of attend_simt_kernel, in floats from the base (doubles first).
 struct AttendSmem {
   int ldr;                                   // pitch of a [k][row] operand
-  size_t w, wpart, q, c, v, s, np, nstay, zt, nseen, sel, list, total;   // offsets in floats
+  size_t w, wpart, q, c, v, s, np, nstay, nseen, sel, list, total;   // offsets in floats
 };
 // RT = 4: 128 query rows at a time (d <= 128), RT = 2: 64 rows.  v == c where the two tiles share one buffer.
 // mma: Q and codewords as bfloat16 rows.
-__host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int block_q, int tile_m,
-                                                         int keep, bool mma) {
+__host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, int M, int P, int tile_m, int keep,
+                                                         bool mma) {
   AttendSmem L;
   L.ldr = 32 * RT + 4;
   const int ntiles = tile_m > 0 ? (M + tile_m - 1) / tile_m : 0;
@@ -549,7 +549,6 @@ __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, 
   L.s = take((size_t)(keep ? (M + kCols - 1) / kCols * kCols : kCols) * L.ldr);
   L.np = take(M);
   L.nstay = take(M);
-  L.zt = take((size_t)block_q * ntiles);
   L.nseen = take(ntiles);
   L.sel = take(M);
   L.list = take(P > 0 ? P : 1);
@@ -588,12 +587,12 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   constexpr int R = 32 * RT, kThreads = kAttThreads;
   const int d = a.d, M = a.M, C = a.C, P = a.P;
   constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
-  const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.block_q, a.tile_m, a.keep, kMma);
+  const AttendSmem L = attend_smem_layout(RT, DT, d, M, P, a.tile_m, a.keep, kMma);
   const int ldr = L.ldr;
   double* w = reinterpret_cast<double*>(sm + L.w);
   double* wpart = reinterpret_cast<double*>(sm + L.wpart);   // [16][64]
   float *qs = sm + L.q, *cs = sm + L.c, *vs = sm + L.v, *ss = sm + L.s;
-  float *npS = sm + L.np, *nstay = sm + L.nstay, *zt = sm + L.zt, *nseen = sm + L.nseen;
+  float *npS = sm + L.np, *nstay = sm + L.nstay, *nseen = sm + L.nseen;
   int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
   constexpr int ldv = DT * 64;
   int* cand = reinterpret_cast<int*>(wpart);              // [M] candidates of the selection (the sums are done by then)
@@ -684,7 +683,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
     sel[j] = 0;
   }
   __syncthreads();
-  if (tid < ntiles) {                                     // keys of each tile; turned into prefix sums after pass A
+  if (tid < ntiles) {                                     // keys of each tile; summed up to a tile where the importance is finished
     float seen = 0.f;
     const int j1 = min(M, (tid + 1) * a.tile_m);
     for (int j = tid * a.tile_m; j < j1; ++j) seen += npS[j];
@@ -692,93 +691,79 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   }
   // the choice of parents needs the importances only if there is one to make
   const bool need_w = (P > 0 && P < M) || a.importance_out != nullptr;
-  // width of the parent tile that starts at c0: it ends where a tile of the tiled importance ends
-  auto width_at = [&](int c0) {
-    int n = min(kCols, M - c0);
-    if (ntiles) n = min(n, (c0 / a.tile_m + 1) * a.tile_m - c0);
-    return n;
-  };
   // with a.keep the tiles start at multiples of 64 (validated by the launcher), so S is [M][rows]
+  // Passes A and B over one tile of the tiled importance (exact importance: one tile of all parents) before the next,
+  // with the maximum and denominator carried on: a tile's weights are taken against the maximum and the denominator seen
+  // up to it, so they stay finite however far a later tile's logits lie above them.
+  const int span = ntiles ? a.tile_m : M;
   for (int rt = 0; rt < nrt && need_w; ++rt) {
     if (rt > 0) { __syncthreads(); load_q(rt); }
-    // ---- pass A
     float m[RT], z[RT];
 #pragma unroll
     for (int i = 0; i < RT; ++i) { m[i] = -INFINITY; z[i] = 0.f; }
-    for (int c0 = 0; c0 < M;) {
-      const int n = width_at(c0);
-      float acc[RT][4];
-      float* s0 = a.keep ? ss + (size_t)c0 * ldr : ss;
-      logits(acc, s0, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
-      if (!kMma && a.keep) store_s(s0, acc);
-      float cnt[4];
+    for (int t0 = 0; t0 < M; t0 += span) {
+      const int t1 = min(M, t0 + span);
+      // ---- pass A
+      for (int c0 = t0; c0 < t1;) {
+        const int n = min(kCols, t1 - c0);
+        float acc[RT][4];
+        float* s0 = a.keep ? ss + (size_t)c0 * ldr : ss;
+        logits(acc, s0, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+        if (!kMma && a.keep) store_s(s0, acc);
+        float cnt[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cnt[j] = tx + 16 * j < n ? npS[c0 + tx + 16 * j] : 0.f;
-      const int t = ntiles ? c0 / a.tile_m : 0;
+        for (int j = 0; j < 4; ++j) cnt[j] = tx + 16 * j < n ? npS[c0 + tx + 16 * j] : 0.f;
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
+          mx = max16(mx);
+          if (mx > m[i]) {                                // uniform over the 16 threads of the row
+            z[i] *= expf(m[i] - mx);
+            m[i] = mx;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) z[i] = fmaf(expf(acc[i][j] - m[i]), cnt[j], z[i]);
+        }
+        c0 += n;
+        __syncthreads();
+      }
+      // exact: the row's full denominator.  Tiled (appendix "Computing Importance with Tiled Codewords"): the
+      // denominator seen up to this codeword's tile (Eq. "aproxdenom").
+      double inv[RT];
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
-        float mx = -INFINITY;
+        const float zi = sum16(z[i]);
+        inv[i] = rt * R + row_of(i) < rows ? 1.0 / (double)zi : 0.0;
+      }
+      // ---- pass B
+      for (int c0 = t0; c0 < t1;) {
+        const int n = min(kCols, t1 - c0);
+        float acc[RT][4];
+        if (a.keep) load_s(ss + (size_t)c0 * ldr, acc);
+        else logits(acc, ss, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
 #pragma unroll
-        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
-        mx = max16(mx);
-        if (mx > m[i]) {                                  // uniform over the 16 threads of the row
-          const float alpha = expf(m[i] - mx);
-          z[i] *= alpha;
-          if (tx == 0)                                    // denominators already recorded follow the reference
-            for (int u = 0; u < t; ++u) if (rt * R + row_of(i) < rows) zt[(size_t)(rt * R + row_of(i)) * ntiles + u] *= alpha;
-          m[i] = mx;
+        for (int j = 0; j < 4; ++j) {
+          double s = 0.0;
+          if (tx + 16 * j < n && npS[c0 + tx + 16 * j] > 0.f) {
+#pragma unroll
+            for (int i = 0; i < RT; ++i)
+              if (rt * R + row_of(i) < rows) s = fma((double)expf(acc[i][j] - m[i]), inv[i], s);
+          }
+          s += __shfl_xor_sync(0xffffffffu, s, 16);
+          if (lane < 16) wpart[warp * kCols + tx + 16 * j] = s;
         }
+        __syncthreads();
+        if (tid < n) {
+          double s = 0.0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) z[i] = fmaf(expf(acc[i][j] - m[i]), cnt[j], z[i]);
-        if (ntiles && (c0 + n == M || (c0 + n) % a.tile_m == 0)) {
-          const float zp = sum16(z[i]);
-          if (tx == 0 && rt * R + row_of(i) < rows) zt[(size_t)(rt * R + row_of(i)) * ntiles + t] = zp;
+          for (int u = 0; u < kThreads / 32; ++u) s += wpart[u * kCols + tid];
+          w[c0 + tid] += s;
         }
+        c0 += n;
+        __syncthreads();
       }
-      c0 += n;
-      __syncthreads();
-    }
-    double inv[RT];
-#pragma unroll
-    for (int i = 0; i < RT; ++i) {
-      const float zi = sum16(z[i]);
-      inv[i] = (!ntiles && rt * R + row_of(i) < rows) ? 1.0 / (double)zi : 0.0;
-    }
-    // ---- pass B
-    int t_inv = -1;
-    for (int c0 = 0; c0 < M;) {
-      const int n = width_at(c0);
-      float acc[RT][4];
-      if (a.keep) load_s(ss + (size_t)c0 * ldr, acc);
-      else logits(acc, ss, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
-      if (ntiles && c0 / a.tile_m != t_inv) {
-        // exact: the row's full denominator.  Tiled (appendix "Computing Importance with Tiled Codewords"):
-        // the denominator seen up to this codeword's tile (Eq. "aproxdenom").
-        t_inv = c0 / a.tile_m;
-#pragma unroll
-        for (int i = 0; i < RT; ++i)
-          inv[i] = rt * R + row_of(i) < rows ? 1.0 / (double)zt[(size_t)(rt * R + row_of(i)) * ntiles + t_inv] : 0.0;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        double s = 0.0;
-        if (tx + 16 * j < n && npS[c0 + tx + 16 * j] > 0.f) {
-#pragma unroll
-          for (int i = 0; i < RT; ++i)
-            if (rt * R + row_of(i) < rows) s = fma((double)expf(acc[i][j] - m[i]), inv[i], s);
-        }
-        s += __shfl_xor_sync(0xffffffffu, s, 16);
-        if (lane < 16) wpart[warp * kCols + tx + 16 * j] = s;
-      }
-      __syncthreads();
-      if (tid < n) {
-        double s = 0.0;
-#pragma unroll
-        for (int u = 0; u < kThreads / 32; ++u) s += wpart[u * kCols + tid];
-        w[c0 + tid] += s;
-      }
-      c0 += n;
-      __syncthreads();
     }
   }
   if (need_w) {
@@ -1059,7 +1044,7 @@ template <typename T, int RT, int DT, bool CORR>
 avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st) {
   constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
   auto bytes = [&](int keep) {
-    return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.block_q, a.tile_m, keep, kMma).total;
+    return sizeof(float) * attend_smem_layout(RT, DT, a.d, a.M, a.P, a.tile_m, keep, kMma).total;
   };
   // The block's logits stay in shared memory when one row tile holds the block and that leaves room for two
   // CTAs per SM (or all of an SM's memory is there for the taking because the grid has a CTA per SM at most).

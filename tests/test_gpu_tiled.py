@@ -43,3 +43,33 @@ def test_one_tile_reproduces_the_plain_forward():
     Y0, topp0, imp0, _ = binding.forward(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], wl.P, wl.block_q, aux=True)
     assert torch.equal(topp, topp0) and torch.allclose(imp, imp0, rtol=1e-5, atol=1e-6)
     assert (Y - Y0).abs().max().item() <= 1e-5
+
+
+@pytest.mark.parametrize("dtype,d,M,tile_m,N,bq", [("f32", 64, 96, 32, 300, 100), ("f32", 36, 200, 64, 260, 64),
+                                                   ("bf16", 64, 256, 128, 300, 128), ("f32", 64, 96, 32, 300, 150)])
+def test_a_later_tile_far_above_an_earlier_one_leaves_finite_importances(dtype, d, M, tile_m, N, bq):
+    """Logits of the last tile lie about 150 (natural log) above those of the tiles before it, more than fp32's
+    exponent holds: the importances of the earlier tiles are ratios of their own and must not come out as 0 / 0."""
+    wl = synth.Workload("far_tile", B=1, H=2, N=N, d=d, M=M, C=2, P=max(2, M // 8), block_q=bq, dtype=dtype, seed=65 + M,
+                        alpha=0.8)
+    x = synth.generate(wl)
+    first = (M - 1) // tile_m * tile_m
+    u = np.zeros(d, dtype=np.float32)
+    u[0] = 1.0
+    lift = 150.0 / wl.scale / 32.0
+    for k, f in (("Cp", slice(None)), ("Cc", slice(None))):
+        x[k][:, first:] += lift * u
+    x["K"] += 0.5 * lift * u                                     # half way: keys on both sides
+    x["K"][:, :, ::2] += 0.5 * lift * u
+    x["K"][:, :, 1::2] -= 0.5 * lift * u
+    x["Q"] += 32.0 * u
+    x = {k: (synth.round_to_bf16(v) if dtype == "bf16" else v) for k, v in x.items()}
+    dv = parity.to_device(x, dtype)
+    Y, topp, imp = binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], wl.P, bq, tile_m, scale=wl.scale)
+    torch.cuda.synchronize()
+    assert torch.isfinite(imp).all()
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], wl.P, bq, wl.scale, form="factorised", tile_m=tile_m)
+    assert (ref["importance"][..., :first] > 0.05).any(axis=-1).all()   # an earlier tile does matter
+    same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
+    rows = np.repeat(same, bq, axis=-1)[..., :N]
+    parity.compare_output(Y.float().cpu().numpy().astype(np.float64), ref["Y"], dtype, rows)
