@@ -519,6 +519,9 @@ struct AttendArgs {
   float scale;
 };
 
+// A running maximum starts at the lowest finite value: while every logit seen is -inf (a product beyond fp32's range) the
+// weights are then exp(-inf) = 0, not exp(-inf + inf).
+constexpr float kLowest = -3.402823466e38f;
 constexpr int kAttThreads = 512;   // 32 x 16: thread (ty, tx) owns rows ty*RT .. , columns tx*4
 
 // Shared memory of attend_simt_kernel, in floats from the base (doubles first).
@@ -700,7 +703,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
     if (rt > 0) { __syncthreads(); load_q(rt); }
     float m[RT], z[RT];
 #pragma unroll
-    for (int i = 0; i < RT; ++i) { m[i] = -INFINITY; z[i] = 0.f; }
+    for (int i = 0; i < RT; ++i) { m[i] = kLowest; z[i] = 0.f; }
     for (int t0 = 0; t0 < M; t0 += span) {
       const int t1 = min(M, t0 + span);
       // ---- pass A
@@ -735,7 +738,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
         const float zi = sum16(z[i]);
-        inv[i] = rt * R + row_of(i) < rows ? 1.0 / (double)zi : 0.0;
+        inv[i] = rt * R + row_of(i) < rows && zi != 0.f ? 1.0 / (double)zi : 0.0;
       }
       // ---- pass B
       for (int c0 = t0; c0 < t1;) {
@@ -857,7 +860,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
     float m[RT], z[RT], o[DT][RT][4];
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
-      m[i] = -INFINITY; z[i] = 0.f;
+      m[i] = kLowest; z[i] = 0.f;
 #pragma unroll
       for (int t = 0; t < DT; ++t)
 #pragma unroll

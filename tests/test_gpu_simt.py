@@ -139,3 +139,22 @@ def test_tile_edges_of_the_register_tiled_kernels(d, M, C, P, bq, N):
     _, topp, imp = binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, bq, 32, scale=wl.scale)
     ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, bq, wl.scale, form="factorised", tile_m=32)
     parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
+
+
+@pytest.mark.parametrize("dtype,flags", [("f32", 0), ("bf16", SIMT)])
+def test_logits_beyond_the_range_of_fp32_weigh_nothing(dtype, flags):
+    """The first 64 parents, a whole codeword tile, and their children have logits of -1e39, -inf in fp32: their weights
+    are 0 as long as any other codeword holds a key."""
+    wl = synth.Workload("neg", B=1, H=2, N=300, d=64, M=130, C=3, P=9, block_q=128, dtype=dtype, seed=91, alpha=0.8)
+    x = synth.generate(wl)
+    for k in ("Q", "K", "Cp", "Cc"):
+        x[k][..., 0] = 0.0
+    x["Q"][..., 0] = 1e31
+    x["Cp"][:, :64, 0] = x["Cc"][:, :64, :, 0] = -1e9
+    x["K"][:, :, ::2, 0] = -1e9                                  # every other key belongs to one of them
+    x = {k: (synth.round_to_bf16(v) if dtype == "bf16" else v) for k, v in x.items()}
+    gpu = parity.gpu_forward(wl, x, flags=flags)
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], wl.P, wl.block_q, wl.scale, form="factorised")
+    assert (ref["np"][..., :64].sum(-1) == 150).all() and (ref["importance"][..., :64] == 0).all()
+    same, _ = parity.compare_selection(gpu, ref)
+    parity.compare_output(gpu["Y"], ref["Y"], dtype, np.repeat(same, wl.block_q, axis=-1)[..., :wl.N])
