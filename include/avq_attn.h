@@ -116,7 +116,7 @@ typedef struct {
  */
 
 /* Bytes of device scratch avq_forward needs for this problem (0 if the problem is invalid).
- * The workspace holds a 256-byte header (device status word), the key indices and the
+ * The workspace holds a 256-byte header (device status words), the key indices and the
  * aggregates between the three stages.  Host function, no CUDA calls. */
 AVQ_API size_t avq_workspace_bytes(const avq_problem* prob, int32_t P, int32_t block_q);
 

@@ -258,7 +258,7 @@ template <int D, int C>
 __global__ void __launch_bounds__(D * ((C == 4) ? 8 : 4))
 finalize_kernel(const float* __restrict__ Vc, const float* __restrict__ nc, float* __restrict__ Vp,
                 float* __restrict__ np_, __nv_bfloat16* __restrict__ Vpb, __nv_bfloat16* __restrict__ Vcb,
-                __nv_bfloat16* __restrict__ Vsb, float* __restrict__ rho, int M) {
+                __nv_bfloat16* __restrict__ Vsb, float* __restrict__ rho, int32_t* wide_word, int M) {
   // One CTA = kPer consecutive parents of one (batch, head); thread (k, mm) owns head-dimension index k of
   // parent mm: C + 1 row loads, C + 2 counts, a handful of stores.  The kernel is a load round trip followed
   // by a little arithmetic, so it wants many short threads, not few long ones.
@@ -279,12 +279,15 @@ finalize_kernel(const float* __restrict__ Vc, const float* __restrict__ nc, floa
   const float stay = tc::ld_after_wait(Vp + row * D + k);   // zero unless keys stay
   const float nstay = tc::ld_after_wait(np_ + row);         // keys that stay
   float s = stay, n = nstay;
+  bool wide = false;                                        // a mean beyond kWideMean, infinite or NaN
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     s += x[c];
     n += cn[c];
     // the attention kernel takes per-codeword MEANS: the count rides in its softmax weights
-    if (Vcb) Vcb[(row * C + c) * D + k] = __float2bfloat16_rn(cn[c] > 0.f ? x[c] * fast_rcp(cn[c]) : 0.f);
+    const float mean = cn[c] > 0.f ? x[c] * fast_rcp(cn[c]) : 0.f;
+    wide |= !(fabsf(mean) <= kWideMean);
+    if (Vcb) Vcb[(row * C + c) * D + k] = __float2bfloat16_rn(mean);
   }
   Vp[row * D + k] = s;
   const float rn = n > 0.f ? fast_rcp(n) : 0.f;
@@ -293,8 +296,10 @@ finalize_kernel(const float* __restrict__ Vc, const float* __restrict__ nc, floa
   // attention kernel is A n_p, so the row is Vbar_stay / n_p and the count n_stay / n_p
   if (Vsb) Vsb[row * D + k] = __float2bfloat16_rn(stay * rn);
   if (rho && k == 0) rho[row] = nstay * rn;
-  __syncthreads();                                     // every thread has read its parent's stay count
+  wide |= !(fabsf(s * rn) <= kWideMean) || !(fabsf(stay * rn) <= kWideMean);
+  const int any_wide = __syncthreads_or(wide);         // every thread has read its parent's stay count
   if (k == 0) np_[row] = n;
+  if (any_wide && wide_word && k == 0 && mm == 0) *wide_word = 1;   // (any CTA: the same value)
 }
 
 // Zeroes the four accumulator arrays of a stand-alone avq_aggregate in one launch (inside avq_forward the
@@ -369,7 +374,8 @@ avq_status run(const avq_problem& p, const void* V, const int32_t* pidx, const i
   dim3 g2(p.M / (C == 4 ? 8 : 4), BH);
   return cuda_ok(tc::launch_pdl(finalize_kernel<D, C>, g2, dim3(D, C == 4 ? 8 : 4), 0, st, true, static_cast<const float*>(Vc),
                                 static_cast<const float*>(nc), Vp, np_, static_cast<__nv_bfloat16*>(Vpb),
-                                static_cast<__nv_bfloat16*>(Vcb), static_cast<__nv_bfloat16*>(Vsb), rho, p.M));
+                                static_cast<__nv_bfloat16*>(Vcb), static_cast<__nv_bfloat16*>(Vsb), rho,
+                                Vpb && status_word ? status_word + kWideWord : nullptr, p.M));
 }
 
 }  // namespace

@@ -198,6 +198,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   };
 
   __shared__ int early_exit;
+  __shared__ int wide;                                   // the aggregation met a mean beyond kWideMean, infinite or NaN
   // This CTA's run of consecutive tiles.  The CTAs with one tile more are the first ones of the grid: CTAs that
   // share an SM are a multiple of the SM count apart, so every SM gets its share of them.
   const int per = p.total_tiles / gridDim.x, more = p.total_tiles - per * gridDim.x;
@@ -333,9 +334,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const bool next_new_bh = has_next && nbh != bh;
     const bool next_new_head = next_new_bh && p.H > 1;
     const bool next_new_cp = has_next && (!kTW || next_new_head || (L::kCodesInCA && PC > 0));
-    const bool next_new_v = has_next && (STAYS || !L::kStageInCC || next_new_bh);
     // V of this tile: loaded behind the last use of the one before (below), except for the first tile
-    const bool new_v = STAYS || !L::kStageInCC || new_bh;
+    const bool new_v = STAYS || !L::kStageInCC || new_bh || wide;
 
     if (new_bh) {
       // ---- Part 2 reads what the earlier kernels of this call wrote: status word, counts, value means.  (Loaded
@@ -353,6 +353,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // no reason to stop)
         const int32_t word = p.status_word != nullptr ? *reinterpret_cast<volatile int32_t*>(p.status_word) : 0;
         early_exit = word != 0 && word != DEV_BAD_INDEX;
+        wide = p.status_word != nullptr ? *reinterpret_cast<volatile int32_t*>(p.status_word + kWideWord) : 0;
       }
       if (tid < CT) {
         cnt[parent_pos(tid)] = n_reg;
@@ -671,6 +672,12 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         *reinterpret_cast<uint4*>(Vs + (ch >> 3) * (M * 128) + sw128_offset(parent_pos(row), (ch & 7) * 8)) =
             __ldg(reinterpret_cast<const uint4*>(p.Vsb + ((size_t)bh * M + row) * D) + ch);
       }
+    } else if (wide) {
+      // a refined parent's weight of zero does not take an infinite value row out of the product: clear the row
+      for (int u = tid; u < (min(P, M) << kLogChunks); u += kThreads) {
+        const int row = sel_list[u >> kLogChunks], ch = u & ((1 << kLogChunks) - 1);
+        *reinterpret_cast<uint4*>(Vs + (ch >> 3) * (M * 128) + sw128_offset(parent_pos(row), (ch & 7) * 8)) = make_uint4(0u, 0u, 0u, 0u);
+      }
     }
     float z_run[4] = {0.f, 0.f, 0.f, 0.f};
     {
@@ -883,7 +890,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (warp == 0 && has_next && elect_one()) {
       // the last value MMA has released the weights (here: the codebook's place) and the parent values
       if (!kTW) issue_cp(nbh, kSubD);
-      if (L::kStageInCC && next_new_v) issue_v(nbh);
+      if (L::kStageInCC && (STAYS || next_new_bh || wide)) issue_v(nbh);
     }
     // The output tile is staged in shared memory in the layout of the Q load and written with TMA tile
     // stores; rows past Nq are clipped by the tensor map.

@@ -257,3 +257,47 @@ def test_children_far_above_the_parents_move_the_reference(d, M, C, P, N):
     c = np.einsum("hnd,hmcd->hnmc", x["Q"][0].astype(np.float64), x["Cc"].astype(np.float64)).max((-1, -2))
     assert ((c - s) * wl.scale * np.log2(np.e) > 80).mean() > 0.5
     parity.full_parity(wl, x=x)
+
+
+@pytest.mark.parametrize("B,d,M,C", [(1, 64, 32, 4), (1, 64, 128, 8), (1, 128, 256, 4), (300, 64, 32, 4), (160, 128, 64, 4)])
+def test_a_refined_parent_with_an_infinite_mean_takes_no_part(B, d, M, C):
+    """Every parent refined.  The sums of half of the parents leave fp32's range although their children's do not, and no
+    query looks that way: the parents' mean rows are infinite, carry no weight and must not reach the output (alone and
+    over chained tiles of one CTA)."""
+    g = np.random.default_rng(d + M)
+    N, H = M * C, 1
+    Cp = (3.0 * g.standard_normal((H, M, d))).astype(np.float32)
+    Cp[:, : M // 2, 0], Cp[:, M // 2:, 0] = 40.0, -40.0
+    Cc = Cp[:, :, None, :] + g.standard_normal((H, M, C, d)).astype(np.float32)
+    Cc[..., 0] = Cp[:, :, None, 0]
+    K = Cc.reshape(1, H, N, d).repeat(B, 0)                      # one key on every child
+    V = g.standard_normal((B, H, N, d)).astype(np.float32)
+    V[:, :, N // 2:] = 3e38
+    Q = g.standard_normal((B, H, 200, d)).astype(np.float32)
+    Q[..., 0] = 40.0                                             # logits of the second half lie 280 (natural log) or more below
+    x = {k: synth.round_to_bf16(np.ascontiguousarray(v)) for k, v in dict(Q=Q, K=K, V=V, Cp=Cp, Cc=Cc).items()}
+    x["V"] = np.minimum(x["V"], np.float32(3.3e38))
+    dv = parity.to_device(x, "bf16")
+    Y, topp, imp, inter = binding.forward(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], M, 128, aux=True)
+    assert not torch.isfinite(inter["Vp"]).all() and torch.isfinite(inter["Vc"]).all()
+    from oracle import avq_oracle as orc
+    for b in sorted({0, B - 1}):
+        ref = orc.forward(x["Q"][b:b + 1], x["K"][b:b + 1], x["V"][b:b + 1], x["Cp"], x["Cc"], M, 128, 1 / np.sqrt(d),
+                          form="factorised")
+        parity.compare_output(Y[b:b + 1].double().cpu().numpy(), ref["Y"], "bf16")
+    assert torch.isfinite(Y.float()).all()
+
+
+def test_an_infinite_value_stays_in_its_dimension():
+    """One key's value is infinite in one dimension; its parent is refined.  Every query gives its child some weight: that
+    dimension of the output is infinite, the others are what they are without it."""
+    wl = synth.C1.with_(B=1, H=2, N=512, seed=57, P=64)
+    x = synth.generate(wl)
+    x["Q"] *= 0.1
+    x["V"][0, :, 100, 7] = 0.0
+    ref = parity.gpu_forward(wl, x)["Y"]
+    x["V"][0, :, 100, 7] = np.inf
+    Y = parity.gpu_forward(wl, x)["Y"]
+    assert np.isposinf(Y[..., 7]).all()
+    rest = np.arange(64) != 7
+    assert np.abs(Y[..., rest] - ref[..., rest]).max() <= 1.6e-2   # (a mean next to a rounding boundary: an ulp of bf16)
