@@ -66,8 +66,8 @@ constexpr size_t kSimtAttendSmemLimit = 200 * 1024;
 
 // ---- tensor-core kernels (avq_tc_*.cu) ----
 // Word of the workspace header that the aggregation sets when a mean value is larger than kWideMean, infinite or NaN (cleared
-// with the header at the start of a forward).  The attention kernel then lets no excluded value row meet a zero weight, at
-// the cost of loads that ordinary values do not need.
+// with the header at the start of a forward).  The attention kernel then lets no excluded value row meet a zero weight and
+// keeps its running sums small, at the cost of loads and turns that ordinary values do not need.
 constexpr int kWideWord = 1;
 constexpr float kWideMean = 1.0995116e12f;                // 2^40
 // zero_base / zero_bytes: a region (multiple of 16 bytes, or none) the assign grid clears on the side

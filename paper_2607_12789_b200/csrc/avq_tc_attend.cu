@@ -786,9 +786,10 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // Any reference value works as long as numerator and denominator share it: the parents' maximum is kept
         // unless the children's weights grow so large against it that fp32 sums could overflow.  That is found out
         // at the barrier that publishes the weights; the rare case goes round the loop once more.
-        constexpr float kLargest = 1.8446744e19f;          // 2^64
+        // 2^64 while no mean exceeds 2^40 (the sums stay below 2^115 then), 2^8 with values beyond that.
+        const float largest = wide ? 256.f : 1.8446744e19f;
         weights_done();
-        if (!__syncthreads_or(fmaxf(fmaxf(zc[0], zc[1]), fmaxf(zc[2], zc[3])) > kLargest)) break;
+        if (!__syncthreads_or(fmaxf(fmaxf(zc[0], zc[1]), fmaxf(zc[2], zc[3])) > largest)) break;
         // ---- row maxima of the chunk (non-empty children); where they exceed the reference it moves up and O and z
         // are rescaled
         float m_c[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};

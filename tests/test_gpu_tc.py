@@ -259,6 +259,33 @@ def test_children_far_above_the_parents_move_the_reference(d, M, C, P, N):
     parity.full_parity(wl, x=x)
 
 
+@pytest.mark.parametrize("d,M,C,P,N", [(64, 64, 4, 16, 300), (64, 96, 8, 40, 260), (128, 64, 4, 5, 250), (128, 256, 4, 48, 400),
+                                       (64, 160, 4, 33, 300)])
+def test_large_values_leave_room_for_children_above_their_parents(d, M, C, P, N):
+    """Values of 1e28 under children whose logits exceed the parents' maximum by tens of powers of two: the running sums
+    must move to the children's reference before they leave fp32's range.  (The output is compared divided by 1e28, which
+    bf16 inputs and fp32 sums carry without a rounding of their own; avq_attend over the same workspace agrees.)"""
+    wl = synth.Workload("large", B=1, H=2, N=N, d=d, M=M, C=C, P=P, block_q=128, seed=950 + M + d, alpha=0.6,
+                        hot_queries=True, sigma_c=7.0)
+    x = synth.generate(wl)
+    s = np.einsum("hnd,hmd->hnm", x["Q"][0].astype(np.float64), x["Cp"].astype(np.float64)).max(-1)
+    c = np.einsum("hnd,hmcd->hnmc", x["Q"][0].astype(np.float64), x["Cc"].astype(np.float64)).max((-1, -2))
+    gap = (c - s) * wl.scale * np.log2(np.e)
+    assert ((gap > 40) & (gap < 62)).mean() > 0.2
+    unit = float(2.0 ** 93)                                      # 9.9e27
+    dv = parity.to_device(x, "bf16")
+    dv["V"] = (dv["V"].float() * unit).to(torch.bfloat16)
+    f = binding.Forward(1, 2, N, N, d, M, C, P, 128, scale=wl.scale, aux=True)
+    Y = f(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"])
+    f.check()
+    Y2 = f.attend(dv["Q"], dv["Cp"], dv["Cc"])
+    assert torch.equal(Y2, Y)
+    from oracle import avq_oracle as orc
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, 128, wl.scale, form="factorised")
+    same, _ = parity.compare_selection(dict(selected=f.topp.cpu().numpy(), importance=f.importance.cpu().numpy()), ref)
+    parity.compare_output((Y.double() / unit).cpu().numpy(), ref["Y"], "bf16", np.repeat(same, 128, axis=-1)[..., :N])
+
+
 @pytest.mark.parametrize("B,d,M,C", [(1, 64, 32, 4), (1, 64, 128, 8), (1, 128, 256, 4), (300, 64, 32, 4), (160, 128, 64, 4)])
 def test_a_refined_parent_with_an_infinite_mean_takes_no_part(B, d, M, C):
     """Every parent refined.  The sums of half of the parents leave fp32's range although their children's do not, and no
