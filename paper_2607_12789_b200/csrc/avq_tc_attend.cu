@@ -674,6 +674,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
     } else if (wide) {
       // a refined parent's weight of zero does not take an infinite value row out of the product: clear the row
+#pragma unroll 1
       for (int u = tid; u < (min(P, M) << kLogChunks); u += kThreads) {
         const int row = sel_list[u >> kLogChunks], ch = u & ((1 << kLogChunks) - 1);
         *reinterpret_cast<uint4*>(Vs + (ch >> 3) * (M * 128) + sw128_offset(parent_pos(row), (ch & 7) * 8)) = make_uint4(0u, 0u, 0u, 0u);
