@@ -106,6 +106,11 @@ struct Plan {
                        oCV = oCC + (kSepCV && !kCodesInCA ? CHW * D * 2 : 0);
   static constexpr int oStage = kStageInCC ? oCC : oV;
   static constexpr int oF = oCV + CHW * D * 2;           // fp32 / word arrays from here
+  // Plans of twice the warps per tile (small grids): two neighbouring warps of a row add the denominator as the one warp of
+  // the other plan does, the second going on from the first's sums, so that which parents are selected does not depend on
+  // how many tiles a call has.
+  static constexpr bool kChain = D == 64 && CT / NQ == 32;
+  static constexpr int chain_floats = kChain ? NQ / 2 * 4 * kRows : 0;
   // TMEM columns: logits, weights (kTW), output.  With 256 logit columns the child logits use half of them and the
   // children's weights go into the other half, so they need not wait for the parents' value MMA.
   static constexpr bool kSepW = CT == 256;
@@ -119,7 +124,7 @@ struct Plan {
 template <int D, int NQ, int CT>
 size_t attend_smem(int MC) {
   using L = Plan<D, NQ, CT>;
-  return L::oF + 4 * ((size_t)2 * CT + CT + L::CHW + CT + 4 * CT + 2 * NQ * kRows + 2 * CT + MC + CT + 32 + 18) + 8 * 6 + 16;
+  return L::oF + 4 * ((size_t)2 * CT + CT + L::CHW + CT + 4 * CT + 2 * NQ * kRows + 2 * CT + MC + CT + 32 + 18 + L::chain_floats) + 8 * 6 + 16;
 }
 
 // STAYS = the PARENT_STAYS rule: a refined parent keeps the keys that stayed with it.
@@ -170,6 +175,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   uint64_t* bars = reinterpret_cast<uint64_t*>(ncand_s + 2);     // [6]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* zchain = reinterpret_cast<float*>(tmem_slot + 2);   // [NQ / 2][4][128] kChain
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
@@ -340,7 +346,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (new_bh) {
       // ---- Part 2 reads what the earlier kernels of this call wrote: status word, counts, value means.  (Loaded
       // with statements the compiler cannot move ahead of the dependency wait.)
-      static_assert(CT <= kThreads && 2 * CT <= 4 * kThreads, "one count load per thread");
+      static_assert(2 * CT <= kThreads, "one count load per thread: M * C / 4 <= 2 CT vectors of four");
       if (first) pdl_wait();
       float n_reg = 0.f;
       float4 nc_reg = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -428,7 +434,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     // m_run is finite: at least one parent holds a key.
 
     // ---- fp32 weights and the exact denominator.  This lane's columns are the codewords t, t + 4, ... of the slice
-    // in ascending order: one chain per row, the quad adds (0 + 1) + (2 + 3).
+    // (kChain: of two warps' slices) in ascending order: one chain per row, the quad adds (0 + 1) + (2 + 3).
     float iz[4];                                         // 1 / z, 0 for rows past the end
     {
       float z[4] = {0.f, 0.f, 0.f, 0.f};
@@ -451,20 +457,48 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
               unpack2(fma2(x, sc2, nm[h]), lo, hi);
               lo = ex2(lo);
               hi = ex2(hi);
-              z[h] = fmaf(hi, n2[b].y, fmaf(lo, n2[b].x, z[h]));
+              if constexpr (!L::kChain) z[h] = fmaf(hi, n2[b].y, fmaf(lo, n2[b].x, z[h]));
               x = pack2(lo, hi);
             }
+        }
+      }
+      constexpr int NZ = L::kChain ? NQ / 2 : NQ;        // chains per row
+      const int cz = L::kChain ? cq >> 1 : cq;
+      if constexpr (L::kChain) {
+        float4* part = reinterpret_cast<float4*>(zchain + cz * 4 * kRows) + q * 32 + lane;
+        auto add = [&]() {
+          if (my_cols > 0)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const float2 n2 = *reinterpret_cast<const float2*>(cnt + colbase + 8 * b + 2 * t4);
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                float lo, hi;
+                unpack2(a[h][b], lo, hi);
+                z[h] = fmaf(hi, n2.y, fmaf(lo, n2.x, z[h]));
+              }
+            }
+        };
+        if ((cq & 1) == 0) {                             // warp-uniform
+          add();
+          *part = make_float4(z[0], z[1], z[2], z[3]);
+        }
+        row_sync<NQ>(q);
+        if (cq & 1) {
+          const float4 first_half = *part;
+          z[0] = first_half.x; z[1] = first_half.y; z[2] = first_half.z; z[3] = first_half.w;
+          add();
         }
       }
 #pragma unroll
       for (int h = 0; h < 4; ++h) z[h] = quad_sum(z[h]);
       float zr;                                          // of row `lane`
       if (NQ > 1) {
-        xz[cq * kRows + q * 32 + g + 8 * t4] = pick4(z, t4);
+        if (!L::kChain || (cq & 1)) xz[cz * kRows + q * 32 + g + 8 * t4] = pick4(z, t4);
         row_sync<NQ>(q);
         zr = xz[r];
 #pragma unroll
-        for (int u = 1; u < NQ; ++u) zr += xz[u * kRows + r];
+        for (int u = 1; u < NZ; ++u) zr += xz[u * kRows + r];
       } else {
         zr = __shfl_sync(0xffffffffu, pick4(z, t4), 4 * (lane & 7) + (lane >> 3));
       }

@@ -328,3 +328,16 @@ def test_an_infinite_value_stays_in_its_dimension():
     assert np.isposinf(Y[..., 7]).all()
     rest = np.arange(64) != 7
     assert np.abs(Y[..., rest] - ref[..., rest]).max() <= 1.6e-2   # (a mean next to a rounding boundary: an ulp of bf16)
+
+
+@pytest.mark.parametrize("M,C,P", [(32, 4, 4), (64, 4, 8), (96, 8, 12), (128, 4, 16)])
+def test_selection_of_a_head_does_not_depend_on_the_rest_of_the_call(M, C, P):
+    """One image alone (a grid that leaves the chip idle takes twice the warps per tile) and the same image in a batch:
+    the importances agree to the last bit, and so do the selections."""
+    wl = synth.Workload("alone", B=5, H=12, N=785, d=64, M=M, C=C, P=P, block_q=128, seed=77 + M, alpha=0.5)
+    dv = parity.to_device(synth.generate(wl), "bf16")
+    _, topp, imp, _ = binding.forward(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, 128, aux=True)
+    for b in (0, 3):
+        one = {k: dv[k][b:b + 1].contiguous() for k in "QKV"}
+        _, topp1, imp1, _ = binding.forward(one["Q"], one["K"], one["V"], dv["Cp"], dv["Cc"], P, 128, aux=True)
+        assert torch.equal(imp1[0], imp[b]) and torch.equal(topp1[0], topp[b])
