@@ -524,10 +524,11 @@ struct AttendArgs {
 constexpr float kLowest = -3.402823466e38f;
 constexpr int kAttThreads = 512;   // 32 x 16: thread (ty, tx) owns rows ty*RT .. , columns tx*4
 
-// Shared memory of attend_simt_kernel, in floats from the base (doubles first).
+// Shared memory of attend_simt_kernel, in floats from the base (doubles first).  All of it is dynamic: the limits the
+// launcher compares it with are those of a CTA's dynamic and static memory together.
 struct AttendSmem {
   int ldr;                                   // pitch of a [k][row] operand
-  size_t w, wpart, q, c, v, s, np, nstay, nseen, sel, list, total;   // offsets in floats
+  size_t w, wpart, q, c, v, s, np, nstay, nseen, sel, list, count, total;   // offsets in floats
 };
 // RT = 4: 128 query rows at a time (d <= 128), RT = 2: 64 rows.  v == c where the two tiles share one buffer.
 // mma: Q and codewords as bfloat16 rows.
@@ -555,6 +556,7 @@ __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, 
   L.nseen = take(ntiles);
   L.sel = take(M);
   L.list = take(P > 0 ? P : 1);
+  L.count = take(33);
   L.total = o;
   return L;
 }
@@ -599,7 +601,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   int *sel = reinterpret_cast<int*>(sm + L.sel), *sel_list = reinterpret_cast<int*>(sm + L.list);
   constexpr int ldv = DT * 64;
   int* cand = reinterpret_cast<int*>(wpart);              // [M] candidates of the selection (the sums are done by then)
-  __shared__ int s_count[32], s_ncand;
+  int *s_count = reinterpret_cast<int*>(sm + L.count), *s_ncand = s_count + 32;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = tid & 15, ty = tid >> 4;
   const int blk = blockIdx.x, bh = blockIdx.y, h = bh % a.H;
@@ -801,7 +803,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
           c = __reduce_add_sync(0xffffffffu, c);
           if (lane == 0) s_count[2 * warp + e] = c;
         }
-        if (tid == 0) s_ncand = 0;
+        if (tid == 0) *s_ncand = 0;
         __syncthreads();
         if (s_count[lane] >= P) bound = key[lane * M / 32];
 #pragma unroll
@@ -811,9 +813,9 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         }
       }
       for (int j = tid; j < M; j += kThreads)
-        if (key[j] >= bound) cand[atomicAdd(&s_ncand, 1)] = j;   // in any order
+        if (key[j] >= bound) cand[atomicAdd(s_ncand, 1)] = j;   // in any order
       __syncthreads();
-      const int nc_ = s_ncand;
+      const int nc_ = *s_ncand;
       int lt = 0;                                         // 2^lt threads share a candidate's scan
       while (lt < 4 && (nc_ << (lt + 1)) <= kThreads) ++lt;
       const int part = tid & ((1 << lt) - 1);

@@ -158,3 +158,12 @@ def test_logits_beyond_the_range_of_fp32_weigh_nothing(dtype, flags):
     assert (ref["np"][..., :64].sum(-1) == 150).all() and (ref["importance"][..., :64] == 0).all()
     same, _ = parity.compare_selection(gpu, ref)
     parity.compare_output(gpu["Y"], ref["Y"], dtype, np.repeat(same, wl.block_q, axis=-1)[..., :wl.N])
+
+
+@pytest.mark.parametrize("dtype,d,M,C,P,bq,flags", [("bf16", 128, 193, 1, 13, 128, SIMT), ("f32", 4, 701, 1, 1, 64, 0)])
+def test_logits_that_just_miss_shared_memory_are_recomputed(dtype, d, M, C, P, bq, flags):
+    """One-wave grids keep a block's logits in shared memory if all of it fits a CTA: at these sizes it exceeds the limit
+    by less than the kernel's own counters take.  The call answers, and so does an ordinary one behind it."""
+    wl = synth.Workload("limit", B=1, H=1, N=300, d=d, M=M, C=C, P=P, block_q=bq, dtype=dtype, seed=92, alpha=0.8)
+    parity.full_parity(wl, flags=flags)
+    parity.full_parity(synth.C0)
