@@ -5,13 +5,15 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "avq_attn.h"
 
 namespace avq {
 
 // Byte offsets of the regions of an avq_forward workspace.
 struct Layout {
-  size_t header = 0;       // 256 bytes; int32 status word at offset 0
+  size_t header = 0;       // 256 bytes; int32 status word at offset 0, word kWideWord behind it
   size_t Vc = 0;           // f32 [B,H,M,C,d]   header, Vc, nc, Vp and np are adjacent: one pass clears them
   size_t nc = 0;           // f32 [B,H,M,C]
   size_t Vp = 0;           // f32 [B,H,M,d]     (accumulates the keys that stay with their parent)
@@ -88,6 +90,27 @@ avq_status tc_attend(const avq_problem& p, const void* Q, const void* Cp, const 
                      void* Y, int32_t* topp_out, float* importance_out, int32_t* status_word,
                      bool chained, const int32_t* perm, cudaStream_t st);   // chained: launched right behind tc_aggregate;
                                                          // perm: see forward_core
+
+// Most shared memory, dynamic and static together, of a CTA on sm_100.
+constexpr size_t kSmemMax = 227 * 1024;
+
+// Opens all of a CTA's shared memory to a kernel, once per device.  (The attribute is the kernel's, not the launch's: were
+// it set to what a launch needs, a thread with a small problem could take it from one about to launch a large one.)
+template <auto Kernel>
+avq_status open_shared_memory() {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  const bool known = dev >= 0 && dev < 64;
+  if (known && done[dev].load(std::memory_order_acquire)) return AVQ_OK;
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess) return AVQ_ERR_CUDA;
+  if (cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemMax - fa.sharedSizeBytes)) !=
+      cudaSuccess)
+    return AVQ_ERR_CUDA;
+  if (known) done[dev].store(true, std::memory_order_release);
+  return AVQ_OK;
+}
 
 inline avq_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AVQ_OK : AVQ_ERR_CUDA; }
 

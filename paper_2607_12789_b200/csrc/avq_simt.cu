@@ -1016,7 +1016,6 @@ size_t simt_attend_smem_bytes(int d, int M, int C, int P, int block_q, int tile_
 
 namespace {
 
-constexpr size_t kSmemMax = 227 * 1024;                   // per CTA on sm_100
 constexpr size_t kSmemHalf = 113 * 1024;                  // two CTAs on an SM
 
 template <typename T>
@@ -1024,8 +1023,8 @@ avq_status launch_assign(const avq_problem& p, const void* K, const void* Cp, co
                          int32_t* pidx, int32_t* cidx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
   const size_t smem = sizeof(float) * assign_smem_floats(p.d, std::is_same<T, __nv_bfloat16>::value);
   auto kern = assign_simt_kernel<T>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return AVQ_ERR_CUDA;
+  const avq_status s = open_shared_memory<assign_simt_kernel<T>>();
+  if (s != AVQ_OK) return s;
   dim3 grid((p.Nk + kAssignKeys - 1) / kAssignKeys, p.B * p.H);
   kern<<<grid, kThreads, smem, st>>>(static_cast<const T*>(K), static_cast<const T*>(Cp),
                                      static_cast<const T*>(Cc), pidx, cidx, p.H, p.Nk, p.d, p.M, p.C,
@@ -1062,8 +1061,9 @@ avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st)
   const size_t smem = bytes(a.keep);
   if (smem > kSmemMax) return AVQ_ERR_UNSUPPORTED;
   auto kern = one_wave ? attend_simt_kernel<T, RT, DT, CORR, true> : attend_simt_kernel<T, RT, DT, CORR, false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return AVQ_ERR_CUDA;
+  const avq_status s = one_wave ? open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, true>>()
+                                : open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, false>>();
+  if (s != AVQ_OK) return s;
   return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kAttThreads), smem, st, chained, a));
 }
 

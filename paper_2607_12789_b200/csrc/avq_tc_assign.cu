@@ -562,15 +562,8 @@ avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const 
                          size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, int nbuf, size_t smem,
                          unsigned grid, cudaStream_t st) {
   auto kern = tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>;
-  // The limit is set once per device and instantiation (setting it again is harmless if two threads race).
-  static size_t configured[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
-  if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return AVQ_ERR_CUDA;
-    if (dev >= 0 && dev < 64) configured[dev] = smem;
-  }
+  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>>();
+  if (s != AVQ_OK) return s;
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
                             static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,

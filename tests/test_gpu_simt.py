@@ -167,3 +167,42 @@ def test_logits_that_just_miss_shared_memory_are_recomputed(dtype, d, M, C, P, b
     wl = synth.Workload("limit", B=1, H=1, N=300, d=d, M=M, C=C, P=P, block_q=bq, dtype=dtype, seed=92, alpha=0.8)
     parity.full_parity(wl, flags=flags)
     parity.full_parity(synth.C0)
+
+
+def test_threads_with_problems_of_different_size_do_not_disturb_each_other():
+    """Eight threads, each with its own stream and workspace, launch the same kernels with small and large shared-memory
+    needs: no call fails, and every output is what the call gives alone."""
+    import threading
+
+    def problem(i):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(i)
+        r = lambda *s: torch.randn(*s, device="cuda", generator=g)
+        M, d = (16, 300, 64, 500)[i % 4], (64, 36)[i // 4]
+        f = binding.Forward(1, 1, 200, 200, d, M, 2, 2, 64, dtype=torch.float32)
+        return f, (r(1, 1, 200, d), r(1, 1, 200, d), r(1, 1, 200, d), r(1, M, d), r(1, M, 2, d))
+
+    problems = [problem(i) for i in range(8)]
+    alone = [f(*args) for f, args in problems]
+    torch.cuda.synchronize()
+    failed, last = [], [None] * 8
+
+    def work(i):
+        f, args = problems[i]
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            for _ in range(600):
+                try:
+                    last[i] = f(*args)
+                except binding.AvqError as e:
+                    failed.append(e)
+        s.synchronize()
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    for y, y0 in zip(last, alone):
+        assert (y - y0).abs().max().item() <= 1e-5               # (the value sums are added in any order)
