@@ -176,17 +176,15 @@ class Forward:
         self.importance = torch.empty((B, H, self.nblk, M), dtype=torch.float32, device=device) if aux else None
         self.dtype, self.device = dtype, device
         self.shape_y = (B, H, Nq, d)
-        self._prob_ref = ctypes.byref(self.prob)
-        self._forward, self._attend = lib().avq_forward, lib().avq_attend
 
     def __call__(self, Q, K, V, Cp, Cc, Y=None):
         _chk(Q, K, V, Cp, Cc)
         if Y is None:
             Y = torch.empty(self.shape_y, dtype=self.dtype, device=Q.device)
         # (addresses as plain integers, which the argument types convert: no object is made for each)
-        st = self._forward(self._prob_ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), self.P,
-                           self.block_q, Y.data_ptr(), _ptr(self.topp), _ptr(self.importance),
-                           self.workspace.data_ptr(), self.workspace.numel(), _raw_stream())
+        st = lib().avq_forward(ctypes.byref(self.prob), Q.data_ptr(), K.data_ptr(), V.data_ptr(), Cp.data_ptr(),
+                               Cc.data_ptr(), self.P, self.block_q, Y.data_ptr(), _ptr(self.topp), _ptr(self.importance),
+                               self.workspace.data_ptr(), self.workspace.numel(), _raw_stream())
         if st != 0:
             raise AvqError(st, "avq_forward")
         return Y
@@ -196,9 +194,9 @@ class Forward:
         _chk(Q, Cp, Cc)
         if Y is None:
             Y = torch.empty(self.shape_y, dtype=self.dtype, device=Q.device)
-        st = self._attend(self._prob_ref, Q.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), self.P, self.block_q, Y.data_ptr(),
-                          _ptr(self.topp), _ptr(self.importance), self.workspace.data_ptr(),
-                          self.workspace.numel(), _raw_stream())
+        st = lib().avq_attend(ctypes.byref(self.prob), Q.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), self.P, self.block_q,
+                              Y.data_ptr(), _ptr(self.topp), _ptr(self.importance), self.workspace.data_ptr(),
+                              self.workspace.numel(), _raw_stream())
         if st != 0:
             raise AvqError(st, "avq_attend")
         return Y

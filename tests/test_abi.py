@@ -1,10 +1,13 @@
 """The C-ABI library builds, loads and exports every symbol the header declares; host-side
 validation rejects unusable arguments before anything is launched (no GPU needed)."""
+import copy
 import ctypes
 import os
+import pickle
 import re
 
 import pytest
+import torch
 
 from paper_2607_12789_b200 import binding, build
 
@@ -87,6 +90,17 @@ def test_null_misaligned_and_small_workspace_are_rejected_on_the_host(lib):
     assert lib.avq_aggregate(ctypes.byref(p), ok, ok, ok, ok, ok, ok, None, None) == 1
     assert lib.avq_check(None, None) == 1
     assert lib.avq_forward_host(ctypes.byref(p), None, ok, ok, ok, ok, 2, 64, ok, ok, ok, ok, ok, ok, 1 << 30, None) == 1
+
+
+def test_a_planned_forward_can_be_copied_and_saved(lib):
+    """Its buffers and its problem are plain data; a copy plans for itself (a change of its problem does not reach the
+    other)."""
+    f = binding.Forward(1, 2, 256, 256, 64, 16, 4, 2, 64, dtype=torch.float32, device="cpu", aux=True)
+    for g in (copy.deepcopy(f), pickle.loads(pickle.dumps(f)), copy.copy(f)):
+        assert (g.prob.M, g.prob.Nk, g.P, g.block_q, g.dtype) == (16, 256, 2, 64, torch.float32)
+        assert g.workspace.shape == f.workspace.shape and g.importance.shape == f.importance.shape
+        g.prob = binding.problem(1, 2, 128, 256, 64, 16, 4, binding.AVQ_F32, 0.5)
+        assert f.prob.Nq == 256 and g.prob.Nq == 128
 
 
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
