@@ -183,6 +183,7 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
   avq_status s;
   const Regions r = carve(workspace, L);
   if (use_tensor_path(p)) {
+    if ((L.zero_end / 16) >> 31) return AVQ_ERR_WORKSPACE;   // header and accumulators: below 32 GiB
     // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
     // The norm table pays for its launch where a head has four waves of tiles to share it and the codebook is not so
     // small that a CTA's own norms are nearly free (8 KB: B8 H12 N1024 d64 M64, whole call 43.6 -> 43.1 us with it;

@@ -112,6 +112,9 @@ avq_status open_shared_memory() {
   return AVQ_OK;
 }
 
+// Share of each of `parts` CTAs in `units` pieces of work.
+inline size_t slice_units(size_t units, size_t parts) { return (units + parts - 1) / parts; }
+
 inline avq_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AVQ_OK : AVQ_ERR_CUDA; }
 
 }  // namespace avq

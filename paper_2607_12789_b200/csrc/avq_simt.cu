@@ -221,12 +221,12 @@ __host__ __device__ inline size_t assign_smem_floats(int d, bool mma) {
 // Parents: 64 keys x 64 codewords at a time, ||k||^2 + ||c||^2 - 2 k.c with float64 rechecks; bfloat16 products on the
 // tensor cores (M512 d64, 16384 keys: 74 us with float32 multiply-adds).  Children: four lanes per key,
 // direct form.  zero_base / zero_units: 16-byte words this grid clears on the side (the accumulators of the
-// aggregation behind it), each CTA an equal slice.
+// aggregation behind it), each CTA a slice of zero_per.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 2)
 assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* __restrict__ Cc,
                    int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int d, int M,
-                   int C, int parent_stays, uint4* __restrict__ zero_base, uint32_t zero_units) {
+                   int C, int parent_stays, uint4* __restrict__ zero_base, size_t zero_units, size_t zero_per) {
   extern __shared__ __align__(16) float smem[];
   constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value;
   const int dpad = (d + 15) & ~15, pitch = dpad + 8;
@@ -243,10 +243,8 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const int bh = blockIdx.y, h = bh % H;
   const int j0 = blockIdx.x * kAssignKeys;
   if (zero_units) {
-    const uint32_t ncta = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const uint32_t per = (zero_units + ncta - 1) / ncta;
-    const uint32_t u0 = cta * per, u1 = min(zero_units, u0 + per);
-    for (uint32_t u = u0 + tid; u < u1; u += kThreads) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
+    const size_t u0 = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * zero_per, u1 = min(zero_units, u0 + zero_per);
+    for (size_t u = u0 + tid; u < u1; u += kThreads) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
   }
   const T* Kb = K + ((size_t)bh * Nk + j0) * d;
   const int rows = min(kAssignKeys, Nk - j0);
@@ -1029,7 +1027,7 @@ avq_status launch_assign(const avq_problem& p, const void* K, const void* Cp, co
   kern<<<grid, kThreads, smem, st>>>(static_cast<const T*>(K), static_cast<const T*>(Cp),
                                      static_cast<const T*>(Cc), pidx, cidx, p.H, p.Nk, p.d, p.M, p.C,
                                      (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0, static_cast<uint4*>(zero_base),
-                                     (uint32_t)(zero_bytes / 16));
+                                     zero_bytes / 16, slice_units(zero_bytes / 16, (size_t)grid.x * grid.y));
   return cuda_ok(cudaGetLastError());
 }
 
@@ -1089,7 +1087,7 @@ avq_status launch_attend(const AttendArgs& a, int B, bool chained, cudaStream_t 
 
 avq_status simt_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
                        int32_t* parent_idx, int32_t* child_idx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
-  if (zero_bytes % 16 != 0 || (zero_bytes / 16) >> 31) return AVQ_ERR_WORKSPACE;
+  if (zero_bytes % 16 != 0) return AVQ_ERR_WORKSPACE;
   return p.dtype == AVQ_F32
              ? launch_assign<float>(p, K, Cp, Cc, parent_idx, child_idx, zero_base, zero_bytes, st)
              : launch_assign<__nv_bfloat16>(p, K, Cp, Cc, parent_idx, child_idx, zero_base, zero_bytes, st);

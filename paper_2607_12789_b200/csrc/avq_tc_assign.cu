@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D))
 tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmCp,
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
                  int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int M, int nblk, int total_tiles,
-                 int nbuf, uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, uint32_t zero_units,
-                 const float* cnorm_g, int beside) {
+                 int nbuf, uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, size_t zero_units,
+                 size_t zero_per, const float* cnorm_g, int beside) {
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -156,13 +156,11 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   const int MH = M >> 1;                             // columns per half (multiple of 16: M % 32 == 0)
   pdl_launch_dependents();   // the next kernel of the call may begin its set-up
   // Inside avq_forward the grid also clears the accumulators of the aggregation that follows (status
-  // header, leaf sums, leaf counts: zero_units 16-byte words), each CTA an equal slice; the stores drain
+  // header, leaf sums, leaf counts: zero_units 16-byte words), each CTA a slice of zero_per; the stores drain
   // while the tile loads.  A bounded wait that expires does so long after CTA 0 has cleared the header.
   if (zero_units) {
-    const uint32_t ncta = gridDim.x, cta = blockIdx.x;
-    const uint32_t per = (zero_units + ncta - 1) / ncta;
-    const uint32_t u0 = cta * per, u1 = min(zero_units, u0 + per);
-    for (uint32_t u = u0 + tid; u < u1; u += kThreadsA) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
+    const size_t u0 = blockIdx.x * zero_per, u1 = min(zero_units, u0 + zero_per);
+    for (size_t u = u0 + tid; u < u1; u += kThreadsA) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
   }
   auto load_keys = [&](int buf, int b, int t) {      // one thread
     mbar_expect_tx(&bar_k[buf], (uint32_t)kKeyBytes);
@@ -568,7 +566,7 @@ avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const 
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
                             static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,
                             p.H, p.Nk, p.M, nblk, total, nbuf, pow2_cols(p.M), status_word,
-                            static_cast<uint4*>(zero_base), (uint32_t)(zero_bytes / 16), cnorm, beside ? 1 : 0));
+                            static_cast<uint4*>(zero_base), zero_bytes / 16, slice_units(zero_bytes / 16, grid), cnorm, beside ? 1 : 0));
 }
 
 template <int D, int NL, bool STAYS>
@@ -639,7 +637,7 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
 avq_status tc_assign(const avq_problem& p, const void* K, const void* Cp, const void* Cc,
                      int32_t* parent_idx, int32_t* child_idx, int32_t* status_word, void* zero_base,
                      size_t zero_bytes, float* cnorm, bool beside, cudaStream_t st) {
-  if (zero_bytes % 16 != 0 || (zero_bytes / 16) >> 31) return AVQ_ERR_WORKSPACE;
+  if (zero_bytes % 16 != 0) return AVQ_ERR_WORKSPACE;
   const bool stays = (p.flags & AVQ_FLAG_PARENT_STAYS) != 0;
 #define AVQ_ASSIGN(DD, NN)                                                                                     \
   (stays ? launch<DD, NN, true>(p, K, Cp, Cc, parent_idx, child_idx, status_word, zero_base, zero_bytes, cnorm, beside, st) \

@@ -51,3 +51,44 @@ def test_update_matches_the_oracle(wl, flags):
     assert (np.abs(Cc2.float().cpu().numpy() - ref["Cc"]) / scale_c).max() <= tol
     if wl.dtype == "f32":
         np.testing.assert_allclose(Cc2.cpu().numpy().mean(axis=2), Cp2.cpu().numpy(), atol=2e-3)
+
+
+@pytest.mark.parametrize("dtype,B,M,C", [("f32", 4096, 1024, 16), ("bf16", 30000, 256, 8)])
+def test_accumulators_beyond_32_gib(dtype, B, M, C):
+    """The sums and counts of a call fill more than 2^31 16-byte words: the update and the CUDA-core forward clear and use
+    all of them (the workspace is filled with NaN first)."""
+    d, Nk = 128, 2
+    need = B * M * (1 + C) * (d + 1) * 4
+    assert need > 2 ** 35
+    if torch.cuda.mem_get_info()[0] < 1.3 * need:
+        pytest.skip("needs 48 GB of free device memory")
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M)
+    Cp = (3 * torch.randn(1, M, d, device="cuda", generator=g)).to(td)
+    Cc = (Cp.float()[:, :, None] + 0.5 * torch.randn(1, M, C, d, device="cuda", generator=g)).to(td)
+    pick = torch.randint(0, M * C, (B * Nk,), device="cuda", generator=g)
+    K = (Cc.view(M * C, d)[pick].float() + 0.3 * torch.randn(B * Nk, d, device="cuda", generator=g)).to(td).view(B, 1, Nk, d)
+    stats = [torch.rand(s, device="cuda", generator=g) for s in ((1, M, d), (1, M), (1, M, C, d), (1, M, C))]
+    before = [s.cpu().numpy() for s in stats]
+    ws_bytes = binding.lib().avq_codebook_update_workspace_bytes(binding.problem(B, 1, Nk, Nk, d, M, C, binding._dtype_code(K),
+                                                                                1.0))
+    torch.empty(ws_bytes, dtype=torch.uint8, device="cuda").fill_(255)   # the allocator hands this block out again
+    Cp2, Cc2 = binding.codebook_update(K, Cp, Cc, *stats, 0.9)
+    host = lambda t: t.float().cpu().numpy()
+    ref = orc.codebook_update(host(K).reshape(1, 1, B * Nk, d), host(Cp), host(Cc), *before, 0.9)
+    for got, key in zip(stats, ("Sp", "Np", "Sc", "Nc")):
+        np.testing.assert_allclose(got.cpu().numpy(), ref[key], rtol=2e-5, atol=2e-3, err_msg=key)
+    torch.cuda.empty_cache()
+    if dtype == "bf16":
+        return
+    f = binding.Forward(B, 1, 1, Nk, d, M, C, 4, 1, dtype=td)
+    f.workspace.fill_(255)
+    Q, V = torch.randn(B, 1, 1, d, device="cuda", generator=g), torch.randn(B, 1, Nk, d, device="cuda", generator=g)
+    Y = f(Q, K, V, Cp, Cc)
+    f.check()
+    for b in (0, B // 2, B - 1):
+        one = binding.forward(Q[b:b + 1], K[b:b + 1], V[b:b + 1], Cp, Cc, 4, 1)
+        assert (Y[b:b + 1] - one).abs().max().item() <= 1e-5
+    del f
+    torch.cuda.empty_cache()
