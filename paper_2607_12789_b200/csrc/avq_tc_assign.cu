@@ -460,7 +460,21 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           if constexpr (TABLE) dp = fmaf(-2.f, dp, cnorm[par[key]]);
         }
         if constexpr (TABLE) {
-          // float64, direct form, a quarter of the dimensions per lane of the key's group
+          // What the products leave open is measured in the direct form in float32, and what that leaves open (relative
+          // 1e-4) in float64; a quarter of the dimensions per lane of the key's group.  (Products alone separate little
+          // where keys lie far from the origin for their distances: B2 H8 N5000 d128 M96 C8 PARENT_STAYS with 32 added to
+          // every dimension, us per call: 190 with float64 straight behind them, 112 so, 118 in the direct form throughout.)
+          auto direct4 = [&](const __nv_bfloat16* c) {
+            float sd = 0.f;
+#pragma unroll
+            for (int u = 0; u < kT; ++u) {
+              const int cu = s4 + 4 * u;
+              sd += sqdiff8(widen8(*reinterpret_cast<const uint4*>(Ks + (cu >> 3) * (kKeys * 128) + sw128_offset(key, (cu & 7) * 8))),
+                            __ldg(reinterpret_cast<const uint4*>(c) + cu));
+            }
+            sd += __shfl_xor_sync(0xffffffffu, sd, 1);
+            return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
+          };
           auto exact4 = [&](const __nv_bfloat16* c) {
             double sd = 0.0;
             for (int u = 0; u < kT; ++u)
@@ -474,23 +488,42 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           };
           const bool live = done && j0 + key < Nk;
           const __nv_bfloat16* Cch = Cc + (head_base + par[key]) * kC * D;
-          bool redo = live && !(e2 - e1 > near);
-          if (__any_sync(0xffffffffu, redo)) {
-            double best = INFINITY;
-            int bi = 0;
+          bool open = live && !(e2 - e1 > near);         // not decided so far
+          if (__any_sync(0xffffffffu, open)) {
+            float f1 = INFINITY, f2 = INFINITY;
+            int fi = 0;
+#pragma unroll 1
             for (int c = 0; c < kC; ++c) {
-              const double sd = exact4(Cch + (size_t)c * D);
-              if (sd < best) { best = sd; bi = c; }
+              const float sd = direct4(Cch + (size_t)c * D);
+              if (sd < f1) { f2 = f1; f1 = sd; fi = c; }
+              else if (sd < f2) { f2 = sd; }
             }
-            if (redo) c1 = bi;
+            if (open) c1 = fi;
+            open = open && !(f2 - f1 > 1e-4f * f2);
+            if (__any_sync(0xffffffffu, open)) {
+              double best = INFINITY;
+              int bi = 0;
+#pragma unroll 1
+              for (int c = 0; c < kC; ++c) {
+                const double sd = exact4(Cch + (size_t)c * D);
+                if (sd < best) { best = sd; bi = c; }
+              }
+              if (open) c1 = bi;
+            }
           }
           if constexpr (STAYS) {
-            // strict '<' against the parent distance; float64 when the two are closer than fp32 separates
+            // strict '<' against the parent distance, decided the same way
             bool moved = e1 < dp;
-            redo = redo || (live && !(fabsf(e1 - dp) > near));
-            if (__any_sync(0xffffffffu, redo)) {
-              const bool closer = exact4(Cch + (size_t)c1 * D) < exact4(Cp + (head_base + par[key]) * D);
-              if (redo) moved = closer;
+            open = live && !(fabsf(e1 - dp) > near);
+            if (__any_sync(0xffffffffu, open)) {
+              const __nv_bfloat16* Cpk = Cp + (head_base + par[key]) * D;
+              const float fc = direct4(Cch + (size_t)c1 * D), fp = direct4(Cpk);
+              if (open) moved = fc < fp;
+              open = open && !(fabsf(fc - fp) > 1e-4f * fmaxf(fc, fp));
+              if (__any_sync(0xffffffffu, open)) {
+                const bool closer = exact4(Cch + (size_t)c1 * D) < exact4(Cpk);
+                if (open) moved = closer;
+              }
             }
             if (!moved) c1 = -1;
           }

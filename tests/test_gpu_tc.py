@@ -341,3 +341,55 @@ def test_selection_of_a_head_does_not_depend_on_the_rest_of_the_call(M, C, P):
         one = {k: dv[k][b:b + 1].contiguous() for k in "QKV"}
         _, topp1, imp1, _ = binding.forward(one["Q"], one["K"], one["V"], dv["Cp"], dv["Cc"], P, 128, aux=True)
         assert torch.equal(imp1[0], imp[b]) and torch.equal(topp1[0], topp[b])
+
+
+def _offset_inputs(B, H, N, d, M, C, offset, seed, twice=True):
+    """Half of the keys hug their parent, half a child; some children stand there twice; everything shifted by `offset`."""
+    g = np.random.default_rng(seed)
+    Cp = 3 * g.standard_normal((H, M, d))
+    Cc = Cp[:, :, None] + 1.2 * g.standard_normal((H, M, C, d))
+    if twice:
+        Cc[:, ::3, C - 1] = Cc[:, ::3, 0]
+    par, chi = g.integers(0, M, (B, H, N)), g.integers(0, C, (B, H, N))
+    head = np.arange(H)[None, :, None]
+    K = np.where((np.arange(N) % 2 == 0)[:, None], Cp[head, par], Cc[head, par, chi]) + 0.05 * g.standard_normal((B, H, N, d))
+    dev = lambda a: (torch.from_numpy(a).float().cuda() + offset).to(torch.bfloat16)
+    return dev(K), dev(Cp), dev(Cc)
+
+
+@pytest.mark.parametrize("B,H,N,d,M,C", [(1, 16, 4736, 64, 64, 4), (2, 16, 2400, 64, 96, 8), (1, 16, 4736, 128, 64, 8),
+                                         (1, 16, 9500, 128, 256, 4)])
+@pytest.mark.parametrize("flags", [0, binding.FLAG_PARENT_STAYS])
+def test_indices_by_the_norm_table_equal_those_of_the_direct_form(B, H, N, d, M, C, flags):
+    """avq_forward measures children by norms and products where the grid is large, avq_assign directly: the same indices,
+    also where keys and codewords share an offset and the products separate little (one tile per CTA and runs of them)."""
+    for offset in (0.0, 4.0, 32.0, 64.0):
+        K, Cp, Cc = _offset_inputs(B, H, N, d, M, C, offset, seed=d + M)
+        pi, ci = binding.assign(K, Cp, Cc, flags=flags)
+        _, _, _, inter = binding.forward(K[:, :, :128].contiguous(), K, K, Cp, Cc, 4, 128, flags=flags, aux=True)
+        assert torch.equal(inter["parent_idx"], pi) and torch.equal(inter["child_idx"], ci)
+
+
+def test_a_common_offset_costs_little_time():
+    """Offsets that bf16 still resolves make the products of the assignment separate less; what they leave open is decided in
+    float32 before float64 is asked.  (2.7 times the time of centred inputs with float64 straight away, 1.3 with
+    float32 in between.)"""
+    def us(offset):
+        K, Cp, Cc = _offset_inputs(2, 8, 5000, 128, 96, 8, offset, seed=3, twice=False)
+        f = binding.Forward(2, 8, 5000, 5000, 128, 96, 8, 12, 128, flags=binding.FLAG_PARENT_STAYS)
+        Y = torch.empty_like(K)
+        for _ in range(10):
+            f(K, K, K, Cp, Cc, Y)
+        times = []
+        for _ in range(30):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            f(K, K, K, Cp, Cc, Y)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        return sorted(times)[len(times) // 2]
+
+    centred, shifted = us(0.0), us(64.0)
+    print(f"centred {centred:.1f} us, shifted {shifted:.1f} us")
+    assert shifted <= 1.6 * centred
