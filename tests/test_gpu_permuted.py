@@ -76,3 +76,24 @@ def test_rows_written_to_their_places_over_chained_tiles(B, H, N, d, M, C, P):
     # the value sums are added in any order: a bf16 mean may fall to the other side of a rounding boundary
     diff = (Y[:, :, perm.long()].float() - Yg.float()).abs()
     assert diff.max().item() <= 1.6e-2 and diff.mean().item() <= 1e-4
+
+
+@pytest.mark.parametrize("B,H,N,d,M,C,P", [(1, 2, 500, 64, 64, 4, 8), (8, 12, 1100, 64, 64, 4, 8), (1, 2, 500, 64, 128, 8, 16),
+                                           (1, 2, 500, 128, 96, 8, 12), (2, 8, 2500, 128, 256, 4, 32), (4, 10, 1111, 128, 64, 8, 5)])
+def test_keys_that_stay_with_their_parent_under_a_token_order(B, H, N, d, M, C, P):
+    """The PARENT_STAYS rule with output rows written to their places, one tile per CTA and chained tiles: equal to the plain
+    forward under the same rule on gathered queries."""
+    wl = synth.Workload("perm_stays", B=B, H=H, N=N, d=d, M=M, C=C, P=P, block_q=128, seed=25 + M, alpha=0.5)
+    x = synth.generate(wl)
+    x["K"][:, :, ::2] = synth.round_to_bf16(x["Cp"][np.arange(H)[None, :, None], np.arange(0, N, 2)[None, None] % M]
+                                            + np.float32(0.03))   # every other key hugs a parent
+    dv = parity.to_device(x, "bf16")
+    perm = torch.from_numpy(np.random.default_rng(4).permutation(N).astype(np.int32)).cuda()
+    flags = binding.FLAG_PARENT_STAYS
+    Y, topp, imp, status = binding.forward_permuted(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, 128, perm, flags=flags)
+    Yg, topp0, imp0, inter = binding.forward(dv["Q"][:, :, perm.long()].contiguous(), dv["K"], dv["V"], dv["Cp"], dv["Cc"],
+                                             P, 128, flags=flags, aux=True)
+    stayed = (inter["child_idx"] < 0).float().mean().item()
+    assert 0.4 < stayed < 0.6 and status == 0 and torch.equal(topp, topp0) and torch.equal(imp, imp0)
+    diff = (Y[:, :, perm.long()].float() - Yg.float()).abs()     # a bf16 mean may fall to the other side of a boundary
+    assert diff.max().item() <= 1.6e-2 and diff.mean().item() <= 1e-4

@@ -206,3 +206,18 @@ def test_threads_with_problems_of_different_size_do_not_disturb_each_other():
     assert not failed
     for y, y0 in zip(last, alone):
         assert (y - y0).abs().max().item() <= 1e-5               # (the value sums are added in any order)
+
+
+@pytest.mark.parametrize("d,M,C,P,bq,N,stays", [(4, 33, 2, 5, 1, 70, False), (36, 65, 3, 7, 50, 131, False), (68, 130, 5, 9, 129, 300, False),
+                                                (132, 65, 2, 65, 64, 200, False), (256, 33, 4, 0, 100, 210, False),
+                                                (64, 64, 4, 8, 64, 200, False), (128, 130, 16, 3, 200, 450, True),
+                                                (36, 33, 4, 6, 50, 260, True)])
+def test_tile_edges_with_bf16_inputs(d, M, C, P, bq, N, stays):
+    """As above for bfloat16 on the CUDA cores: products by 16 x 8 x 16 tiles (head dimensions that are no multiple of 16,
+    padded rows and columns), every row-tile variant, both child rules."""
+    wl = synth.Workload("edges16", B=1, H=2, N=N, d=d, M=M, C=C, P=P, block_q=bq, dtype="bf16", seed=170 + d, alpha=0.6)
+    x = synth.generate(wl)
+    if stays:                                                    # every other key hugs a parent: it stays
+        x["K"][:, :, ::2] = synth.round_to_bf16(x["Cp"][None, :, np.arange(0, N, 2) % M] + np.float32(0.03))
+    rep = parity.full_parity(wl, flags=SIMT | (STAYS if stays else 0), parent_stays=stays, x=x)
+    assert not stays or 0.8 * N < rep["stay_count"] < 1.2 * N
