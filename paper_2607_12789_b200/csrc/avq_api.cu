@@ -185,9 +185,11 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
   if (use_tensor_path(p)) {
     if ((L.zero_end / 16) >> 31) return AVQ_ERR_WORKSPACE;   // header and accumulators: below 32 GiB
     // status header, leaf sums and leaf counts are adjacent: the assign grid clears them on the side
-    // The norm table pays for its launch where a head has four waves of tiles to share it and the codebook is not so
-    // small that a CTA's own norms are nearly free (8 KB: B8 H12 N1024 d64 M64, whole call 43.6 -> 43.1 us with it;
-    // 4 KB: B8 H12 N10167 d64 M32 C8, 270 us without, 276 with).
+    // The norm table costs a launch and halves the instructions per child.  From four tiles per SM over all heads (592 on
+    // 148 SMs) the two about cancel or it pays; us per call without and with it: d64 M64 C4 192 tiles 22.9 and 24.5, 768 43.4
+    // and 43.6, 1536 70.3 and 69.7; d64 M128 C8 192 tiles 29.1 and 29.7, 1024 68.9 and 68.9; d128 M256 C4 592 tiles 98.9 and
+    // 97.5, 1536 256.8 and 253.4; d128 M96 C8 1536 tiles 200.1 and 201.6.  A 4 KB codebook is too small for it (B8 H12
+    // N10167 d64 M32 C8: 270 and 276).
     const bool norms_pass = (size_t)p.M * p.d >= 4096 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
     s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);
     if (s != AVQ_OK) return s;

@@ -1058,9 +1058,12 @@ avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st)
   a.keep = (a.block_q <= 32 * RT && (a.tile_m == 0 || a.tile_m % kCols == 0) && bytes(1) <= most) ? 1 : 0;
   const size_t smem = bytes(a.keep);
   if (smem > kSmemMax) return AVQ_ERR_UNSUPPORTED;
-  auto kern = one_wave ? attend_simt_kernel<T, RT, DT, CORR, true> : attend_simt_kernel<T, RT, DT, CORR, false>;
-  const avq_status s = one_wave ? open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, true>>()
-                                : open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, false>>();
+  // (the wide variant differs where a CTA may have half an SM's registers otherwise, and in the float32 operand loads)
+  constexpr bool kHasWide = !kMma || (DT == 1 && !CORR);
+  const bool wide = kHasWide && one_wave;
+  auto kern = wide ? attend_simt_kernel<T, RT, DT, CORR, kHasWide> : attend_simt_kernel<T, RT, DT, CORR, false>;
+  const avq_status s = wide ? open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, kHasWide>>()
+                            : open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, false>>();
   if (s != AVQ_OK) return s;
   return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kAttThreads), smem, st, chained, a));
 }

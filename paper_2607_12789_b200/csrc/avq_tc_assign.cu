@@ -1,7 +1,7 @@
 // Tensor-core key assignment (Algorithm 1, parent and child argmin) for bf16 inputs.
 //
-// One CTA takes a run of tiles of 128 consecutive keys of one (batch, head), 8 warps.  TMA stages the key tiles (two
-// buffers where they fit) and, once per head, the head's parent codebook in shared memory (K-major, 128-byte swizzle); one elected thread issues the
+// One CTA takes a tile of 128 consecutive keys of one (batch, head), or a run of them, 8 warps.  TMA stages each key tile
+// and, once per head, the head's parent codebook in shared memory (K-major, 128-byte swizzle); one elected thread issues the
 // tcgen05 MMA chain  D[128 x M] = K_tile . Cp^T  into TMEM.
 //   parent   warp w holds keys 32 (w % 4) .. +31 of the column half w / 4 and reads the products in the fragment layout
 //            (4 keys x column pairs per lane).  Two passes over ||c||^2 - 2 k.c: the minimum of the row; then the
@@ -9,8 +9,9 @@
 //            when there is more than one such column are all M distances redone in float64 in the direct form
 //            (lowest index wins ties).  Three instructions per column and row instead of the six of a running best,
 //            runner-up and index, and half of them off the ALU pipe, which bounded the kernel.
-//   child    fp32 direct form sum (k - c)^2 on CUDA cores (2 C d flops per key; a second MMA over all
-//            M C children would cost C times the parent GEMM), float64 recheck for near-ties.
+//   child    on CUDA cores (a second MMA over all M C children would cost C times the parent GEMM): ||c||^2 - 2 k.c where
+//            a norm table is at hand, near-ties in the direct form sum (k - c)^2 in float32 and then in float64; else
+//            the direct form throughout, near-ties in float64.
 //            Four lanes per key, each over a quarter of the head dimension for all C children of the
 //            key's parent (one running sum per child); a transposing butterfly merges the four lanes.
 #include <type_traits>
@@ -120,15 +121,15 @@ __global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D))
 tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmCp,
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
                  int32_t* __restrict__ pidx, int32_t* __restrict__ cidx, int H, int Nk, int M, int nblk, int total_tiles,
-                 int nbuf, uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, size_t zero_units,
+                 uint32_t tmem_cols, int32_t* status_word, uint4* __restrict__ zero_base, size_t zero_units,
                  size_t zero_per, const float* cnorm_g, int beside) {
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int kSub = D / 64;                       // 64-column sub-tiles along the head dimension
   constexpr int kKeyBytes = kSub * kKeys * 128;
-  if constexpr (!RUNS) nbuf = 1;
-  unsigned char* Cs = smem + nbuf * kKeyBytes;       // kSub x [M x 128 B]; before it nbuf key tiles, kSub x [128 x 128 B] each
+  const unsigned char* Ks = smem;                    // key tile: kSub x [128 x 128 B]
+  unsigned char* Cs = smem + kKeyBytes;              // kSub x [M x 128 B]
   float* cnorm = reinterpret_cast<float*>(Cs + kSub * M * 128);   // [M]
   float* xd = cnorm + M;                             // [2][128] smallest distance of each column half
   float* xs = xd + 2 * kKeys;                        // [2][128] columns close to the minimum: sum of 256 + index
@@ -137,9 +138,9 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   int* chi = par + kKeys;                            // [128] final child of each key
   uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(chi + kKeys);   // max ||c||^2 (non-negative float bits)
   uint32_t* tmem_slot = cmax_bits + 1;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [4]
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 4);
-  uint64_t *bar_k = bars, *bar_mma = bars + 2, *bar_c = bars + 3;   // key tile (per buffer), products, codebook
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [3]
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 3);
+  uint64_t *bar_k = bars, *bar_mma = bars + 1, *bar_c = bars + 2;   // key tile, products, codebook
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
@@ -162,10 +163,10 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const size_t u0 = blockIdx.x * zero_per, u1 = min(zero_units, u0 + zero_per);
     for (size_t u = u0 + tid; u < u1; u += kThreadsA) zero_base[u] = make_uint4(0u, 0u, 0u, 0u);
   }
-  auto load_keys = [&](int buf, int b, int t) {      // one thread
-    mbar_expect_tx(&bar_k[buf], (uint32_t)kKeyBytes);
+  auto load_keys = [&](int b, int t) {               // one thread
+    mbar_expect_tx(bar_k, (uint32_t)kKeyBytes);
 #pragma unroll
-    for (int s = 0; s < kSub; ++s) tma_load_3d(smem + buf * kKeyBytes + s * kKeys * 128, &tmK, s * 64, t * kKeys, b, &bar_k[buf]);
+    for (int s = 0; s < kSub; ++s) tma_load_3d(smem + s * kKeys * 128, &tmK, s * 64, t * kKeys, b, bar_k);
   };
   auto load_codes = [&](int b) {
     mbar_expect_tx(bar_c, (uint32_t)(kSub * M * 128));
@@ -176,13 +177,12 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmCp);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) mbar_init(&bars[i], 1);
+    for (int i = 0; i < 3; ++i) mbar_init(&bars[i], 1);
     mbar_fence_init();
     *abort_flag = 0;
     *cmax_bits = 0;
-    load_keys(0, bh, blk);
+    load_keys(bh, blk);
     load_codes(bh);
-    if (RUNS && nbuf == 2 && tile0 + 1 < tile1) load_keys(1, blk + 1 == nblk ? bh + 1 : bh, blk + 1 == nblk ? 0 : blk + 1);
   }
   // tcgen05.alloc blocks while the SM's columns are taken (four CTAs of 256 columns share an SM at d = 64,
   // M > 128: two run, two wait here).  The holders need nothing from the waiters and free their columns
@@ -196,11 +196,11 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   tc_fence_after();
 
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-  auto issue_mma = [&](const unsigned char* keys) {  // one warp
+  auto issue_mma = [&]() {                           // one warp
     if (elect_one()) {
       tc_fence_after();
       const uint32_t idesc = umma_idesc_bf16(kKeys, M);
-      const uint64_t kd = umma_desc_sw128(smem_u32(keys)), cd = umma_desc_sw128(smem_u32(Cs));
+      const uint64_t kd = umma_desc_sw128(smem_u32(Ks)), cd = umma_desc_sw128(smem_u32(Cs));
 #pragma unroll
       for (int k = 0; k < D / 16; ++k)
         umma_bf16(tmem_base, kd + (uint64_t)((k / 4) * (kKeys * 8) + (k % 4) * 2),
@@ -209,13 +209,12 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
     __syncwarp();
   };
-  uint32_t ph_k = 0, ph_mma = 0, ph_c = 0;           // ph_k: bit per buffer
-  bool new_head = true, mma_issued = false;
-  for (int tile = tile0, buf = 0;; ++tile, buf = RUNS && nbuf == 2 ? buf ^ 1 : 0) {
+  uint32_t ph_k = 0, ph_mma = 0, ph_c = 0;
+  bool new_head = true;
+  for (int tile = tile0;; ++tile) {
   const int h = bh % H, j0 = blk * kKeys;
   const int nbh = blk + 1 == nblk ? bh + 1 : bh, nblk_ = blk + 1 == nblk ? 0 : blk + 1;
   const bool has_next = RUNS && tile + 1 < tile1, next_new_head = has_next && nbh != bh && H > 1;
-  const unsigned char* Ks = smem + buf * kKeyBytes;
   // ||c_m||^2 (and its maximum) of a head: from the array the kernel ahead of this one filled, or from the staged
   // codebook
   bool codes = true;
@@ -238,10 +237,9 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       atomicMax(cmax_bits, __float_as_uint(s));
     }
   }
-  const bool loaded = mbar_wait(&bar_k[buf], (ph_k >> buf) & 1u, abort_flag, status_word, DEV_TIMEOUT_ASSIGN) && codes;
-  ph_k ^= 1u << buf;
-  if (warp == 0 && loaded && !mma_issued) issue_mma(Ks);   // (all lanes wait for the same barriers and agree)
-  mma_issued = false;
+  const bool loaded = mbar_wait(bar_k, ph_k, abort_flag, status_word, DEV_TIMEOUT_ASSIGN) && codes;
+  ph_k ^= 1;
+  if (warp == 0 && loaded) issue_mma();              // (all lanes wait for the same barriers and agree)
 
   {                                                  // half of ||k||^2 per thread
     float s = 0.f;
@@ -319,15 +317,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   if (warp == 1 && !has_next) tmem_dealloc(tmem_base, tmem_cols);
-  // the products have been read: those of the next tile, if its keys have a buffer of their own, run beside the rest
-  if (nbuf == 2 && has_next && !next_new_head) {
-    if (warp == 0 && mbar_wait(&bar_k[buf ^ 1], (ph_k >> (buf ^ 1)) & 1u, abort_flag, status_word, DEV_TIMEOUT_ASSIGN)) {
-      tc_fence_after();
-      issue_mma(smem + (buf ^ 1) * kKeyBytes);
-    }
-    mma_issued = true;
-  }
-
   const __nv_bfloat16* Cph = Cp + (size_t)h * M * D;
   if (hf == 0) {
     const float s = xs[r] + xs[kKeys + r];           // < 512: a single column, 256 + index
@@ -565,8 +554,7 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   }
   // every thread is past its last read of this key tile (and of the codebook): refill
   if (warp == 0 && has_next && elect_one()) {
-    if (nbuf == 1) load_keys(0, nbh, nblk_);
-    else if (tile + 2 < tile1) load_keys(buf, nblk_ + 1 == nblk ? nbh + 1 : nbh, nblk_ + 1 == nblk ? 0 : nblk_ + 1);
+    load_keys(nbh, nblk_);
     if (next_new_head) {
       *cmax_bits = 0;
       load_codes(nbh);
@@ -590,7 +578,7 @@ uint32_t pow2_cols(int n) {
 template <int D, int NL, bool STAYS, bool RUNS, bool TABLE>
 avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const avq_problem& p, const void* Cp,
                          const void* Cc, int32_t* pidx, int32_t* cidx, int32_t* status_word, void* zero_base,
-                         size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, int nbuf, size_t smem,
+                         size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, size_t smem,
                          unsigned grid, cudaStream_t st) {
   auto kern = tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>;
   const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>>();
@@ -598,7 +586,7 @@ avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const 
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
                             static_cast<const __nv_bfloat16*>(Cp), static_cast<const __nv_bfloat16*>(Cc), pidx, cidx,
-                            p.H, p.Nk, p.M, nblk, total, nbuf, pow2_cols(p.M), status_word,
+                            p.H, p.Nk, p.M, nblk, total, pow2_cols(p.M), status_word,
                             static_cast<uint4*>(zero_base), zero_bytes / 16, slice_units(zero_bytes / 16, grid), cnorm, beside ? 1 : 0));
 }
 
@@ -620,13 +608,8 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
     avq_status s = make_tmap_bf16(&tmCp, Cp, 2, dims, box);
     if (s != AVQ_OK) return s;
   }
-  // Key tiles: two buffers where that does not cost a resident CTA.
-  auto bytes = [&](int nbuf) {
-    return (size_t)(D / 64) * (nbuf * kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys) + 96;
-  };
-  constexpr size_t kSmSmem = 227 * 1024;
-  auto resident = [&](int nbuf) { return (int)min((size_t)assign_min_ctas(D), kSmSmem / (bytes(nbuf) + 1024)); };
-  const uint32_t cols = pow2_cols(p.M);
+  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys) + 96;
+  const int resident = (int)min((size_t)assign_min_ctas(D), kSmemMax / (smem + 1024));   // CTAs on an SM
   int sms = 148;
   {
     static int sm_count[64] = {};
@@ -641,17 +624,13 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   const int nblk = (p.Nk + kKeys - 1) / kKeys;
   if ((uint64_t)nblk * BH > 0x7fffffffull) return AVQ_ERR_UNSUPPORTED;
   const int total = (int)(nblk * BH);
-  // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, pays from four tiles per
-  // CTA on (N16384 H16 d128 M256, 6.9 tiles: 72 -> 63 us); with fewer the uneven last round costs more than the
-  // set-up it saves (B2 H8 N5000 d128, 2.2 tiles: whole call 111 -> 130 us), and where the columns of the resident
-  // CTAs exceed TMEM, so that they take them in turn, it costs too (N65536 d64 M256: whole call 780 -> 960 us).  A
-  // codebook below 64 KB is set up faster than the loop state costs (B8 H12 N10167 d64 M32: this kernel 122 us with
-  // one tile per CTA, 130 with runs and the norm table).
-  const int nbuf2 = resident(2) >= resident(1) ? 2 : 1;
-  const bool shared_cols = (int)cols * resident(1) > 512;
-  const bool runs = !shared_cols && p.M * D >= 32768 && (int64_t)total >= 4ll * resident(nbuf2) * sms;
-  const int nbuf = runs ? nbuf2 : 1;
-  const size_t smem = bytes(nbuf);
+  // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, for the largest codebook
+  // (64 KB: d128 M256) from four tiles per CTA on (N16384 H16, 6.9 tiles: 72 -> 63 us); with fewer the uneven last round
+  // costs more than the set-up it saves (B2 H8 N5000 d128 M96, 2.2 tiles: whole call 111 -> 130 us).  Below M256 the gain
+  // is smaller (H16 N16384 d128 C4, whole call with one tile per CTA and with runs: M64 126 and 123, M128 182 and 178, M224
+  // 229 and 222) and runs are not taken.  At d64 they cost: M32 by their loop state (B8 H12 N10167: this kernel 122 us and
+  // 130), M256 because the resident CTAs take the TMEM columns in turn (N65536: whole call 780 and 960).
+  const bool runs = D == 128 && p.M == 256 && (int64_t)total >= 4ll * resident * sms;
   if (cnorm) {
     const int parents = p.H * p.M, rows = parents * (1 + p.C);
     if (launch_pdl(code_norms_kernel<D>, dim3((rows * 8 + 255) / 256), dim3(256), 0, st, beside,
@@ -659,10 +638,11 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
                    rows) != cudaSuccess)
       return AVQ_ERR_CUDA;
   }
-  auto go = cnorm ? (runs ? launch_kernel<D, NL, STAYS, true, true> : launch_kernel<D, NL, STAYS, false, true>)
-                  : (runs ? launch_kernel<D, NL, STAYS, true, false> : launch_kernel<D, NL, STAYS, false, false>);
-  return go(tmK, tmCp, p, Cp, Cc, pidx, cidx, status_word, zero_base, zero_bytes, cnorm, beside, nblk, total, nbuf, smem,
-            (unsigned)(runs ? resident(nbuf) * sms : total), st);
+  auto go = cnorm ? launch_kernel<D, NL, STAYS, false, true> : launch_kernel<D, NL, STAYS, false, false>;
+  if constexpr (D == 128)
+    if (runs) go = cnorm ? launch_kernel<D, NL, STAYS, true, true> : launch_kernel<D, NL, STAYS, true, false>;
+  return go(tmK, tmCp, p, Cp, Cc, pidx, cidx, status_word, zero_base, zero_bytes, cnorm, beside, nblk, total, smem,
+            (unsigned)(runs ? resident * sms : total), st);
 }
 
 }  // namespace

@@ -19,7 +19,7 @@ EncodeTiledFn encode_tiled_fn() {
 }
 
 namespace {
-// Encoding a tensor map costs a few microseconds of host time and a forward needs seven of them, so
+// Encoding a tensor map costs a few microseconds of host time and a forward needs six of them, so
 // recent encodings are kept: the result depends only on (base, rank, dims, strides, box).
 constexpr int kMaxRank = 4;
 struct TmapKey {
