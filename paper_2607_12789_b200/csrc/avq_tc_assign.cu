@@ -3,7 +3,7 @@
 // One CTA takes a tile of 128 consecutive keys of one (batch, head), or a run of them, 8 warps.  TMA stages each key tile
 // and, once per head, the head's parent codebook in shared memory (K-major, 128-byte swizzle); one elected thread issues the
 // tcgen05 MMA chain  D[128 x M] = K_tile . Cp^T  into TMEM.
-//   parent   warp w holds keys 32 (w % 4) .. +31 of the column half w / 4 and reads the products in the fragment layout
+//   parent   (beyond 64 parents; up to that best, runner-up and index by a key per lane) warp w holds keys 32 (w % 4) .. +31 of the column half w / 4 and reads the products in the fragment layout
 //            (4 keys x column pairs per lane).  Two passes over ||c||^2 - 2 k.c: the minimum of the row; then the
 //            number and the index of the columns within the MMA's rounding of it, added up in one register.  Only
 //            when there is more than one such column are all M distances redone in float64 in the direct form
@@ -88,6 +88,75 @@ __device__ double exact_dist_smem(const unsigned char* Ks, int row, const __nv_b
   return s;
 }
 
+// float64, direct form, by the four lanes (s4) of a key's group: a quarter of the dimensions each
+template <int D>
+__device__ __forceinline__ double exact4(const unsigned char* Ks, int key, int s4, const __nv_bfloat16* c) {
+  double sd = 0.0;
+  for (int u = 0; u < D / 32; ++u)
+    for (int e = 0; e < 8; ++e) {
+      const int col = 8 * (s4 + 4 * u) + e;
+      const double x = (double)key_elem<D>(Ks, key, col) - (double)__bfloat162float(c[col]);
+      sd += x * x;
+    }
+  sd += __shfl_xor_sync(0xffffffffu, sd, 1);
+  return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
+}
+
+// PARENT_STAYS, one warp, four lanes per key: the child of key row `key` (-1: it stays) where norms and products leave open
+// which child is nearest or (stay_open) whether that is closer than the parent.  Measured in the direct form in float32, and
+// what that leaves open (relative 1e-4) in float64.  Keys that hug their parent are about equally far from its children, and
+// products separate little where keys lie far from the origin for their distances: B2 H8 N5000 d128 M96 C8 with 32 added to
+// every dimension, us per call: 190 with float64 straight behind the products, 114 so, 118 in the direct form throughout.  (Keys
+// that moved are close to one child: without PARENT_STAYS such offsets cost nothing.)  Out of line: keys around the origin
+// hardly ever come here, and inlined it took registers from the loop that calls it.
+template <int D, int C>
+__device__ __noinline__ int settle_child(const unsigned char* Ks, int key, int s4, const __nv_bfloat16* Cch,
+                                         const __nv_bfloat16* Cpk, int c1, bool open, bool stay_open, bool moved) {
+  auto direct4 = [&](const __nv_bfloat16* c) {
+    float sd = 0.f;
+#pragma unroll
+    for (int u = 0; u < D / 32; ++u) {
+      const int cu = s4 + 4 * u;
+      sd += sqdiff8(widen8(*reinterpret_cast<const uint4*>(Ks + (cu >> 3) * (kKeys * 128) + sw128_offset(key, (cu & 7) * 8))),
+                    __ldg(reinterpret_cast<const uint4*>(c) + cu));
+    }
+    sd += __shfl_xor_sync(0xffffffffu, sd, 1);
+    return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
+  };
+  if (__any_sync(0xffffffffu, open)) {
+    float f1 = INFINITY, f2 = INFINITY;
+    int fi = 0;
+#pragma unroll 1
+    for (int c = 0; c < C; ++c) {
+      const float sd = direct4(Cch + (size_t)c * D);
+      if (sd < f1) { f2 = f1; f1 = sd; fi = c; }
+      else if (sd < f2) { f2 = sd; }
+    }
+    if (open) c1 = fi;
+    open = open && !(f2 - f1 > 1e-4f * f2);
+    if (__any_sync(0xffffffffu, open)) {
+      double best = INFINITY;
+      int bi = 0;
+#pragma unroll 1
+      for (int c = 0; c < C; ++c) {
+        const double sd = exact4<D>(Ks, key, s4, Cch + (size_t)c * D);
+        if (sd < best) { best = sd; bi = c; }
+      }
+      if (open) c1 = bi;
+    }
+  }
+  if (__any_sync(0xffffffffu, stay_open)) {
+    const float fc = direct4(Cch + (size_t)c1 * D), fp = direct4(Cpk);
+    if (stay_open) moved = fc < fp;
+    stay_open = stay_open && !(fabsf(fc - fp) > 1e-4f * fmaxf(fc, fp));
+    if (__any_sync(0xffffffffu, stay_open)) {
+      const bool closer = exact4<D>(Ks, key, s4, Cch + (size_t)c1 * D) < exact4<D>(Ks, key, s4, Cpk);
+      if (stay_open) moved = closer;
+    }
+  }
+  return moved ? c1 : -1;
+}
+
 // ||c||^2 of every codeword of every head, once per call: parents [H, M], then children [H, M, C].  Eight lanes per
 // codeword row.
 template <int D>
@@ -110,13 +179,15 @@ __global__ void __launch_bounds__(256) code_norms_kernel(const __nv_bfloat16* __
   pdl_wait();                // this grid's completion implies that of the one it ran beside
 }
 
+enum Form { kOne, kRuns, kSmall };
 // NL = 16-byte loads per lane that cover one parent's C x d block of children: C * d / 256.
 // STAYS: Algorithm 1's masked scatter - a key moves to its nearest child only if that child is strictly
 // closer than the parent (child index -1 otherwise).
-// RUNS: a CTA takes a run of tiles (else one: no loop state in registers).
+// FORM: kOne, one tile per CTA; kRuns, a CTA takes a run of tiles (more loop state in registers); kSmall, one tile per CTA and
+// the parents' distances with a key per lane: best, runner-up and index in one pass.
 // TABLE: cnorm_g holds the squared norms of all codewords (parents [H, M], then children [H, M, C]); the child distances
 // are then ||c||^2 - 2 k.c at one mixed-precision multiply-add per element, half the instructions of the direct form.
-template <int D, int NL, bool STAYS, bool RUNS, bool TABLE>
+template <int D, int NL, bool STAYS, Form FORM, bool TABLE>
 __global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D))
 tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmCp,
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
@@ -126,13 +197,14 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   // 1024-byte alignment (swizzle atoms) is requested from the launch, not computed from the pointer, so
   // that the compiler keeps every access in the shared address space.
   extern __shared__ __align__(1024) unsigned char smem[];
+  constexpr bool RUNS = FORM == kRuns;
   constexpr int kSub = D / 64;                       // 64-column sub-tiles along the head dimension
   constexpr int kKeyBytes = kSub * kKeys * 128;
   const unsigned char* Ks = smem;                    // key tile: kSub x [128 x 128 B]
   unsigned char* Cs = smem + kKeyBytes;              // kSub x [M x 128 B]
   float* cnorm = reinterpret_cast<float*>(Cs + kSub * M * 128);   // [M]
   float* xd = cnorm + M;                             // [2][128] smallest distance of each column half
-  float* xs = xd + 2 * kKeys;                        // [2][128] columns close to the minimum: sum of 256 + index
+  float* xs = xd + 2 * kKeys;                        // [2][128] columns close to the minimum: sum of 256 + index (kSmall: runner-up)
   float* xkn = xs + 2 * kKeys;                       // [2][128] halves of ||k||^2
   int* par = reinterpret_cast<int*>(xkn + 2 * kKeys);   // [128] final parent of each key
   int* chi = par + kKeys;                            // [128] final child of each key
@@ -260,6 +332,23 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   // ---- parents: minimum of ||c||^2 - 2 k.c over this warp's half of the columns
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * MH);
   const float* cnh = cnorm + hf * MH;
+  if constexpr (FORM == kSmall) {
+    float d1 = INFINITY, d2 = INFINITY;
+    int i1 = 0;
+    for (int c0 = 0; c0 < MH; c0 += 16) {
+      float dot[16];
+      tmem_ld16(trow + c0, dot);                     // warp-collective: executed by every lane
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        const float dist = fmaf(-2.f, dot[e], cnh[c0 + e]);
+        d2 = fminf(d2, fmaxf(dist, d1));             // runner-up: second smallest so far
+        if (dist < d1) { d1 = dist; i1 = hf * MH + c0 + e; }
+      }
+    }
+    xd[hf * kKeys + r] = d1;
+    xs[hf * kKeys + r] = d2;
+    par[hf * kKeys + r] = i1;                        // (par and chi, adjacent: [2][128])
+  } else {
   const f32x2 minus2 = pack2(-2.f, -2.f);
   float m[4];
 #pragma unroll
@@ -314,14 +403,25 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
   for (int h4 = 0; h4 < 4; ++h4) hits[h4] = quad_sum(hits[h4]);
   xs[hf * kKeys + q * 32 + g + 8 * t4] = pick4(hits, t4);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 1 && !has_next) tmem_dealloc(tmem_base, tmem_cols);
   const __nv_bfloat16* Cph = Cp + (size_t)h * M * D;
   if (hf == 0) {
-    const float s = xs[r] + xs[kKeys + r];           // < 512: a single column, 256 + index
-    int i1 = (s >= 256.f && s < 512.f) ? (int)s - 256 : 0;
-    if (done && j0 + r < Nk && !(s >= 256.f && s < 512.f)) {
+    int i1;
+    bool open;                                       // more than one parent within the MMA's rounding of the nearest
+    if constexpr (FORM == kSmall) {                  // (the lower half holds the lower indices: it wins ties)
+      const float a1 = xd[r], a2 = xs[r], b1 = xd[kKeys + r], b2 = xs[kKeys + r];
+      i1 = b1 < a1 ? chi[r] : par[r];
+      const float close = 2e-4f * (xkn[r] + xkn[kKeys + r] + __uint_as_float(*cmax_bits));
+      open = !(fminf(fmaxf(a1, b1), fminf(a2, b2)) - fminf(a1, b1) > close);
+    } else {
+      const float s = xs[r] + xs[kKeys + r];         // < 512: a single column, 256 + index
+      open = !(s >= 256.f && s < 512.f);
+      i1 = open ? 0 : (int)s - 256;
+    }
+    if (done && j0 + r < Nk && open) {
       double best = INFINITY;
       int bi = 0;
       for (int mm = 0; mm < M; ++mm) {
@@ -449,72 +549,23 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           if constexpr (TABLE) dp = fmaf(-2.f, dp, cnorm[par[key]]);
         }
         if constexpr (TABLE) {
-          // What the products leave open is measured in the direct form in float32, and what that leaves open (relative
-          // 1e-4) in float64; a quarter of the dimensions per lane of the key's group.  (Products alone separate little
-          // where keys lie far from the origin for their distances: B2 H8 N5000 d128 M96 C8 PARENT_STAYS with 32 added to
-          // every dimension, us per call: 190 with float64 straight behind them, 112 so, 118 in the direct form throughout.)
-          auto direct4 = [&](const __nv_bfloat16* c) {
-            float sd = 0.f;
-#pragma unroll
-            for (int u = 0; u < kT; ++u) {
-              const int cu = s4 + 4 * u;
-              sd += sqdiff8(widen8(*reinterpret_cast<const uint4*>(Ks + (cu >> 3) * (kKeys * 128) + sw128_offset(key, (cu & 7) * 8))),
-                            __ldg(reinterpret_cast<const uint4*>(c) + cu));
-            }
-            sd += __shfl_xor_sync(0xffffffffu, sd, 1);
-            return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
-          };
-          auto exact4 = [&](const __nv_bfloat16* c) {
-            double sd = 0.0;
-            for (int u = 0; u < kT; ++u)
-              for (int e = 0; e < 8; ++e) {
-                const int col = 8 * (s4 + 4 * u) + e;
-                const double x = (double)key_elem<D>(Ks, key, col) - (double)__bfloat162float(c[col]);
-                sd += x * x;
-              }
-            sd += __shfl_xor_sync(0xffffffffu, sd, 1);
-            return sd + __shfl_xor_sync(0xffffffffu, sd, 2);
-          };
           const bool live = done && j0 + key < Nk;
+          const bool open = live && !(e2 - e1 > near);   // not decided by the products
           const __nv_bfloat16* Cch = Cc + (head_base + par[key]) * kC * D;
-          bool open = live && !(e2 - e1 > near);         // not decided so far
-          if (__any_sync(0xffffffffu, open)) {
-            float f1 = INFINITY, f2 = INFINITY;
-            int fi = 0;
-#pragma unroll 1
+          if constexpr (STAYS) {                         // strict '<' against the parent distance
+            const bool moved = e1 < dp, stay_open = live && !(fabsf(e1 - dp) > near);
+            if (__any_sync(0xffffffffu, open || stay_open))
+              c1 = settle_child<D, kC>(Ks, key, s4, Cch, Cp + (head_base + par[key]) * D, c1, open, stay_open, moved);
+            else if (!moved)
+              c1 = -1;
+          } else if (__any_sync(0xffffffffu, open)) {
+            double best = INFINITY;
+            int bi = 0;
             for (int c = 0; c < kC; ++c) {
-              const float sd = direct4(Cch + (size_t)c * D);
-              if (sd < f1) { f2 = f1; f1 = sd; fi = c; }
-              else if (sd < f2) { f2 = sd; }
+              const double sd = exact4<D>(Ks, key, s4, Cch + (size_t)c * D);
+              if (sd < best) { best = sd; bi = c; }
             }
-            if (open) c1 = fi;
-            open = open && !(f2 - f1 > 1e-4f * f2);
-            if (__any_sync(0xffffffffu, open)) {
-              double best = INFINITY;
-              int bi = 0;
-#pragma unroll 1
-              for (int c = 0; c < kC; ++c) {
-                const double sd = exact4(Cch + (size_t)c * D);
-                if (sd < best) { best = sd; bi = c; }
-              }
-              if (open) c1 = bi;
-            }
-          }
-          if constexpr (STAYS) {
-            // strict '<' against the parent distance, decided the same way
-            bool moved = e1 < dp;
-            open = live && !(fabsf(e1 - dp) > near);
-            if (__any_sync(0xffffffffu, open)) {
-              const __nv_bfloat16* Cpk = Cp + (head_base + par[key]) * D;
-              const float fc = direct4(Cch + (size_t)c1 * D), fp = direct4(Cpk);
-              if (open) moved = fc < fp;
-              open = open && !(fabsf(fc - fp) > 1e-4f * fmaxf(fc, fp));
-              if (__any_sync(0xffffffffu, open)) {
-                const bool closer = exact4(Cch + (size_t)c1 * D) < exact4(Cpk);
-                if (open) moved = closer;
-              }
-            }
-            if (!moved) c1 = -1;
+            if (open) c1 = bi;
           }
           if (s4 == 0) chi[key] = c1;
         } else if (s4 == 0) {
@@ -575,13 +626,13 @@ uint32_t pow2_cols(int n) {
   return c;
 }
 
-template <int D, int NL, bool STAYS, bool RUNS, bool TABLE>
+template <int D, int NL, bool STAYS, Form FORM, bool TABLE>
 avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const avq_problem& p, const void* Cp,
                          const void* Cc, int32_t* pidx, int32_t* cidx, int32_t* status_word, void* zero_base,
                          size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, size_t smem,
                          unsigned grid, cudaStream_t st) {
-  auto kern = tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>;
-  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, RUNS, TABLE>>();
+  auto kern = tc_assign_kernel<D, NL, STAYS, FORM, TABLE>;
+  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, FORM, TABLE>>();
   if (s != AVQ_OK) return s;
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
@@ -638,9 +689,16 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
                    rows) != cudaSuccess)
       return AVQ_ERR_CUDA;
   }
-  auto go = cnorm ? launch_kernel<D, NL, STAYS, false, true> : launch_kernel<D, NL, STAYS, false, false>;
+  // Up to 64 parents the fragment layout's exchanges cost more than its cheaper columns save (this kernel alone, us, fragments
+  // and a key per lane: H16 d64 C4 N65536 M32 97.8 and 95.2, M64 106.2 and 104.5; d128 N16384 M32 54.0 and 51.9, M64 56.0 and
+  // 54.6; beyond, in the form the kernel had with a key per lane throughout: d64 M128 118.5 and 120.8, M256 151 and 166).
+  // With the norm table at d64 the loop behind has no registers to spare (whole call N65536 M64 C8: 301.7 and 304.5).
+  const bool small = p.M <= 64 && !(D == 64 && cnorm);
+  constexpr Form kSmallTable = D == 64 ? kOne : kSmall;
+  auto go = cnorm ? (small ? launch_kernel<D, NL, STAYS, kSmallTable, true> : launch_kernel<D, NL, STAYS, kOne, true>)
+                  : (small ? launch_kernel<D, NL, STAYS, kSmall, false> : launch_kernel<D, NL, STAYS, kOne, false>);
   if constexpr (D == 128)
-    if (runs) go = cnorm ? launch_kernel<D, NL, STAYS, true, true> : launch_kernel<D, NL, STAYS, true, false>;
+    if (runs) go = cnorm ? launch_kernel<D, NL, STAYS, kRuns, true> : launch_kernel<D, NL, STAYS, kRuns, false>;
   return go(tmK, tmCp, p, Cp, Cc, pidx, cidx, status_word, zero_base, zero_bytes, cnorm, beside, nblk, total, smem,
             (unsigned)(runs ? resident * sms : total), st);
 }
