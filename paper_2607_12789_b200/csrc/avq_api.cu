@@ -189,8 +189,11 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
     // 148 SMs) the two about cancel or it pays; us per call without and with it: d64 M64 C4 192 tiles 22.9 and 24.5, 768 43.4
     // and 43.6, 1536 70.3 and 69.7; d64 M128 C8 192 tiles 29.1 and 29.7, 1024 68.9 and 68.9; d128 M256 C4 592 tiles 98.9 and
     // 97.5, 1536 256.8 and 253.4; d128 M96 C8 1536 tiles 200.1 and 201.6.  A 4 KB codebook is too small for it (B8 H12
-    // N10167 d64 M32 C8: 270 and 276).
-    const bool norms_pass = (size_t)p.M * p.d >= 4096 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592;
+    // N10167 d64 M32 C8: 270 and 276), and so are keys that do not outnumber the codewords of a head (its batch together)
+    // four to one: H96 N1024, ratio 0.9: d128 M128 C8 121.5 and 126.3; 1.8: d64 M64 C8 50.5 and 52.5; 3.2: d64 M64 C4
+    // 44.2 and 44.4; ratio 14: H16 N16384 d64 M128 C8 128.7 and 126.9.
+    const bool norms_pass = (size_t)p.M * p.d >= 4096 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592 &&
+                            (size_t)p.B * p.Nk >= 4 * (size_t)p.M * (1 + p.C);
     s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);
     if (s != AVQ_OK) return s;
     s = tc_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, r.Vpb, r.Vcb, r.Vsb, r.rho, true, false, r.status_word, st);
