@@ -21,7 +21,7 @@
 //             O = (A n) . mean_p           tcgen05.mma
 //   children  of the selected parents, in chunks of <= CHW columns: gathered codeword rows,
 //             S_c = Q . Cc_sel^T, bf16 weights, O += A_c . Vbar_c   (Algorithm 2, child loop); O is rescaled in
-//             TMEM only if the children's weights against the row's reference pass 2^64
+//             TMEM only if the children's weights against the row's reference pass 2^64 (2^8 where a mean exceeds 2^40)
 //   Y = O / z, z accumulated from the same bf16-rounded weights as the numerator.
 // Empty codewords are excluded from every maximum and contribute nothing (their logit is -inf, their count and
 // value sum are zero) - appendix on numerical stability.
@@ -79,7 +79,7 @@ __device__ __forceinline__ void row_sync(int q) {
 // Shared-memory and TMEM plan of one instantiation.
 // NQ = warps (column slices) per 32 query rows: 1, 2 or 4.  Small tiles take NQ = 1 so that four CTAs share an SM and
 // overlap each other's load / MMA / softmax phases; the largest take NQ = 4.
-// CT = parent tile width (64, 128 or 256, >= M), a compile-time constant so that every shared-memory
+// CT = parent tile width (32, 64, 128 or 256, >= M), a compile-time constant so that every shared-memory
 // offset folds into the instruction stream instead of occupying a register.
 template <int D, int NQ, int CT>
 struct Plan {
@@ -88,36 +88,37 @@ struct Plan {
   static constexpr int CHW = CT < 128 ? CT : 128;        // child chunk width
   static constexpr int QT = kSubD * kRows * 128;         // bytes of a query / output tile
   // Weights as the A operand in TMEM: nothing to swizzle or fence, the MMA reads half the shared memory, and the
-  // codebook survives the tile.  The smallest tile has no TMEM columns left (four CTAs of 128 columns share an
-  // SM): its weights overwrite the codebook in shared memory, which is then loaded again (8 KB).
+  // codebook survives the tile.  64 parents with one warp per row have no TMEM columns left (four CTAs of 128 columns share
+  // an SM): their weights overwrite the codebook in shared memory, which is then loaded again (8 KB).
   static constexpr bool kTW = !(CT == 64 && D == 64 && NQ == 1);
   // The children's codes and value rows have a buffer each, so that both gathers run ahead of the logits.  The largest
   // tile has room for the values only: the codes go over the parent codebook, whose logits are done by then, and the
-  // overwritten half of the codebook is loaded again behind the child logits.  The smallest gathers the values into
-  // the codes' place once the child logits are done (four CTAs fill each other's gaps).
+  // overwritten half of the codebook is loaded again behind the child logits.  The tile without weights in TMEM gathers
+  // the values into the codes' place once the child logits are done (four CTAs fill each other's gaps).
   static constexpr bool kCodesInCA = CT == 256 && D == 128;
   static constexpr bool kSepCV = kTW;
-  // The output tile is staged in the child buffers where they are as large as a query tile, else across the
-  // parent values and the child buffer (the parent values are then loaded again).
+  // The output tile is staged in the child buffers, padded to its size where needed, or, without buffers for both, across
+  // the parent values and the child buffer (the parent values are then loaded again).
   static constexpr bool kStageInCC = CT >= 128 || kSepCV;
+  static constexpr int child_bytes = CHW * D * 2 * (kSepCV && !kCodesInCA ? 2 : 1);
+  static constexpr int stage_pad = kStageInCC && child_bytes < QT ? QT - child_bytes : 0;   // (32 parents only)
   static constexpr int cp_bytes = CT * D * 2;
   static constexpr int ca_bytes = kTW ? cp_bytes : (cp_bytes > kRows * CT * 2 ? cp_bytes : kRows * CT * 2);
   static constexpr int oQ = 0, oCA = QT, oV = oCA + ca_bytes, oCC = oV + CT * D * 2,
                        oCV = oCC + (kSepCV && !kCodesInCA ? CHW * D * 2 : 0);
   static constexpr int oStage = kStageInCC ? oCC : oV;
-  static constexpr int oF = oCV + CHW * D * 2;           // fp32 / word arrays from here
+  static constexpr int oF = oCV + CHW * D * 2 + stage_pad;   // fp32 / word arrays from here
   // Plans of twice the warps per tile (small grids): two neighbouring warps of a row add the denominator as the one warp of
   // the other plan does, the second going on from the first's sums, so that which parents are selected does not depend on
   // how many tiles a call has.
-  static constexpr bool kChain = D == 64 && CT / NQ == 32;
+  static constexpr bool kChain = D == 64 && NQ > 1 && CT / NQ == 32;
   static constexpr int chain_floats = kChain ? NQ / 2 * 4 * kRows : 0;
   // TMEM columns: logits, weights (kTW), output.  With 256 logit columns the child logits use half of them and the
   // children's weights go into the other half, so they need not wait for the parents' value MMA.
   static constexpr bool kSepW = CT == 256;
-  static constexpr int tW = kTW ? CT : 0, tWc = kSepW ? 128 : tW, tO = kTW ? CT + CT / 2 : CT;
+  static constexpr int tW = kTW ? CT : 0, tWc = kSepW ? 128 : tW, tO = CT == 32 ? 64 : (kTW ? CT + CT / 2 : CT);
   static constexpr int tmem_used = tO + D;
   static constexpr uint32_t tmem_cols = tmem_used <= 128 ? 128 : (tmem_used <= 256 ? 256 : 512);
-  static_assert(CHW * D * 2 * (kSepCV && !kCodesInCA ? 2 : 1) >= QT || !kStageInCC, "the output tile fits its staging area");
   static_assert(kStageInCC || CT * D * 2 + CHW * D * 2 >= QT, "the output tile fits its staging area");
 };
 
@@ -340,7 +341,16 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const bool next_new_bh = has_next && nbh != bh;
     const bool next_new_head = next_new_bh && p.H > 1;
     const bool next_new_cp = has_next && (!kTW || next_new_head || (L::kCodesInCA && PC > 0));
-    // V of this tile: loaded behind the last use of the one before (below), except for the first tile
+    // V of this tile: loaded behind the last use of the one before (below), except for the first tile.  Where its place is the
+    // staging area: as soon as the store of the tile before has read that.  (Only ahead of the gather, where the other
+    // plans wait for their stores, nothing covered the load: N65536 H16 d64 M64 P0 attend 81.7 -> 75.3 us.)
+    if (!L::kStageInCC && warp == 0 && store_pending) {
+      if (elect_one()) {
+        tma_store_wait_read();
+        issue_v(bh);
+      }
+      store_pending = false;
+    }
     const bool new_v = STAYS || !L::kStageInCC || new_bh || wide;
 
     if (new_bh) {
@@ -639,10 +649,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     // the output tile of the tile before must have left its staging area before that is refilled (its store was
     // issued a whole parent pass ago, so this does not wait in practice)
     if (warp == 0 && store_pending) {
-      if (elect_one()) {
-        tma_store_wait_read();
-        if (!L::kStageInCC) issue_v(bh);                 // this tile's values: their buffer was the staging area
-      }
+      if (elect_one()) tma_store_wait_read();
       store_pending = false;
     }
     __syncthreads();
@@ -652,15 +659,15 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const __nv_bfloat16* Cch = p.Cc + (size_t)(bh % p.H) * M * C * D;
     const __nv_bfloat16* Vch = p.Vcb + (size_t)bh * M * C * D;
     int ncols = min(PC, CHW);
-    int np32 = (ncols + 31) & ~31;
-    // Rows of a chunk, gathered into a row-per-codeword tile of np32 rows (kSubD sub-tiles of 64 columns): local
+    int np16 = (ncols + 15) & ~15;
+    // Rows of a chunk, gathered into a row-per-codeword tile of np16 rows (kSubD sub-tiles of 64 columns): local
     // row e = src[sel_list[(e_first+e)/C] * C + (e_first+e)%C, :]; padding rows are zero.  A thread keeps its
     // 16-byte chunk column and walks down the rows (kThreads is a multiple of the chunks per row).
     auto gather_rows = [&](unsigned char* dst_tile, const __nv_bfloat16* src, int e_first) {
       constexpr int kRowsPerPass = kThreads >> kLogChunks;   // a multiple of 8: a thread's swizzle phase is fixed
       constexpr int kPasses = (CHW + kRowsPerPass - 1) / kRowsPerPass;
       const int ch = tid & ((1 << kLogChunks) - 1), row0 = tid >> kLogChunks;
-      const uint32_t dst0 = smem_u32(dst_tile) + (uint32_t)((ch >> 3) * (np32 * 128)) + sw128_offset(row0, (ch & 7) * 8);
+      const uint32_t dst0 = smem_u32(dst_tile) + (uint32_t)((ch >> 3) * (np16 * 128)) + sw128_offset(row0, (ch & 7) * 8);
       const __nv_bfloat16* src_col = src + ch * 8;
       int sel[kPasses];
 #pragma unroll
@@ -676,7 +683,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           const int e = e_first + row;
           const uint32_t off = (uint32_t)(((sel[it] << logC) + (e & (C - 1))) << kLogD);   // elements: < 2^31
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src_col + off) : "memory");
-        } else if (row < np32) {
+        } else if (row < np16) {
           asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
         }
       }
@@ -756,7 +763,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       else asm volatile("bar.arrive 5, 64;" ::: "memory");
     };
     if (warp == 0 && PC > 0) {
-      issue_sc(np32);
+      issue_sc(np16);
       pair_barrier(false);
     }
     if (kSepCV && PC > 0) gather_rows(CV, Vch, 0);         // while the logits are computed
@@ -783,7 +790,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       else if (e0 > 0) gather_rows(CV, Vch, e0);
       tc_fence_after();
       bool o_done = L::kSepW || e0 > 0;                    // the weights' columns are free
-      const int my_c = min(max(np32 - cq * QWC, 0), QWC);  // multiple of 32
+      const int my_c = min(max(np16 - cq * QWC, 0), QWC);  // multiple of 16
       float zc[4];
       for (;;) {
         // bf16 weights exp2(s - m + log2 n) of the children, their sum
@@ -801,10 +808,15 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             for (int b = 0; b < 4; ++b) ln[b] = *reinterpret_cast<const f32x2*>(l2n + cq * QWC + 32 * c + 8 * b + 2 * t4);
             tmem_ld_wait_frag<4>(s);
             uint32_t pk[4][4];
+            const bool whole = 32 * c + 16 < my_c;         // else the last 16 columns are not there (no logits, weight zero)
 #pragma unroll
             for (int b = 0; b < 4; ++b)
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
+                if (b >= 2 && !whole) {
+                  pk[b][h] = 0u;
+                  continue;
+                }
                 const f32x2 x = pack2u(s[h >> 1][4 * b + 2 * (h & 1)], s[h >> 1][4 * b + 2 * (h & 1) + 1]);
                 float lo, hi;
                 unpack2(add2(fma2(x, sc2, nm[h]), ln[b]), lo, hi);
@@ -885,17 +897,17 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       for (int h = 0; h < 4; ++h) z_run[h] += zc[h];
 
       // ---- O += A_c . Vbar_c
-      if (warp == kVWarp) issue_o(kSepCV ? CV : CC, np32, L::tWc, true, bar_pv);
+      if (warp == kVWarp) issue_o(kSepCV ? CV : CC, np16, L::tWc, true, bar_pv);
       if (!last) {
         ncols = min(PC - e0 - CHW, CHW);
-        np32 = (ncols + 31) & ~31;
+        np16 = (ncols + 15) & ~15;
         if constexpr (!kSepCV) mbar_wait(bar_pv, ph_pv, abort_flag, p.status_word, DEV_TIMEOUT_ATTEND);   // values have left CC
         gather_codes(e0 + CHW);
         cp_async_wait_all();
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
-        if (warp == 0) issue_sc(np32);
+        if (warp == 0) issue_sc(np16);
       }
     }
 
@@ -1067,6 +1079,9 @@ avq_status launch(const avq_problem& p, const void* Q, const void* Cp, const voi
     return AVQ_ERR_CUDA;
   if constexpr (D == 64) {
     if (CT == 64 && a.total_tiles <= 2 * sms) return launch_nq<D, 2, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
+    // (in the 64-parent plan such calls load the codebook again for every tile and wait for their children's values: H16 C4
+    // N65536 attend P0 77.4 -> 53.1 us, P4 115 -> 88; N16384 P4 34.0 -> 27.9)
+    if (p.M == 32) return launch_nq<D, 1, 32>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
     if (CT == 128 && a.total_tiles <= sms) return launch_nq<D, 4, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
     if (CT == 64) return launch_nq<D, 1, 64>(tmQ, tmCp, tmVpb, tmY, a, chained, st);
     if (CT == 128) return launch_nq<D, 2, 128>(tmQ, tmCp, tmVpb, tmY, a, chained, st);

@@ -61,7 +61,7 @@ def test_out_of_range_entries_are_skipped_and_reported():
     assert (Y[:, :, 7] == 0).all() and (Y[:, :, 300] == 0).all()  # the rows nothing was scattered to stay as they were
 
 
-@pytest.mark.parametrize("B,H,N,d,M,C,P", [(8, 12, 1100, 64, 64, 4, 8), (2, 16, 1500, 64, 128, 8, 16),
+@pytest.mark.parametrize("B,H,N,d,M,C,P", [(8, 12, 1100, 64, 64, 4, 8), (6, 16, 1100, 64, 32, 8, 9), (2, 16, 1500, 64, 128, 8, 16),
                                            (2, 8, 2500, 128, 256, 4, 32), (4, 10, 1111, 128, 64, 8, 5)])
 def test_rows_written_to_their_places_over_chained_tiles(B, H, N, d, M, C, P):
     """More query tiles than one wave of CTAs, so that output rows leave the staging area of every plan while the next
@@ -78,7 +78,7 @@ def test_rows_written_to_their_places_over_chained_tiles(B, H, N, d, M, C, P):
     assert diff.max().item() <= 1.6e-2 and diff.mean().item() <= 1e-4
 
 
-@pytest.mark.parametrize("B,H,N,d,M,C,P", [(1, 2, 500, 64, 64, 4, 8), (8, 12, 1100, 64, 64, 4, 8), (1, 2, 500, 64, 128, 8, 16),
+@pytest.mark.parametrize("B,H,N,d,M,C,P", [(1, 2, 500, 64, 64, 4, 8), (8, 12, 1100, 64, 64, 4, 8), (6, 16, 1100, 64, 32, 4, 8), (1, 2, 500, 64, 128, 8, 16),
                                            (1, 2, 500, 128, 96, 8, 12), (2, 8, 2500, 128, 256, 4, 32), (4, 10, 1111, 128, 64, 8, 5)])
 def test_keys_that_stay_with_their_parent_under_a_token_order(B, H, N, d, M, C, P):
     """The PARENT_STAYS rule with output rows written to their places, one tile per CTA and chained tiles: equal to the plain

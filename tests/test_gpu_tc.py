@@ -210,6 +210,20 @@ def test_random_shapes_full_parity(wl):
     parity.full_parity(wl)
 
 
+@pytest.mark.parametrize("C,P", [(4, 4), (4, 17), (8, 32)])
+@pytest.mark.parametrize("flags", [0, binding.FLAG_PARENT_STAYS])
+def test_smallest_codebook_over_chained_tiles(C, P, flags):
+    """32 parents with more tiles than small grids have: one child chunk of 16 columns, several chunks with a ragged last
+    one, every parent refined; more tiles than CTAs, and children that move the reference."""
+    wl = synth.Workload("m32", B=3, H=16, N=1700, d=64, M=32, C=C, P=P, block_q=128, seed=58 + C + P, alpha=0.6,
+                        hot_queries=True, sigma_c=0.5 if P < 32 else 20.0)
+    x = synth.generate(wl)
+    if flags:                                                     # every other key hugs a parent: it stays
+        x["K"][:, :, ::2] = synth.round_to_bf16(x["Cp"][np.arange(16)[None, :, None], np.arange(0, 1700, 2)[None, None] % 32]
+                                                + np.float32(0.03))
+    parity.full_parity(wl, flags=flags, parent_stays=bool(flags), x=x)
+
+
 def test_long_ragged_head_uses_chunked_aggregate_end_to_end():
     """A ragged long head over few leaves (the chunked aggregate inside avq_forward), sampled against the oracle."""
     wl = synth.sweep_point(16384, 32, 4).with_(H=2, N=16384 + 77, name="ragged_long")
@@ -330,7 +344,7 @@ def test_an_infinite_value_stays_in_its_dimension():
     assert np.abs(Y[..., rest] - ref[..., rest]).max() <= 1.6e-2   # (a mean next to a rounding boundary: an ulp of bf16)
 
 
-@pytest.mark.parametrize("M,C,P", [(32, 4, 4), (64, 4, 8), (96, 8, 12), (128, 4, 16)])
+@pytest.mark.parametrize("M,C,P", [(32, 4, 4), (32, 8, 9), (64, 4, 8), (96, 8, 12), (128, 4, 16)])
 def test_selection_of_a_head_does_not_depend_on_the_rest_of_the_call(M, C, P):
     """One image alone (a grid that leaves the chip idle takes twice the warps per tile) and the same image in a batch:
     the importances agree to the last bit, and so do the selections."""
