@@ -351,7 +351,7 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
       store_pending = false;
     }
-    const bool new_v = STAYS || !L::kStageInCC || new_bh || wide;
+    const bool new_v = STAYS || !L::kStageInCC || (new_bh | (wide != 0));   // (one load, waited for where it is used)
 
     if (new_bh) {
       // ---- Part 2 reads what the earlier kernels of this call wrote: status word, counts, value means.  (Loaded
@@ -792,6 +792,9 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       bool o_done = L::kSepW || e0 > 0;                    // the weights' columns are free
       const int my_c = min(max(np16 - cq * QWC, 0), QWC);  // multiple of 16
       float zc[4];
+      // Largest partial sum of the children's weights before the reference moves: 2^64 while no mean exceeds 2^40 (the sums
+      // stay below 2^115 then), 2^8 with values beyond that.
+      const float largest = wide ? 256.f : 1.8446744e19f;
       for (;;) {
         // bf16 weights exp2(s - m + log2 n) of the children, their sum
         const f32x2 sc2 = pack2(sc, sc);
@@ -833,8 +836,6 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // Any reference value works as long as numerator and denominator share it: the parents' maximum is kept
         // unless the children's weights grow so large against it that fp32 sums could overflow.  That is found out
         // at the barrier that publishes the weights; the rare case goes round the loop once more.
-        // 2^64 while no mean exceeds 2^40 (the sums stay below 2^115 then), 2^8 with values beyond that.
-        const float largest = wide ? 256.f : 1.8446744e19f;
         weights_done();
         if (!__syncthreads_or(fmaxf(fmaxf(zc[0], zc[1]), fmaxf(zc[2], zc[3])) > largest)) break;
         // ---- row maxima of the chunk (non-empty children); where they exceed the reference it moves up and O and z
