@@ -27,7 +27,8 @@
 // value sum are zero) - appendix on numerical stability.
 // A CTA takes a run of consecutive tiles: codebook, parent values and counts stay in shared memory while the
 // (batch, head) does not change.
-// Bound by issue slots and by the latency of a tile's phases one after the other, not by the tensor cores.  Against one
+// Bound by the latency of a tile's phases one after the other (issue slots about half used, tensor pipe 7 to 17 %, no
+// memory above a third), not by the tensor cores.  Against one
 // row per lane with the weights in shared memory: B1 H16 N16384 d128 M256 C4 P32 183 -> 148 us (floor 31.5, tensor),
 // N65536 d64 M256 P64 827 -> 615, B2 H16 N4096 d64 M128 C8 P16 43.5 -> 37.
 #include "avq_tc_common.cuh"
