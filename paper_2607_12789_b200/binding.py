@@ -181,10 +181,11 @@ class Forward:
         _chk(Q, K, V, Cp, Cc)
         if Y is None:
             Y = torch.empty(self.shape_y, dtype=self.dtype, device=Q.device)
-        # (addresses as plain integers, which the argument types convert: no object is made for each)
-        st = lib().avq_forward(ctypes.byref(self.prob), Q.data_ptr(), K.data_ptr(), V.data_ptr(), Cp.data_ptr(),
-                               Cc.data_ptr(), self.P, self.block_q, Y.data_ptr(), _ptr(self.topp), _ptr(self.importance),
-                               self.workspace.data_ptr(), self.workspace.numel(), _raw_stream())
+        # (addresses as plain integers and the problem itself, which the argument types convert: no object is made for each)
+        st = (_lib or lib()).avq_forward(self.prob, Q.data_ptr(), K.data_ptr(), V.data_ptr(), Cp.data_ptr(),
+                                         Cc.data_ptr(), self.P, self.block_q, Y.data_ptr(), _ptr(self.topp),
+                                         _ptr(self.importance), self.workspace.data_ptr(), self.workspace.numel(),
+                                         _raw_stream())
         if st != 0:
             raise AvqError(st, "avq_forward")
         return Y
@@ -194,9 +195,9 @@ class Forward:
         _chk(Q, Cp, Cc)
         if Y is None:
             Y = torch.empty(self.shape_y, dtype=self.dtype, device=Q.device)
-        st = lib().avq_attend(ctypes.byref(self.prob), Q.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), self.P, self.block_q,
-                              Y.data_ptr(), _ptr(self.topp), _ptr(self.importance), self.workspace.data_ptr(),
-                              self.workspace.numel(), _raw_stream())
+        st = (_lib or lib()).avq_attend(self.prob, Q.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), self.P, self.block_q,
+                                        Y.data_ptr(), _ptr(self.topp), _ptr(self.importance), self.workspace.data_ptr(),
+                                        self.workspace.numel(), _raw_stream())
         if st != 0:
             raise AvqError(st, "avq_attend")
         return Y

@@ -97,10 +97,8 @@ constexpr size_t kSmemMax = 227 * 1024;
 // Opens all of a CTA's shared memory to a kernel, once per device.  (The attribute is the kernel's, not the launch's: were
 // it set to what a launch needs, a thread with a small problem could take it from one about to launch a large one.)
 template <auto Kernel>
-avq_status open_shared_memory() {
+avq_status open_shared_memory(int dev) {                  // dev: the current device
   static std::atomic<bool> done[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
   const bool known = dev >= 0 && dev < 64;
   if (known && done[dev].load(std::memory_order_acquire)) return AVQ_OK;
   cudaFuncAttributes fa;

@@ -1022,7 +1022,9 @@ avq_status launch_assign(const avq_problem& p, const void* K, const void* Cp, co
                          int32_t* pidx, int32_t* cidx, void* zero_base, size_t zero_bytes, cudaStream_t st) {
   const size_t smem = sizeof(float) * assign_smem_floats(p.d, std::is_same<T, __nv_bfloat16>::value);
   auto kern = assign_simt_kernel<T>;
-  const avq_status s = open_shared_memory<assign_simt_kernel<T>>();
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  const avq_status s = open_shared_memory<assign_simt_kernel<T>>(dev);
   if (s != AVQ_OK) return s;
   dim3 grid((p.Nk + kAssignKeys - 1) / kAssignKeys, p.B * p.H);
   kern<<<grid, kThreads, smem, st>>>(static_cast<const T*>(K), static_cast<const T*>(Cp),
@@ -1063,8 +1065,8 @@ avq_status launch_attend_rdc(AttendArgs a, int B, bool chained, cudaStream_t st)
   constexpr bool kHasWide = !kMma || (DT == 1 && !CORR);
   const bool wide = kHasWide && one_wave;
   auto kern = wide ? attend_simt_kernel<T, RT, DT, CORR, kHasWide> : attend_simt_kernel<T, RT, DT, CORR, false>;
-  const avq_status s = wide ? open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, kHasWide>>()
-                            : open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, false>>();
+  const avq_status s = wide ? open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, kHasWide>>(dev)
+                            : open_shared_memory<attend_simt_kernel<T, RT, DT, CORR, false>>(dev);
   if (s != AVQ_OK) return s;
   return cuda_ok(tc::launch_pdl(kern, dim3(a.nblk, B * a.H), dim3(kAttThreads), smem, st, chained, a));
 }

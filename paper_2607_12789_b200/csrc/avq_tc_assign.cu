@@ -634,7 +634,9 @@ avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const 
                          size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, size_t smem,
                          unsigned grid, cudaStream_t st) {
   auto kern = tc_assign_kernel<D, NL, STAYS, FORM, TABLE>;
-  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, FORM, TABLE>>();
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, FORM, TABLE>>(dev);
   if (s != AVQ_OK) return s;
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,

@@ -1005,12 +1005,12 @@ avq_status launch_plan(const CUtensorMap& tmQ, const CUtensorMap& tmCp, const CU
                        const CUtensorMap& tmY, const AttendParams& a, bool chained, cudaStream_t st) {
   auto kern = tc_attend_kernel<D, NQ, CT, STAYS, PERM>;
   const size_t smem = attend_smem<D, NQ, CT>(a.M * a.C);
-  const avq_status s = open_shared_memory<tc_attend_kernel<D, NQ, CT, STAYS, PERM>>();
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
+  const avq_status s = open_shared_memory<tc_attend_kernel<D, NQ, CT, STAYS, PERM>>(dev);
   if (s != AVQ_OK) return s;
   // Grid: one wave of CTAs (4 / NQ per SM), each taking an equal run of tiles.
   static int sm_count[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
   int sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
   if (sms <= 0) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AVQ_ERR_CUDA;
