@@ -250,6 +250,8 @@ avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void*
   if (s != AVQ_OK) return s;
   s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
   if (s != AVQ_OK) return s;
+  if (tc_tiled_fits(p, P, block_q, tile_m))
+    return tc_attend_tiled(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, r.status_word, st);
   return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, true, st);
 }
 

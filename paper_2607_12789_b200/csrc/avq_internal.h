@@ -91,6 +91,13 @@ avq_status tc_attend(const avq_problem& p, const void* Q, const void* Cp, const 
                      bool chained, const int32_t* perm, cudaStream_t st);   // chained: launched right behind tc_aggregate;
                                                          // perm: see forward_core
 
+// The attention pass of avq_forward_tiled on the tensor cores, launched right behind simt_aggregate: whether it takes the
+// problem, and the call.
+bool tc_tiled_fits(const avq_problem& p, int32_t P, int32_t block_q, int32_t tile_m);
+avq_status tc_attend_tiled(const avq_problem& p, const void* Q, const void* Cp, const void* Cc, const float* Vp, const float* np_,
+                           const float* Vc, const float* nc, int32_t P, int32_t block_q, void* Y, int32_t* topp_out,
+                           float* importance_out, int32_t tile_m, int32_t* status_word, cudaStream_t st);
+
 // Most shared memory, dynamic and static together, of a CTA on sm_100.
 constexpr size_t kSmemMax = 227 * 1024;
 

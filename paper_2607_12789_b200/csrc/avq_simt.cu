@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "avq_internal.h"
+#include "avq_select.cuh"
 #include "avq_tc_common.cuh"
 
 namespace avq {
@@ -520,7 +521,7 @@ struct AttendArgs {
 // A running maximum starts at the lowest finite value: while every logit seen is -inf (a product beyond fp32's range) the
 // weights are then exp(-inf) = 0, not exp(-inf + inf).
 constexpr float kLowest = -3.402823466e38f;
-constexpr int kAttThreads = 512;   // 32 x 16: thread (ty, tx) owns rows ty*RT .. , columns tx*4
+constexpr int kAttThreads = kSelThreads;   // 32 x 16: thread (ty, tx) owns rows ty*RT .. , columns tx*4
 
 // Shared memory of attend_simt_kernel, in floats from the base (doubles first).  All of it is dynamic: the limits the
 // launcher compares it with are those of a CTA's dynamic and static memory together.
@@ -784,73 +785,10 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   }
   __syncthreads();
 
-  // ---- top-P (ties -> lower index), then an ascending list.  Non-negative doubles order like their bit patterns.
-  if (P > 0) {
-    // Only candidates are ranked, those at or above a bound that at least P keys reach: the largest of 32 sample keys
-    // that has P keys at or above it.  (Ranking all of them took 16 of 230 us at M = 512.)
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(w);
-    if (P >= M) {
-      for (int j = tid; j < M; j += kThreads) sel[j] = 1;
-    } else {
-      unsigned long long bound = 0;
-      {
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const unsigned long long smp = key[(2 * warp + e) * M / 32];
-          int c = 0;
-          for (int j = lane; j < M; j += 32) c += key[j] >= smp;
-          c = __reduce_add_sync(0xffffffffu, c);
-          if (lane == 0) s_count[2 * warp + e] = c;
-        }
-        if (tid == 0) *s_ncand = 0;
-        __syncthreads();
-        if (s_count[lane] >= P) bound = key[lane * M / 32];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, bound, o);
-          bound = other > bound ? other : bound;
-        }
-      }
-      for (int j = tid; j < M; j += kThreads)
-        if (key[j] >= bound) cand[atomicAdd(s_ncand, 1)] = j;   // in any order
-      __syncthreads();
-      const int nc_ = *s_ncand;
-      int lt = 0;                                         // 2^lt threads share a candidate's scan
-      while (lt < 4 && (nc_ << (lt + 1)) <= kThreads) ++lt;
-      const int part = tid & ((1 << lt) - 1);
-      for (int i0_ = 0; i0_ < nc_; i0_ += kThreads >> lt) {   // uniform
-        const int i = i0_ + (tid >> lt);
-        const int j = i < nc_ ? cand[i] : 0;
-        const unsigned long long kj = key[j];
-        int rank = 0;
-        if (i < nc_) {
-#pragma unroll 4
-          for (int q = part; q < nc_; q += 1 << lt) {
-            const int k = cand[q];
-            const unsigned long long kk = key[k];
-            rank += (kk > kj) | ((kk == kj) & (k < j));
-          }
-        }
-        for (int o = 1; o < (1 << lt); o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-        if (i < nc_ && part == 0 && rank < P) sel[j] = 1;
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      int base = 0;
-      for (int j = lane; j < ((M + 31) & ~31); j += 32) {
-        const bool on = j < M && sel[j] != 0;
-        const uint32_t bal = __ballot_sync(0xffffffffu, on);
-        if (on) sel_list[base + __popc(bal & ((1u << lane) - 1u))] = j;
-        base += __popc(bal);
-      }
-    }
-    __syncthreads();
-    if (a.topp_out) {
-      int32_t* to = a.topp_out + ((size_t)bh * a.nblk + blk) * P;
-      for (int r = tid; r < P; r += kThreads) to[r] = sel_list[r];
-    }
-  }
+  // ---- top-P (ties -> lower index), then an ascending list
+  if (P > 0)
+    select_parents(w, M, P, sel, sel_list, cand, s_count, s_ncand,
+                   a.topp_out ? a.topp_out + ((size_t)bh * a.nblk + blk) * P : nullptr, [] { __syncthreads(); });
 
   // ---- pass C: merged softmax over unrefined parents, stay residuals and children of refined parents
   T* Yb = static_cast<T*>(a.Y) + ((size_t)bh * a.Nq + i0) * d;

@@ -73,3 +73,43 @@ def test_a_later_tile_far_above_an_earlier_one_leaves_finite_importances(dtype, 
     same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
     rows = np.repeat(same, bq, axis=-1)[..., :N]
     parity.compare_output(Y.float().cpu().numpy().astype(np.float64), ref["Y"], dtype, rows)
+
+
+@pytest.mark.parametrize("M,C,P,bq,tile_m,N,flags", [(5, 1, 2, 17, 32, 64, 0),           # one narrow tile, children in one too
+                                                     (130, 3, 20, 100, 96, 250, 0),      # ragged tiles of 96, blocks of 100 rows
+                                                     (300, 16, 40, 50, 256, 330, 0),     # two code tiles per importance tile
+                                                     (256, 2, 32, 64, 64, 300, binding.FLAG_PARENT_STAYS),
+                                                     (40, 5, 40, 128, 32, 129, 0),       # every parent refined
+                                                     (512, 4, 0, 128, 128, 300, 0)])     # none
+def test_tensor_core_tiles_at_their_edges(M, C, P, bq, tile_m, N, flags):
+    """bf16, d = 64: importance tiles, code tiles, query blocks and child tiles with remainders."""
+    wl = synth.Workload("edges", B=1, H=2, N=N, d=64, M=M, C=C, P=P, block_q=bq, seed=66 + M, alpha=0.5, hot_queries=True)
+    x = synth.generate(wl)
+    stays = bool(flags & binding.FLAG_PARENT_STAYS)
+    if stays:
+        x["K"][:, :, ::2] = synth.round_to_bf16((x["Cp"][:, :1] + 0.05 * x["V"][0, :, : len(x["K"][0, 0, ::2])]).astype(np.float32))
+    dv = parity.to_device(x, "bf16")
+    Y, topp, imp = binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, bq, tile_m, scale=wl.scale, flags=flags)
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, bq, wl.scale, parent_stays=stays, form="factorised", tile_m=tile_m)
+    same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
+    rows = np.repeat(same, bq, axis=-1)[..., :N]
+    parity.compare_output(Y.float().cpu().numpy().astype(np.float64), ref["Y"], "bf16", rows)
+
+
+def test_values_that_are_not_finite_leave_the_other_dimensions_alone():
+    """A tile with an infinite value sum takes its product on the CUDA cores: an infinity times the part of a weight that
+    happens to be zero must not become NaN, and nothing leaks into other dimensions or heads."""
+    wl = synth.Workload("inf", B=1, H=2, N=300, d=64, M=256, C=4, P=32, block_q=128, seed=67, alpha=0.5)
+    x = synth.generate(wl)
+    x["Q"] *= 0.1                                                # every key has some weight
+    run = lambda: binding.forward_tiled(*(parity.to_device(x, "bf16")[k] for k in ("Q", "K", "V", "Cp", "Cc")), wl.P, 128, 128,
+                                        scale=wl.scale)[0].float().cpu().numpy()
+    x["V"][0, 0, 100, 7] = 0.0
+    plain = run()
+    x["V"][0, 0, 100, 7] = np.inf
+    Y = run()
+    assert np.isposinf(Y[0, 0, :, 7]).all()
+    rest = np.arange(64) != 7
+    assert np.array_equal(Y[0, 1], plain[0, 1])
+    # the tile's sum in another order (float32), then one bf16 rounding: an ulp (2^-8) where a value is next to a boundary
+    assert np.abs(Y[0, 0][:, rest] - plain[0, 0][:, rest]).max() <= 2 ** -8 * np.abs(plain).max()
