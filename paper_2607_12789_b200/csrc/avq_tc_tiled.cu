@@ -46,6 +46,7 @@ struct TiledArgs {
   float* importance_out;
   int32_t* status_word;
   int H, Nq, M, C, P, block_q, nblk, stays, tile_m, Nk;
+  uint32_t inv_C;                              // 2^18 / C rounded up
   float scale;
 };
 
@@ -263,7 +264,8 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       rows_sync(q);
       to_frag((xz[r] + xz[kRows + r]) + (xz[2 * kRows + r] + xz[3 * kRows + r]), z);
     };
-    // This thread's logits of the tile at TMEM column `col`: e[h][2 b + u]; cnt[2 b + u] of its columns (0: not there).
+    // This thread's logits of the tile at TMEM column `col`: e[h][2 b + u], -inf where no key stands behind the column (its
+    // weight is then exp(-inf) = 0 against any reference, without a branch); cnt[2 b + u] of its columns.
     auto load_logits = [&](int col, const float* counts, int n, float (&e)[4][8], float (&cnt)[8]) {
       if (32 * cq < n) {                                   // warp-uniform
         uint32_t s[2][16];
@@ -281,13 +283,13 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int u = 0; u < 2; ++u)
-              e[i][2 * b + u] = __uint_as_float(s[i >> 1][4 * b + 2 * (i & 1) + u]) * a.scale;
+              e[i][2 * b + u] = cnt[2 * b + u] > 0.f ? __uint_as_float(s[i >> 1][4 * b + 2 * (i & 1) + u]) * a.scale : -INFINITY;
       } else {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           cnt[c] = 0.f;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) e[i][c] = 0.f;
+          for (int i = 0; i < 4; ++i) e[i][c] = -INFINITY;
         }
       }
     };
@@ -331,9 +333,8 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           load_logits(s * kTile, npS + t0 + s * kTile, width - s * kTile, e, cnt);
 #pragma unroll
           for (int c = 0; c < 8; ++c)
-            if (cnt[c] > 0.f)
 #pragma unroll
-              for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
+            for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
         }
         row_max(mx);
 #pragma unroll
@@ -347,7 +348,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
           for (int c = 0; c < 8; ++c)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) e[i][c] = cnt[c] > 0.f && valid[i] ? expf(e[i][c] - m[i]) : 0.f;
+            for (int i = 0; i < 4; ++i) e[i][c] = expf(e[i][c] - m[i]);
         };
         float zs[4] = {0.f, 0.f, 0.f, 0.f};
         for (int s = 0; s < subs; ++s) {
@@ -372,8 +373,11 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           }
           double d[8];
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
-            d[c] = fma((double)e[3][c], inv[3], fma((double)e[2][c], inv[2], fma((double)e[1][c], inv[1], (double)e[0][c] * inv[0])));
+          for (int c = 0; c < 8; ++c) {
+            d[c] = 0.0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[c] = fma((double)(valid[i] ? e[i][c] : 0.f), inv[i], d[c]);
+          }
           // over the 8 lanes of a column: lane 4 g + t keeps column 8 (g / 2) + 2 t + g % 2
 #pragma unroll
           for (int n = 4, bit = 16; n; n >>= 1, bit >>= 1) {
@@ -405,7 +409,10 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // ---- pass C: merged softmax over unrefined parents, stay residuals and children of refined parents
     auto first_of = [&](int k) { return k >= ptiles ? (k - ptiles) * kTile : k * kTile; };
     auto width_of = [&](int k) { return min(kTile, (k >= ptiles ? P * C : M) - first_of(k)); };
-    auto child_row = [&](int e) { return sel_list[e / C] * C + e % C; };
+    auto child_row = [&](int e) {                          // (e < 2^13, C <= 16: the division by multiplication is exact)
+      const int f = (int)(((uint32_t)e * a.inv_C) >> 18);
+      return sel_list[f] * C + (e - f * C);
+    };
     // keys that stand behind column c of tile k
     auto count_of = [&](int k, int c) {
       if (c >= width_of(k)) return 0.f;
@@ -536,9 +543,8 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
       for (int c = 0; c < 8; ++c)
-        if (cnt[c] > 0.f)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
+        for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
       row_max(mx);
       float alpha[4];
 #pragma unroll
@@ -554,7 +560,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       for (int c = 0; c < 8; ++c)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          e[i][c] = cnt[c] > 0.f ? expf(e[i][c] - m[i]) : 0.f;
+          e[i][c] = expf(e[i][c] - m[i]);
           z[i] = fmaf(e[i][c], cnt[c], z[i]);
         }
       if (k > 0) take_product(k - 1);                      // and with it the weights' columns
@@ -642,6 +648,7 @@ avq_status tc_attend_tiled(const avq_problem& p, const void* Q, const void* Cp, 
   a.stays = (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0;
   a.tile_m = tile_m;
   a.Nk = p.Nk;
+  a.inv_C = ((1u << 18) + (uint32_t)p.C - 1) / (uint32_t)p.C;
   a.scale = p.scale;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
