@@ -23,14 +23,15 @@ __device__ __forceinline__ void select_parents(const double* w, int M, int P, in
   } else {
     unsigned long long bound = 0;
     {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const unsigned long long smp = key[(2 * warp + e) * M / 32];
-        int c = 0;
-        for (int j = lane; j < M; j += 32) c += key[j] >= smp;
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (lane == 0) s_count[2 * warp + e] = c;
+      const unsigned long long smp0 = key[2 * warp * M / 32], smp1 = key[(2 * warp + 1) * M / 32];
+      int c = 0;                                            // keys at or above the two samples, 16 bits each
+#pragma unroll 4
+      for (int j = lane; j < M; j += 32) {
+        const unsigned long long kj = key[j];
+        c += (kj >= smp0) + ((kj >= smp1) << 16);
       }
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (lane < 2) s_count[2 * warp + lane] = (c >> (16 * lane)) & 0xFFFF;
       if (tid == 0) *s_ncand = 0;
       sync();
       if (s_count[lane] >= P) bound = key[lane * M / 32];

@@ -34,6 +34,7 @@ constexpr int kIssuer = kCompute / 32;         // the warp that issues loads and
 constexpr int kThreadsT = kCompute + 32;
 constexpr int kTileBytes = kTile * kD * 2;     // rows of 128 bytes
 constexpr int kMaxTiles = 80;                  // M + P C <= 8192
+constexpr int kStayRow = 1 << 28, kChildRow = 1 << 29;
 // TMEM columns: two logit tiles, three weight parts, the value product
 constexpr int kColW = 256, kColO = 448;
 constexpr float kLowest = -3.402823466e38f;    // a running maximum starts at the lowest finite value (weights of -inf logits are then 0)
@@ -51,7 +52,7 @@ struct TiledArgs {
 };
 
 struct TiledSmem {
-  size_t q, c, v, w, wpart, tcnt, np, nstay, xm, xz, nseen, sel, list, count, bad, bars, total;   // byte offsets
+  size_t q, c, v, raw, w, wpart, tcnt, trow, np, nstay, xm, xz, nseen, sel, list, count, bad, bars, total;   // byte offsets
 };
 __host__ __device__ inline TiledSmem tiled_smem_layout(int M, int P, int tile_m) {
   TiledSmem L;
@@ -60,9 +61,11 @@ __host__ __device__ inline TiledSmem tiled_smem_layout(int M, int P, int tile_m)
   L.q = take(kTileBytes);
   L.c = take(2 * kTileBytes);
   L.v = take(2 * 3 * kTileBytes);
+  L.raw = take(4 * kTile * kD);
   L.w = take(8 * (size_t)M);
   L.wpart = take(8 * 4 * kTile > 4 * (size_t)M ? 8 * 4 * kTile : 4 * (size_t)M);   // also the candidates of the selection
-  L.tcnt = take(4 * 2 * kTile);
+  L.tcnt = take(4 * 4 * kTile);
+  L.trow = take(4 * 4 * kTile);
   L.np = take(4 * (size_t)M);
   L.nstay = take(4 * (size_t)M);
   L.xm = take(4 * 4 * kRows);
@@ -72,7 +75,7 @@ __host__ __device__ inline TiledSmem tiled_smem_layout(int M, int P, int tile_m)
   L.list = take(4 * (size_t)(P > 0 ? P : 1));
   L.count = take(4 * 33);
   L.bad = take(4 * kMaxTiles);
-  L.bars = take(8 * 5 + 8);
+  L.bars = take(8 * 6 + 8);
   L.total = o;
   return L;
 }
@@ -102,12 +105,12 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   float *tcnt = reinterpret_cast<float*>(smem + L.tcnt), *npS = reinterpret_cast<float*>(smem + L.np);
   float *nstay = reinterpret_cast<float*>(smem + L.nstay), *xm = reinterpret_cast<float*>(smem + L.xm);
   float *xz = reinterpret_cast<float*>(smem + L.xz), *nseen = reinterpret_cast<float*>(smem + L.nseen);
-  int *sel = reinterpret_cast<int*>(smem + L.sel), *sel_list = reinterpret_cast<int*>(smem + L.list);
+  int *trow = reinterpret_cast<int*>(smem + L.trow), *sel = reinterpret_cast<int*>(smem + L.sel), *sel_list = reinterpret_cast<int*>(smem + L.list);
   int *s_count = reinterpret_cast<int*>(smem + L.count);
   volatile int* bad = reinterpret_cast<volatile int*>(smem + L.bad);   // [tile] it holds a value sum that is not finite
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
-  uint64_t *bar_q = bars, *bar_c = bars + 1, *bar_s = bars + 3, *bar_o = bars + 4;   // query tile, codes [2], logits, product
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
+  uint64_t *bar_q = bars, *bar_c = bars + 1, *bar_s = bars + 3, *bar_o = bars + 5;   // query tile, codes [2], logits [2], product
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, lane = tid & 31;
@@ -126,7 +129,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (elect_one()) {
       prefetch_tmap(&tmQ);
       prefetch_tmap(&tmCp);
-      for (int i = 0; i < 5; ++i) mbar_init(&bars[i], 1);
+      for (int i = 0; i < 6; ++i) mbar_init(&bars[i], 1);
       mbar_fence_init();
       *abort_flag = 0;
     }
@@ -155,12 +158,12 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       }
       __syncwarp();
     };
-    uint32_t ph_c[2] = {0, 0}, ph_s = 0;
+    uint32_t ph_c = 0, ph_s = 0;                           // a bit per barrier
     bool ok = true;
     auto logits = [&](int u, int n, int col, bool loaded) {
       if (loaded) {
-        ok = wait(&bar_c[u & 1], ph_c[u & 1]) && ok;
-        ph_c[u & 1] ^= 1;
+        ok = wait(&bar_c[u & 1], (ph_c >> (u & 1)) & 1) && ok;
+        ph_c ^= 1u << (u & 1);
       }
       tc_fence_after();
       if (ok && elect_one()) {
@@ -175,9 +178,19 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (elect_one()) umma_commit(bar);
       __syncwarp();
     };
-    auto logits_done = [&]() {
-      ok = wait(bar_s, ph_s) && ok;
-      ph_s ^= 1;
+    auto logits_done = [&](int i) {
+      ok = wait(&bar_s[i], (ph_s >> i) & 1) && ok;
+      ph_s ^= 1u << i;
+    };
+    // tile k of pass C (its codes have landed), two ahead of the weights; then the load that takes its buffer
+    auto tile_logits = [&](int k) {
+      const bool child = k >= ptiles;
+      logits(na + k, child ? min(kTile, P * C - (k - ptiles) * kTile) : min(kTile, M - k * kTile), (k & 1) * kTile, !child);
+      commit(&bar_s[k & 1]);
+    };
+    auto next_codes = [&](int k) {
+      logits_done(k & 1);
+      load_codes(na + k + 2);
     };
     if (elect_one()) {
       mbar_expect_tx(bar_q, kTileBytes);
@@ -192,24 +205,20 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (t > 0) ready_wait();                             // the logits of the tile before have been read
       for (int s = 0; s < subs; ++s) logits(u + s, min(kTile, min(tile_m, M - t0) - s * kTile), s * kTile, true);
       commit(bar_s);
-      logits_done();
+      logits_done(0);
       for (int s = 0; s < subs; ++s) load_codes(u + s + 2);
       u += subs;
     }
     if (need_w) ready_wait();
-    logits(na, min(kTile, M), 0, true);
-    commit(bar_s);
-    logits_done();
-    load_codes(na + 2);
+    tile_logits(0);
+    if (ptiles > 1) tile_logits(1);
+    next_codes(0);
+    if (ptiles > 1) next_codes(1);
     const uint32_t idesc_o = umma_idesc_bf16(kRows, kD) | (1u << 16);   // B (the value rows) is MN-major
     for (int k = 0; k < tiles; ++k) {
-      ready_wait();                                        // weights and values of tile k, gathered codes of tile k + 1
-      const bool child = k + 1 >= ptiles;
-      if (k + 1 < tiles) {
-        const int n = child ? min(kTile, P * C - (k + 1 - ptiles) * kTile) : min(kTile, M - (k + 1) * kTile);
-        logits(na + k + 1, n, ((k + 1) & 1) * kTile, !child);
-        commit(bar_s);
-      }
+      ready_wait();                                        // weights and values of tile k, gathered codes of tile k + 2
+      if (k == 0 && ptiles == 1 && tiles > 1) tile_logits(1);
+      if (k + 2 < tiles) tile_logits(k + 2);
       const int n = k >= ptiles ? min(kTile, P * C - (k - ptiles) * kTile) : min(kTile, M - k * kTile);
       if (ok && !bad[k] && elect_one()) {
         const uint32_t v0 = smem_u32(Vs + (k & 1) * 3 * kTileBytes);
@@ -231,10 +240,8 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       }
       __syncwarp();
       commit(bar_o);
-      if (k + 1 < tiles) {
-        logits_done();
-        load_codes(na + k + 3);
-      }
+      if (k == 0 && ptiles == 1 && tiles > 1) next_codes(1);
+      if (k + 2 < tiles) next_codes(k + 2);
     }
   } else {
     const int q = warp & 3, cq = warp >> 2, r = q * 32 + lane;
@@ -316,7 +323,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
     // ---- pass A: importance, tile by tile: a tile's weights against the maximum and the denominator seen up to it (Eq.
     // "aproxdenom"), so they stay finite however far a later tile's logits lie above them
-    uint32_t ph_s = 0;
+    uint32_t ph_s = 0;                                     // a bit per barrier
     if (need_w) {
       float m[4] = {kLowest, kLowest, kLowest, kLowest}, z[4] = {0.f, 0.f, 0.f, 0.f};
       bool valid[4];                                       // rows of this block
@@ -324,7 +331,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       for (int i = 0; i < 4; ++i) valid[i] = q * 32 + g + 8 * i < rows;
       for (int t0 = 0; t0 < M; t0 += tile_m) {
         const int width = min(tile_m, M - t0), subs = (width + kTile - 1) / kTile;
-        wait(bar_s, ph_s);
+        wait(bar_s, ph_s & 1);
         ph_s ^= 1;
         tc_fence_after();
         float e[4][8], cnt[8];
@@ -413,40 +420,65 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const int f = (int)(((uint32_t)e * a.inv_C) >> 18);
       return sel_list[f] * C + (e - f * C);
     };
-    // keys that stand behind column c of tile k
-    auto count_of = [&](int k, int c) {
-      if (c >= width_of(k)) return 0.f;
-      const int e = first_of(k) + c;
-      if (k >= ptiles) return ld_after_wait(nc + child_row(e));
-      return sel[e] ? (a.stays ? nstay[e] : 0.f) : npS[e];
+    // What stands behind column tid of tile k (prepared two tiles ahead, four tiles kept): the keys, and the row of their value
+    // sums, a child's (kChildRow) or a parent's, less the children's where the parent is refined (kStayRow); -1: none.
+    auto describe = [&](int k) {
+      if (tid >= kTile || k >= tiles) return;
+      float n = 0.f;
+      int row = -1;
+      if (tid < width_of(k)) {
+        const int e = first_of(k) + tid;
+        if (k >= ptiles) {
+          const int cr = child_row(e);
+          n = ld_after_wait(nc + cr);
+          row = cr | kChildRow;
+        } else {
+          n = sel[e] ? (a.stays ? nstay[e] : 0.f) : npS[e];
+          if (n > 0.f) row = sel[e] ? e | kStayRow : e;
+        }
+      }
+      tcnt[(k & 3) * kTile + tid] = n;
+      trow[(k & 3) * kTile + tid] = row;
     };
-    // value sums 4 ch .. + 3 of column c of tile k (a refined parent: of the keys that stay)
-    auto value_of = [&](int k, int c, int ch) {
+    // value sums 4 ch .. + 3 of such a row
+    auto value_of = [&](int row, int ch) {
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c >= width_of(k)) return v;
-      const int e = first_of(k) + c;
-      if (k >= ptiles) return ld_after_wait(reinterpret_cast<const float4*>(Vc + (size_t)child_row(e) * kD) + ch);
-      if ((sel[e] ? (a.stays ? nstay[e] : 0.f) : npS[e]) > 0.f) {
-        v = ld_after_wait(reinterpret_cast<const float4*>(Vp + (size_t)e * kD) + ch);
-        if (sel[e])
+      if (row >= 0) {
+        const int j = row & (kStayRow - 1);
+        v = ld_after_wait(reinterpret_cast<const float4*>((row & kChildRow ? Vc : Vp) + (size_t)j * kD) + ch);
+        if (row & kStayRow)
           for (int cc = 0; cc < C; ++cc) {
-            const float4 x = ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)e * C + cc) * kD) + ch);
+            const float4 x = ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)j * C + cc) * kD) + ch);
             v.x -= x.x; v.y -= x.y; v.z -= x.z; v.w -= x.w;
           }
       }
       return v;
     };
-    float4 val[4];                                         // rows tid / 16 + 32 i, dimensions 4 (tid % 16) .. + 3
+    // Value sums of tile k on their way: rows tid / 16 + 32 i, dimensions 4 (tid % 16) .. + 3, each thread its own.
+    const uint32_t own_v = smem_u32(smem + L.raw) + 16 * tid;
     auto load_values = [&](int k) {
+      int row[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) val[i] = value_of(k, (tid >> 4) + 32 * i, tid & 15);
-      if (tid < kTile) tcnt[(k & 1) * kTile + tid] = count_of(k, tid);
+      for (int i = 0; i < 4; ++i) row[i] = trow[(k & 3) * kTile + (tid >> 4) + 32 * i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t dst = own_v + 16 * kCompute * i;
+        if (row[i] >= 0 && (row[i] & kStayRow)) {
+          const float4 v = value_of(row[i], tid & 15);
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+        } else {                                           // (no row: nothing is read, zeros are written)
+          const int j = row[i] < 0 ? 0 : row[i] & (kStayRow - 1);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst),
+                       "l"((row[i] & kChildRow ? Vc : Vp) + (size_t)j * kD + 4 * (tid & 15)), "r"(row[i] < 0 ? 0 : 16) : "memory");
+        }
+      }
     };
     auto store_values = [&](int k) {
       bool finite = true;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float x[4] = {val[i].x, val[i].y, val[i].z, val[i].w};
+        float x[4];
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(own_v + 16 * kCompute * i) : "memory");
         uint32_t p[4][3];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -514,7 +546,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
           const int col = 16 * cq + 8 * b + 2 * t4;
-          const float4 v = value_of(k, c, col >> 2);
+          const float4 v = value_of(trow[(k & 3) * kTile + c], col >> 2);
           const float v0 = (col & 2) ? v.z : v.x, v1 = (col & 2) ? v.w : v.y;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -529,17 +561,21 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       // its buffer held a code tile of pass A, whose logits are done, or nothing yet
       gather_codes(1);
     }
+    describe(0);
+    describe(1);
+    compute_sync();
     load_values(0);
-    compute_sync();                                        // the counts of tile 0
+    cp_async_wait_all();
     for (int k = 0; k < tiles; ++k) {
-      wait(bar_s, ph_s);
-      ph_s ^= 1;
+      wait(&bar_s[k & 1], (ph_s >> (k & 1)) & 1);
+      ph_s ^= 1u << (k & 1);
       tc_fence_after();
       if (k + 2 < tiles && k + 2 >= ptiles) gather_codes(k + 2);
       store_values(k);
       if (k + 1 < tiles) load_values(k + 1);
+      describe(k + 2);
       float e[4][8], cnt[8];
-      load_logits((k & 1) * kTile, tcnt + (k & 1) * kTile, width_of(k), e, cnt);
+      load_logits((k & 1) * kTile, tcnt + (k & 3) * kTile, width_of(k), e, cnt);
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
       for (int c = 0; c < 8; ++c)
@@ -549,11 +585,9 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       float alpha[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        alpha[i] = 1.f;
-        if (mx[i] > m[i]) {
-          alpha[i] = expf(m[i] - mx[i]);
-          m[i] = mx[i];
-        }
+        const float up = fmaxf(m[i], mx[i]);               // (mx may be -inf, m is finite or +inf)
+        alpha[i] = up > m[i] ? expf(m[i] - up) : 1.f;
+        m[i] = up;
         z[i] *= alpha[i];
       }
 #pragma unroll
