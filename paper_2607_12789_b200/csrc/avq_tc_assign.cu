@@ -9,7 +9,8 @@
 //            when there is more than one such column are all M distances redone in float64 in the direct form
 //            (lowest index wins ties).  Three instructions per column and row instead of the six of a running best,
 //            runner-up and index, and half of them off the ALU pipe, which bounded the kernel.
-//   child    on CUDA cores (a second MMA over all M C children would cost C times the parent GEMM): ||c||^2 - 2 k.c where
+//   child    (PARENT_STAYS: by warp-level tensor-core products over the keys in the order of their parents, see there)
+//            on CUDA cores (a second MMA over all M C children would cost C times the parent GEMM): ||c||^2 - 2 k.c where
 //            a norm table is at hand, near-ties in the direct form sum (k - c)^2 in float32 and then in float64; else
 //            the direct form throughout, near-ties in float64.
 //            Four lanes per key, each over a quarter of the head dimension for all C children of the
@@ -50,6 +51,11 @@ __device__ __forceinline__ void dot_bf16x8(float& s, const uint4& k, const uint4
   for (int e = 0; e < 4; ++e)
     asm("{\n\t.reg .b16 a, b, c, d;\n\tmov.b32 {a, b}, %1;\n\tmov.b32 {c, d}, %2;\n\tfma.rn.f32.bf16 %0, a, c, %0;\n\tfma.rn.f32.bf16 %0, b, d, %0;\n\t}"
         : "+f"(s) : "r"(x[e]), "r"(y[e]));
+}
+// One warp: c += a (16 x 16) . b (16 x 8), exact products, fp32 sums
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 struct KeyChunk { f32x2 p[4]; };      // 8 key elements as four fp32 pairs
 __device__ __forceinline__ KeyChunk widen8(const uint4& a) {
@@ -210,7 +216,10 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   float* xkn = xs + 2 * kKeys;                       // [2][128] halves of ||k||^2
   int* par = reinterpret_cast<int*>(xkn + 2 * kKeys);   // [128] final parent of each key
   int* chi = par + kKeys;                            // [128] final child of each key
-  uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(chi + kKeys);   // max ||c||^2 (non-negative float bits)
+  int* hist = chi + kKeys;                           // STAYS: [M] keys per parent
+  int* offs = reinterpret_cast<int*>(xs);            // [M] first place of a parent's keys in `order`
+  uint8_t* order = reinterpret_cast<uint8_t*>(hist + M);   // STAYS: [128] keys by parent
+  uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(STAYS ? order + kKeys : reinterpret_cast<uint8_t*>(hist));   // max ||c||^2 (non-negative float bits)
   uint32_t* tmem_slot = cmax_bits + 1;
   uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [3]
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 3);
@@ -315,6 +324,8 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   ph_k ^= 1;
   if (warp == 0 && loaded) issue_mma();              // (all lanes wait for the same barriers and agree)
 
+  if (STAYS)
+    for (int m = tid; m < M; m += kThreadsA) hist[m] = 0;
   {                                                  // half of ||k||^2 per thread
     float s = 0.f;
     constexpr int kChunksHalf = D / 16;              // 16-byte chunks in half a row
@@ -433,10 +444,160 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       i1 = bi;
     }
     par[r] = i1;
+    if constexpr (STAYS) {
+      xd[r] = open ? NAN : fminf(xd[r], xd[kKeys + r]);   // distance to the parent, less ||k||^2
+      // ---- the keys in the order of their parents (within a parent any): counting sort by the warps of the lower half
+      const int rank = atomicAdd(&hist[i1], 1);
+      asm volatile("bar.sync 5, 128;" ::: "memory");
+      const int per = M >> 5;                          // bins per lane
+      int before = 0, n = 0;
+      for (int u = 0; u < per; ++u) n += hist[lane * per + u];
+      before = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += up;
+      }
+      before -= n;
+      if (lane >> 3 == q)                              // a quarter of the bins per warp
+        for (int u = 0; u < per; ++u) {
+          offs[lane * per + u] = before;
+          before += hist[lane * per + u];
+        }
+      asm volatile("bar.sync 5, 128;" ::: "memory");
+      order[offs[i1] + rank] = (uint8_t)r;
+    }
   }
   __syncthreads();
 
-  {
+  if constexpr (STAYS) {
+    // ---- children, PARENT_STAYS: a warp takes 16 keys in the order of their parents.  k . c for all 16 and the children of
+    // each parent among them, one (eight children) or two (four) parents per warp-level tensor-core product: 16 keys x 8
+    // children; a key takes the columns of its own parent.  Both operands hold the head dimension in the order in which a lane
+    // reads 16-byte chunks (lane t of a quad: chunks t, t + 4, ...).  The distance to the parent comes from the parents' products.
+    // Bound by the latency of the child rows, one product ahead.  Against four lanes per key in the loop below, with the
+    // parent's row read too, us per call: B2 H8 N5000 d128 M96 C8 98.3 -> 88.4, H12 N400 d128 M256 C8 67.7 -> 47.7, B8 H12
+    // N10167 d64 M32 C8 268 -> 230, B2 H16 N4096 d64 M128 C8 81.0 -> 77.1, H16 N65536 d64 M256 C4 700 and 700.  Where no key
+    // may stay the loop below keeps more loads in flight: H16 N65536 d64 M256 C4 771 and 789, B2 H16 N4096 d64 M128 C8 69.3
+    // and 68.7, B8 H12 N1254 d64 M256 C4 44.1 and 46.7.
+    constexpr int kC = NL * 256 / D;                   // children per parent (4 or 8)
+    constexpr int kPar = 8 / kC;                       // parents per product
+    constexpr int kB = D / 32;                         // 16-byte chunks per lane and row
+    const int mk = order[warp * 16 + (lane & 15)], mp = par[mk];
+    const int prev = __shfl_up_sync(0xffffffffu, mp, 1);
+    const uint32_t heads = __ballot_sync(0xffffffffu, lane < 16 && (lane == 0 || mp != prev));   // first key of each parent
+    const int nd = __popc(heads);
+    int key[2], own[2], cid[2];                        // rows g, g + 8: key, parent, this lane's first child of it
+    bool mine[2];                                      // this lane holds children of the row's own parent
+    int ord[2];                                        // which of the parents the row's is
+    uint4 ka[2][kB];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      key[i] = __shfl_sync(0xffffffffu, mk, g + 8 * i);
+      own[i] = __shfl_sync(0xffffffffu, mp, g + 8 * i);
+      ord[i] = __popc(heads & ((2u << (g + 8 * i)) - 1u)) - 1;
+      mine[i] = kPar == 1 || (ord[i] & 1) == (t4 >> 1);
+      cid[i] = kPar == 1 ? 2 * t4 : 2 * (t4 & 1);
+#pragma unroll
+      for (int b = 0; b < kB; ++b) {
+        const int ch = t4 + 4 * b;
+        ka[i][b] = *reinterpret_cast<const uint4*>(Ks + (ch >> 3) * (kKeys * 128) + sw128_offset(key[i], (ch & 7) * 8));
+      }
+    }
+    const size_t head_base = (size_t)h * M;
+    float nrm[2][2], dot[2][2];                        // of children cid, cid + 1
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      dot[i][0] = dot[i][1] = nrm[i][0] = nrm[i][1] = 0.f;
+      if constexpr (TABLE) {
+        const float2 n2 = ld_after_wait(reinterpret_cast<const float2*>(cnorm_g + (size_t)H * M + (head_base + own[i]) * kC + cid[i]));
+        nrm[i][0] = n2.x;
+        nrm[i][1] = n2.y;
+      }
+    }
+    uint32_t rest = heads;
+    auto fetch = [&](uint4 (&z)[kB]) {                 // the next product's children: lane 4 g + t, row g
+      int src = __ffs(rest) - 1;
+      rest &= rest - 1;
+      if constexpr (kPar == 2) {
+        if (rest && g >= 4) src = __ffs(rest) - 1;
+        rest &= rest - 1;
+      }
+      const int pp = __shfl_sync(0xffffffffu, mp, src);
+      const uint4* row = reinterpret_cast<const uint4*>(Cc + ((head_base + pp) * kC + (g & (kC - 1))) * D) + t4;
+#pragma unroll
+      for (int b = 0; b < kB; ++b) z[b] = __ldg(row + 4 * b);
+    };
+    auto product = [&](const uint4 (&z)[kB], int u) {
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int b = 0; b < kB; ++b) {
+        mma_bf16(c, ka[0][b].x, ka[1][b].x, ka[0][b].y, ka[1][b].y, z[b].x, z[b].y);
+        mma_bf16(c, ka[0][b].z, ka[1][b].z, ka[0][b].w, ka[1][b].w, z[b].z, z[b].w);
+      }
+      float n0 = 0.f, n1 = 0.f;
+      if constexpr (!TABLE) {                          // ||c||^2 of row g, then of this lane's columns 2 t, 2 t + 1
+        float n = 0.f;
+#pragma unroll
+        for (int b = 0; b < kB; ++b) n = norm_bf16x8(n, z[b]);
+        n = quad_sum(n);
+        n0 = __shfl_sync(0xffffffffu, n, 8 * t4);
+        n1 = __shfl_sync(0xffffffffu, n, 8 * t4 + 4);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (ord[i] / kPar == u) {
+          dot[i][0] = c[2 * i];
+          dot[i][1] = c[2 * i + 1];
+          if constexpr (!TABLE) { nrm[i][0] = n0; nrm[i][1] = n1; }
+        }
+    };
+    uint4 z[2][kB];
+    fetch(z[0]);
+    for (int u = 0; u * kPar < nd; u += 2) {
+      if ((u + 1) * kPar < nd) fetch(z[1]);
+      product(z[0], u);
+      if ((u + 1) * kPar < nd) {
+        if ((u + 2) * kPar < nd) fetch(z[0]);
+        product(z[1], u + 1);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float a = mine[i] ? fmaf(-2.f, dot[i][0], nrm[i][0]) : INFINITY;
+      const float b = mine[i] ? fmaf(-2.f, dot[i][1], nrm[i][1]) : INFINITY;
+      float e1 = fminf(a, b), e2 = fmaxf(a, b);
+      int c1 = b < a ? cid[i] + 1 : cid[i];
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        const float b1 = __shfl_xor_sync(0xffffffffu, e1, o);
+        const float b2 = __shfl_xor_sync(0xffffffffu, e2, o);
+        const int cb = __shfl_xor_sync(0xffffffffu, c1, o);
+        e2 = fminf(fmaxf(e1, b1), fminf(e2, b2));
+        if (b1 < e1 || (b1 == e1 && cb < c1)) { e1 = b1; c1 = cb; }
+      }
+      // Closer than this two distances are measured again, in the direct form in float32 and then in float64.  A tensor-core
+      // product adds 16 exact products to the sum and rounds each of the 17 terms by at most 2^-24 of the largest of them and
+      // of the sum: D / 16 steps are off by at most 17 D / 16 2^-24 |k||c|, the norm (chains of at most D / 4 and three
+      // additions) by (D/4 + 3) 2^-24 |c|^2, so a distance by less than 1.05e-5 (|k|^2 + |c|^2) at D = 128 and two of them by
+      // less than 2.1e-5 (|k|^2 + max |c|^2).
+      float cmx = mine[i] ? fmaxf(nrm[i][0], nrm[i][1]) : 0.f;
+      cmx = quad_max(cmx);
+      cmx = fmaxf(cmx, cnorm[own[i]]);
+      const float near = 2.5e-5f * (xkn[key[i]] + xkn[kKeys + key[i]] + cmx);
+      const bool live = done && j0 + key[i] < Nk;
+      const bool open = live && !(e2 - e1 > near);     // not decided by the products
+      const float dp = xd[key[i]];                     // the parent's distance (NaN where that was decided in float64)
+      const bool moved = e1 < dp;                      // strictly closer
+      const bool stay_open = live && !(fabsf(e1 - dp) > near);
+      if (__any_sync(0xffffffffu, open || stay_open))
+        c1 = settle_child<D, kC>(Ks, key[i], t4, Cc + (head_base + own[i]) * kC * D, Cp + (head_base + own[i]) * D, c1, open,
+                                 stay_open, moved);
+      else if (!moved)
+        c1 = -1;
+      if (t4 == 0) chi[key[i]] = c1;
+    }
+  } else {
     // ---- child argmin, four lanes per key: a warp takes 8 keys at a time (two passes over its 16 keys).
     // Lane s of a key's group covers the 16-byte chunks s, s + 4, ... of the key row and of each of the
     // parent's C children (the group reads 64 contiguous bytes of a child row per load), keeps one running
@@ -458,7 +619,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       for (int c = 0; c < 4; ++c) dst[c] = __ldg(src + c * kChunks);
     };
     float sum[kC];
-    float sum_p = 0.f;                                   // STAYS: the same for the parent itself
     issue(0, buf4[0]);
     float ncv[2][kC / 4];                                // TABLE: norms of child s4 (and s4 + 4) of this lane's keys
     if constexpr (TABLE) {
@@ -477,7 +637,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       if (t == 0 && f == 0) {
 #pragma unroll
         for (int c = 0; c < kC; ++c) sum[c] = 0.f;
-        sum_p = 0.f;
       }
       const int ch = s4 + 4 * t;
       if (f == 0) {
@@ -489,13 +648,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       for (int c = 0; c < 4; ++c) {
         if constexpr (TABLE) dot_bf16x8(sum[4 * f + c], kv, buf4[step & 1][c]);
         else sum[4 * f + c] += sqdiff8(kv, buf4[step & 1][c]);
-      }
-      if constexpr (STAYS) {
-        if (f == 0) {
-          const uint4 pw = __ldg(reinterpret_cast<const uint4*>(Cp + (head_base + par[key]) * D) + ch);
-          if constexpr (TABLE) dot_bf16x8(sum_p, kv, pw);
-          else sum_p += sqdiff8(kv, pw);
-        }
       }
       if (t == kT - 1 && f == kF - 1) {
         // transpose-reduce over the group: after the two exchanges lane s holds the total of child s
@@ -521,7 +673,7 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // two of them by less than 1e-5 (|k|^2 + max |c|^2).
         float near = 0.f;
         if constexpr (TABLE) {
-          float cmx = STAYS ? cnorm[par[key]] : 0.f;
+          float cmx = 0.f;
 #pragma unroll
           for (int i = 0; i < kC / 4; ++i) {
             cmx = fmaxf(cmx, ncv[pass][i]);
@@ -544,23 +696,11 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           e2 = fminf(fmaxf(e1, b1), fminf(e2, b2));
           if (b1 < e1 || (b1 == e1 && cb < c1)) { e1 = b1; c1 = cb; }
         }
-        float dp = 0.f;
-        if constexpr (STAYS) {
-          dp = sum_p + __shfl_xor_sync(0xffffffffu, sum_p, 1);
-          dp += __shfl_xor_sync(0xffffffffu, dp, 2);
-          if constexpr (TABLE) dp = fmaf(-2.f, dp, cnorm[par[key]]);
-        }
         if constexpr (TABLE) {
           const bool live = done && j0 + key < Nk;
           const bool open = live && !(e2 - e1 > near);   // not decided by the products
           const __nv_bfloat16* Cch = Cc + (head_base + par[key]) * kC * D;
-          if constexpr (STAYS) {                         // strict '<' against the parent distance
-            const bool moved = e1 < dp, stay_open = live && !(fabsf(e1 - dp) > near);
-            if (__any_sync(0xffffffffu, open || stay_open))
-              c1 = settle_child<D, kC>(Ks, key, s4, Cch, Cp + (head_base + par[key]) * D, c1, open, stay_open, moved);
-            else if (!moved)
-              c1 = -1;
-          } else if (__any_sync(0xffffffffu, open)) {
+          if (__any_sync(0xffffffffu, open)) {
             double best = INFINITY;
             int bi = 0;
             for (int c = 0; c < kC; ++c) {
@@ -571,7 +711,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           }
           if (s4 == 0) chi[key] = c1;
         } else if (s4 == 0) {
-          bool rechecked = false;
           double best = INFINITY;
           if (done && j0 + key < Nk && !(e2 - e1 > 1e-4f * e2)) {
             const __nv_bfloat16* Cch = Cc + (head_base + par[key]) * kC * D;
@@ -581,16 +720,6 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
               if (sd < best) { best = sd; bi = c; }
             }
             c1 = bi;
-            rechecked = true;
-          }
-          if constexpr (STAYS) {
-            // strict '<' against the parent distance; float64 when the two are closer than fp32 separates
-            bool moved = e1 < dp;
-            if (done && j0 + key < Nk && (rechecked || !(fabsf(e1 - dp) > 1e-4f * fmaxf(e1, dp)))) {
-              if (!rechecked) best = exact_dist_smem<D>(Ks, key, Cc + ((head_base + par[key]) * kC + c1) * D);
-              moved = best < exact_dist_smem<D>(Ks, key, Cp + (head_base + par[key]) * D);
-            }
-            if (!moved) c1 = -1;
           }
           chi[key] = c1;
         }
@@ -663,7 +792,7 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
     avq_status s = make_tmap_bf16(&tmCp, Cp, 2, dims, box);
     if (s != AVQ_OK) return s;
   }
-  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys) + 96;
+  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys + (STAYS ? p.M + kKeys / 4 : 0)) + 96;
   const int resident = (int)min((size_t)assign_min_ctas(D), kSmemMax / (smem + 1024));   // CTAs on an SM
   int sms = 148;
   {

@@ -147,6 +147,27 @@ def test_parent_stays_on_the_tensor_core_path(wl):
     assert np.abs(gpu_rep["Y"] - gpu_st["Y"]).max() > 1e-3
 
 
+@pytest.mark.parametrize("d,M,C", [(64, 32, 8), (64, 256, 4), (128, 96, 4), (128, 128, 8)])
+@pytest.mark.parametrize("spread", ["one_parent", "all_parents", "two_per_sixteen"])
+def test_parent_stays_with_few_and_many_parents_per_tile(d, M, C, spread):
+    """The child step takes a tile's keys in the order of their parents, 16 per warp: a tile of one parent, tiles whose keys
+    have a parent each, and a ragged last tile, half of the keys close to their parent."""
+    from oracle import avq_oracle as orc
+    g = np.random.default_rng(d + M + C)
+    N = 333
+    Cp = synth.round_to_bf16(3 * g.standard_normal((M, d)).astype(np.float32))
+    Cc = synth.round_to_bf16((Cp[:, None] + 0.8 * g.standard_normal((M, C, d))).astype(np.float32))
+    par = {"one_parent": np.full(N, M - 1), "all_parents": g.permutation(N) % M, "two_per_sixteen": np.arange(N) // 8 % M}[spread]
+    K = Cc[par, g.integers(0, C, N)] + 0.2 * g.standard_normal((N, d))
+    K[::2] = Cp[par[::2]] + 0.05 * g.standard_normal((len(K[::2]), d))
+    K = synth.round_to_bf16(K.astype(np.float32))
+    ref = orc.assign_head(K, Cp, Cc, parent_stays=True)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a[None])).cuda().to(torch.bfloat16)
+    pi, ci = binding.assign(t(K[None]), t(Cp), t(Cc), flags=binding.FLAG_PARENT_STAYS)
+    assert np.array_equal(pi.cpu().numpy()[0, 0], ref["parent_idx"])
+    assert np.array_equal(ci.cpu().numpy()[0, 0], ref["child_idx"])
+
+
 def test_tensor_core_and_cuda_core_paths_agree_at_full_size():
     wl = synth.C3.with_(H=4)
     dv = parity.to_device(synth.generate(wl), "bf16")
