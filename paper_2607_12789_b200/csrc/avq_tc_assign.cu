@@ -9,8 +9,8 @@
 //            when there is more than one such column are all M distances redone in float64 in the direct form
 //            (lowest index wins ties).  Three instructions per column and row instead of the six of a running best,
 //            runner-up and index, and half of them off the ALU pipe, which bounded the kernel.
-//   child    (PARENT_STAYS: by warp-level tensor-core products over the keys in the order of their parents, see there)
-//            on CUDA cores (a second MMA over all M C children would cost C times the parent GEMM): ||c||^2 - 2 k.c where
+//   child    large grids with eight children, and PARENT_STAYS: by warp-level tensor-core products over the keys in the order
+//            of their parents (see there).  Else on CUDA cores (a second MMA over all M C children would cost C times the parent GEMM): ||c||^2 - 2 k.c where
 //            a norm table is at hand, near-ties in the direct form sum (k - c)^2 in float32 and then in float64; else
 //            the direct form throughout, near-ties in float64.
 //            Four lanes per key, each over a quarter of the head dimension for all C children of the
@@ -195,7 +195,8 @@ enum Form { kOne, kRuns, kSmall };
 // the parents' distances with a key per lane: best, runner-up and index in one pass.
 // TABLE: cnorm_g holds the squared norms of all codewords (parents [H, M], then children [H, M, C]); the child distances
 // are then ||c||^2 - 2 k.c at one mixed-precision multiply-add per element, half the instructions of the direct form.
-template <int D, int NL, bool STAYS, Form FORM, bool TABLE>
+// SORTED: children by products over the keys in the order of their parents (always under PARENT_STAYS).
+template <int D, int NL, bool STAYS, Form FORM, bool TABLE, bool SORTED>
 __global__ void __launch_bounds__(kThreadsA, assign_min_ctas(D))
 tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmCp,
                  const __nv_bfloat16* __restrict__ Cp, const __nv_bfloat16* __restrict__ Cc,
@@ -216,10 +217,10 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   float* xkn = xs + 2 * kKeys;                       // [2][128] halves of ||k||^2
   int* par = reinterpret_cast<int*>(xkn + 2 * kKeys);   // [128] final parent of each key
   int* chi = par + kKeys;                            // [128] final child of each key
-  int* hist = chi + kKeys;                           // STAYS: [M] keys per parent
+  int* hist = chi + kKeys;                           // SORTED: [M] keys per parent
   int* offs = reinterpret_cast<int*>(xs);            // [M] first place of a parent's keys in `order`
-  uint8_t* order = reinterpret_cast<uint8_t*>(hist + M);   // STAYS: [128] keys by parent
-  uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(STAYS ? order + kKeys : reinterpret_cast<uint8_t*>(hist));   // max ||c||^2 (non-negative float bits)
+  uint8_t* order = reinterpret_cast<uint8_t*>(hist + M);   // SORTED: [128] keys by parent
+  uint32_t* cmax_bits = reinterpret_cast<uint32_t*>(SORTED ? order + kKeys : reinterpret_cast<uint8_t*>(hist));   // max ||c||^2 (non-negative float bits)
   uint32_t* tmem_slot = cmax_bits + 1;
   uint64_t* bars = reinterpret_cast<uint64_t*>(tmem_slot + 1);      // [3]
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 3);
@@ -324,7 +325,7 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   ph_k ^= 1;
   if (warp == 0 && loaded) issue_mma();              // (all lanes wait for the same barriers and agree)
 
-  if (STAYS)
+  if (SORTED)
     for (int m = tid; m < M; m += kThreadsA) hist[m] = 0;
   {                                                  // half of ||k||^2 per thread
     float s = 0.f;
@@ -444,8 +445,8 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       i1 = bi;
     }
     par[r] = i1;
-    if constexpr (STAYS) {
-      xd[r] = open ? NAN : fminf(xd[r], xd[kKeys + r]);   // distance to the parent, less ||k||^2
+    if constexpr (SORTED) {
+      if (STAYS) xd[r] = open ? NAN : fminf(xd[r], xd[kKeys + r]);   // distance to the parent, less ||k||^2
       // ---- the keys in the order of their parents (within a parent any): counting sort by the warps of the lower half
       const int rank = atomicAdd(&hist[i1], 1);
       asm volatile("bar.sync 5, 128;" ::: "memory");
@@ -470,16 +471,12 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   }
   __syncthreads();
 
-  if constexpr (STAYS) {
-    // ---- children, PARENT_STAYS: a warp takes 16 keys in the order of their parents.  k . c for all 16 and the children of
+  if constexpr (SORTED) {
+    // ---- children, SORTED: a warp takes 16 keys in the order of their parents.  k . c for all 16 and the children of
     // each parent among them, one (eight children) or two (four) parents per warp-level tensor-core product: 16 keys x 8
     // children; a key takes the columns of its own parent.  Both operands hold the head dimension in the order in which a lane
     // reads 16-byte chunks (lane t of a quad: chunks t, t + 4, ...).  The distance to the parent comes from the parents' products.
-    // Bound by the latency of the child rows, one product ahead.  Against four lanes per key in the loop below, with the
-    // parent's row read too, us per call: B2 H8 N5000 d128 M96 C8 98.3 -> 88.4, H12 N400 d128 M256 C8 67.7 -> 47.7, B8 H12
-    // N10167 d64 M32 C8 268 -> 230, B2 H16 N4096 d64 M128 C8 81.0 -> 77.1, H16 N65536 d64 M256 C4 700 and 700.  Where no key
-    // may stay the loop below keeps more loads in flight: H16 N65536 d64 M256 C4 771 and 789, B2 H16 N4096 d64 M128 C8 69.3
-    // and 68.7, B8 H12 N1254 d64 M256 C4 44.1 and 46.7.
+    // Bound by the latency of the child rows, one product ahead (the rule and what both forms take: beside the launch).
     constexpr int kC = NL * 256 / D;                   // children per parent (4 or 8)
     constexpr int kPar = 8 / kC;                       // parents per product
     constexpr int kB = D / 32;                         // 16-byte chunks per lane and row
@@ -583,13 +580,13 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       // less than 2.1e-5 (|k|^2 + max |c|^2).
       float cmx = mine[i] ? fmaxf(nrm[i][0], nrm[i][1]) : 0.f;
       cmx = quad_max(cmx);
-      cmx = fmaxf(cmx, cnorm[own[i]]);
+      if (STAYS) cmx = fmaxf(cmx, cnorm[own[i]]);
       const float near = 2.5e-5f * (xkn[key[i]] + xkn[kKeys + key[i]] + cmx);
       const bool live = done && j0 + key[i] < Nk;
       const bool open = live && !(e2 - e1 > near);     // not decided by the products
-      const float dp = xd[key[i]];                     // the parent's distance (NaN where that was decided in float64)
-      const bool moved = e1 < dp;                      // strictly closer
-      const bool stay_open = live && !(fabsf(e1 - dp) > near);
+      const float dp = STAYS ? xd[key[i]] : INFINITY;  // the parent's distance (NaN where that was decided in float64)
+      const bool moved = !STAYS || e1 < dp;            // strictly closer
+      const bool stay_open = STAYS && live && !(fabsf(e1 - dp) > near);
       if (__any_sync(0xffffffffu, open || stay_open))
         c1 = settle_child<D, kC>(Ks, key[i], t4, Cc + (head_base + own[i]) * kC * D, Cp + (head_base + own[i]) * D, c1, open,
                                  stay_open, moved);
@@ -751,21 +748,31 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   if (beside) pdl_wait();    // this grid's completion then implies that of the one it ran beside
 }
 
+int sm_count() {                                      // of the current device; 0: unknown
+  static int known[64] = {};
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev >= 0 && dev < 64 && known[dev] > 0) return known[dev];
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (dev >= 0 && dev < 64) known[dev] = n;
+  return n;
+}
+
 uint32_t pow2_cols(int n) {
   uint32_t c = 32;
   while ((int)c < n) c <<= 1;
   return c;
 }
 
-template <int D, int NL, bool STAYS, Form FORM, bool TABLE>
+template <int D, int NL, bool STAYS, Form FORM, bool TABLE, bool SORTED>
 avq_status launch_kernel(const CUtensorMap& tmK, const CUtensorMap& tmCp, const avq_problem& p, const void* Cp,
                          const void* Cc, int32_t* pidx, int32_t* cidx, int32_t* status_word, void* zero_base,
                          size_t zero_bytes, const float* cnorm, bool beside, int nblk, int total, size_t smem,
                          unsigned grid, cudaStream_t st) {
-  auto kern = tc_assign_kernel<D, NL, STAYS, FORM, TABLE>;
+  auto kern = tc_assign_kernel<D, NL, STAYS, FORM, TABLE, SORTED>;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
-  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, FORM, TABLE>>(dev);
+  const avq_status s = open_shared_memory<tc_assign_kernel<D, NL, STAYS, FORM, TABLE, SORTED>>(dev);
   if (s != AVQ_OK) return s;
   // launched as a dependent of the norms kernel when there is one: set-up, loads and the MMA overlap it
   return cuda_ok(launch_pdl(kern, dim3(grid), dim3(kThreadsA), smem, st, cnorm != nullptr || beside, tmK, tmCp,
@@ -792,22 +799,23 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
     avq_status s = make_tmap_bf16(&tmCp, Cp, 2, dims, box);
     if (s != AVQ_OK) return s;
   }
-  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys + (STAYS ? p.M + kKeys / 4 : 0)) + 96;
-  const int resident = (int)min((size_t)assign_min_ctas(D), kSmemMax / (smem + 1024));   // CTAs on an SM
-  int sms = 148;
-  {
-    static int sm_count[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return AVQ_ERR_CUDA;
-    sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
-    if (sms <= 0) {
-      if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return AVQ_ERR_CUDA;
-      if (dev >= 0 && dev < 64) sm_count[dev] = sms;
-    }
-  }
+  // Children by products over sorted keys.  Under PARENT_STAYS, where the loop over each key's children reads the parent's row as
+  // well, always (us per call, loop and products: B2 H8 N5000 d128 M96 C8 98.3 and 88.4, H12 N400 d128 M256 C8 67.7 and 47.7,
+  // B8 H12 N10167 d64 M32 C8 268 and 230, B2 H16 N4096 d64 M128 C8 81.0 and 77.1, H16 N65536 d64 M256 C4 700 and 700).  Where
+  // every key moves, for eight children and grids that hide the sort: d128 H16 N20000 M32 167.7 and 142.6, M64 179.5 and
+  // 157.8, M128 247.5 and 234.7, M256 303.4 and 299.4; 288 tiles M64 34.4 and 33.3, M256 56.2 and 53.9, but 48 tiles M64 23.3
+  // and 24.0; d64 H16 N20000 M32 92.0 and 85.1, M64 111.3 and 105.4, M128 144.9 and 142.6, M256 224.0 and 224.8; 288 tiles M64
+  // 25.7 and 26.5.  With four children the two about cancel or products lose: d64 H16 N20000 M64 96.5 and 97.9, M256 204.5
+  // and 211.5; d128 M128 215.0 and 214.5, M256 256.8 and 259.8.
+  constexpr bool kSortedAtAll = STAYS || NL * 256 / D == 8;
   const int nblk = (p.Nk + kKeys - 1) / kKeys;
   if ((uint64_t)nblk * BH > 0x7fffffffull) return AVQ_ERR_UNSUPPORTED;
   const int total = (int)(nblk * BH);
+  const int sms = sm_count();
+  if (sms <= 0) return AVQ_ERR_CUDA;
+  const bool sorted = STAYS || (kSortedAtAll && (D == 128 ? 2 * total >= 3 * sms : total >= 4 * sms && p.M <= 128));
+  const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys + (sorted ? p.M + kKeys / 4 : 0)) + 96;
+  const int resident = (int)min((size_t)assign_min_ctas(D), kSmemMax / (smem + 1024));   // CTAs on an SM
   // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, for the largest codebook
   // (64 KB: d128 M256) from four tiles per CTA on (N16384 H16, 6.9 tiles: 72 -> 63 us); with fewer the uneven last round
   // costs more than the set-up it saves (B2 H8 N5000 d128 M96, 2.2 tiles: whole call 111 -> 130 us).  Below M256 the gain
@@ -828,10 +836,17 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   // With the norm table at d64 the loop behind has no registers to spare (whole call N65536 M64 C8: 301.7 and 304.5).
   const bool small = p.M <= 64 && !(D == 64 && cnorm);
   constexpr Form kSmallTable = D == 64 ? kOne : kSmall;
-  auto go = cnorm ? (small ? launch_kernel<D, NL, STAYS, kSmallTable, true> : launch_kernel<D, NL, STAYS, kOne, true>)
-                  : (small ? launch_kernel<D, NL, STAYS, kSmall, false> : launch_kernel<D, NL, STAYS, kOne, false>);
-  if constexpr (D == 128)
-    if (runs) go = cnorm ? launch_kernel<D, NL, STAYS, kRuns, true> : launch_kernel<D, NL, STAYS, kRuns, false>;
+  auto choose = [&](auto sorted_) {
+    constexpr bool kSorted = decltype(sorted_)::value;
+    auto go = cnorm ? (small ? launch_kernel<D, NL, STAYS, kSmallTable, true, kSorted> : launch_kernel<D, NL, STAYS, kOne, true, kSorted>)
+                    : (small ? launch_kernel<D, NL, STAYS, kSmall, false, kSorted> : launch_kernel<D, NL, STAYS, kOne, false, kSorted>);
+    if constexpr (D == 128)
+      if (runs) go = cnorm ? launch_kernel<D, NL, STAYS, kRuns, true, kSorted> : launch_kernel<D, NL, STAYS, kRuns, false, kSorted>;
+    return go;
+  };
+  auto go = choose(std::integral_constant<bool, STAYS>{});
+  if constexpr (kSortedAtAll && !STAYS)
+    if (sorted) go = choose(std::true_type{});
   return go(tmK, tmCp, p, Cp, Cc, pidx, cidx, status_word, zero_base, zero_bytes, cnorm, beside, nblk, total, smem,
             (unsigned)(runs ? resident * sms : total), st);
 }

@@ -405,6 +405,17 @@ def test_indices_by_the_norm_table_equal_those_of_the_direct_form(B, H, N, d, M,
         assert torch.equal(inter["parent_idx"], pi) and torch.equal(inter["child_idx"], ci)
 
 
+@pytest.mark.parametrize("H,N,d,M", [(24, 1200, 128, 32), (10, 3000, 128, 256), (37, 2001, 64, 96)])
+def test_eight_children_over_sorted_keys_equal_the_cuda_core_assignment(H, N, d, M):
+    """Large grids take eight children by products over keys in the order of their parents: the indices of the CUDA-core
+    kernel, which measures every child directly, also with near-ties (an offset) and duplicated children."""
+    for offset in (0.0, 32.0):
+        K, Cp, Cc = _offset_inputs(1, H, N, d, M, 8, offset, seed=d + M + N)
+        pi, ci = binding.assign(K, Cp, Cc)
+        pr, cr = binding.assign(K, Cp, Cc, flags=binding.FLAG_SIMT)
+        assert torch.equal(pi, pr) and torch.equal(ci, cr)
+
+
 def test_a_common_offset_costs_little_time():
     """Offsets that bf16 still resolves make the products of the assignment separate less; what they leave open is decided in
     float32 before float64 is asked.  (2.7 times the time of centred inputs with float64 straight away, 1.3 with
