@@ -20,6 +20,20 @@ __device__ __forceinline__ void select_parents(const double* w, int M, int P, in
   const unsigned long long* key = reinterpret_cast<const unsigned long long*>(w);
   if (P >= M) {
     for (int j = tid; j < M; j += kSelThreads) sel[j] = 1;
+  } else if (4 * M <= kSelThreads) {
+    // Few parents: four or more threads rank each of them at once, without a bound and its barriers.
+    int lt = 2;                                             // 2^lt threads share a parent's scan
+    while (lt < 4 && (M << (lt + 1)) <= kSelThreads) ++lt;
+    const int j = tid >> lt, part = tid & ((1 << lt) - 1);
+    const unsigned long long kj = key[min(j, M - 1)];
+    int rank = 0;
+#pragma unroll 4
+    for (int k = part; k < M; k += 1 << lt) {
+      const unsigned long long kk = key[k];
+      rank += (kk > kj) | ((kk == kj) & (k < j));
+    }
+    for (int o = 1; o < (1 << lt); o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (j < M && part == 0 && rank < P) sel[j] = 1;
   } else {
     unsigned long long bound = 0;
     {

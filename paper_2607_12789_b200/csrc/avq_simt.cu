@@ -514,6 +514,7 @@ struct AttendArgs {
   int correcting; // Algorithm 2's literal child pass: mean-recovered parent logit and Delta A = A_c - A_p
   int tile_m;     // 0: exact importance; else parents visited in tiles of tile_m (Eq. "aproxdenom")
   int Nk;
+  uint32_t inv_C; // 2^18 / C rounded up: e / C = e inv_C >> 18 for e < 2^13, C <= 16
   int keep;       // the block's parent logits stay in shared memory between the passes
   float scale;
 };
@@ -560,6 +561,12 @@ __host__ __device__ inline AttendSmem attend_smem_layout(int RT, int DT, int d, 
   return L;
 }
 
+// Logits of columns without keys become -inf: their weight is then exp(-inf) = 0 against any reference, without a branch per
+// element around the exponential.
+__device__ __forceinline__ void mask_empty(float (&acc)[4], const float (&cnt)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) acc[j] = cnt[j] > 0.f ? acc[j] : -INFINITY;
+}
 __device__ __forceinline__ float max16(float v) {         // over the 16 threads of a row
 #pragma unroll
   for (int o = 8; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -720,16 +727,17 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         for (int j = 0; j < 4; ++j) cnt[j] = tx + 16 * j < n ? npS[c0 + tx + 16 * j] : 0.f;
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
+          mask_empty(acc[i], cnt);
           float mx = -INFINITY;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
+          for (int j = 0; j < 4; ++j) mx = fmaxf(mx, acc[i][j]);
           mx = max16(mx);
           if (mx > m[i]) {                                // uniform over the 16 threads of the row
             z[i] *= expf(m[i] - mx);
             m[i] = mx;
           }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) z[i] = fmaf(expf(acc[i][j] - m[i]), cnt[j], z[i]);
+          for (int j = 0; j < 4; ++j) z[i] = fmaf(expf(acc[i][j] - m[i]), cnt[j], z[i]);
         }
         c0 += n;
         __syncthreads();
@@ -748,14 +756,23 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         float acc[RT][4];
         if (a.keep) load_s(ss + (size_t)c0 * ldr, acc);
         else logits(acc, ss, n, [&](int c) { return Cph + (size_t)(c0 + c) * d; });
+        float cnt[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cnt[j] = tx + 16 * j < n ? npS[c0 + tx + 16 * j] : 0.f;
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {                    // (rows past the end: their weights do not count)
+          mask_empty(acc[i], cnt);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float e = expf(acc[i][j] - m[i]);
+            acc[i][j] = rt * R + row_of(i) < rows ? e : 0.f;
+          }
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           double s = 0.0;
-          if (tx + 16 * j < n && npS[c0 + tx + 16 * j] > 0.f) {
 #pragma unroll
-            for (int i = 0; i < RT; ++i)
-              if (rt * R + row_of(i) < rows) s = fma((double)expf(acc[i][j] - m[i]), inv[i], s);
-          }
+          for (int i = 0; i < RT; ++i) s = fma((double)acc[i][j], inv[i], s);
           s += __shfl_xor_sync(0xffffffffu, s, 16);
           if (lane < 16) wpart[warp * kCols + tx + 16 * j] = s;
         }
@@ -793,6 +810,10 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   // ---- pass C: merged softmax over unrefined parents, stay residuals and children of refined parents
   T* Yb = static_cast<T*>(a.Y) + ((size_t)bh * a.Nq + i0) * d;
   const int child_w = (kCols / C) * C;                    // whole families per tile
+  auto child_row = [&](int e) {                           // e-th child of the selected parents
+    const int f = (int)(((uint32_t)e * a.inv_C) >> 18);
+    return sel_list[f] * C + (e - f * C);
+  };
   const int vch = d >> 2;
   for (int rt = 0; rt < nrt; ++rt) {
     if (rt > 0 || (nrt > 1 && need_w)) { __syncthreads(); load_q(rt); }
@@ -805,11 +826,25 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
 #pragma unroll
         for (int j = 0; j < 4; ++j) o[t][i][j] = 0.f;
     }
-    // value rows of a tile (padding rows and columns zero): vs[c][k]
-    auto load_v = [&](auto val) {
+    // Value rows of a tile (padding rows and columns zero): vs[c][k], copied without waiting, except a refined parent's (the sum
+    // of the keys that stay).  row(c): the row's address, nullptr for zeros; stay(c): it is to be reduced by its children's.
+    auto load_v = [&](auto row, auto stay) {
       for (int u = tid; u < kCols * (ldv / 4); u += kThreads) {
         const int c = u / (ldv / 4), ch = u - c * (ldv / 4);
-        *reinterpret_cast<float4*>(vs + c * ldv + 4 * ch) = ch < vch ? val(c, ch) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float* to = vs + c * ldv + 4 * ch;
+        const float* from = ch < vch ? row(c) : nullptr;
+        if (from == nullptr) {
+          *reinterpret_cast<float4*>(to) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else if (const float* child = stay(c)) {
+          float4 v = ld_after_wait(reinterpret_cast<const float4*>(from) + ch);
+          for (int cc = 0; cc < C; ++cc) {
+            const float4 x = ld_after_wait(reinterpret_cast<const float4*>(child + (size_t)cc * d) + ch);
+            v.x -= x.x; v.y -= x.y; v.z -= x.z; v.w -= x.w;
+          }
+          *reinterpret_cast<float4*>(to) = v;
+        } else {
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(to)), "l"(from + 4 * ch) : "memory");
+        }
       }
     };
     const int ptiles = (M + kCols - 1) / kCols;
@@ -820,34 +855,22 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       const int n = child ? min(child_w, P * C - c0) : min(kCols, M - c0);
       float acc[RT][4], cnt[4];
       float* sw = ss;                                     // weights of this tile, [column][row]
-      auto val_parent = [&](int c, int ch) {
-        const int j = c0 + c;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < n) {
-          const bool refined = sel[j] != 0 && !CORR;
-          const float nn = refined ? (a.stays ? nstay[j] : 0.f) : npS[j];
-          if (nn > 0.f) {
-            v = ld_after_wait(reinterpret_cast<const float4*>(Vp + (size_t)j * d) + ch);
-            if (refined)
-              for (int cc = 0; cc < C; ++cc) {
-                const float4 x = ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)j * C + cc) * d) + ch);
-                v.x -= x.x; v.y -= x.y; v.z -= x.z; v.w -= x.w;
-              }
-          }
+      auto load_values = [&]() {
+        if (child) {
+          load_v([&](int c) { return c < n ? Vc + (size_t)child_row(c0 + c) * d : nullptr; },
+                 [](int) { return (const float*)nullptr; });
+        } else {
+          load_v([&](int c) -> const float* {
+                   if (c >= n) return nullptr;
+                   const bool refined = sel[c0 + c] != 0 && !CORR;
+                   return (refined ? (a.stays ? nstay[c0 + c] : 0.f) : npS[c0 + c]) > 0.f ? Vp + (size_t)(c0 + c) * d : nullptr;
+                 },
+                 [&](int c) { return sel[c0 + c] && !CORR ? Vc + (size_t)(c0 + c) * C * d : nullptr; });
         }
-        return v;
       };
-      auto val_child = [&](int c, int ch) {
-        if (c >= n) return make_float4(0.f, 0.f, 0.f, 0.f);
-        const int e = c0 + c, p = sel_list[e / C];
-        return ld_after_wait(reinterpret_cast<const float4*>(Vc + ((size_t)p * C + e % C) * d) + ch);
-      };
-      if (DT <= 2) {                                      // its own buffer: loads fly together with the codewords'
-        if (child) load_v(val_child);
-        else load_v(val_parent);
-      }
+      if (DT <= 2) load_values();                         // its own buffer: the copies fly with the codewords' loads
       if (child) {
-        logits(acc, sw, n, [&](int c) { const int e = c0 + c; return Cch + ((size_t)sel_list[e / C] * C + e % C) * d; });
+        logits(acc, sw, n, [&](int c) { return Cch + (size_t)child_row(c0 + c) * d; });
       } else if (a.keep && need_w) {
         sw = ss + (size_t)c0 * ldr;                       // the tile's logits, overwritten by its weights
         load_s(sw, acc);
@@ -860,8 +883,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         cnt[j] = 0.f;
         if (c < n) {
           if (child) {
-            const int e = c0 + c;
-            cnt[j] = ld_after_wait(nc + (size_t)sel_list[e / C] * C + e % C);
+            cnt[j] = ld_after_wait(nc + child_row(c0 + c));
           } else {
             // correcting form: every parent keeps its full term here, the children add differences below
             cnt[j] = (sel[c0 + c] && !CORR) ? (a.stays ? nstay[c0 + c] : 0.f) : npS[c0 + c];
@@ -888,9 +910,10 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       }
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
+        mask_empty(acc[i], cnt);
         float mx = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) if (cnt[j] > 0.f) mx = fmaxf(mx, acc[i][j]);
+        for (int j = 0; j < 4; ++j) mx = fmaxf(mx, acc[i][j]);
         mx = max16(mx);
         if (mx > m[i]) {
           const float alpha = expf(m[i] - mx);
@@ -903,20 +926,18 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          float av = 0.f;
-          if (cnt[j] > 0.f) {
-            av = expf(acc[i][j] - m[i]);
-            if (CORR && child) av -= expf(mean[CORR ? i : 0][j] - m[i]);
-            z[i] = fmaf(av, cnt[j], z[i]);
-          }
+          float av = expf(acc[i][j] - m[i]);
+          if (CORR && child) av = cnt[j] > 0.f ? av - expf(mean[CORR ? i : 0][j] - m[i]) : 0.f;
+          z[i] = fmaf(av, cnt[j], z[i]);
           acc[i][j] = av;
         }
       }
       store_s(sw, acc);
+      if (DT <= 2) tc::cp_async_wait_all();
       __syncthreads();
       if (DT > 2) {                                       // shared buffer: the codewords are done with
-        if (child) load_v(val_child);
-        else load_v(val_parent);
+        load_values();
+        tc::cp_async_wait_all();
         __syncthreads();
       }
 #pragma unroll
@@ -1067,6 +1088,7 @@ avq_status simt_attend(const avq_problem& p, const void* Q, const void* Cp, cons
   a.stays = (p.flags & AVQ_FLAG_PARENT_STAYS) ? 1 : 0;
   a.correcting = (p.flags & AVQ_FLAG_CORRECTING) ? 1 : 0;
   a.keep = 0;
+  a.inv_C = ((1u << 18) + (uint32_t)p.C - 1) / (uint32_t)p.C;
   a.scale = p.scale;
   return p.dtype == AVQ_F32 ? launch_attend<float>(a, p.B, chained, st)
                             : launch_attend<__nv_bfloat16>(a, p.B, chained, st);
