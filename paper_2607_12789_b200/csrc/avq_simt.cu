@@ -55,11 +55,11 @@ constexpr int kLdC = kCols + 4;    // row pitch of a [k][column] operand, floats
 // the shared-memory operand, so that a narrow tile costs only the columns it has.
 __device__ __forceinline__ int code_pos(int c) { return ((c & 15) << 2) | (c >> 4); }
 
-// Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][r] (CODES: dst[k][code_pos(r)]), k < d: the transposed
+// Copies `rows` rows of d elements (row r at src(r), nullptr = zeros) into dst[k][place(r)], k < d: the transposed
 // operand of the register-tiled products.  A warp takes 8 rows x 4 chunks of 4 elements: 64-byte pieces of a
 // row in global memory, at most two-way bank conflicts in shared memory.
-template <int THREADS, int BATCH, bool CODES, typename Src>
-__device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Src src) {
+template <int THREADS, int BATCH, typename Place, typename Src>
+__device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, int d, Place place, Src src) {
   constexpr int kWarps = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kc = lane & 3, rr = lane >> 2;
@@ -74,7 +74,7 @@ __device__ __forceinline__ void load_transposed(float* dst, int ld, int rows, in
       at[e] = -1;
       v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (ue < units && c < chunks) {
-        at[e] = 4 * c * ld + (CODES ? code_pos(r) : r);
+        at[e] = 4 * c * ld + place(r);
         const auto* p = src(r);
         if (p) v[e] = ld4(p + 4 * c);
       }
@@ -153,6 +153,18 @@ __device__ double exact_dist(const T* krow, const T* c, int d) {
   return s;
 }
 
+// The same asynchronously (cp.async; the caller waits), each row in pieces of 8 bytes.
+template <int THREADS, typename Src>
+__device__ __forceinline__ void load_rows_async(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
+  const int per = dpad >> 2;
+  for (int u = threadIdx.x; u < rows * per; u += THREADS) {
+    const int r = u / per, c = u - r * per;
+    const __nv_bfloat16* p = src(r);
+    const bool there = p != nullptr && 4 * c < d;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(dst + r * pitch + 4 * c)),
+                 "l"(there ? p + 4 * c : src(0)), "r"(there ? 8 : 0) : "memory");
+  }
+}
 // `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
 template <int THREADS, typename Src>
 __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
@@ -213,10 +225,14 @@ __device__ __forceinline__ void mma_block(float* s, int ldr, const __nv_bfloat16
 // ------------------------------------------------------------------------------- assign
 constexpr int kAssignKeys = 64;    // keys per CTA
 
-// Shared memory: float32, keys and codewords as [k][row]; bfloat16, both as rows, and the products [column][key]; norms.
+// bfloat16: the next tile of codewords is copied while one is used, as long as that leaves two CTAs on an SM (H4 N4096 M512, this
+// kernel, us, waiting for each tile and copying ahead: d128 43.9 and 39.3, d256 68.6 and 82.9).
+__host__ __device__ inline bool assign_two_tiles(int d) { return d <= 192; }
+// Shared memory: float32, keys and codewords as [k][row]; bfloat16, both as rows, two tiles of codewords, and the products
+// [column][key]; norms.
 __host__ __device__ inline size_t assign_smem_floats(int d, bool mma) {
   if (!mma) return 2 * (size_t)d * kLdC + kAssignKeys + kCols;
-  return 2 * (size_t)kAssignKeys * ((size_t)(d + 15) / 16 * 8 + 4) + (size_t)kCols * kLdC + kAssignKeys + kCols;
+  return (assign_two_tiles(d) ? 3 : 2) * (size_t)kAssignKeys * ((size_t)(d + 15) / 16 * 8 + 4) + (size_t)kCols * kLdC + kAssignKeys + kCols;
 }
 
 // Parents: 64 keys x 64 codewords at a time, ||k||^2 + ||c||^2 - 2 k.c with float64 rechecks; bfloat16 products on the
@@ -233,7 +249,9 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const int dpad = (d + 15) & ~15, pitch = dpad + 8;
   float* ks = smem;                                               // [d][kLdC] keys, or rows of pitch bfloat16
   float* cs = ks + (kMma ? (size_t)kAssignKeys * pitch / 2 : (size_t)d * kLdC);   // codewords of the current tile, alike
-  float* prod = cs + (size_t)kCols * pitch / 2;                   // bfloat16: [kCols][kLdC] products
+  const bool two = kMma && assign_two_tiles(d);
+  float* cs_next = two ? cs + (size_t)kCols * pitch / 2 : cs;     // bfloat16: of the tile behind it, on their way
+  float* prod = cs_next + (size_t)kCols * pitch / 2;              // bfloat16: [kCols][kLdC] products
   float* kn = kMma ? prod + (size_t)kCols * kLdC : cs + (size_t)d * kLdC;   // [kAssignKeys] key norms
   float* cn = kn + kAssignKeys;                                   // [kCols] codeword norms (float32: by code_pos)
   __shared__ int s_par[kAssignKeys];
@@ -251,8 +269,24 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const int rows = min(kAssignKeys, Nk - j0);
   const T* Cph = Cp + (size_t)h * M * d;
   auto key_row = [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; };
-  if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(ks), pitch, kAssignKeys, d, dpad, key_row);
-  else load_transposed<kThreads, 4, false>(ks, kLdC, kAssignKeys, d, key_row);
+  auto load_codes = [&](float* to, int m0) {              // bfloat16: a tile of codewords, not waited for
+    const int w = min(kCols, M - m0);
+    load_rows_async<kThreads>(reinterpret_cast<__nv_bfloat16*>(to), pitch, kCols, d, dpad, [&](int r) {
+      return r < w ? reinterpret_cast<const __nv_bfloat16*>(Cph) + (size_t)(m0 + r) * d : (const __nv_bfloat16*)nullptr;
+    });
+  };
+  if constexpr (kMma) {
+    load_codes(cs, 0);
+    load_rows<kThreads>(reinterpret_cast<T*>(ks), pitch, kAssignKeys, d, dpad, key_row);
+  } else {                                                // the keys and the first codewords in one go (cs is behind ks)
+    const int w = min(kCols, M);
+    load_transposed<kThreads, 8>(ks, kLdC, kAssignKeys + code_rows(w), d,
+                                 [&](int r) { return r < kAssignKeys ? r : d * kLdC + code_pos(r - kAssignKeys); },
+                                 [&](int r) {
+                                   if (r < kAssignKeys) return key_row(r);
+                                   return r - kAssignKeys < w ? Cph + (size_t)(r - kAssignKeys) * d : (const T*)nullptr;
+                                 });
+  }
   // squared norm of a staged row (float32: column), four lanes per row (row tid / 4)
   auto row_norm = [&](const float* base) {
     float s = 0.f;
@@ -281,11 +315,21 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   for (int i = 0; i < 4; ++i) { d1[i] = INFINITY; d2[i] = INFINITY; i1[i] = 0; }
   for (int m0 = 0; m0 < M; m0 += kCols) {
     const int w = min(kCols, M - m0);
-    if (m0 > 0) __syncthreads();
-    auto code_row = [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; };
-    if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(cs), pitch, kCols, d, dpad, code_row);
-    else load_transposed<kThreads, 4, true>(cs, kLdC, code_rows(w), d, code_row);
-    __syncthreads();
+    if (!kMma && m0 > 0) __syncthreads();
+    if constexpr (kMma) {
+      if (m0 > 0) {
+        if (two) { float* t = cs; cs = cs_next; cs_next = t; }
+        else { __syncthreads(); load_codes(cs, m0); }
+      }
+      tc::cp_async_wait_all();
+      __syncthreads();
+      if (two && m0 + kCols < M) load_codes(cs_next, m0 + kCols);   // (the tile before has been read)
+    } else {
+      if (m0 > 0)
+        load_transposed<kThreads, 4>(cs, kLdC, code_rows(w), d, [](int r) { return code_pos(r); },
+                                     [&](int r) { return r < w ? Cph + (size_t)(m0 + r) * d : (const T*)nullptr; });
+      __syncthreads();
+    }
     float acc[4][4] = {};
     if (m0 == 0) {
       const float s = row_norm(ks);
@@ -373,54 +417,63 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   const int key = tid >> 2, s4 = tid & 3;
   const int par = s_par[key];
   const T* Cch = Cc + ((size_t)h * M + par) * C * d;
-  // distance to one codeword row, this lane's chunks; four loads in flight
-  auto dist_part = [&](const T* c) {
-    float s = 0.f;
-    for (int c0 = s4; c0 < (d >> 2); c0 += 16) {
-      float4 v[4];
+  // distances to nr (at most 4) codeword rows c, c + d, ..., this lane's chunks; all loads of 64 elements in flight
+  auto dist_part = [&](const T* c, auto nr, int rows_there, float (&sum)[decltype(nr)::value]) {
+    constexpr int N = decltype(nr)::value;
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (c0 + 4 * e < (d >> 2)) v[e] = ld4(c + 4 * (c0 + 4 * e));
+    for (int x = 0; x < N; ++x) sum[x] = 0.f;
+    for (int c0 = s4; c0 < (d >> 2); c0 += 16) {
+      float4 v[N][4];
+#pragma unroll
+      for (int x = 0; x < N; ++x)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (x < rows_there && c0 + 4 * e < (d >> 2)) v[x][e] = ld4(c + (size_t)x * d + 4 * (c0 + 4 * e));
 #pragma unroll
       for (int e = 0; e < 4; ++e)
         if (c0 + 4 * e < (d >> 2)) {
           const int k = 4 * (c0 + 4 * e);
-          float4 x;
+          float4 kv;
           if constexpr (kMma) {
             const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const T*>(ks) + key * pitch + k);
-            x = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
-                            __uint_as_float(u.y & 0xFFFF0000u));
+            kv = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                             __uint_as_float(u.y & 0xFFFF0000u));
           } else {
             const float* kp = ks + (size_t)k * kLdC + key;
-            x = make_float4(kp[0], kp[kLdC], kp[2 * kLdC], kp[3 * kLdC]);
+            kv = make_float4(kp[0], kp[kLdC], kp[2 * kLdC], kp[3 * kLdC]);
           }
-          x.x -= v[e].x; x.y -= v[e].y; x.z -= v[e].z; x.w -= v[e].w;
-          s = fmaf(x.x, x.x, s); s = fmaf(x.y, x.y, s); s = fmaf(x.z, x.z, s); s = fmaf(x.w, x.w, s);
+#pragma unroll
+          for (int x = 0; x < N; ++x)
+            if (x < rows_there) {
+              const float4 y = make_float4(kv.x - v[x][e].x, kv.y - v[x][e].y, kv.z - v[x][e].z, kv.w - v[x][e].w);
+              sum[x] = fmaf(y.x, y.x, sum[x]); sum[x] = fmaf(y.y, y.y, sum[x]);
+              sum[x] = fmaf(y.z, y.z, sum[x]); sum[x] = fmaf(y.w, y.w, sum[x]);
+            }
         }
     }
-    return s;
+#pragma unroll
+    for (int x = 0; x < N; ++x) {                         // the four lanes
+      sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], 1);
+      sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], 2);
+    }
   };
   float e1 = INFINITY, e2 = INFINITY;
   int c1 = 0;
-  for (int c = 0; c < C; c += 2) {                        // two children at a time
-    float sa = dist_part(Cch + (size_t)c * d);
-    float sb = c + 1 < C ? dist_part(Cch + (size_t)(c + 1) * d) : INFINITY;
-    sa += __shfl_xor_sync(0xffffffffu, sa, 1);
-    sb += __shfl_xor_sync(0xffffffffu, sb, 1);
-    sa += __shfl_xor_sync(0xffffffffu, sa, 2);
-    sb += __shfl_xor_sync(0xffffffffu, sb, 2);
-    if (sa < e1) { e2 = e1; e1 = sa; c1 = c; }
-    else if (sa < e2) { e2 = sa; }
-    if (c + 1 < C) {
-      if (sb < e1) { e2 = e1; e1 = sb; c1 = c + 1; }
-      else if (sb < e2) { e2 = sb; }
-    }
+  for (int c = 0; c < C; c += 4) {                        // four children at a time
+    float sum[4];
+    dist_part(Cch + (size_t)c * d, std::integral_constant<int, 4>{}, C - c, sum);
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      if (c + x < C) {
+        if (sum[x] < e1) { e2 = e1; e1 = sum[x]; c1 = c + x; }
+        else if (sum[x] < e2) { e2 = sum[x]; }
+      }
   }
   float dpar = 0.f;                                       // the parent's distance in the same form
   if (parent_stays) {
-    dpar = dist_part(Cph + (size_t)par * d);
-    dpar += __shfl_xor_sync(0xffffffffu, dpar, 1);
-    dpar += __shfl_xor_sync(0xffffffffu, dpar, 2);
+    float sum[1];
+    dist_part(Cph + (size_t)par * d, std::integral_constant<int, 1>{}, 1, sum);
+    dpar = sum[0];
   }
   double dc64 = -1.0;
   const bool redo = C > 1 && key < rows && !(e2 - e1 > kNearTie * e2);
@@ -629,7 +682,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
   auto load_q = [&](int rt) {
     auto row = [&](int r) { return rt * R + r < rows ? Qb + (size_t)(rt * R + r) * d : (const T*)nullptr; };
     if constexpr (kMma) load_rows<kThreads>(reinterpret_cast<T*>(qs), pitch, R, d, dpad, row);
-    else load_transposed<kThreads, WIDE ? 4 : 2, false>(qs, ldr, R, d, row);
+    else load_transposed<kThreads, WIDE ? 4 : 2>(qs, ldr, R, d, [](int r) { return r; }, row);
   };
   auto store_s = [&](float* s0, const float (&acc)[RT][4]) {
 #pragma unroll
@@ -667,7 +720,7 @@ __global__ void __launch_bounds__(kAttThreads, (DT == 1 && !CORR && !WIDE) ? 2 :
       __syncthreads();
       load_s(s0, acc);
     } else {
-      load_transposed<kThreads, 2, true>(cs, kLdC, code_rows(n), d, row);
+      load_transposed<kThreads, 2>(cs, kLdC, code_rows(n), d, [](int c) { return code_pos(c); }, row);
       __syncthreads();
 #pragma unroll
       for (int i = 0; i < RT; ++i)
