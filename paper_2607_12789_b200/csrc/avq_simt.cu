@@ -153,16 +153,21 @@ __device__ double exact_dist(const T* krow, const T* c, int d) {
   return s;
 }
 
-// The same asynchronously (cp.async; the caller waits), each row in pieces of 8 bytes.
-template <int THREADS, typename Src>
+// The same asynchronously (cp.async; the caller waits), each row in pieces of 16 bytes (8 where d is no multiple of 8).
+template <int THREADS, int PIECE, typename Src>
 __device__ __forceinline__ void load_rows_async(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
-  const int per = dpad >> 2;
-  for (int u = threadIdx.x; u < rows * per; u += THREADS) {
-    const int r = u / per, c = u - r * per;
+  const int per = dpad / PIECE, step_r = THREADS / per, step_c = THREADS - step_r * per;
+  int r = threadIdx.x / per, c = threadIdx.x - r * per;
+  for (; r < rows; r += step_r, c += step_c) {
+    if (c >= per) { c -= per; if (++r >= rows) break; }
     const __nv_bfloat16* p = src(r);
-    const bool there = p != nullptr && 4 * c < d;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(dst + r * pitch + 4 * c)),
-                 "l"(there ? p + 4 * c : src(0)), "r"(there ? 8 : 0) : "memory");
+    const bool there = p != nullptr && PIECE * c < d;
+    const uint32_t to = tc::smem_u32(dst + r * pitch + PIECE * c);
+    const __nv_bfloat16* from = there ? p + PIECE * c : src(0);
+    if constexpr (PIECE == 8)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
+    else
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(to), "l"(from), "r"(there ? 8 : 0) : "memory");
   }
 }
 // `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
@@ -271,9 +276,11 @@ assign_simt_kernel(const T* __restrict__ K, const T* __restrict__ Cp, const T* _
   auto key_row = [&](int r) { return r < rows ? Kb + (size_t)r * d : (const T*)nullptr; };
   auto load_codes = [&](float* to, int m0) {              // bfloat16: a tile of codewords, not waited for
     const int w = min(kCols, M - m0);
-    load_rows_async<kThreads>(reinterpret_cast<__nv_bfloat16*>(to), pitch, kCols, d, dpad, [&](int r) {
+    auto row = [&](int r) {
       return r < w ? reinterpret_cast<const __nv_bfloat16*>(Cph) + (size_t)(m0 + r) * d : (const __nv_bfloat16*)nullptr;
-    });
+    };
+    if (d % 8 == 0) load_rows_async<kThreads, 8>(reinterpret_cast<__nv_bfloat16*>(to), pitch, kCols, d, dpad, row);
+    else load_rows_async<kThreads, 4>(reinterpret_cast<__nv_bfloat16*>(to), pitch, kCols, d, dpad, row);
   };
   if constexpr (kMma) {
     load_codes(cs, 0);
