@@ -648,7 +648,8 @@ __device__ __forceinline__ float sum16(float v) {
 // logit, operands read from global memory for every product: whole forward fp32 B2 H12 N1024 d64 M64 C4 P8
 // 2660 -> 82 us, tiled bf16 B1 H4 N4096 d64 M512 C4 P64 12.1 -> 0.36 ms (84 us and 0.40 ms with
 // 256 threads); with the bfloat16 logits on the tensor cores 0.27 ms; with the steps since (narrow tiles, candidates only
-// ranked, packed multiply-adds, importance tile by tile) 78 us and 0.185 ms.
+// ranked, packed multiply-adds, importance tile by tile) 78 us and 0.185 ms; without branches around the exponentials, value
+// rows copied asynchronously and small selections ranked at once, 74.6 us (the tiled one has a kernel of its own).
 // 512 threads with 4 rows each rather than 256 with 8: the same products per second, twice the warps for everything
 // that is a latency (operand loads, exponentials, exchanges), which was most of the time.
 // WIDE: one CTA per SM with twice the registers, for grids of a wave at most (they measured 3 % faster there, fp32
