@@ -542,11 +542,12 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       if (tid < M) {
         const int c = parent_pos(tid);
         wj = cnt[c] * ((wpart[c] + wpart[CT + c]) + (wpart[2 * CT + c] + wpart[3 * CT + c]));
-        w[tid] = wj;
+        w[tid] = fabsf(wj);                              // (a NaN's sign would not order)
         const uint32_t m_ = __ballot_sync(0xffffffffu, wj > 0.f);   // M is a multiple of 32
         if (lane == 0) { nzmask[warp] = m_; selmask[warp] = 0u; }
         if (p.importance_out) p.importance_out[((size_t)bh * p.nblk + blk) * M + tid] = wj;
       }
+      if (CT <= 64 && tid >= M && tid < CT) w[tid] = 0.f;
       if (tid == 0) *ncand_s = 0;
       key = __float_as_uint(wj);
       nz = __syncthreads_count(wj > 0.f);
@@ -584,55 +585,80 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           }
         }
       } else {
-        // Only candidates are ranked, those at or above a bound that at least P keys reach.  The bound is the
-        // largest of 32 sample keys (the first 32 parents') that has at least P keys at or above it, else the
-        // smallest key above zero; each warp counts for its share of the samples.
-        constexpr int kPer = 32 / (kThreads / 32);       // samples per warp
-        uint32_t kk[CT / 32];
+        int rank = P, j = 0;                             // parent j of this thread, if it is to be listed
+        if constexpr (CT <= 64) {
+          // Few parents: 2^kLt threads rank each of them against a share of the others, with no barrier in between.
+          // (Candidates as below and all parents so, us per call: H16 N20000 d64 M32 C8 85.2 and 82.6, N65536 M64 259.8 and
+          // 256.4, B1 H12 N785 M64 19.0 and 18.6; but N20000 M128 137.2 and 140.7, N9000 M96 71.1 and 73.3.)
+          constexpr int kLt = kThreads / CT == 2 ? 1 : 2, kShare = CT >> kLt;
+          static_assert((CT << kLt) == kThreads, "every thread has a parent and a share");
+          const int part = tid & ((1 << kLt) - 1);
+          j = tid >> kLt;
+          const uint32_t mine = reinterpret_cast<const uint32_t*>(w)[j];   // (zero from M on: above no other)
+          int above = 0;
 #pragma unroll
-        for (int k = 0; k < CT / 32; ++k) kk[k] = k < K ? reinterpret_cast<const uint32_t*>(w)[32 * k + lane] : 0u;
+          for (int v = 0; v < kShare / 4; ++v) {
+            const uint4 x = reinterpret_cast<const uint4*>(w)[part * (kShare / 4) + v];
+            const int k = part * kShare + 4 * v;
+            above += (x.x + (k < j) > mine) + (x.y + (k + 1 < j) > mine) + (x.z + (k + 2 < j) > mine) + (x.w + (k + 3 < j) > mine);
+          }
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-          const uint32_t smp = __shfl_sync(0xffffffffu, kk[0], warp * kPer + j);
-          int c = 0;
+          for (int o = 1; o < (1 << kLt); o <<= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
+          if (part == 0) rank = above;
+        } else {
+          // Only candidates are ranked, those at or above a bound that at least P keys reach.  The bound is the
+          // largest of 32 sample keys (the first 32 parents') that has at least P keys at or above it, else the
+          // smallest key above zero; each warp counts for its share of the samples.
+          constexpr int kPer = 32 / (kThreads / 32);       // samples per warp
+          uint32_t kk[CT / 32];
 #pragma unroll
-          for (int k = 0; k < CT / 32; ++k) c += kk[k] >= smp;
-          c = __reduce_add_sync(0xffffffffu, c);
-          if (lane == 0) wcount[warp * kPer + j] = smp > 0u ? c : 0;
-        }
-        __syncthreads();
-        const uint32_t bound = max(__reduce_max_sync(0xffffffffu, wcount[lane] >= P ? kk[0] : 0u), 1u);
-        if (warp < K) {                                  // candidates of this warp's 32 parents -> list, in any order
-          const uint32_t mk = __ballot_sync(0xffffffffu, key >= bound);
-          int base = 0;
-          if (lane == 0) base = atomicAdd(ncand_s, __popc(mk));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          // importance above, complement of the index below: larger means refined earlier, no two are equal
-          if ((mk >> lane) & 1u) cand[base + __popc(mk & below)] = ((uint64_t)key << 32) | (uint32_t)(0xFFFF - tid);
-        }
-        __syncthreads();
-        // rank of every candidate among them; 2^lt threads share a candidate.  The list of refined parents is
-        // ordered by rank.
-        const int ncand = *ncand_s;
-        constexpr int kLogT = NQ == 4 ? 9 : (NQ == 2 ? 8 : 7);
-        const int lt = max(0, min(4, kLogT - (32 - __clz(ncand - 1))));
-        const int i = tid >> lt, part = tid & ((1 << lt) - 1);
-        const uint64_t mine = i < ncand ? cand[i] : 0;
-        int rank = 0;
-        for (int k = part; k < ncand; k += 4 << lt) {    // four in flight; past the end only the comparison is masked
+          for (int k = 0; k < CT / 32; ++k) kk[k] = k < K ? reinterpret_cast<const uint32_t*>(w)[32 * k + lane] : 0u;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int ku = k + (u << lt);
-            rank += (cand[min(ku, CT - 1)] > mine) & (ku < ncand);
+          for (int e = 0; e < kPer; ++e) {
+            const uint32_t smp = __shfl_sync(0xffffffffu, kk[0], warp * kPer + e);
+            int c = 0;
+#pragma unroll
+            for (int k = 0; k < CT / 32; ++k) c += kk[k] >= smp;
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0) wcount[warp * kPer + e] = smp > 0u ? c : 0;
+          }
+          __syncthreads();
+          const uint32_t bound = max(__reduce_max_sync(0xffffffffu, wcount[lane] >= P ? kk[0] : 0u), 1u);
+          if (warp < K) {                                  // candidates of this warp's 32 parents -> list, in any order
+            const uint32_t mk = __ballot_sync(0xffffffffu, key >= bound);
+            int base = 0;
+            if (lane == 0) base = atomicAdd(ncand_s, __popc(mk));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            // importance above, complement of the index below: larger means refined earlier, no two are equal
+            if ((mk >> lane) & 1u) cand[base + __popc(mk & below)] = ((uint64_t)key << 32) | (uint32_t)(0xFFFF - tid);
+          }
+          __syncthreads();
+          // rank of every candidate among them; 2^lt threads share a candidate.  The list of refined parents is
+          // ordered by rank.
+          const int ncand = *ncand_s;
+          constexpr int kLogT = NQ == 4 ? 9 : (NQ == 2 ? 8 : 7);
+          const int lt = max(0, min(4, kLogT - (32 - __clz(ncand - 1))));
+          const int i = tid >> lt, part = tid & ((1 << lt) - 1);
+          const uint64_t mine = i < ncand ? cand[i] : 0;
+          int above = 0;
+          for (int k = part; k < ncand; k += 4 << lt) {    // four in flight; past the end only the comparison is masked
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int ku = k + (u << lt);
+              above += (cand[min(ku, CT - 1)] > mine) & (ku < ncand);
+            }
+          }
+#pragma unroll
+          for (int o = 1; o <= 8; o <<= 1) {
+            const int other = __shfl_xor_sync(0xffffffffu, above, o);
+            if (o < (1 << lt)) above += other;
+          }
+          if (i < ncand && part == 0) {
+            rank = above;
+            j = 0xFFFF - (int)((uint32_t)mine & 0xFFFFu);
           }
         }
-#pragma unroll
-        for (int o = 1; o <= 8; o <<= 1) {
-          const int other = __shfl_xor_sync(0xffffffffu, rank, o);
-          if (o < (1 << lt)) rank += other;
-        }
-        if (i < ncand && part == 0 && rank < P) {
-          const int j = 0xFFFF - (int)((uint32_t)mine & 0xFFFFu);
+        if (rank < P) {
           choose(j, rank);
           if (topp_out) atomicOr(&selmask[j >> 5], 1u << (j & 31));
         }
