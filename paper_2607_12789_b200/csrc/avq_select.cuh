@@ -55,8 +55,15 @@ __device__ __forceinline__ void select_parents(const double* w, int M, int P, in
         bound = other > bound ? other : bound;
       }
     }
-    for (int j = tid; j < M; j += kSelThreads)
-      if (key[j] >= bound) cand[atomicAdd(s_ncand, 1)] = j;   // in any order
+    for (int j0 = 0; j0 < M; j0 += kSelThreads) {            // in any order, one addition per warp
+      const int j = j0 + tid;
+      const bool on = j < M && key[j] >= bound;
+      const uint32_t bal = __ballot_sync(0xffffffffu, on);
+      int base = 0;
+      if (lane == 0 && bal) base = atomicAdd(s_ncand, __popc(bal));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (on) cand[base + __popc(bal & ((1u << lane) - 1u))] = j;
+    }
     sync();
     const int nc_ = *s_ncand;
     int lt = 0;                                             // 2^lt threads share a candidate's scan
@@ -80,13 +87,23 @@ __device__ __forceinline__ void select_parents(const double* w, int M, int P, in
     }
   }
   sync();
-  if (warp == 0) {
-    int base = 0;
-    for (int j = lane; j < ((M + 31) & ~31); j += 32) {
-      const bool on = j < M && sel[j] != 0;
-      const uint32_t bal = __ballot_sync(0xffffffffu, on);
-      if (on) sel_list[base + __popc(bal & ((1u << lane) - 1u))] = j;
-      base += __popc(bal);
+  // the ascending list: a warp per 32 parents (M <= 1024: at most 32 words of s_count)
+  const int words = (M + 31) >> 5;
+  uint32_t mine[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int j = 32 * (warp + 16 * u) + lane;
+    mine[u] = __ballot_sync(0xffffffffu, j < M && sel[min(j, M - 1)] != 0);
+    if (lane == 0) s_count[warp + 16 * u] = (int)mine[u];
+  }
+  sync();
+  const int ones = __popc((uint32_t)s_count[lane]);         // (words past the last are zero)
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int word = warp + 16 * u;
+    if (word < words) {
+      const int base = __reduce_add_sync(0xffffffffu, lane < word ? ones : 0);
+      if ((mine[u] >> lane) & 1u) sel_list[base + __popc(mine[u] & ((1u << lane) - 1u))] = 32 * word + lane;
     }
   }
   sync();
