@@ -36,6 +36,7 @@ constexpr int kIssuer = kCompute / 32;         // the warp that issues loads and
 constexpr int kThreadsT = kCompute + 32;
 constexpr int kTileBytes = kTile * kD * 2;     // rows of 128 bytes
 constexpr int kMaxTiles = 80;                  // M + P C <= 8192
+constexpr int kSlots = 8;                      // tiles described at a time (the reason: at describe() below)
 constexpr int kStayRow = 1 << 28, kChildRow = 1 << 29;
 // TMEM columns: two logit tiles, three weight parts, the value product
 constexpr int kColW = 256, kColO = 448;
@@ -66,8 +67,8 @@ __host__ __device__ inline TiledSmem tiled_smem_layout(int M, int P, int tile_m)
   L.raw = take(4 * kTile * kD);
   L.w = take(8 * (size_t)M);
   L.wpart = take(8 * 4 * kTile > 4 * (size_t)M ? 8 * 4 * kTile : 4 * (size_t)M);   // also the candidates of the selection
-  L.tcnt = take(4 * 4 * kTile);
-  L.trow = take(4 * 4 * kTile);
+  L.tcnt = take(kSlots * 4 * kTile);
+  L.trow = take(kSlots * 4 * kTile);
   L.np = take(4 * (size_t)M);
   L.nstay = take(4 * (size_t)M);
   L.xm = take(4 * 4 * kRows);
@@ -422,8 +423,13 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const int f = (int)(((uint32_t)e * a.inv_C) >> 18);
       return sel_list[f] * C + (e - f * C);
     };
-    // What stands behind column tid of tile k (prepared two tiles ahead, four tiles kept): the keys, and the row of their value
-    // sums, a child's (kChildRow) or a parent's, less the children's where the parent is refined (kStayRow); -1: none.
+    // What stands behind column tid of tile k: the keys, and the row of their value sums, a child's (kChildRow) or a parent's, less
+    // the children's where the parent is refined (kStayRow); -1: none.
+    // Tiles 0 to 2 are described before the loop, ahead of a barrier, tile k + 3 in turn k.  No barrier joins all warps in a
+    // turn; what orders them is take_product(k - 1) in turn k: it waits for a product that the issuing warp starts behind the
+    // arrivals of all warps in turn k - 1.  A warp in turn k therefore knows every other to be through turn k - 2, in which
+    // tile k + 1, the furthest it reads (load_values), was described.  And it overwrites the slot of tile k - 5, which was last read
+    // in turn k - 4 (a product on the CUDA cores, a turn behind its tile); six slots would do.
     auto describe = [&](int k) {
       if (tid >= kTile || k >= tiles) return;
       float n = 0.f;
@@ -439,8 +445,8 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           if (n > 0.f) row = sel[e] ? e | kStayRow : e;
         }
       }
-      tcnt[(k & 3) * kTile + tid] = n;
-      trow[(k & 3) * kTile + tid] = row;
+      tcnt[(k & (kSlots - 1)) * kTile + tid] = n;
+      trow[(k & (kSlots - 1)) * kTile + tid] = row;
     };
     // value sums 4 ch .. + 3 of such a row
     auto value_of = [&](int row, int ch) {
@@ -461,7 +467,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     auto load_values = [&](int k) {
       int row[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) row[i] = trow[(k & 3) * kTile + (tid >> 4) + 32 * i];
+      for (int i = 0; i < 4; ++i) row[i] = trow[(k & (kSlots - 1)) * kTile + (tid >> 4) + 32 * i];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const uint32_t dst = own_v + 16 * kCompute * i;
@@ -548,7 +554,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
           const int col = 16 * cq + 8 * b + 2 * t4;
-          const float4 v = value_of(trow[(k & 3) * kTile + c], col >> 2);
+          const float4 v = value_of(trow[(k & (kSlots - 1)) * kTile + c], col >> 2);
           const float v0 = (col & 2) ? v.z : v.x, v1 = (col & 2) ? v.w : v.y;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -563,8 +569,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       // its buffer held a code tile of pass A, whose logits are done, or nothing yet
       gather_codes(1);
     }
-    describe(0);
-    describe(1);
+    for (int k = 0; k < 3; ++k) describe(k);
     compute_sync();
     load_values(0);
     cp_async_wait_all();
@@ -575,9 +580,9 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (k + 2 < tiles && k + 2 >= ptiles) gather_codes(k + 2);
       store_values(k);
       if (k + 1 < tiles) load_values(k + 1);
-      describe(k + 2);
+      describe(k + 3);
       float e[4][8], cnt[8];
-      load_logits((k & 1) * kTile, tcnt + (k & 3) * kTile, width_of(k), e, cnt);
+      load_logits((k & 1) * kTile, tcnt + (k & (kSlots - 1)) * kTile, width_of(k), e, cnt);
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
       for (int c = 0; c < 8; ++c)

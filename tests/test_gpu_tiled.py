@@ -113,3 +113,56 @@ def test_values_that_are_not_finite_leave_the_other_dimensions_alone():
     assert np.array_equal(Y[0, 1], plain[0, 1])
     # the tile's sum in another order (float32), then one bf16 rounding: an ulp (2^-8) where a value is next to a boundary
     assert np.abs(Y[0, 0][:, rest] - plain[0, 0][:, rest]).max() <= 2 ** -8 * np.abs(plain).max()
+
+
+def _neighbouring_parents_refined(M, C, P, bq, N, seed):
+    """Half of the keys close to a parent, half to a child; queries around P parents with consecutive indices, which are then
+    the refined ones: with PARENT_STAYS their value rows (the keys that stay) fill whole groups of a tile's columns."""
+    wl = synth.Workload("neighbours", B=1, H=2, N=N, d=64, M=M, C=C, P=P, block_q=bq, seed=seed)
+    x = synth.generate(wl)
+    g = np.random.default_rng(seed)
+    for h in range(2):
+        hot = M // 4 + np.arange(N) % P
+        x["K"][0, h, ::2] = x["Cp"][h, g.permutation(hot)[::2]] + 0.05 * g.standard_normal(((N + 1) // 2, 64))
+        x["Q"][0, h] = 0.3 * x["Cp"][h, hot] + 0.3 * g.standard_normal((N, 64))
+    return wl, {k: synth.round_to_bf16(v.astype(np.float32)) for k, v in x.items()}
+
+
+@pytest.mark.parametrize("M,C,P,tile_m", [(512, 8, 64, 128), (512, 16, 48, 256), (160, 16, 100, 32), (1024, 4, 32, 128)])
+def test_keys_that_stay_under_refined_neighbours(M, C, P, tile_m):
+    """Eight and more code tiles with rows that take 1 + C loads each, in some warps and not in others; forty calls agree."""
+    wl, x = _neighbouring_parents_refined(M, C, P, 128, 700, seed=70 + M + C)
+    dv = parity.to_device(x, "bf16")
+    call = lambda: binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, 128, tile_m, scale=wl.scale,
+                                         flags=binding.FLAG_PARENT_STAYS)
+    Y, topp, imp = call()
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, 128, wl.scale, parent_stays=True, form="factorised", tile_m=tile_m)
+    assert (np.diff(ref["selected"][:, :, 0]) == 1).mean() > 0.5 and 100 < (ref["child_idx"] < 0).sum() < 1300
+    same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
+    rows = np.repeat(same, 128, axis=-1)[..., :wl.N]
+    parity.compare_output(Y.float().cpu().numpy().astype(np.float64), ref["Y"], "bf16", rows)
+    # (the value sums are added up by atomics, in any order: a last bit of float32, then at most one of bfloat16)
+    for _ in range(40):
+        Y2, topp2, imp2 = call()
+        assert torch.equal(topp, topp2) and torch.equal(imp, imp2)
+        assert (Y2.float() - Y.float()).abs().max().item() <= 2 ** -7 * Y.float().abs().max().item()
+
+
+@pytest.mark.parametrize("M,C,P", [(512, 4, 64), (1024, 8, 64)])
+def test_a_value_that_is_not_finite_in_the_first_of_many_tiles(M, C, P):
+    """The tile's product then runs on the CUDA cores, slowly, while other warps are up to a turn ahead: six and twelve code tiles,
+    so that the descriptions of the tiles are overwritten meanwhile.  The other dimensions are the oracle's."""
+    wl = synth.Workload("inf_first", B=1, H=2, N=900, d=64, M=M, C=C, P=P, block_q=128, seed=71 + M, alpha=0.8)
+    x = synth.generate(wl)
+    x["Q"] = synth.round_to_bf16(0.1 * x["Q"])                   # every key has some weight
+    dv = parity.to_device(x, "bf16")
+    first = int((binding.assign(dv["K"], dv["Cp"], dv["Cc"], flags=binding.FLAG_SIMT)[0][0, 0] < 128).nonzero()[0])
+    ref = orc.forward(x["Q"], x["K"], x["V"], x["Cp"], x["Cc"], P, 128, wl.scale, form="factorised", tile_m=128)
+    dv["V"][0, 0, first, 7] = float("inf")
+    Y, topp, imp = binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, 128, 128, scale=wl.scale)
+    same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy(), importance=imp.cpu().numpy()), ref)
+    rows = np.repeat(same, 128, axis=-1)[..., :wl.N]
+    Y = Y.float().cpu().numpy().astype(np.float64)
+    assert np.isposinf(Y[0, 0, :, 7]).all()
+    Y[0, 0, :, 7] = ref["Y"][0, 0, :, 7]
+    parity.compare_output(Y, ref["Y"], "bf16", rows)
