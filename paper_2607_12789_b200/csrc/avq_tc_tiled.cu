@@ -71,7 +71,7 @@ __host__ __device__ inline TiledSmem tiled_smem_layout(int M, int P, int tile_m)
   L.trow = take(kSlots * 4 * kTile);
   L.np = take(4 * (size_t)M);
   L.nstay = take(4 * (size_t)M);
-  L.xm = take(4 * 4 * kRows);
+  L.xm = take(2 * 4 * 4 * kRows);
   L.xz = take(4 * 4 * kRows);
   L.nseen = take(4 * (size_t)((M + tile_m - 1) / tile_m));
   L.sel = take(4 * (size_t)M);
@@ -260,12 +260,15 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
       for (int i = 0; i < 4; ++i) out[i] = __shfl_sync(0xffffffffu, v, g + 8 * i);
     };
-    auto row_max = [&](float (&m)[4]) {                    // over the quad and the four warps of a row
+    // Over the quad and the four warps of a row, through buffer `buf` of xm.  In pass C a warp may be a turn ahead of one that
+    // still reads the maxima of the turn before: the turns take the buffers alternately (through turn k - 2 all are, see describe()).
+    auto row_max = [&](float (&m)[4], int buf) {
+      float* xb = xm + buf * 4 * kRows;
 #pragma unroll
       for (int i = 0; i < 4; ++i) m[i] = quad_max(m[i]);
-      xm[cq * kRows + q * 32 + g + 8 * t4] = pick4(m, t4);
+      xb[cq * kRows + q * 32 + g + 8 * t4] = pick4(m, t4);
       rows_sync(q);
-      to_frag(fmaxf(fmaxf(xm[r], xm[kRows + r]), fmaxf(xm[2 * kRows + r], xm[3 * kRows + r])), m);
+      to_frag(fmaxf(fmaxf(xb[r], xb[kRows + r]), fmaxf(xb[2 * kRows + r], xb[3 * kRows + r])), m);
     };
     auto row_sum = [&](float (&z)[4]) {
 #pragma unroll
@@ -346,7 +349,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
             for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
         }
-        row_max(mx);
+        row_max(mx, 0);                                    // (barriers of all warps at the end of each turn)
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           if (mx[i] > m[i]) {
@@ -588,7 +591,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       for (int c = 0; c < 8; ++c)
 #pragma unroll
         for (int i = 0; i < 4; ++i) mx[i] = fmaxf(mx[i], e[i][c]);
-      row_max(mx);
+      row_max(mx, k & 1);
       float alpha[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {

@@ -166,3 +166,29 @@ def test_a_value_that_is_not_finite_in_the_first_of_many_tiles(M, C, P):
     assert np.isposinf(Y[0, 0, :, 7]).all()
     Y[0, 0, :, 7] = ref["Y"][0, 0, :, 7]
     parity.compare_output(Y, ref["Y"], "bf16", rows)
+
+
+@pytest.mark.parametrize("M,C,P,tile_m", [(1024, 8, 128, 256), (96, 16, 96, 96)])
+def test_many_tiles_in_many_blocks_come_out_the_same_every_time(M, C, P, tile_m):
+    """Sixteen and thirteen code tiles in 96 blocks, each tile's logits above those of the tile before it in half of the rows:
+    were a warp to take a maximum of another turn, its weights would be off by powers of e."""
+    wl = synth.Workload("ladder", B=2, H=3, N=2048, d=64, M=M, C=C, P=P, block_q=128, seed=72 + M, alpha=0.8)
+    x = synth.generate(wl)
+    lift = np.zeros((M, 64), dtype=np.float32)
+    lift[:, 0] = 8.0 * np.arange(M) / M
+    x["Cp"], x["Cc"] = x["Cp"] + lift, x["Cc"] + lift[:, None]
+    x["Q"][..., ::2, 0] += 6.0
+    x["Q"][..., 1::2, 0] -= 6.0
+    x = {k: synth.round_to_bf16(v) for k, v in x.items()}
+    dv = parity.to_device(x, "bf16")
+    call = lambda: binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, 128, tile_m, scale=wl.scale)
+    Y, topp, imp = call()
+    for _ in range(40):
+        Y2, topp2, imp2 = call()
+        assert torch.equal(topp, topp2) and torch.equal(imp, imp2)
+        assert (Y2.float() - Y.float()).abs().max().item() <= 2 ** -7 * Y.float().abs().max().item()
+    ref = orc.forward_head(x["Q"][1, 2], x["K"][1, 2], x["V"][1, 2], x["Cp"][2], x["Cc"][2], P, 128, wl.scale, form="factorised",
+                           tile_m=tile_m)
+    head = lambda t: t.float().cpu().numpy()[1, 2]
+    same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy()[1, 2], importance=head(imp)), ref)
+    parity.compare_output(head(Y).astype(np.float64), ref["Y"], "bf16", np.repeat(same, 128))
