@@ -376,7 +376,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           z[i] += zs[i];
-          inv[i] = z[i] != 0.f ? 1.0 / (double)z[i] : 0.0;
+          inv[i] = valid[i] && z[i] != 0.f ? 1.0 / (double)z[i] : 0.0;   // (a row of the next block may be NaN)
         }
         for (int s = subs - 1; s >= 0; --s) {              // the last code tile's weights are still there
           if (s < subs - 1) weights(s);

@@ -192,3 +192,23 @@ def test_many_tiles_in_many_blocks_come_out_the_same_every_time(M, C, P, tile_m)
     head = lambda t: t.float().cpu().numpy()[1, 2]
     same, _ = parity.compare_selection(dict(selected=topp.cpu().numpy()[1, 2], importance=head(imp)), ref)
     parity.compare_output(head(Y).astype(np.float64), ref["Y"], "bf16", np.repeat(same, 128))
+
+
+@pytest.mark.parametrize("bq,P,bad", [(64, 32, float("nan")), (100, 32, float("inf")), (50, 0, float("nan"))])
+def test_a_query_that_is_not_finite_spoils_no_other_block(bq, P, bad):
+    """Blocks of fewer than 128 queries: the tile's further rows hold the next block's queries, which must not count here."""
+    wl = synth.Workload("bad_query", B=1, H=2, N=400, d=64, M=256, C=4, P=P, block_q=bq, seed=73 + bq, alpha=0.5)
+    x = synth.generate(wl)
+    run = lambda q: binding.forward_tiled(q, *(dv[k] for k in ("K", "V", "Cp", "Cc")), P, bq, 128, scale=wl.scale)
+    dv = parity.to_device(x, "bf16")
+    Y0, topp0, imp0 = run(dv["Q"])
+    Q = dv["Q"].clone()
+    Q[0, 0, bq + 3] = bad                                        # in block 1 of head 0 only
+    Y, topp, imp = run(Q)
+    assert not torch.isfinite(Y[0, 0, bq + 3]).any()
+    keep = torch.ones(1, 2, imp.shape[2], dtype=torch.bool, device="cuda")
+    keep[0, 0, 1] = False
+    assert torch.equal(imp[keep], imp0[keep]) and torch.equal(topp[keep], topp0[keep])
+    rows = keep.repeat_interleave(bq, dim=-1)[..., :400]
+    # (value sums added up in any order: at most an ulp of bfloat16)
+    assert (Y.float() - Y0.float())[rows].abs().max().item() <= 2 ** -7 * Y0.float().abs().max().item()
