@@ -274,7 +274,8 @@ def forward_permuted(Q, K, V, Cp, Cc, P: int, block_q: int, perm, scale=None, fl
 
 
 def forward_tiled(Q, K, V, Cp, Cc, P: int, block_q: int, tile_m: int, scale=None, flags: int = 0):
-    """avq_forward_tiled: selection from the tiled importance.  Returns (Y, topp, importance)."""
+    """avq_forward_tiled: selection from the tiled importance (FLAG_SIMT: CUDA-core kernels throughout).
+    Returns (Y, topp, importance)."""
     _chk(Q, K, V, Cp, Cc)
     prob = _problem_from(Q, K, Cp, Cc, scale, flags | FLAG_SIMT)
     B, H, Nq, d = Q.shape
@@ -283,6 +284,7 @@ def forward_tiled(Q, K, V, Cp, Cc, P: int, block_q: int, tile_m: int, scale=None
     if nbytes == 0:
         raise AvqError(lib().avq_workspace_layout(ctypes.byref(prob), P, block_q, None, None, None, None, None, None)
                        or 3, "avq_workspace_bytes")
+    prob.flags = flags                     # (FLAG_SIMT above sizes the workspace)
     ws = torch.empty(nbytes, dtype=torch.uint8, device=Q.device)
     Y = torch.empty_like(Q)
     topp = torch.empty((B, H, nblk, P), dtype=torch.int32, device=Q.device)

@@ -232,7 +232,7 @@ avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void*
                              size_t workspace_bytes, void* stream) {
   if (!prob) return AVQ_ERR_NULL;
   avq_problem p = *prob;
-  p.flags |= AVQ_FLAG_SIMT;                        // the tiled importance lives in the CUDA-core attention kernel
+  p.flags |= AVQ_FLAG_SIMT;                        // envelope, workspace and the stages before are those of the CUDA cores
   avq_status s = validate_forward(&p, P, block_q);
   if (s != AVQ_OK) return s;
   if (tile_m < 32 || tile_m % 32 != 0) return AVQ_ERR_SHAPE;
@@ -250,7 +250,7 @@ avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void*
   if (s != AVQ_OK) return s;
   s = simt_aggregate(p, V, r.pidx, r.cidx, r.Vp, r.np_, r.Vc, r.nc, true, r.status_word, st);
   if (s != AVQ_OK) return s;
-  if (tc_tiled_fits(p, P, block_q, tile_m))
+  if (!(prob->flags & AVQ_FLAG_SIMT) && tc_tiled_fits(p, P, block_q, tile_m))   // the caller's flag asks for the CUDA cores throughout
     return tc_attend_tiled(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, r.status_word, st);
   return simt_attend(p, Q, Cp, Cc, r.Vp, r.np_, r.Vc, r.nc, P, block_q, Y, topp_out, importance_out, tile_m, true, st);
 }

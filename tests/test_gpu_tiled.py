@@ -212,3 +212,20 @@ def test_a_query_that_is_not_finite_spoils_no_other_block(bq, P, bad):
     rows = keep.repeat_interleave(bq, dim=-1)[..., :400]
     # (value sums added up in any order: at most an ulp of bfloat16)
     assert (Y.float() - Y0.float())[rows].abs().max().item() <= 2 ** -7 * Y0.float().abs().max().item()
+
+
+@pytest.mark.parametrize("M,C,P,bq,tile_m,flags", [(768, 8, 64, 128, 128, 0), (544, 3, 50, 100, 160, 0),
+                                                   (768, 8, 64, 128, 256, binding.FLAG_PARENT_STAYS)])
+def test_the_cuda_core_flag_selects_the_cuda_core_kernel_and_both_agree(M, C, P, bq, tile_m, flags):
+    wl = synth.Workload("both", B=1, H=2, N=1000, d=64, M=M, C=C, P=P, block_q=bq, seed=74 + M, alpha=0.8, hot_queries=True)
+    dv = parity.to_device(synth.generate(wl), "bf16")
+    call = lambda f: binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, bq, tile_m, scale=wl.scale, flags=flags | f)
+    Y, topp, imp = call(0)
+    Y1, topp1, imp1 = call(binding.FLAG_SIMT)
+    # importances added up in another order: float32's last bits differ somewhere, and no more than those of some thousand terms
+    assert not torch.equal(imp, imp1) and torch.allclose(imp, imp1, rtol=2e-4, atol=1e-5)
+    same = (topp == topp1).all(-1)
+    assert same.float().mean().item() > 0.9                      # (a near-tie may fall either way)
+    rows = same.repeat_interleave(bq, dim=-1)[..., :wl.N]
+    # one bfloat16 rounding each: an ulp where float32 results fall on either side of a boundary
+    assert ((Y.float() - Y1.float()).abs()[rows] <= 2 ** -7 * Y1.float().abs()[rows] + 1e-5).all()
