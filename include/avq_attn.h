@@ -182,8 +182,8 @@ AVQ_API avq_status avq_forward_permuted(const avq_problem* prob, const void* Q, 
  * and the P parents with the largest w are refined.  The output is the exact refined attention for that
  * selection; only the selection (and importance_out) differs from avq_forward.  tile_m: a multiple of 32;
  * tile_m >= M reproduces avq_forward.  Runs the CUDA-core kernels for either dtype (M up to 1024), bfloat16 with d = 64,
- * block_q <= 128 and tile_m <= 256 the tensor cores in the attention pass, to the same precision, unless
- * AVQ_FLAG_SIMT asks for the CUDA cores there too.  The workspace is that of avq_forward for the same
+ * block_q <= 128 and tile_m <= 256 the tensor cores in the attention pass, to the same precision, where codebook
+ * and blocks are large enough for that to pay and unless AVQ_FLAG_SIMT asks for the CUDA cores there too.  The workspace is that of avq_forward for the same
  * problem with AVQ_FLAG_SIMT set. */
 AVQ_API avq_status avq_forward_tiled(const avq_problem* prob, const void* Q, const void* K, const void* V,
                              const void* Cp, const void* Cc, int32_t P, int32_t block_q, int32_t tile_m,

@@ -656,11 +656,25 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   if (warp == kIssuer) tmem_dealloc(tmem_base, 512);
 }
 
+// A block costs this kernel a tile of 128 rows and tiles of 128 codewords whatever it has of them, on an SM of its own; the CUDA-core
+// kernel takes 64 of each at a time, two blocks to an SM.  So small blocks and small codebooks stay there.  Us per call here
+// and there, H4 N4096 and H12 N8192, C4, importance tiles of min(M, 128) unless said otherwise:
+//   128 rows  M64 P8 39.0 and 39.0, 117.7 and 112.0 (H16 N4096); tiles of 32 0.91 and 0.93 times the other's time
+//             M64 P16 0.99 and 1.00 times; M80 P4 0.91 and 0.82 times; M128 P16 0.80 and 0.73 times
+//   64 rows   M64 P8 55.9 and 43.1; M128 P16 1.03 and 1.01 times; M160 P16 1.09 and 1.08 times, M200 P10 0.87 and 0.85
+//             (tiles of 32: 1.03 and 1.02) times; M128 P28 0.92 and 0.91 times; M256 P64 0.70 and 0.69 times
+//   16 rows   M64 P8 144.0 and 99.0; M160 P16 1.09 and 1.10 times, M200 P10 0.83 and 0.83 times, M512 P64 0.61 times
+bool tc_tiled_pays(const avq_problem& p, int32_t P, int32_t block_q, int32_t tile_m) {
+  const int64_t columns = (int64_t)p.M + (int64_t)P * p.C;
+  if (block_q <= 64) return columns >= 240;
+  return p.M > (tile_m < 64 ? tile_m : 64) || columns >= 128;
+}
+
 }  // namespace
 
 bool tc_tiled_fits(const avq_problem& p, int32_t P, int32_t block_q, int32_t tile_m) {
   return p.dtype == AVQ_BF16 && p.d == kD && block_q <= kRows && tile_m <= 2 * kTile && !(p.flags & AVQ_FLAG_CORRECTING) &&
-         tiled_smem_layout(p.M, P, tile_m).total <= kSmemMax;
+         tiled_smem_layout(p.M, P, tile_m).total <= kSmemMax && tc_tiled_pays(p, P, block_q, tile_m);
 }
 
 avq_status tc_attend_tiled(const avq_problem& p, const void* Q, const void* Cp, const void* Cc, const float* Vp, const float* np_,

@@ -229,3 +229,19 @@ def test_the_cuda_core_flag_selects_the_cuda_core_kernel_and_both_agree(M, C, P,
     rows = same.repeat_interleave(bq, dim=-1)[..., :wl.N]
     # one bfloat16 rounding each: an ulp where float32 results fall on either side of a boundary
     assert ((Y.float() - Y1.float()).abs()[rows] <= 2 ** -7 * Y1.float().abs()[rows] + 1e-5).all()
+
+
+@pytest.mark.parametrize("M,C,P,bq,tile_m,tensor", [(64, 4, 8, 128, 64, False), (64, 4, 8, 128, 32, True), (64, 4, 16, 65, 64, True),
+                                                    (63, 4, 16, 128, 256, False), (65, 1, 0, 128, 128, True), (32, 3, 20, 100, 32, False),
+                                                    (33, 1, 2, 100, 32, True), (160, 4, 19, 64, 128, False), (160, 4, 20, 64, 128, True),
+                                                    (64, 4, 8, 16, 32, False), (512, 4, 64, 16, 128, True)])
+def test_small_codebooks_and_blocks_stay_on_the_cuda_cores(M, C, P, bq, tile_m, tensor):
+    """Where the tensor-core kernel takes longer (up to 1.5 times at 64 parents and blocks of 8 to 64 queries) it is not used: the
+    importances then are those of the CUDA-core kernel bit for bit; elsewhere some last bit differs."""
+    wl = synth.Workload("rule", B=1, H=4, N=500, d=64, M=M, C=C, P=P, block_q=bq, seed=75 + M, alpha=0.8, hot_queries=True)
+    dv = parity.to_device(synth.generate(wl), "bf16")
+    call = lambda f: binding.forward_tiled(dv["Q"], dv["K"], dv["V"], dv["Cp"], dv["Cc"], P, bq, tile_m, scale=wl.scale, flags=f)
+    (Y, _, imp), (Y1, _, imp1) = call(0), call(binding.FLAG_SIMT)
+    assert torch.equal(imp, imp1) == (not tensor)
+    assert torch.allclose(imp, imp1, rtol=2e-4, atol=1e-5)
+    assert ((Y.float() - Y1.float()).abs() <= 2 ** -7 * Y1.float().abs() + 1e-5).float().mean().item() > 0.98   # (near-tied selections)
