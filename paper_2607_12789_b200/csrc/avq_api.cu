@@ -191,7 +191,10 @@ avq_status forward_core(const avq_problem& p, const void* Q, const void* K, cons
     // 97.5, 1536 256.8 and 253.4; d128 M96 C8 1536 tiles 200.1 and 201.6.  A 4 KB codebook is too small for it (B8 H12
     // N10167 d64 M32 C8: 270 and 276), and so are keys that do not outnumber the codewords of a head (its batch together)
     // four to one: H96 N1024, ratio 0.9: d128 M128 C8 121.5 and 126.3; 1.8: d64 M64 C8 50.5 and 52.5; 3.2: d64 M64 C4
-    // 44.2 and 44.4; ratio 14: H16 N16384 d64 M128 C8 128.7 and 126.9.
+    // 44.2 and 44.4; ratio 14: H16 N16384 d64 M128 C8 128.7 and 126.9.  The figures of eight children are those of the loop over a
+    // key's children; by products over sorted keys, which larger grids take, the table pays as it does there: H16 N20000 d64
+    // M64 C8 105.5 and 104.5, d128 M64 158.6 and 155.9, M128 232.5 and 229.7, M256 293.6 and 292.0; PARENT_STAYS H16 N12000
+    // d64 M128 C8 115.5 and 112.3, d128 M128 C4 160.6 and 158.8.
     const bool norms_pass = (size_t)p.M * p.d >= 4096 && (size_t)p.B * p.H * ((p.Nk + 127) / 128) >= 592 &&
                             (size_t)p.B * p.Nk >= 4 * (size_t)p.M * (1 + p.C);
     s = tc_assign(p, K, Cp, Cc, r.pidx, r.cidx, r.status_word, workspace, L.zero_end, norms_pass ? r.cnorm : nullptr, perm != nullptr, st);

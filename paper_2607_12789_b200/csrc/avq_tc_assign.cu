@@ -805,7 +805,10 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   // every key moves, for eight children and grids that hide the sort: d128 H16 N20000 M32 167.7 and 142.6, M64 179.5 and
   // 157.8, M128 247.5 and 234.7, M256 303.4 and 299.4; 288 tiles M64 34.4 and 33.3, M256 56.2 and 53.9, but 48 tiles M64 23.3
   // and 24.0; d64 H16 N20000 M32 92.0 and 85.1, M64 111.3 and 105.4, M128 144.9 and 142.6, M256 224.0 and 224.8; 288 tiles M64
-  // 25.7 and 26.5.  With four children the two about cancel or products lose: d64 H16 N20000 M64 96.5 and 97.9, M256 204.5
+  // 25.7 and 26.5.  Those keys crowd around few parents; where every parent has as many, a warp's 16 keys have more parents and
+  // the products gain less: with the norm table H16 N20000 d64 M64 112.4 and 108.6, M128 140.1 and 143.8, d128 M128 246.5 and
+  // 245.2; without it, this kernel alone, d64 M64 45.6 and 45.5, M96 48.6 and 52.0, M128 50.3 and 56.4 (crowded keys 49.6 and
+  // 49.6), d128 M128 90.6 and 92.7 (91.8 and 82.0).  So at d64 not above 64 parents without the table.  With four children the two about cancel or products lose: d64 H16 N20000 M64 96.5 and 97.9, M256 204.5
   // and 211.5; d128 M128 215.0 and 214.5, M256 256.8 and 259.8.
   constexpr bool kSortedAtAll = STAYS || NL * 256 / D == 8;
   const int nblk = (p.Nk + kKeys - 1) / kKeys;
@@ -813,7 +816,7 @@ avq_status launch(const avq_problem& p, const void* K, const void* Cp, const voi
   const int total = (int)(nblk * BH);
   const int sms = sm_count();
   if (sms <= 0) return AVQ_ERR_CUDA;
-  const bool sorted = STAYS || (kSortedAtAll && (D == 128 ? 2 * total >= 3 * sms : total >= 4 * sms && p.M <= 128));
+  const bool sorted = STAYS || (kSortedAtAll && (D == 128 ? 2 * total >= 3 * sms : total >= 4 * sms && p.M <= (cnorm ? 128 : 64)));
   const size_t smem = (size_t)(D / 64) * (kKeys + p.M) * 128 + sizeof(float) * (p.M + 6 * kKeys) + sizeof(int) * (2 * kKeys + (sorted ? p.M + kKeys / 4 : 0)) + 96;
   const int resident = (int)min((size_t)assign_min_ctas(D), kSmemMax / (smem + 1024));   // CTAs on an SM
   // A wave of CTAs with runs of tiles, the codebook and its norms staying in shared memory, for the largest codebook

@@ -405,7 +405,8 @@ def test_indices_by_the_norm_table_equal_those_of_the_direct_form(B, H, N, d, M,
         assert torch.equal(inter["parent_idx"], pi) and torch.equal(inter["child_idx"], ci)
 
 
-@pytest.mark.parametrize("H,N,d,M", [(24, 1200, 128, 32), (10, 3000, 128, 256), (37, 2001, 64, 96)])
+@pytest.mark.parametrize("H,N,d,M", [(24, 1200, 128, 32), (10, 3000, 128, 256), (37, 2001, 64, 96),
+                                     (37, 2001, 64, 64)])
 def test_eight_children_over_sorted_keys_equal_the_cuda_core_assignment(H, N, d, M):
     """Large grids take eight children by products over keys in the order of their parents: the indices of the CUDA-core
     kernel, which measures every child directly, also with near-ties (an offset) and duplicated children."""
@@ -439,3 +440,40 @@ def test_a_common_offset_costs_little_time():
     centred, shifted = us(0.0), us(64.0)
     print(f"centred {centred:.1f} us, shifted {shifted:.1f} us")
     assert shifted <= 1.6 * centred
+
+
+def test_assignment_takes_no_longer_where_every_parent_has_as_many_keys():
+    """d = 64, 128 parents of eight children: products over keys in the order of their parents cost 1.5 times as much where the keys
+    spread over all parents as where a sixteenth of the parents has all of them (56.5 and 37.4 us); the loop over a key's
+    children 1.05 times (50.3 and 47.9)."""
+    H, N, M, C = 16, 20000, 128, 8
+    _, Cp, Cc = _offset_inputs(1, H, 1, 64, M, C, 0.0, seed=4, twice=False)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+
+    def keys(parents):
+        at = torch.randint(0, parents * C, (H, N, 1), device="cuda", generator=g).expand(H, N, 64)
+        near = Cc.float().view(H, M * C, 64).gather(1, at) + 0.3 * torch.randn(H, N, 64, device="cuda", generator=g)
+        return near.to(torch.bfloat16)[None].contiguous()
+
+    def us(K):
+        prob = binding.problem(1, H, N, N, 64, M, C, binding.AVQ_BF16, 1.0)
+        pi, ci = torch.empty(2, 1, H, N, dtype=torch.int32, device="cuda")
+        call = lambda: binding.lib().avq_assign(prob, K.data_ptr(), Cp.data_ptr(), Cc.data_ptr(), pi.data_ptr(), ci.data_ptr(),
+                                                binding._raw_stream())
+        for _ in range(10):
+            assert call() == 0
+        times = []
+        for _ in range(30):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 1e2)
+        return sorted(times)[len(times) // 2]
+
+    spread, few = us(keys(M)), us(keys(M // 16))
+    print(f"spread {spread:.1f} us, crowded {few:.1f} us")
+    assert spread <= 1.2 * few
