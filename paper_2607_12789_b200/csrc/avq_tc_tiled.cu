@@ -8,15 +8,21 @@
 // issues the TMA loads and every tcgen05.mma, so that none of the others waits for the tensor pipe.
 //   logits   S = Q . C^T, one tcgen05.mma chain per tile; parents' codes by TMA, children's by cp.async gathers, two buffers
 //   pass A   per importance tile: maximum, denominator, float64 column sums (importance)
-//   pass C   weights and value sums enter the value product as three bfloat16 parts each.  Truncation splits a float32 exactly
-//            (8 + 8 + 8 significant bits); of the nine products the six above 2^-24 are added, the smallest first.  A tile's product
-//            starts from zero and is added to float32 registers while the next tile's weights are computed.
+//   pass C   weights and value sums enter the value product as three bfloat16 parts each, rounded to nearest, which hold a
+//            float32 exactly (below 2^-110, to 2^-134).  Second and third part are at most 2^-8 and 2^-17 of it.  Of the nine products
+//            six are added, the smallest first; the others are at most 2^-24 of the term together, what a float32 multiply-add
+//            rounds off.  A tile's product starts from zero and is added to float32 registers while the next tile's weights
+//            are computed.
+//            Relative error of the float32 output (before its rounding to bfloat16) against 64 bits, CUDA-core kernel and here: M512
+//            to M1024 P32 to P64, queries N(0, 1) 4.2e-7 to 4.8e-7 and 3.7e-7 to 4.0e-7, around a few parents 4.2e-7 to 6.7e-7
+//            for both; P0 and peaked weights, sums of one or two terms, 1.6e-7 and 1.7e-7.  (Parts cut off instead of
+//            rounded left out up to 2^-21 of a term.  Adding the two products of 2^-25 too changed nothing and took 1 us.)
 // Bound by the phases of a tile one after the other (exponentials 2000 to 3300 cycles per code tile, splits 1300, column sums
 // 2100), with 128 blocks on as many SMs.  B1 H4 N4096 M512 C4 P64, importance tiles of 128, both cold: 167 us in the CUDA-core
 // kernel (whose value product alone takes 55 at the float32 rate), 66 here.  A dedicated issuing warp: the 48 instructions
 // of a tile's value product hold their issuer up for 2000 to 3000 cycles.
-// A tile with an infinite or NaN value sum takes its product on the CUDA cores (an infinity times a part that happens to be
-// zero would be NaN).
+// A tile with a value sum that is infinite, NaN or beyond bfloat16's largest takes its product on the CUDA cores (an infinity
+// times a part that happens to be zero would be NaN).
 #include <math.h>
 
 #include "avq_internal.h"
@@ -40,6 +46,7 @@ constexpr int kSlots = 8;                      // tiles described at a time (the
 constexpr int kStayRow = 1 << 28, kChildRow = 1 << 29;
 // TMEM columns: two logit tiles, three weight parts, the value product
 constexpr int kColW = 256, kColO = 448;
+constexpr float kLargestBf16 = 3.38953139e38f; // 0x7F7F0000
 constexpr float kLowest = -3.402823466e38f;    // a running maximum starts at the lowest finite value (weights of -inf logits are then 0)
 
 struct TiledArgs {
@@ -89,14 +96,18 @@ __device__ __forceinline__ void ready_arrive() { asm volatile("bar.arrive 8, %0;
 __device__ __forceinline__ void ready_wait() { asm volatile("bar.sync 8, %0;" ::"n"(kThreadsT) : "memory"); }
 __device__ __forceinline__ void rows_sync(int q) { asm volatile("bar.sync %0, 128;" ::"r"(q + 1) : "memory"); }
 
-// x = sum of three bfloat16 (the upper halves of the results), exactly
-__device__ __forceinline__ void split3(float x, uint32_t (&p)[3]) {
-  p[0] = __float_as_uint(x);
-  const float r = x - __uint_as_float(p[0] & 0xFFFF0000u);
-  p[1] = __float_as_uint(r);
-  p[2] = __float_as_uint(r - __uint_as_float(p[1] & 0xFFFF0000u));
+// Two float32 as three pairs of bfloat16 (low half: lo) that add up to them exactly: each rounds to nearest what the ones before
+// leave over, which has at most 16 and 7 significant bits.
+__device__ __forceinline__ void split3(float lo, float hi, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[j]) : "f"(hi), "f"(lo));
+    if (j < 2) {
+      lo -= __uint_as_float(p[j] << 16);
+      hi -= __uint_as_float(p[j] & 0xFFFF0000u);
+    }
+  }
 }
-__device__ __forceinline__ uint32_t upper_halves(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
 
 __global__ void __launch_bounds__(kThreadsT, 1)
 attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmCp, const TiledArgs a) {
@@ -110,7 +121,7 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   float *xz = reinterpret_cast<float*>(smem + L.xz), *nseen = reinterpret_cast<float*>(smem + L.nseen);
   int *trow = reinterpret_cast<int*>(smem + L.trow), *sel = reinterpret_cast<int*>(smem + L.sel), *sel_list = reinterpret_cast<int*>(smem + L.list);
   int *s_count = reinterpret_cast<int*>(smem + L.count);
-  volatile int* bad = reinterpret_cast<volatile int*>(smem + L.bad);   // [tile] it holds a value sum that is not finite
+  volatile int* bad = reinterpret_cast<volatile int*>(smem + L.bad);   // [tile] it holds a value sum that bfloat16 does not reach
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
   uint64_t *bar_q = bars, *bar_c = bars + 1, *bar_s = bars + 3, *bar_o = bars + 5;   // query tile, codes [2], logits [2], product
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
@@ -485,24 +496,22 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       }
     };
     auto store_values = [&](int k) {
-      bool finite = true;
+      bool fits = true;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         float x[4];
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(own_v + 16 * kCompute * i) : "memory");
-        uint32_t p[4][3];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          finite = finite && fabsf(x[e]) <= 3.402823466e38f;
-          split3(x[e], p[e]);
-        }
+        for (int e = 0; e < 4; ++e) fits = fits && fabsf(x[e]) <= kLargestBf16;
+        uint32_t p[2][3];
+        split3(x[0], x[1], p[0]);
+        split3(x[2], x[3], p[1]);
         const uint32_t at = smem_u32(Vs + (k & 1) * 3 * kTileBytes) + sw128_offset((tid >> 4) + 32 * i, 4 * (tid & 15));
 #pragma unroll
         for (int j = 0; j < 3; ++j)
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + j * kTileBytes), "r"(upper_halves(p[0][j], p[1][j])),
-                       "r"(upper_halves(p[2][j], p[3][j])) : "memory");
+          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + j * kTileBytes), "r"(p[0][j]), "r"(p[1][j]) : "memory");
       }
-      if (!finite) bad[k] = 1;
+      if (!fits) bad[k] = 1;
     };
     auto gather_codes = [&](int k) {                       // children's codeword rows of tile k, zeros behind them
       const int n = width_of(k), n16 = (n + 15) & ~15;
@@ -618,11 +627,10 @@ attend_tiled_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         for (int b = 0; b < 4; ++b)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            uint32_t lo[3], hi[3];
-            split3(e[i][2 * b], lo);
-            split3(e[i][2 * b + 1], hi);
+            uint32_t p[3];
+            split3(e[i][2 * b], e[i][2 * b + 1], p);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) part[j][i >> 1][2 * b + (i & 1)] = upper_halves(lo[j], hi[j]);
+            for (int j = 0; j < 3; ++j) part[j][i >> 1][2 * b + (i & 1)] = p[j];
           }
 #pragma unroll
         for (int j = 0; j < 3; ++j) tmem_st_weights(t_row + kColW + j * (kTile / 2) + 16 * cq, part[j]);

@@ -245,3 +245,59 @@ def test_small_codebooks_and_blocks_stay_on_the_cuda_cores(M, C, P, bq, tile_m, 
     assert torch.equal(imp, imp1) == (not tensor)
     assert torch.allclose(imp, imp1, rtol=2e-4, atol=1e-5)
     assert ((Y.float() - Y1.float()).abs() <= 2 ** -7 * Y1.float().abs() + 1e-5).float().mean().item() > 0.98   # (near-tied selections)
+
+
+def test_the_value_product_rounds_like_float32_multiply_adds():
+    """Three parents with the same weight w and value sums a, b and -(a + b) of 24 significant bits: the output is what the value
+    product rounds off.  Three float32 multiply-adds leave 0.36 2^-24 w (root mean square, on these numbers), products of
+    bfloat16 parts 0.46 where the parts are cut off and 0.10 where they are rounded to nearest."""
+    g = np.random.default_rng(76)
+    M, N, d = 128, 128, 64
+    rng = lambda n: g.integers(2 ** 23, 2 ** 24, n)
+    a = rng(d) * 2.0 ** -25                                      # in [1/4, 1/2), multiples of 2^-25
+    b = (rng(d) // 2 * 2 * 2.0 ** -25) + (a * 2.0 ** 25 % 2) * 2.0 ** -25   # a + b: a multiple of 2^-24
+    x = np.stack([np.zeros(d), a, b, -(a + b)])
+    assert (x.astype(np.float32) == x).all()
+    parts, rest = [], x.copy()                                   # each as the sum of three bfloat16: the values of three keys
+    for _ in range(3):
+        p = synth.round_to_bf16(rest.astype(np.float32)).astype(np.float64)
+        parts.append(p)
+        rest = rest - p
+    assert (rest == 0).all()
+    Cp = np.zeros((M, d))
+    Cp[:, 1] = np.arange(M) * 4.0 + 100.0                        # far away and without keys
+    for j in range(4):
+        Cp[j] = 0.0
+        Cp[j, 2 + j] = 8.0                                       # (queries are zero there)
+    Cp[0, 0] = 2.0
+    Cp[1:4, 0] = 1.0
+    K = np.repeat(Cp[:4], 3, axis=0)
+    V = np.stack([parts[i][j] for j in range(4) for i in range(3)])
+    Q = np.zeros((N, d))
+    Q[:, 0] = 8.0 * (0.05 + 3.0 * g.random(N))
+    t = lambda v: torch.from_numpy(np.ascontiguousarray(v[None])).float().cuda().to(torch.bfloat16)
+    Q, K, V, Cp_ = t(Q[None]), t(K[None]), t(V[None]), t(Cp)
+    Y, _, _ = binding.forward_tiled(Q, K, V, Cp_, Cp_[:, :, None].contiguous(), 0, 128, 128, scale=0.125)
+    w = np.exp(-Q[0, 0, :, 0].double().cpu().numpy() / 8)
+    left = Y[0, 0].double().cpu().numpy() * ((3 + 9 * w) / w)[:, None]      # times the denominator, over the weight
+    rms = np.sqrt((left ** 2).mean()) * 2.0 ** 24
+    print(f"rms {rms:.2f} 2^-24")
+    assert 0 < rms <= 0.36
+
+
+def test_value_sums_beyond_the_largest_bfloat16():
+    """A finite float32 sum that rounds to infinity as a bfloat16 is not split: the output stays finite."""
+    wl = synth.Workload("large", B=1, H=1, N=256, d=64, M=256, C=4, P=0, block_q=128, seed=77, alpha=0.5)
+    x = synth.generate(wl)
+    x["Q"] = synth.round_to_bf16(0.1 * x["Q"])
+    dv = parity.to_device(x, "bf16")
+    par = binding.assign(dv["K"], dv["Cp"], dv["Cc"], flags=binding.FLAG_SIMT)[0][0, 0]
+    two = (par == par[0]).nonzero().flatten()[:2].tolist()
+    assert len(two) == 2
+    dv["V"][0, 0, :, 7] = 0.0
+    dv["V"][0, 0, two[0], 7], dv["V"][0, 0, two[1], 7] = 3.3895e38, 1.2e36   # the largest bfloat16, and less than half a step
+    call = lambda f: binding.forward_tiled(*(dv[k] for k in ("Q", "K", "V", "Cp", "Cc")), 0, 128, 128, scale=wl.scale, flags=f)[0]
+    Y, Y1 = call(0).float(), call(binding.FLAG_SIMT).float()
+    assert torch.isfinite(Y).all() and (Y[..., 7] > 1e34).all()
+    # one bfloat16 rounding each
+    assert ((Y - Y1).abs() <= 2 ** -7 * Y1.abs() + 1e-5).all()
