@@ -153,23 +153,6 @@ __device__ double exact_dist(const T* krow, const T* c, int d) {
   return s;
 }
 
-// The same asynchronously (cp.async; the caller waits), each row in pieces of 16 bytes (8 where d is no multiple of 8).
-template <int THREADS, int PIECE, typename Src>
-__device__ __forceinline__ void load_rows_async(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
-  const int per = dpad / PIECE, step_r = THREADS / per, step_c = THREADS - step_r * per;
-  int r = threadIdx.x / per, c = threadIdx.x - r * per;
-  for (; r < rows; r += step_r, c += step_c) {
-    if (c >= per) { c -= per; if (++r >= rows) break; }
-    const __nv_bfloat16* p = src(r);
-    const bool there = p != nullptr && PIECE * c < d;
-    const uint32_t to = tc::smem_u32(dst + r * pitch + PIECE * c);
-    const __nv_bfloat16* from = there ? p + PIECE * c : src(0);
-    if constexpr (PIECE == 8)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
-    else
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(to), "l"(from), "r"(there ? 8 : 0) : "memory");
-  }
-}
 // `rows` rows of d bfloat16 (row r at src(r), nullptr = zeros) into dst[r][k], k < dpad, zeros from d on.
 template <int THREADS, typename Src>
 __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
@@ -190,6 +173,23 @@ __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, int pitch, int row
 #pragma unroll
     for (int e = 0; e < 2; ++e)
       if (at[e] >= 0) *reinterpret_cast<uint2*>(dst + at[e]) = v[e];
+  }
+}
+// The same asynchronously (cp.async; the caller waits), each row in pieces of 16 bytes (8 where d is no multiple of 8).
+template <int THREADS, int PIECE, typename Src>
+__device__ __forceinline__ void load_rows_async(__nv_bfloat16* dst, int pitch, int rows, int d, int dpad, Src src) {
+  const int per = dpad / PIECE, step_r = THREADS / per, step_c = THREADS - step_r * per;
+  int r = threadIdx.x / per, c = threadIdx.x - r * per;
+  for (; r < rows; r += step_r, c += step_c) {
+    if (c >= per) { c -= per; if (++r >= rows) break; }
+    const __nv_bfloat16* p = src(r);
+    const bool there = p != nullptr && PIECE * c < d;
+    const uint32_t to = tc::smem_u32(dst + r * pitch + PIECE * c);
+    const __nv_bfloat16* from = there ? p + PIECE * c : src(0);
+    if constexpr (PIECE == 8)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(there ? 16 : 0) : "memory");
+    else
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(to), "l"(from), "r"(there ? 8 : 0) : "memory");
   }
 }
 __device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p) {

@@ -15,8 +15,9 @@
 //            the direct form throughout, near-ties in float64.
 //            Four lanes per key, each over a quarter of the head dimension for all C children of the
 //            key's parent (one running sum per child); a transposing butterfly merges the four lanes.
-// Bound by L1 and shared memory (58 to 73 % busy) and the latency of the child loads; L2 is at 12 to 19 %, issue slots at 40
-// to 48 %.
+// Bound, with the loop over a key's children, by L1 and shared memory (56 to 69 % busy) and the latency of the child loads, issue
+// slots at 39 to 59 %; with products over sorted keys by latency, the barriers around the sort first (2.7 to 3.5 warps wait at one
+// per instruction issued), L1 at 39 to 50 %, issue slots at 29 to 52 %.  L2 is at 9 to 19 %.
 #include <type_traits>
 
 #include "avq_tc_common.cuh"
@@ -577,7 +578,9 @@ tc_assign_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       // product adds 16 exact products to the sum and rounds each of the 17 terms by at most 2^-24 of the largest of them and
       // of the sum: D / 16 steps are off by at most 17 D / 16 2^-24 |k||c|, the norm (chains of at most D / 4 and three
       // additions) by (D/4 + 3) 2^-24 |c|^2, so a distance by less than 1.05e-5 (|k|^2 + |c|^2) at D = 128 and two of them by
-      // less than 2.1e-5 (|k|^2 + max |c|^2).
+      // less than 2.1e-5 (|k|^2 + max |c|^2).  A parent's norm is one chain of D where there is no table, off by 7.7e-6 |c|^2:
+      // its distance and a child's together by less than 3.3e-5 |k| |c| + 1.0e-5 |c|^2 with the larger |c|, which is
+      // below 2.5e-5 (|k|^2 + |c|^2) for every |k| and |c| (2.5 k^2 - 3.3 k c + 1.5 c^2 has no zero).
       float cmx = mine[i] ? fmaxf(nrm[i][0], nrm[i][1]) : 0.f;
       cmx = quad_max(cmx);
       if (STAYS) cmx = fmaxf(cmx, cnorm[own[i]]);

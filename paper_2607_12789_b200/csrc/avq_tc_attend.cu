@@ -178,6 +178,8 @@ tc_attend_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* zchain = reinterpret_cast<float*>(tmem_slot + 2);   // [NQ / 2][4][128] kChain
+  // it is read in pieces of 16 bytes: the words in front of it, apart from the M C (M is a multiple of 32)
+  static_assert(L::oF % 16 == 0 && (11 * CT + CHW + 2 * NQ * kRows + 32 + 8 + 8 + 2 + 2 * 6 + 2) % 4 == 0, "zchain is aligned");
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
